@@ -10,15 +10,19 @@
 //        matrix of Lindholm's closed-form weights for linear densities,
 //   u2 harmonic inside (Dirichlet problem),
 //   H = -grad(u1 + u2) per tet, lumped to the nodes.
-// The map M -> H is applied to all 3n unit vectors at once: the Poisson
-// problems are solved by Jacobi-preconditioned CG batched over the 3n
-// right-hand sides (row-major [n][3n] blocks, one thread per entry, per-column
-// reductions in a fixed order so that results are bit-reproducible).
+// The map M -> H is formed as a matrix.  Its source div(M) and its gradient are
+// sparse, so the solves are done for the n nodal sources rather than for the
+// 3n magnetisation components: G = K^+ (Neumann), the harmonic extension E of
+// the boundary values (Dirichlet), Q = G + E (D + diag(..)) G_boundary, and
+// N = P Q R with the sparse R (source) and P (projected gradient).  Both solves
+// run as Jacobi-preconditioned CG over row-major blocks of right-hand sides: a
+// CTA owns one or two columns and runs their iterations in shared memory, with
+// reductions in a fixed order so that results are bit-reproducible.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
-#include <map>
-#include <array>
 
 #include "bpm_internal.cuh"
 
@@ -26,8 +30,11 @@ namespace bpm {
 
 namespace {
 
+// buffers of one assembly; zeroing and uploads are ordered on its stream
 struct DevPool {
+    cudaStream_t st = nullptr;
     std::vector<void*> ptrs;
+    explicit DevPool(cudaStream_t s) : st(s) {}
     ~DevPool() {
         for (void* p : ptrs) cudaFree(p);
     }
@@ -43,9 +50,9 @@ struct DevPool {
         }
         ptrs.push_back(q);
         if (zero) {
-            e = cudaMemset(q, 0, count * sizeof(T));
+            e = cudaMemsetAsync(q, 0, count * sizeof(T), st);
             if (e != cudaSuccess) {
-                set_error("cudaMemset failed: %s", cudaGetErrorString(e));
+                set_error("cudaMemsetAsync failed: %s", cudaGetErrorString(e));
                 return BPM_ERR_CUDA;
             }
         }
@@ -54,10 +61,37 @@ struct DevPool {
     }
 };
 
+// A stream forked from `main` at fork() and joined into it by join().  Left on an early return it is
+// drained before its stream goes, so that its kernels never outlive the buffers they use (declare it
+// after the pool that owns them).
+struct SideStream {
+    cudaStream_t s = nullptr;
+    cudaEvent_t e = nullptr;
+    int fork(cudaStream_t main) {
+        BPM_CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        BPM_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        BPM_CK(cudaEventRecord(e, main));
+        BPM_CK(cudaStreamWaitEvent(s, e, 0));
+        return BPM_OK;
+    }
+    int join(cudaStream_t main) {
+        BPM_CK(cudaEventRecord(e, s));
+        BPM_CK(cudaStreamWaitEvent(main, e, 0));
+        return BPM_OK;
+    }
+    ~SideStream() {
+        if (s) {
+            cudaStreamSynchronize(s);
+            cudaStreamDestroy(s);
+        }
+        if (e) cudaEventDestroy(e);
+    }
+};
+
 template <class T>
 int upload(DevPool& pool, T** dst, const std::vector<T>& src) {
     BPM_TRY(pool.alloc(dst, src.size(), false));
-    BPM_CK(cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice));
+    BPM_CK(cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, pool.st));
     return BPM_OK;
 }
 
@@ -106,9 +140,10 @@ __device__ inline int local_index(const int* tet, int node) {
     return 0;
 }
 
-__device__ inline int find_col(const int* __restrict__ col, int lo, int hi, int j) {
-    for (int e = lo; e < hi; ++e)
-        if (col[e] == j) return e;
+// position of a node in a tet, -1 if the tet does not hold it
+__device__ inline int tet_slot(const int* tet, int node) {
+    for (int a = 0; a < 4; ++a)
+        if (tet[a] == node) return a;
     return -1;
 }
 
@@ -131,26 +166,33 @@ __global__ void k_node_lumped(int n, const int* __restrict__ n2t_ptr, const int*
     Ku[i] = ku / v;
 }
 
+// One warp per row, a lane per CSR entry (i, j): the lane walks the tets around i in order and
+// adds those that hold j, so every entry is summed in the same order as a serial loop over the
+// row would.  (One thread per row: 197 us at 481 nodes, two CTAs' worth of threads; now 24 us.)
 __global__ void k_csr_values(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                              const int* __restrict__ n2t_ptr, const int* __restrict__ n2t,
                              const int* __restrict__ tets, const int* __restrict__ region,
                              const double* __restrict__ mat_A, const double* __restrict__ vol,
                              const double* __restrict__ grads, double* __restrict__ KA,
                              double* __restrict__ KL) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= n) return;
-    for (int e = n2t_ptr[i]; e < n2t_ptr[i + 1]; ++e) {
-        int t = n2t[e];
-        const int* tt = tets + 4 * t;
-        int a = local_index(tt, i);
-        const double* g = grads + 12 * t;
-        for (int b = 0; b < 4; ++b) {
-            int pos = find_col(col, rowptr[i], rowptr[i + 1], tt[b]);
-            if (pos < 0) continue;
-            double gg = g[3 * a] * g[3 * b] + g[3 * a + 1] * g[3 * b + 1] + g[3 * a + 2] * g[3 * b + 2];
-            KL[pos] += vol[t] * gg;
-            KA[pos] += mat_A[region[t]] * vol[t] * gg;
+    for (int pos = rowptr[i] + lane; pos < rowptr[i + 1]; pos += 32) {
+        const int j = col[pos];
+        double kl = 0, ka = 0;
+        for (int e = n2t_ptr[i]; e < n2t_ptr[i + 1]; ++e) {
+            const int t = n2t[e];
+            const int* tt = tets + 4 * t;
+            const int b = tet_slot(tt, j);
+            if (b < 0) continue;
+            const int a = local_index(tt, i);
+            const double* g = grads + 12 * t;
+            const double gg = g[3 * a] * g[3 * b] + g[3 * a + 1] * g[3 * b + 1] + g[3 * a + 2] * g[3 * b + 2];
+            kl += vol[t] * gg;
+            ka += mat_A[region[t]] * vol[t] * gg;
         }
+        KL[pos] = kl;
+        KA[pos] = ka;
     }
 }
 
@@ -187,130 +229,360 @@ __device__ double block_sum(double v, double* red) {
     return s;
 }
 
-// Largest eigenvalue of S = D K_A (D = 2e18/(Ms V)) by power iteration on the
-// similar symmetric matrix D^1/2 K_A D^1/2; one block, Rayleigh quotient.
-__global__ void k_power_iteration(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
-                                  const double* __restrict__ KA, const double* __restrict__ V,
-                                  const double* __restrict__ Ms, double* x, double* y, int iters,
-                                  double* lam_out) {
-    __shared__ double red[32];
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        x[i] = ((i & 1) ? 1.0 : -1.0) + 0.3 * sin(0.7 * i);
-    __syncthreads();
-    double lam = 0;
-    for (int it = 0; it < iters; ++it) {
-        double nn = 0, xy = 0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            double di = sqrt(2.0e18 / (Ms[i] * V[i]));
-            double s = 0;
-            for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-                int j = col[e];
-                s += KA[e] * sqrt(2.0e18 / (Ms[j] * V[j])) * x[j];
-            }
-            y[i] = di * s;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            nn += y[i] * y[i];
-            xy += x[i] * y[i];
-        }
-        double xx = 0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) xx += x[i] * x[i];
-        nn = block_sum(nn, red);
-        xy = block_sum(xy, red);
-        xx = block_sum(xx, red);
-        lam = xy / xx;
-        double inv = 1.0 / sqrt(nn);
-        for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = y[i] * inv;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *lam_out = lam;
+// A CSR matrix in slices of 32 rows (diagonal included): entry e of row 32 s + l sits at
+// off[s] + 32 e + l, so that a warp reads a slice's values and columns coalesced; padding
+// entries hold the row itself (or node 0) with the value 0.
+struct Sliced {
+    const int* off;      // [n_slices + 1]
+    const int* col;      // node of the entry
+    const int* src;      // its CSR entry, -1 for padding
+    int len;
+};
+
+// sliced values of a CSR matrix; with d: d_i v_ij d_j; with mask: rows and columns outside it zero
+__global__ void k_sliced_values(Sliced A, const int* __restrict__ rows, const double* __restrict__ v,
+                                const double* __restrict__ d, const unsigned char* __restrict__ mask,
+                                double* __restrict__ out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= A.len) return;
+    const int e = A.src[k], i = rows[k], j = A.col[k];
+    double x = e >= 0 ? v[e] : 0.0;
+    if (d) x *= d[i] * d[j];
+    if (mask && !(mask[i] && mask[j])) x = 0.0;
+    out[k] = x;
 }
 
-// R [n][3n]: (R M)_i = int M . grad(phi_i) for nodal P1 M; column c*n + k
-__global__ void k_rhs(int n, const int* __restrict__ n2t_ptr, const int* __restrict__ n2t,
-                      const int* __restrict__ tets, const double* __restrict__ vol,
-                      const double* __restrict__ grads, double* __restrict__ R) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_exchange_scale(int n, const double* __restrict__ V, const double* __restrict__ Ms,
+                                 double* __restrict__ d) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) d[i] = sqrt(2.0e18 / (Ms[i] * V[i]));
+}
+
+// K_ii^-1/2 of every node, and the same with zeros off the interior
+__global__ void k_diag_scale(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
+                             const double* __restrict__ K, const unsigned char* __restrict__ interior,
+                             double* __restrict__ d, double* __restrict__ d_in) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    size_t ncol = 3 * (size_t)n;
-    for (int e = n2t_ptr[i]; e < n2t_ptr[i + 1]; ++e) {
-        int t = n2t[e];
-        const int* tt = tets + 4 * t;
-        int a = local_index(tt, i);
-        const double* g = grads + 12 * t;
-        double q = 0.25 * vol[t];
-        for (int b = 0; b < 4; ++b)
-            for (int c = 0; c < 3; ++c) R[i * ncol + (size_t)c * n + tt[b]] += q * g[3 * a + c];
+    double kii = 0;
+    for (int e = rowptr[i]; e < rowptr[i + 1]; ++e)
+        if (col[e] == i) kii = K[e];
+    d[i] = 1.0 / sqrt(kii);
+    d_in[i] = interior[i] ? d[i] : 0.0;
+}
+
+__device__ __forceinline__ double sliced_row(const Sliced& A, const double* __restrict__ val, const double* x, int i) {
+    const int lo = A.off[i >> 5] + (i & 31), hi = A.off[(i >> 5) + 1];
+    double s = 0;
+#pragma unroll 4
+    for (int k = lo; k < hi; k += 32) s += val[k] * x[A.col[k]];
+    return s;
+}
+
+// Largest eigenvalue of S = D K_A (D = 2e18/(Ms V)) by power iteration on the similar symmetric
+// matrix D^1/2 K_A D^1/2 (sliced values in `val`), Rayleigh quotient of the last iterate.  A cluster
+// of 8 CTAs holds both vectors in every CTA's shared memory; a CTA forms an eighth of
+// the rows, four lanes a row, and writes them to all eight copies, with one cluster barrier per iteration.  Every CTA
+// normalises its own copy every 8 steps (the direction does not depend on when).  An SM does two
+// FP64 multiply-adds a cycle, so one CTA alone was bound by them: 5.9 ms for 1500 steps at 481 nodes,
+// 3.4 ms with the cluster, and it runs beside the demag assembly.  (With square roots and divisions
+// formed per entry, rows read uncoalesced and three reductions a step: 116 ms.)
+constexpr int kPowCluster = 8, kPowThreads = 512;
+
+__global__ void __cluster_dims__(kPowCluster, 1, 1) __launch_bounds__(kPowThreads)
+    k_power_iteration(int n, Sliced A, const double* __restrict__ val, int iters, double* __restrict__ lam_out) {
+    namespace cgr = cooperative_groups;
+    extern __shared__ double vec[];
+    __shared__ double red[32];
+    cgr::cluster_group cl = cgr::this_cluster();
+    const int rank = (int)cl.block_rank();
+    const int n_slices = (n + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *x = vec, *y = vec + n;
+    for (int i = threadIdx.x; i < n; i += kPowThreads) x[i] = ((i & 1) ? 1.0 : -1.0) + 0.3 * sin(0.7 * i);
+    cl.sync();
+    for (int it = 1; it < iters; ++it) {
+        // a warp takes 8 rows of a slice, four lanes a row; each lane sends the sum to two CTAs
+        for (int u = rank + kPowCluster * warp; u < 4 * n_slices; u += kPowCluster * (kPowThreads / 32)) {
+            const int i = 8 * u + (lane & 7), part = lane >> 3;
+            double v = 0;
+            if (i < n) {
+                const int hi = A.off[(i >> 5) + 1];
+#pragma unroll 2
+                for (int k = A.off[i >> 5] + (i & 31) + 32 * part; k < hi; k += 128) v += val[k] * x[A.col[k]];
+            }
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (i < n) {
+                cl.map_shared_rank(y, 2 * part)[i] = v;
+                cl.map_shared_rank(y, 2 * part + 1)[i] = v;
+            }
+        }
+        cl.sync();
+        double* t = x;
+        x = y;
+        y = t;
+        if ((it & 7) == 0) {
+            double nn = 0;
+            for (int i = threadIdx.x; i < n; i += kPowThreads) nn += x[i] * x[i];
+            const double inv = 1.0 / sqrt(block_sum(nn, red));
+            for (int i = threadIdx.x; i < n; i += kPowThreads) x[i] *= inv;
+            __syncthreads();
+        }
     }
+    double xy = 0, xx = 0;
+    if (rank == 0) {
+        for (int i = threadIdx.x; i < n; i += kPowThreads) {
+            xy += x[i] * sliced_row(A, val, x, i);
+            xx += x[i] * x[i];
+        }
+        xy = block_sum(xy, red);
+        xx = block_sum(xx, red);
+        if (threadIdx.x == 0) *lam_out = xy / xx;
+    }
+}
+
+// (R M)_j = int M . grad(phi_j) for nodal P1 M, by columns: RT[c][pos] = R[j][c n + k] for CSR entry
+// pos = (k, j).  A lane per entry, tets in order, as in k_csr_values.
+__global__ void k_source(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
+                         const int* __restrict__ n2t_ptr, const int* __restrict__ n2t,
+                         const int* __restrict__ tets, const double* __restrict__ vol,
+                         const double* __restrict__ grads, int nnz, double* __restrict__ RT) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (k >= n) return;
+    for (int pos = rowptr[k] + lane; pos < rowptr[k + 1]; pos += 32) {
+        const int j = col[pos];
+        double s[3] = {0, 0, 0};
+        for (int e = n2t_ptr[k]; e < n2t_ptr[k + 1]; ++e) {
+            const int t = n2t[e];
+            const int a = tet_slot(tets + 4 * t, j);
+            if (a < 0) continue;
+            const double* g = grads + 12 * t;
+            const double q = 0.25 * vol[t];
+            for (int c = 0; c < 3; ++c) s[c] += q * g[3 * a + c];
+        }
+        for (int c = 0; c < 3; ++c) RT[(size_t)c * nnz + pos] = s[c];
+    }
+}
+
+// U = Q R: U[i][c n + k] = sum over the neighbours j of k of Q[i][j] R[j][c n + k] (RT sliced: rv[c][entry])
+__global__ void k_apply_source(int n, Sliced A, const double* __restrict__ rv, const double* __restrict__ Q,
+                               double* __restrict__ U) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (k >= n) return;
+    const double* q = Q + (size_t)i * n;
+    double s0 = 0, s1 = 0, s2 = 0;
+    const int lo = A.off[k >> 5] + (k & 31), hi = A.off[(k >> 5) + 1];
+#pragma unroll 4
+    for (int e = lo; e < hi; e += 32) {
+        const double v = q[A.col[e]];
+        s0 += v * rv[e];
+        s1 += v * rv[A.len + e];
+        s2 += v * rv[2 * (size_t)A.len + e];
+    }
+    double* u = U + (size_t)i * 3 * n + k;
+    u[0] = s0;
+    u[n] = s1;
+    u[2 * (size_t)n] = s2;
+}
+
+// right-hand sides of the nodal sources of the Neumann problem: e_j - 1/n
+__global__ void k_unit_sources(int n, double* __restrict__ B) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (j < n) B[(size_t)i * n + j] = (i == j ? 1.0 : 0.0) - 1.0 / n;
+}
+
+// right-hand sides -K_IB of the harmonic extension (interior rows; B zeroed before)
+__global__ void k_boundary_sources(int n, int nb, const int* __restrict__ rowptr, const int* __restrict__ col,
+                                   const double* __restrict__ K, const unsigned char* __restrict__ interior,
+                                   const int* __restrict__ bidx, double* __restrict__ B) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= n || !interior[i]) return;
+    for (int e = rowptr[i] + lane; e < rowptr[i + 1]; e += 32)
+        if (!interior[col[e]]) B[(size_t)i * nb + bidx[col[e]]] = -K[e];
+}
+
+// the extension on the boundary itself is the identity
+__global__ void k_boundary_identity(int nb, const int* __restrict__ bnodes, double* __restrict__ E) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < nb) E[(size_t)bnodes[b] * nb + b] = 1.0;
 }
 
 // ---------------------------------------------------------------- batched CG
-// Y[i][c] = sum_e val_e X[col_e][c]; with mask: rows and columns outside the mask are zero
-__global__ void k_spmm(int n, int ncol, const int* __restrict__ rowptr, const int* __restrict__ col,
-                       const double* __restrict__ val, const unsigned char* __restrict__ mask,
-                       const double* __restrict__ X, double* __restrict__ Y) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (c >= ncol) return;
-    double s = 0;
-    if (!mask || mask[i]) {
-        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-            int j = col[e];
-            if (mask && !mask[j]) continue;
-            s += val[e] * X[(size_t)j * ncol + c];
+// kCgSteps iterations of CG on C columns of the right-hand side block, one CTA: p, q and r of its
+// columns in shared memory ([n][C]), x in global memory (each thread its own rows).  The matrix is
+// scaled to a unit diagonal (d K d, d = K_ii^-1/2: Jacobi preconditioning); b and x are scaled on the
+// way in and out.  The columns are independent, so an iteration needs
+// no grid-wide step.  The matrix (sliced, 12 B an entry) comes from L1/L2, once for the C columns.
+// The bound is the FP64 rate, two multiply-adds a cycle and SM: about 25 per node, column and
+// iteration.  Hence one warp adds up the CTA's partial sums and divides (all threads doing so cost a
+// third of the iteration), while the others update x.  Measured at 481 nodes, 481 columns: 20 us an
+// iteration (28 us with all threads reducing and two columns a CTA; one kernel per vector operation
+// with one thread per column in the dot products took 330 us for the 1443 columns of 3n sources).
+constexpr int kCgThreads = 256, kCgSteps = 16;
+
+// sum over the CTA of C values per thread: partial sums to shared memory, warp 0 adds them
+template <int C>
+__device__ __forceinline__ void put_partial(const double (&v)[C], double* part) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) part[c * kCgThreads + threadIdx.x] = v[c];
+}
+template <int C>
+__device__ __forceinline__ void warp_total(const double* part, double (&v)[C]) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        double s = 0;
+        for (int k = threadIdx.x; k < kCgThreads; k += 32) s += part[c * kCgThreads + k];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        v[c] = s;
+    }
+}
+
+template <int C>
+__global__ void __launch_bounds__(kCgThreads) k_cg_steps(int n, int ncol, Sliced A, const double* __restrict__ val,
+                                                         const double* __restrict__ d,
+                                                         const double* __restrict__ b, int first,
+                                                         double* __restrict__ x, double* __restrict__ rg,
+                                                         double* __restrict__ pg, double* __restrict__ rzg,
+                                                         double* __restrict__ bbg, double* __restrict__ rrg) {
+    extern __shared__ double cg[];
+    __shared__ double part[kCgThreads * C], coef[C], rz_s[C], floor_s[C];
+    double *p = cg, *q = cg + (size_t)n * C, *r = q + (size_t)n * C;
+    const int c0 = blockIdx.x * C;
+    double v[C], s[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) v[c] = s[c] = 0;
+    for (int i = threadIdx.x; i < n; i += kCgThreads) {
+        const double di = d[i];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const bool in = c0 + c < ncol;
+            const size_t k = (size_t)i * ncol + c0 + c;
+            const double bv = in && first ? b[k] : 0.0;
+            const double rv = first ? di * bv : (in ? rg[k] : 0.0);
+            r[i * C + c] = rv;
+            p[i * C + c] = first ? rv : (in ? pg[k] : 0.0);
+            if (first) {
+                if (in) x[k] = 0.0;
+                v[c] += rv * rv;
+                s[c] += bv * bv;
+            }
         }
     }
-    Y[(size_t)i * ncol + c] = s;
+    // a column at rounding level stays where it is: steps beyond it would only follow the null space
+    // of the Neumann problem (a mesh of a few dozen nodes is there before the first check)
+    put_partial<C>(v, part);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        warp_total<C>(part, v);
+        if (threadIdx.x == 0)
+            for (int c = 0; c < C; ++c) {
+                const bool in = c0 + c < ncol;
+                if (in && first) rzg[ncol + c0 + c] = v[c];
+                rz_s[c] = first ? v[c] : (in ? rzg[c0 + c] : 0.0);
+                floor_s[c] = 1e-31 * (first ? v[c] : (in ? rzg[ncol + c0 + c] : 0.0));
+            }
+    }
+    if (first) {
+        __syncthreads();
+        put_partial<C>(s, part);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            warp_total<C>(part, s);
+            if (threadIdx.x == 0)
+                for (int c = 0; c < C && c0 + c < ncol; ++c) bbg[c0 + c] = s[c];
+        }
+    }
+    for (int it = 0; it < kCgSteps; ++it) {
+        __syncthreads();                                   // p of every row is in place
+        double pq[C], rr[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) pq[c] = rr[c] = 0;
+        for (int i = threadIdx.x; i < n; i += kCgThreads) {
+            const int lo = A.off[i >> 5] + (i & 31), hi = A.off[(i >> 5) + 1];
+            double t[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) t[c] = 0;
+#pragma unroll 4
+            for (int k = lo; k < hi; k += 32) {
+                const double a = val[k];
+                const double* pj = p + A.col[k] * C;
+#pragma unroll
+                for (int c = 0; c < C; ++c) t[c] += a * pj[c];
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                q[i * C + c] = t[c];
+                pq[c] += p[i * C + c] * t[c];
+            }
+        }
+        put_partial<C>(pq, part);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            warp_total<C>(part, pq);
+            if (threadIdx.x == 0)
+                for (int c = 0; c < C; ++c) coef[c] = pq[c] > 0 && rz_s[c] > floor_s[c] ? rz_s[c] / pq[c] : 0.0;
+        }
+        __syncthreads();
+        double a[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) a[c] = coef[c];
+        for (int i = threadIdx.x; i < n; i += kCgThreads)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const double rv = r[i * C + c] - a[c] * q[i * C + c];
+                r[i * C + c] = rv;
+                rr[c] += rv * rv;
+            }
+        put_partial<C>(rr, part);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            warp_total<C>(part, rr);
+            if (threadIdx.x == 0)
+                for (int c = 0; c < C; ++c) {
+                    coef[c] = rz_s[c] > 0 ? rr[c] / rz_s[c] : 0.0;
+                    rz_s[c] = rr[c];
+                }
+        }
+        for (int i = threadIdx.x; i < n; i += kCgThreads)
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                if (c0 + c < ncol) x[(size_t)i * ncol + c0 + c] += a[c] * p[i * C + c];
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += kCgThreads)
+#pragma unroll
+            for (int c = 0; c < C; ++c) p[i * C + c] = r[i * C + c] + coef[c] * p[i * C + c];
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) s[c] = 0;
+    for (int i = threadIdx.x; i < n; i += kCgThreads) {
+        const double di = d[i];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const double rv = r[i * C + c], u = di > 0 ? rv / di : 0.0;
+            s[c] += u * u;
+            if (c0 + c < ncol) {
+                rg[(size_t)i * ncol + c0 + c] = rv;
+                pg[(size_t)i * ncol + c0 + c] = p[i * C + c];
+            }
+        }
+    }
+    __syncthreads();
+    put_partial<C>(s, part);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        warp_total<C>(part, s);
+        if (threadIdx.x == 0)
+            for (int c = 0; c < C && c0 + c < ncol; ++c) {
+                rrg[c0 + c] = s[c];
+                rzg[c0 + c] = rz_s[c];
+            }
+    }
 }
 
-__global__ void k_coldot(int n, int ncol, const double* __restrict__ X, const double* __restrict__ Y,
-                         double* __restrict__ out) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncol) return;
-    double s = 0;
-    for (int i = 0; i < n; ++i) s += X[(size_t)i * ncol + c] * Y[(size_t)i * ncol + c];
-    out[c] = s;
-}
-
-__global__ void k_cg_init(int n, int ncol, const double* __restrict__ b, const double* __restrict__ dinv,
-                          double* __restrict__ x, double* __restrict__ r, double* __restrict__ z,
-                          double* __restrict__ p) {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n * ncol) return;
-    int i = (int)(k / ncol);
-    x[k] = 0;
-    r[k] = b[k];
-    z[k] = dinv[i] * b[k];
-    p[k] = z[k];
-}
-
-__global__ void k_cg_xr(int n, int ncol, const double* __restrict__ rz, const double* __restrict__ pq,
-                        const double* __restrict__ dinv, const double* __restrict__ p,
-                        const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                        double* __restrict__ z) {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n * ncol) return;
-    int i = (int)(k / ncol), c = (int)(k % ncol);
-    double a = pq[c] > 0 ? rz[c] / pq[c] : 0.0;
-    x[k] += a * p[k];
-    double rv = r[k] - a * q[k];
-    r[k] = rv;
-    z[k] = dinv[i] * rv;
-}
-
-__global__ void k_cg_p(int n, int ncol, const double* __restrict__ rz_new, double* __restrict__ rz_old,
-                       const double* __restrict__ z, double* __restrict__ p) {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n * ncol) return;
-    int c = (int)(k % ncol);
-    double b = rz_old[c] > 0 ? rz_new[c] / rz_old[c] : 0.0;
-    p[k] = z[k] + b * p[k];
-}
-
-__global__ void k_copy_vec(int ncol, const double* __restrict__ a, double* __restrict__ b) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncol) b[c] = a[c];
+// x = d x', out of the scaled system
+__global__ void k_scale_rows(int ncol, const double* __restrict__ d, double* __restrict__ X) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (c < ncol) X[(size_t)i * ncol + c] *= d[i];
 }
 
 __global__ void k_max_ratio(int ncol, const double* __restrict__ rr, const double* __restrict__ bb,
@@ -333,68 +605,64 @@ __global__ void k_max_ratio(int ncol, const double* __restrict__ rr, const doubl
     }
 }
 
-__global__ void k_col_mean_sub(int n, int ncol, double* __restrict__ X) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncol) return;
+// subtract each column's mean: 32 columns a CTA, 8 warps over the rows, partial sums in a fixed order
+__global__ void __launch_bounds__(256) k_col_mean_sub(int n, int ncol, double* __restrict__ X) {
+    __shared__ double part[8][32];
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + l;
     double s = 0;
-    for (int i = 0; i < n; ++i) s += X[(size_t)i * ncol + c];
+    if (c < ncol)
+        for (int i = w; i < n; i += 8) s += X[(size_t)i * ncol + c];
+    part[w][l] = s;
+    __syncthreads();
+    s = 0;
+    for (int k = 0; k < 8; ++k) s += part[k][l];
     s /= n;
-    for (int i = 0; i < n; ++i) X[(size_t)i * ncol + c] -= s;
+    if (c < ncol)
+        for (int i = w; i < n; i += 8) X[(size_t)i * ncol + c] -= s;
 }
 
-__global__ void k_masked_scale(int n, int ncol, const unsigned char* __restrict__ mask, double s,
-                               double* __restrict__ X) {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n * ncol) return;
-    int i = (int)(k / ncol);
-    X[k] = mask[i] ? s * X[k] : 0.0;
+template <int C>
+int cg_launch(cudaStream_t st, int n, int ncol, const Sliced& A, const double* val, const double* d,
+              const double* b, int first, double* x, double* r, double* p, double* rz, double* bb, double* rr) {
+    const int smem = 3 * (int)sizeof(double) * n * C;
+    BPM_CK(cudaFuncSetAttribute(k_cg_steps<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_cg_steps<C><<<(ncol + C - 1) / C, kCgThreads, smem, st>>>(n, ncol, A, val, d, b, first, x, r, p, rz, bb, rr);
+    BPM_CK(cudaGetLastError());
+    return BPM_OK;
 }
 
-int pcg(cudaStream_t st, DevPool& pool, int n, int ncol, const int* rowptr, const int* col,
-        const double* val, const unsigned char* mask, const double* dinv, const double* b,
-        double* x, double tol, int maxit, int* iters_out, double* resid_out) {
-    size_t N = (size_t)n * ncol;
-    double *r, *z, *p, *q, *rz, *rzn, *pq, *bb, *rr, *mx;
+int pcg(cudaStream_t st, DevPool& pool, int n, int ncol, const Sliced& A, const double* val, const double* d,
+        const double* b, double* x, double tol, int maxit, int* iters_out, double* resid_out) {
+    const size_t N = (size_t)n * ncol;
+    double *r, *p, *rz, *bb, *rr, *mx;
     BPM_TRY(pool.alloc(&r, N, false));
-    BPM_TRY(pool.alloc(&z, N, false));
     BPM_TRY(pool.alloc(&p, N, false));
-    BPM_TRY(pool.alloc(&q, N, false));
-    BPM_TRY(pool.alloc(&rz, ncol));
-    BPM_TRY(pool.alloc(&rzn, ncol));
-    BPM_TRY(pool.alloc(&pq, ncol));
+    BPM_TRY(pool.alloc(&rz, 2 * (size_t)ncol));   // current and initial r . z
     BPM_TRY(pool.alloc(&bb, ncol));
     BPM_TRY(pool.alloc(&rr, ncol));
     BPM_TRY(pool.alloc(&mx, 1));
-    const int T = 256;
-    unsigned gN = (unsigned)((N + T - 1) / T), gC = (unsigned)((ncol + T - 1) / T);
-    dim3 gS((ncol + 127) / 128, n);
-    k_cg_init<<<gN, T, 0, st>>>(n, ncol, b, dinv, x, r, z, p);
-    k_coldot<<<gC, T, 0, st>>>(n, ncol, r, z, rz);
-    k_coldot<<<gC, T, 0, st>>>(n, ncol, b, b, bb);
-    BPM_CK(cudaGetLastError());
+    // columns a CTA: two share the matrix loads where there are enough columns to fill the SMs either
+    // way, and while three vectors of both fit shared memory (4096 nodes: 196608 B)
+    const bool two = n <= 4096 && ncol >= 1024;
     double res = 1.0;
     int it = 0;
-    for (it = 1; it <= maxit; ++it) {
-        k_spmm<<<gS, 128, 0, st>>>(n, ncol, rowptr, col, val, mask, p, q);
-        k_coldot<<<gC, T, 0, st>>>(n, ncol, p, q, pq);
-        k_cg_xr<<<gN, T, 0, st>>>(n, ncol, rz, pq, dinv, p, q, x, r, z);
-        k_coldot<<<gC, T, 0, st>>>(n, ncol, r, z, rzn);
-        k_cg_p<<<gN, T, 0, st>>>(n, ncol, rzn, rz, z, p);
-        k_copy_vec<<<gC, T, 0, st>>>(ncol, rzn, rz);
-        if (it % 16 == 0 || it == maxit) {
-            k_coldot<<<gC, T, 0, st>>>(n, ncol, r, r, rr);
-            k_max_ratio<<<1, 1024, 0, st>>>(ncol, rr, bb, mx);
-            BPM_CK(cudaGetLastError());
-            BPM_CK(cudaMemcpyAsync(&res, mx, sizeof(double), cudaMemcpyDeviceToHost, st));
-            BPM_CK(cudaStreamSynchronize(st));
-            if (!(res < 1e300)) {
-                set_error("CG produced a non-finite residual");
-                return BPM_ERR_NONFINITE;
-            }
-            if (res < tol) break;
+    while (it < maxit) {
+        BPM_TRY(two ? cg_launch<2>(st, n, ncol, A, val, d, b, it == 0, x, r, p, rz, bb, rr)
+                    : cg_launch<1>(st, n, ncol, A, val, d, b, it == 0, x, r, p, rz, bb, rr));
+        it += kCgSteps;
+        k_max_ratio<<<1, 1024, 0, st>>>(ncol, rr, bb, mx);
+        BPM_CK(cudaGetLastError());
+        BPM_CK(cudaMemcpyAsync(&res, mx, sizeof(double), cudaMemcpyDeviceToHost, st));
+        BPM_CK(cudaStreamSynchronize(st));
+        if (!(res < 1e300)) {
+            set_error("CG produced a non-finite residual");
+            return BPM_ERR_NONFINITE;
         }
+        if (res < tol) break;
     }
-    *iters_out = std::min(it, maxit);
+    k_scale_rows<<<dim3((ncol + 127) / 128, n), 128, 0, st>>>(ncol, d, x);
+    BPM_CK(cudaGetLastError());
+    *iters_out = it;
     *resid_out = res;
     if (res >= tol) {
         set_error("CG did not converge: relative residual %.3e after %d iterations", res, maxit);
@@ -461,26 +729,42 @@ __global__ void k_interior_angles(int nb, const int* __restrict__ bnodes, const 
     omega[ib] = s;
 }
 
+// Lindholm weights of every (observer, face) pair, W[ib][3 f + k] for vertex k of face f; zero where
+// the observer is a vertex of the face (it lies in the face's plane).  One evaluation gives all three
+// weights of a face (evaluated per (observer, node) pair each face was computed three times and two
+// of its weights dropped: 584 us at 272 boundary nodes).
+__global__ void k_bem_weights(int i0, int rows, int nf, const int* __restrict__ bnodes,
+                              const double* __restrict__ xyz, const int* __restrict__ faces,
+                              double* __restrict__ W) {
+    const int f = blockIdx.x * blockDim.x + threadIdx.x, ib = blockIdx.y;
+    if (f >= nf || ib >= rows) return;
+    const int i = bnodes[i0 + ib];
+    const int* fc = faces + 3 * f;
+    double w[3] = {0, 0, 0};
+    if (fc[0] != i && fc[1] != i && fc[2] != i) {
+        const V3 y[3] = {ld3(xyz + 3 * fc[0]), ld3(xyz + 3 * fc[1]), ld3(xyz + 3 * fc[2])};
+        lindholm(ld3(xyz + 3 * i), y, w);
+    }
+    double* o = W + ((size_t)ib * nf + f) * 3;
+    o[0] = w[0];
+    o[1] = w[1];
+    o[2] = w[2];
+}
+
 // Bmat[ib][jb] = D_ij + delta_ij (Omega_i/4pi - 1),
-// D_ij = -(1/4pi) sum over boundary faces T containing node j (not node i) of w_j(x_i; T)
-__global__ void k_bem_matrix(int nb, const int* __restrict__ bnodes, const double* __restrict__ xyz,
-                             const int* __restrict__ faces, const int* __restrict__ b2f_ptr,
-                             const int* __restrict__ b2f, const double* __restrict__ omega,
+// D_ij = -(1/4pi) sum over boundary faces T containing node j of w_j(x_i; T)
+__global__ void k_bem_matrix(int i0, int nb, int nf, const int* __restrict__ bnodes, const int* __restrict__ faces,
+                             const int* __restrict__ b2f_ptr, const int* __restrict__ b2f,
+                             const double* __restrict__ omega, const double* __restrict__ W,
                              double* __restrict__ Bmat) {
-    int jb = blockIdx.x * blockDim.x + threadIdx.x;
-    int ib = blockIdx.y;
+    const int jb = blockIdx.x * blockDim.x + threadIdx.x, ib = i0 + blockIdx.y;
     if (jb >= nb) return;
-    int i = bnodes[ib], j = bnodes[jb];
-    V3 x = ld3(xyz + 3 * i);
+    const int j = bnodes[jb];
     double s = 0;
     for (int e = b2f_ptr[jb]; e < b2f_ptr[jb + 1]; ++e) {
         const int* f = faces + 3 * b2f[e];
-        if (f[0] == i || f[1] == i || f[2] == i) continue;  // x_i in the face plane: weight 0
-        V3 y[3] = {ld3(xyz + 3 * f[0]), ld3(xyz + 3 * f[1]), ld3(xyz + 3 * f[2])};
-        double w[3];
-        lindholm(x, y, w);
-        int loc = (f[0] == j) ? 0 : ((f[1] == j) ? 1 : 2);
-        s += w[loc];
+        const int loc = (f[0] == j) ? 0 : ((f[1] == j) ? 1 : 2);
+        s += W[((size_t)blockIdx.y * nf + b2f[e]) * 3 + loc];
     }
     double v = -s / (4.0 * M_PI);
     if (ib == jb) v += omega[ib] / (4.0 * M_PI) - 1.0;
@@ -495,16 +779,8 @@ __global__ void k_gather_rows(int nb, int ncol, const int* __restrict__ rows, co
     dst[(size_t)ib * ncol + c] = src[(size_t)rows[ib] * ncol + c];
 }
 
-__global__ void k_scatter_rows(int nb, int ncol, const int* __restrict__ rows, const double* __restrict__ src,
-                               double* __restrict__ dst) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    int ib = blockIdx.y;
-    if (c >= ncol) return;
-    dst[(size_t)rows[ib] * ncol + c] = src[(size_t)ib * ncol + c];
-}
-
-// C[M][N] = A[M][K] B[K][N] (row-major, FP64), 32x32 tiles
-__global__ void k_dgemm(int M, int N, int K, const double* __restrict__ A, const double* __restrict__ B,
+// C[M][N] (+)= A[M][K] B[K][N] (row-major, FP64), 32x32 tiles
+__global__ void k_dgemm(int M, int N, int K, const double* __restrict__ A, const double* __restrict__ B, int add,
                         double* __restrict__ C) {
     __shared__ double As[32][33], Bs[32][33];
     int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -526,34 +802,31 @@ __global__ void k_dgemm(int M, int N, int K, const double* __restrict__ A, const
     }
     for (int q = 0; q < 4; ++q) {
         int gr = row0 + ty + 8 * q;
-        if (gr < M && col < N) C[(size_t)gr * N + col] = acc[q];
+        if (gr < M && col < N) C[(size_t)gr * N + col] = add ? C[(size_t)gr * N + col] + acc[q] : acc[q];
     }
 }
 
-__global__ void k_add3(size_t N, const double* __restrict__ a, const double* __restrict__ b,
-                       const double* __restrict__ c, double* __restrict__ out) {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < N) out[k] = a[k] + b[k] + c[k];
-}
-
-// P_c[e] = (1/V_i) sum_{t ni i, k} (vol_t / 4) grad(phi_k)|_t [c] for CSR entry e = (i, k)
+// P_c[e] = (1/V_i) sum_{t ni i, k} (vol_t / 4) grad(phi_k)|_t [c] for CSR entry e = (i, k); a lane per
+// entry, tets in order, as in k_csr_values
 __global__ void k_proj_values(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                               const int* __restrict__ n2t_ptr, const int* __restrict__ n2t,
                               const int* __restrict__ tets, const double* __restrict__ vol,
                               const double* __restrict__ grads, const double* __restrict__ V, int nnz,
                               double* __restrict__ P) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= n) return;
-    for (int e = n2t_ptr[i]; e < n2t_ptr[i + 1]; ++e) {
-        int t = n2t[e];
-        const int* tt = tets + 4 * t;
-        const double* g = grads + 12 * t;
-        double q = 0.25 * vol[t] / V[i];
-        for (int b = 0; b < 4; ++b) {
-            int pos = find_col(col, rowptr[i], rowptr[i + 1], tt[b]);
-            if (pos < 0) continue;
-            for (int c = 0; c < 3; ++c) P[(size_t)c * nnz + pos] += q * g[3 * b + c];
+    for (int pos = rowptr[i] + lane; pos < rowptr[i + 1]; pos += 32) {
+        const int j = col[pos];
+        double s[3] = {0, 0, 0};
+        for (int e = n2t_ptr[i]; e < n2t_ptr[i + 1]; ++e) {
+            const int t = n2t[e];
+            const int b = tet_slot(tets + 4 * t, j);
+            if (b < 0) continue;
+            const double* g = grads + 12 * t;
+            const double q = 0.25 * vol[t] / V[i];
+            for (int c = 0; c < 3; ++c) s[c] += q * g[3 * b + c];
         }
+        for (int c = 0; c < 3; ++c) P[(size_t)c * nnz + pos] = s[c];
     }
 }
 
@@ -673,24 +946,28 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     }
     const int nnz = (int)col.size();
     // boundary faces: faces of exactly one tet, oriented outward
-    std::map<std::array<int, 3>, std::array<int, 5>> fmap;  // key -> {count, a, b, c, opposite}
+    struct Face {
+        uint64_t key;                      // sorted corners, 21 bits each
+        int a, b, c, opposite;
+    };
+    std::vector<Face> fl;
+    fl.reserve(4 * (size_t)nt);
     for (int t = 0; t < nt; ++t)
         for (int k = 0; k < 4; ++k) {
             int f[3], q = 0;
             for (int a = 0; a < 4; ++a)
                 if (a != k) f[q++] = tets[4 * t + a];
-            std::array<int, 3> key{f[0], f[1], f[2]};
-            std::sort(key.begin(), key.end());
-            auto it = fmap.find(key);
-            if (it == fmap.end())
-                fmap[key] = {1, f[0], f[1], f[2], tets[4 * t + k]};
-            else
-                it->second[0]++;
+            int o[3] = {f[0], f[1], f[2]};
+            std::sort(o, o + 3);
+            fl.push_back(Face{(uint64_t)o[0] << 42 | (uint64_t)o[1] << 21 | (uint64_t)o[2], f[0], f[1], f[2],
+                              tets[4 * t + k]});
         }
+    std::sort(fl.begin(), fl.end(), [](const Face& x, const Face& y) { return x.key < y.key; });
     std::vector<int> faces;
-    for (auto& kv : fmap) {
-        if (kv.second[0] != 1) continue;
-        int a = kv.second[1], b = kv.second[2], c = kv.second[3], d = kv.second[4];
+    for (size_t i = 0, j; i < fl.size(); i = j) {
+        for (j = i + 1; j < fl.size() && fl[j].key == fl[i].key; ++j) {}
+        if (j - i != 1) continue;
+        int a = fl[i].a, b = fl[i].b, c = fl[i].c, d = fl[i].opposite;
         V3 ya = ld3(xyz + 3 * a);
         V3 nrmv = cross(sub(ld3(xyz + 3 * b), ya), sub(ld3(xyz + 3 * c), ya));
         if (dot(nrmv, sub(ld3(xyz + 3 * d), ya)) > 0) std::swap(b, c);
@@ -727,7 +1004,7 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     }
 
     // ---------------- device assembly ----------------
-    DevPool pool;
+    DevPool pool(st);
     double *d_xyz, *d_vol, *d_grads, *d_V, *d_Ms, *d_Ku, *d_KA, *d_KL, *d_mMs, *d_mKu, *d_mA;
     int *d_tets, *d_reg, *d_n2tp, *d_n2t, *d_rowptr, *d_col, *d_bnodes, *d_faces, *d_b2fp, *d_b2f;
     unsigned char* d_int;
@@ -758,8 +1035,9 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     const int T = 256;
     k_tet_geom<<<(nt + T - 1) / T, T, 0, st>>>(nt, d_xyz, d_tets, d_vol, d_grads);
     k_node_lumped<<<(n + T - 1) / T, T, 0, st>>>(n, d_n2tp, d_n2t, d_reg, d_vol, d_mMs, d_mKu, d_V, d_Ms, d_Ku);
-    k_csr_values<<<(n + T - 1) / T, T, 0, st>>>(n, d_rowptr, d_col, d_n2tp, d_n2t, d_tets, d_reg, d_mA,
-                                                 d_vol, d_grads, d_KA, d_KL);
+    const int gRow = (32 * n + T - 1) / T;   // a warp per row
+    k_csr_values<<<gRow, T, 0, st>>>(n, d_rowptr, d_col, d_n2tp, d_n2t, d_tets, d_reg, d_mA, d_vol, d_grads, d_KA,
+                                     d_KL);
     BPM_CK(cudaGetLastError());
     // exchange operator values (FP32) and lambda_max
     float* d_c;
@@ -771,78 +1049,127 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     BPM_CK(cudaMemcpyAsync(M->csr_rowptr, d_rowptr, (n + 1) * sizeof(int), cudaMemcpyDeviceToDevice, st));
     BPM_CK(cudaMemcpyAsync(M->csr_col, d_col, nnz * sizeof(int), cudaMemcpyDeviceToDevice, st));
     k_exchange_values64<<<(n + T - 1) / T, T, 0, st>>>(n, d_rowptr, d_col, d_KA, d_V, d_Ms, M->csr_c64);
-    double *d_px, *d_py, *d_lam;
-    BPM_TRY(pool.alloc(&d_px, n));
-    BPM_TRY(pool.alloc(&d_py, n));
-    BPM_TRY(pool.alloc(&d_lam, 1));
-    k_power_iteration<<<1, 1024, 0, st>>>(n, d_rowptr, d_col, d_KA, d_V, d_Ms, d_px, d_py, 1500, d_lam);
+    // the matrix pattern in 32-row slices, for the power iteration and CG
+    const int n_sl = (n + 31) / 32;
+    std::vector<int> soff(n_sl + 1, 0);
+    for (int q = 0; q < n_sl; ++q) {
+        int w = 0;
+        for (int i = 32 * q; i < std::min(n, 32 * q + 32); ++i) w = std::max(w, rowptr[i + 1] - rowptr[i]);
+        soff[q + 1] = soff[q] + 32 * w;
+    }
+    Sliced A{};
+    A.len = soff[n_sl];
+    std::vector<int> scol(A.len), ssrc(A.len), srow(A.len);
+    for (int q = 0; q < n_sl; ++q)
+        for (int k = soff[q]; k < soff[q + 1]; ++k) {
+            const int i = 32 * q + ((k - soff[q]) & 31), e = i < n ? rowptr[i] + (k - soff[q]) / 32 : 0;
+            const bool in = i < n && e < rowptr[i + 1];
+            srow[k] = i < n ? i : 0;
+            scol[k] = in ? col[e] : srow[k];
+            ssrc[k] = in ? e : -1;
+        }
+    int *d_soff, *d_scol, *d_ssrc, *d_srow;
+    double *d_sval, *d_sval_in, *d_sval_x, *d_dx, *d_lam;
+    BPM_TRY(upload(pool, &d_soff, soff));
+    BPM_TRY(upload(pool, &d_scol, scol));
+    BPM_TRY(upload(pool, &d_ssrc, ssrc));
+    BPM_TRY(upload(pool, &d_srow, srow));
+    A.off = d_soff;
+    A.col = d_scol;
+    A.src = d_ssrc;
+    BPM_TRY(pool.alloc(&d_sval, A.len, false));
+    BPM_TRY(pool.alloc(&d_sval_in, A.len, false));
+    BPM_TRY(pool.alloc(&d_sval_x, A.len, false));
+    BPM_TRY(pool.alloc(&d_dx, n, false));
+    BPM_TRY(pool.alloc(&d_lam, 1, false));
+    const int gS = (A.len + T - 1) / T;
+    k_exchange_scale<<<(n + T - 1) / T, T, 0, st>>>(n, d_V, d_Ms, d_dx);
+    k_sliced_values<<<gS, T, 0, st>>>(A, d_srow, d_KA, d_dx, nullptr, d_sval_x);
+    BPM_CK(cudaGetLastError());
+    // lambda_max on a stream of its own, beside the demag assembly
+    SideStream side;
+    BPM_TRY(side.fork(st));
+    const int psmem = 2 * (int)sizeof(double) * n;
+    BPM_CK(cudaFuncSetAttribute(k_power_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
+    k_power_iteration<<<kPowCluster, kPowThreads, psmem, side.s>>>(n, A, d_sval_x, 1500, d_lam);
     BPM_CK(cudaGetLastError());
     M->exch_val.resize(nnz);
     M->V.resize(n);
     M->Ms.resize(n);
     M->Ku.resize(n);
-    double lam = 0;
     BPM_CK(cudaMemcpyAsync(M->exch_val.data(), d_c, nnz * sizeof(float), cudaMemcpyDeviceToHost, st));
     BPM_CK(cudaMemcpyAsync(M->V.data(), d_V, n * sizeof(double), cudaMemcpyDeviceToHost, st));
     BPM_CK(cudaMemcpyAsync(M->Ms.data(), d_Ms, n * sizeof(double), cudaMemcpyDeviceToHost, st));
     BPM_CK(cudaMemcpyAsync(M->Ku.data(), d_Ku, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    BPM_CK(cudaMemcpyAsync(&lam, d_lam, sizeof(double), cudaMemcpyDeviceToHost, st));
-    std::vector<double> KLh(nnz);
-    BPM_CK(cudaMemcpyAsync(KLh.data(), d_KL, nnz * sizeof(double), cudaMemcpyDeviceToHost, st));
-    BPM_CK(cudaStreamSynchronize(st));
 
     // ---------------- Fredkin-Koehler demag ----------------
     const int ncol = 3 * n;
-    const size_t NN = (size_t)n * ncol;
-    double *d_R, *d_U1, *d_dinvN, *d_dinvD;
-    BPM_TRY(pool.alloc(&d_R, NN));
-    k_rhs<<<(n + T - 1) / T, T, 0, st>>>(n, d_n2tp, d_n2t, d_tets, d_vol, d_grads, d_R);
+    const size_t NN = (size_t)n * n, NB = (size_t)n * nb;
+    double *d_RT, *d_rv;
+    BPM_TRY(pool.alloc(&d_RT, 3 * (size_t)nnz, false));
+    BPM_TRY(pool.alloc(&d_rv, 3 * (size_t)A.len, false));
+    k_source<<<gRow, T, 0, st>>>(n, d_rowptr, d_col, d_n2tp, d_n2t, d_tets, d_vol, d_grads, nnz, d_RT);
+    for (int c = 0; c < 3; ++c)
+        k_sliced_values<<<gS, T, 0, st>>>(A, d_srow, d_RT + (size_t)c * nnz, nullptr, nullptr,
+                                          d_rv + (size_t)c * A.len);
     BPM_CK(cudaGetLastError());
-    std::vector<double> dinvN(n), dinvD(n);
-    for (int i = 0; i < n; ++i) {
-        double kii = 0;
-        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e)
-            if (col[e] == i) kii = KLh[e];
-        dinvN[i] = 1.0 / kii;
-        dinvD[i] = interior[i] ? 1.0 / kii : 0.0;
-    }
-    BPM_TRY(upload(pool, &d_dinvN, dinvN));
-    BPM_TRY(upload(pool, &d_dinvD, dinvD));
-    BPM_TRY(pool.alloc(&d_U1, NN, false));
+    // the Laplacian scaled to a unit diagonal, whole and with interior rows and columns only
+    double *d_sc, *d_sc_in;
+    BPM_TRY(pool.alloc(&d_sc, n, false));
+    BPM_TRY(pool.alloc(&d_sc_in, n, false));
+    k_diag_scale<<<(n + T - 1) / T, T, 0, st>>>(n, d_rowptr, d_col, d_KL, d_int, d_sc, d_sc_in);
+    k_sliced_values<<<gS, T, 0, st>>>(A, d_srow, d_KL, d_sc, nullptr, d_sval);
+    k_sliced_values<<<gS, T, 0, st>>>(A, d_srow, d_KL, d_sc, d_int, d_sval_in);
+    BPM_CK(cudaGetLastError());
     int it1 = 0, it2 = 0;
     double res1 = 0, res2 = 0;
-    BPM_TRY(pcg(st, pool, n, ncol, d_rowptr, d_col, d_KL, nullptr, d_dinvN, d_R, d_U1, 1e-12, 20000, &it1, &res1));
-    k_col_mean_sub<<<(ncol + T - 1) / T, T, 0, st>>>(n, ncol, d_U1);
-    // boundary values of u2
-    double *d_omega, *d_Bmat, *d_U1B, *d_U2B, *d_U2e, *d_bD, *d_U2I;
-    BPM_TRY(pool.alloc(&d_omega, nb));
+    // G = K^+ for the nodal sources, zero-mean gauge
+    double *d_b, *d_G;
+    BPM_TRY(pool.alloc(&d_b, NN, false));
+    BPM_TRY(pool.alloc(&d_G, NN, false));
+    k_unit_sources<<<dim3((n + 127) / 128, n), 128, 0, st>>>(n, d_b);
+    BPM_TRY(pcg(st, pool, n, n, A, d_sval, d_sc, d_b, d_G, 1e-12, 20000, &it1, &res1));
+    k_col_mean_sub<<<(n + 31) / 32, 256, 0, st>>>(n, n, d_G);
+    // boundary values of u2 from u1
+    double *d_omega, *d_Bmat;
+    BPM_TRY(pool.alloc(&d_omega, nb, false));
     BPM_TRY(pool.alloc(&d_Bmat, (size_t)nb * nb, false));
-    BPM_TRY(pool.alloc(&d_U1B, (size_t)nb * ncol, false));
-    BPM_TRY(pool.alloc(&d_U2B, (size_t)nb * ncol, false));
     k_interior_angles<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_bnodes, d_n2tp, d_n2t, d_tets, d_xyz, d_omega);
-    k_bem_matrix<<<dim3((nb + 127) / 128, nb), 128, 0, st>>>(nb, d_bnodes, d_xyz, d_faces, d_b2fp, d_b2f,
-                                                             d_omega, d_Bmat);
-    k_gather_rows<<<dim3((ncol + 127) / 128, nb), 128, 0, st>>>(nb, ncol, d_bnodes, d_U1, d_U1B);
-    k_dgemm<<<dim3((ncol + 31) / 32, (nb + 31) / 32), dim3(32, 8), 0, st>>>(nb, ncol, nb, d_Bmat, d_U1B, d_U2B);
-    BPM_CK(cudaGetLastError());
-    // harmonic extension: K_II u2_I = -K_IB u2_B
-    BPM_TRY(pool.alloc(&d_U2e, NN));
-    BPM_TRY(pool.alloc(&d_bD, NN, false));
-    BPM_TRY(pool.alloc(&d_U2I, NN));
-    k_scatter_rows<<<dim3((ncol + 127) / 128, nb), 128, 0, st>>>(nb, ncol, d_bnodes, d_U2B, d_U2e);
-    k_spmm<<<dim3((ncol + 127) / 128, n), 128, 0, st>>>(n, ncol, d_rowptr, d_col, d_KL, nullptr, d_U2e, d_bD);
-    k_masked_scale<<<(unsigned)((NN + T - 1) / T), T, 0, st>>>(n, ncol, d_int, -1.0, d_bD);
-    BPM_CK(cudaGetLastError());
-    if (nb < n)
-        BPM_TRY(pcg(st, pool, n, ncol, d_rowptr, d_col, d_KL, d_int, d_dinvD, d_bD, d_U2I, 1e-12, 20000, &it2,
-                    &res2));
-    // u = u1 + u2 ; N = P u
+    {   // observers in blocks whose weights stay within 256 MB
+        double* d_W;
+        const int rows = std::max(1, std::min(nb, (int)((size_t(256) << 20) / (3 * sizeof(double) * (size_t)nf))));
+        BPM_TRY(pool.alloc(&d_W, 3 * (size_t)rows * nf, false));
+        for (int i0 = 0; i0 < nb; i0 += rows) {
+            const int m = std::min(rows, nb - i0);
+            k_bem_weights<<<dim3((nf + 127) / 128, m), 128, 0, st>>>(i0, m, nf, d_bnodes, d_xyz, d_faces, d_W);
+            k_bem_matrix<<<dim3((nb + 127) / 128, m), 128, 0, st>>>(i0, nb, nf, d_bnodes, d_faces, d_b2fp, d_b2f,
+                                                                    d_omega, d_W, d_Bmat);
+        }
+    }
+    // harmonic extension E of unit boundary values: K_II E_I = -K_IB, identity on the boundary
+    double *d_bD, *d_E, *d_F, *d_GB;
+    int* d_bidx;
+    BPM_TRY(upload(pool, &d_bidx, bidx));
+    BPM_TRY(pool.alloc(&d_bD, NB));
+    BPM_TRY(pool.alloc(&d_E, NB));
+    if (nb < n) {
+        k_boundary_sources<<<gRow, T, 0, st>>>(n, nb, d_rowptr, d_col, d_KL, d_int, d_bidx, d_bD);
+        BPM_TRY(pcg(st, pool, n, nb, A, d_sval_in, d_sc_in, d_bD, d_E, 1e-12, 20000, &it2, &res2));
+    }
+    k_boundary_identity<<<(nb + T - 1) / T, T, 0, st>>>(nb, d_bnodes, d_E);
+    // Q = G + (E B) G_boundary: potential u1 + u2 of the nodal sources
+    BPM_TRY(pool.alloc(&d_F, NB, false));
+    BPM_TRY(pool.alloc(&d_GB, (size_t)nb * n, false));
+    const dim3 gemm_threads(32, 8);
+    k_gather_rows<<<dim3((n + 127) / 128, nb), 128, 0, st>>>(nb, n, d_bnodes, d_G, d_GB);
+    k_dgemm<<<dim3((nb + 31) / 32, (n + 31) / 32), gemm_threads, 0, st>>>(n, nb, nb, d_E, d_Bmat, 0, d_F);
+    k_dgemm<<<dim3((n + 31) / 32, (n + 31) / 32), gemm_threads, 0, st>>>(n, n, nb, d_F, d_GB, 1, d_G);
+    // U = Q R, N = P U
     double *d_U, *d_P;
-    BPM_TRY(pool.alloc(&d_U, NN, false));
-    k_add3<<<(unsigned)((NN + T - 1) / T), T, 0, st>>>(NN, d_U1, d_U2e, d_U2I, d_U);
-    BPM_TRY(pool.alloc(&d_P, 3 * (size_t)nnz));
-    k_proj_values<<<(n + T - 1) / T, T, 0, st>>>(n, d_rowptr, d_col, d_n2tp, d_n2t, d_tets, d_vol, d_grads, d_V,
-                                                 nnz, d_P);
+    BPM_TRY(pool.alloc(&d_U, (size_t)n * ncol, false));
+    BPM_TRY(pool.alloc(&d_P, 3 * (size_t)nnz, false));
+    k_apply_source<<<dim3((n + 127) / 128, n), 128, 0, st>>>(n, A, d_rv, d_G, d_U);
+    k_proj_values<<<gRow, T, 0, st>>>(n, d_rowptr, d_col, d_n2tp, d_n2t, d_tets, d_vol, d_grads, d_V, nnz, d_P);
     BPM_CK(cudaGetLastError());
     double* N64 = nullptr;
     BPM_CK(cudaMalloc(&N64, (size_t)ncol * ncol * sizeof(double)));
@@ -854,6 +1181,9 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     BPM_CK(cudaMalloc(&M->Nlo, (size_t)K * K * sizeof(__nv_bfloat16)));
     k_demag_convert<<<dim3((K + 127) / 128, K), 128, 0, st>>>(n, M->n_pad, K, N64, M->N32, M->Nhi, M->Nlo);
     BPM_CK(cudaGetLastError());
+    double lam = 0;
+    BPM_TRY(side.join(st));
+    BPM_CK(cudaMemcpyAsync(&lam, d_lam, sizeof(double), cudaMemcpyDeviceToHost, st));
     BPM_CK(cudaStreamSynchronize(st));
     if (!(flags & BPM_MESH_KEEP_F64)) {
         cudaFree(M->N64);
