@@ -345,14 +345,15 @@ enum { BPM_RASTER_AUTO = 0, BPM_RASTER_M = 1, BPM_RASTER_N = 2 };
  * gemm_k_block 32, gemm_pair 0, and streams 2 for a one-mesh batch, 1 for a
  * multi-mesh batch (the fastest on the census and uneven batches measured). */
 typedef struct {
-    int32_t gemm_tile_n;     /* output columns per demag-GEMM CTA: 256 or 128 */
+    int32_t gemm_tile_n;     /* islands per demag-GEMM tile at most: 256 or 128 (the library takes
+                                narrower tiles where wide ones would leave SMs idle) */
     int32_t stage_threads;   /* threads per Heun-stage CTA: 128, 256 or 512 */
     int32_t gemm_raster;     /* BPM_RASTER_*: tile order of the tensor-core GEMM */
     int32_t stage_islands;   /* islands per Heun-stage CTA: 1 (0 = 1), or 2 with 256 threads */
     int32_t gemm_k_block;    /* K depth of a tensor-core GEMM pipeline stage: 32 (0 = 32) or 64 */
     int32_t gemm_pair;       /* 1: 256 x 256 GEMM tiles on the two SMs of a CTA pair (tcgen05
-                                cta_group::2; needs gemm_tile_n 256), 0: 128 x gemm_tile_n tiles
-                                on one SM */
+                                cta_group::2; needs gemm_tile_n 256), 0: tiles of 128 operator rows
+                                by up to gemm_tile_n islands on one SM */
     int32_t streams;         /* 2 .. 4: the interval graph integrates the batch as up to that many
                                 chains, each on its own stream, so that one chain's GEMM overlaps
                                 another chain's stage kernels: a one-mesh batch cut into chunks of

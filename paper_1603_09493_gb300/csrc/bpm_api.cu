@@ -110,6 +110,7 @@ using namespace bpm;
 struct Group {
     Mesh* mesh = nullptr;
     int B = 0, Bp = 0;
+    int splits = 1;               // planes of Hd: slices of the tensor-core demag product's K
     std::vector<int> user_idx;    // batch island index of each group row
     int* d_idx = nullptr;
     float4* isl = nullptr;
@@ -183,10 +184,13 @@ int setup_grouped_gemm(bpm_batch* bt) {
     std::vector<GemmOperands> ops;
     for (auto& g : bt->groups) {
         const int K = g.mesh->K();
-        ops.push_back(GemmOperands{g.Ahi, g.Alo, g.mesh->Nhi, g.mesh->Nlo, g.Hd, g.Bp, K, K});
+        ops.push_back(GemmOperands{g.Ahi, g.Alo, g.mesh->Nhi, g.mesh->Nlo, g.Hd, g.B, g.Bp, K, K, g.splits,
+                                   (size_t)g.Bp * K});
+        g.args.hd_planes = bt->pair ? 1 : g.splits;   // the CTA-pair kernel does not slice K
+        g.args.hd_plane = (size_t)g.Bp * K;
     }
     return grouped_gemm_setup(&bt->gg, ops, bt->tile_n, bt->p.precision == BPM_PREC_BF16X3 ? 3 : 1, bt->raster,
-                              bt->k_block, bt->ctx->l2_bytes, bt->pair);
+                              bt->k_block, bt->ctx->sm_count, bt->pair);
 }
 
 // The chains of a multi-stream batch: the one group's islands cut into `streams` chunks of a
@@ -215,6 +219,8 @@ int setup_chains(bpm_batch* bt) {
             return BPM_ERR_CUDA;
         }
     const int products = bt->p.precision == BPM_PREC_BF16X3 ? 3 : 1;
+    // the chains' products run side by side: each picks its tiles for its share of the SMs (tiles for
+    // all of them made 1024 census islands 27 % slower)
     if (ng > 1) {
         // a multi-mesh batch: its groups dealt to the chains, largest GEMM first, each to the chain
         // with the least GEMM work so far (rows x K^2)
@@ -233,10 +239,11 @@ int setup_chains(bpm_batch* bt) {
             for (int i : bt->chain_groups[c]) {
                 const Group& q = bt->groups[i];
                 const int K = q.mesh->K();
-                ops.push_back(GemmOperands{q.Ahi, q.Alo, q.mesh->Nhi, q.mesh->Nlo, q.Hd, q.Bp, K, K});
+                ops.push_back(GemmOperands{q.Ahi, q.Alo, q.mesh->Nhi, q.mesh->Nlo, q.Hd, q.B, q.Bp, K, K, q.splits,
+                                           (size_t)q.Bp * K});
             }
             BPM_TRY(grouped_gemm_setup(&bt->gg_chain[c], ops, bt->tile_n, products, bt->raster, bt->k_block,
-                                       bt->ctx->l2_bytes, bt->pair));
+                                       bt->ctx->sm_count, bt->pair, chains));
         }
         bt->chains = chains;
         return BPM_OK;
@@ -245,12 +252,12 @@ int setup_chains(bpm_batch* bt) {
     const int K = g.mesh->K();
     for (int c = 0; c < chains; ++c) {
         const int b0 = c * chunk;
-        const int rows = c + 1 < chains ? chunk : g.Bp - b0;   // the last chunk's GEMM covers the padding
+        const int rows = c + 1 < chains ? chunk : g.Bp - b0;
         const size_t off = (size_t)b0 * K, S = (size_t)b0 * 3 * g.mesh->n_pad;
         std::vector<GemmOperands> ops{GemmOperands{g.Ahi + off, g.Alo + off, g.mesh->Nhi, g.mesh->Nlo, g.Hd + off,
-                                                   rows, K, K}};
+                                                   std::min(chunk, g.B - b0), rows, K, K, g.splits, 0}};
         BPM_TRY(grouped_gemm_setup(&bt->gg_chain[c], ops, bt->tile_n, products, bt->raster, bt->k_block,
-                                   bt->ctx->l2_bytes, bt->pair));
+                                   bt->ctx->sm_count, bt->pair, chains));
         StepArgs a = g.args;
         a.B = std::min(chunk, g.B - b0);
         a.isl += 3 * (size_t)b0;
@@ -878,7 +885,8 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
         chk(dalloc(&g.isl, 3 * (size_t)g.B));
         chk(dalloc(&g.m, S));
         chk(dalloc(&g.k1, S));
-        chk(dalloc(&g.Hd, S));
+        if (tensor_core_precision(bt)) g.splits = gemm_splits(g.B, M->K(), ctx->sm_count);
+        chk(dalloc(&g.Hd, g.splits * S));
         if (p->precision == BPM_PREC_FP32) {
             chk(dalloc(&g.A32, S));
         } else {
@@ -928,6 +936,7 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
         a.m = g.m;
         a.k1 = g.k1;
         a.Hd = g.Hd;
+        a.hd_planes = 1;
         a.A32 = g.A32;
         a.Ahi = g.Ahi;
         a.Alo = g.Alo;

@@ -2,23 +2,39 @@
 //
 // One launch computes, for every mesh group g of a batch (uneven mesh sizes),
 //   C_g[M_g][N_g] = sum of the BF16 split products of A_g[M_g][K_g] and W_g[N_g][K_g]^T
-// (3 products hi*hi + lo*hi + hi*lo, or 1), FP32 accumulate in TMEM.  The
-// 128 x TN output tiles of all groups form one list; each CTA (one per SM)
-// walks it with a stride of the grid size.  Within a group the tiles run
-// M-major or N-major (chosen per group), so that a wave of CTAs shares the
-// larger operand's rows in L2 and it is read from HBM once.  Warp roles:
-//   warp 0  one lane streams the k-blocks of every tile with TMA into a ring of
-//           shared-memory stages (the ring runs across tile boundaries);
-//   warp 1  allocates two TMEM accumulators; one lane issues the MMAs, tile i
+// (3 products hi*hi + lo*hi + hi*lo, or 1), FP32 accumulate in TMEM: M_g islands,
+// N_g = K_g operator rows.  The operator's rows are the MMA's M side (128 a tile),
+// the islands its N side, nb of them a tile, any multiple of 16 up to TN.  Island
+// counts are what varies (one island to thousands, ragged over design variants),
+// and an MMA costs nearly in proportion to N, so no tile computes padding beyond
+// 15 islands (with the islands on the M side a group of 135 took 256 rows: eight
+// design variants of 135 islands 35.1 ms an interval, 30.2 so).  A tile's accumulator holds operator rows in lanes, so a warp
+// stores 128 contiguous bytes of an island's field per instruction.
+//
+// A group of at most 128 islands has only N_g / 128 tiles, each a serial walk over
+// K.  Its K is cut into up to four slices (gemm_splits), each an item of its own
+// writing its own plane of C; the stage kernels add the planes in order.  The
+// slices depend on K alone, not on what else is in the batch.  One island of 209
+// nodes: 374 -> 172 us an interval of 6 steps; nine of 481 nodes: 689 -> 330 us of
+// 8 steps; 60 of 1547 nodes: 5.2 -> 2.7 ms of 28 steps.
+//
+// The items of all groups form one list; each CTA (one per SM) walks it with a
+// stride of the grid size.  Within a group the tiles run M-major or N-major (chosen
+// per group), so that a wave of CTAs shares the larger operand's rows in L2 and it
+// is read from HBM once.  Warp roles:
+//   warp 0  one lane streams the k-blocks of every item with TMA into a ring of
+//           shared-memory stages (the ring runs across item boundaries);
+//   warp 1  allocates two TMEM accumulators; one lane issues the MMAs, item i
 //           into accumulator i % 2;
 //   warps 2-5  read an accumulator back (tcgen05.ld) and store it, while the
-//           MMAs of the next tile run into the other accumulator.
+//           MMAs of the next item run into the other accumulator.
 // Per-group tensor maps live in a device array (64-byte aligned entries).
 // Every wait is bounded; on timeout the kernel raises the error flag, drains
 // its copies and MMAs, frees TMEM and exits, and later launches return at once.
 // The waits of normal progress take the launch's limit (wait_ns); the drains
 // always take the fixed limit, so that copies and MMAs land before shared
 // memory or TMEM is given up.
+#include <algorithm>
 #include <cstring>
 
 #include "bpm_tc_ptx.cuh"
@@ -32,10 +48,11 @@ using namespace tc;
 constexpr int kGThreads = 192;
 
 // KB: K depth of a stage (64: 128 B rows, 128-byte swizzle; 32: 64 B rows, 64-byte swizzle)
+// TN: islands per tile at most
 template <int P, int TN, int KB>
 struct GCfg {
-    static constexpr int A_BYTES = TM * KB * 2;
-    static constexpr int W_BYTES = TN * KB * 2;
+    static constexpr int W_BYTES = TM * KB * 2;
+    static constexpr int A_BYTES = TN * KB * 2;
     static constexpr int stage_bytes = (P == 3 ? 2 : 1) * (A_BYTES + W_BYTES);
     static constexpr int stages = (192 * 1024) / stage_bytes;
     static constexpr int smem = stages * stage_bytes + 1024 + 256;
@@ -53,13 +70,14 @@ __device__ __forceinline__ int find_group(const GemmGroupDev* __restrict__ G, in
     return g;
 }
 
-// output tile lt of group gg -> first row (M) and column (N)
-template <int TN>
-__device__ __forceinline__ void tile_origin(const GemmGroupDev& gg, int lt, int& m0, int& n0) {
+// item it of group gg -> first island, first operator row, k-slice
+__device__ __forceinline__ void item_origin(const GemmGroupDev& gg, int it, int& b0, int& r0, int& slice) {
+    slice = it % gg.splits;
+    const int lt = it / gg.splits;
     const int mt = gg.n_major ? lt % gg.tiles_m : lt / gg.tiles_n;
     const int nt = gg.n_major ? lt / gg.tiles_m : lt % gg.tiles_n;
-    m0 = mt * TM;
-    n0 = nt * TN;
+    b0 = mt * gg.nb;
+    r0 = nt * TM;
 }
 
 template <int P, int TN, int KB>
@@ -86,10 +104,10 @@ __global__ void __launch_bounds__(kGThreads, 1)
     auto acce_bar = [&](int a) { return bar0 + 8u * (2 * S + 2 + a); };
     const uint32_t done_bar = bar0 + 8u * (2 * S + 4);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + S * CF::stage_bytes + 8 * (2 * S + 5));
-    auto sAhi = [&](int s) { return base + s * CF::stage_bytes; };
-    auto sWhi = [&](int s) { return base + s * CF::stage_bytes + A_TILE; };
-    auto sAlo = [&](int s) { return base + s * CF::stage_bytes + A_TILE + W_TILE; };
-    auto sWlo = [&](int s) { return base + s * CF::stage_bytes + 2 * A_TILE + W_TILE; };
+    auto sWhi = [&](int s) { return base + s * CF::stage_bytes; };
+    auto sAhi = [&](int s) { return base + s * CF::stage_bytes + W_TILE; };
+    auto sWlo = [&](int s) { return base + s * CF::stage_bytes + W_TILE + A_TILE; };
+    auto sAlo = [&](int s) { return base + s * CF::stage_bytes + 2 * W_TILE + A_TILE; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -122,20 +140,21 @@ __global__ void __launch_bounds__(kGThreads, 1)
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
-            int m0, n0;
-            tile_origin<TN>(gg, t - gg.tile_begin, m0, n0);
-            const int nk = gg.K / KB;
-            for (int kb = 0; kb < nk; ++kb, ++kbg) {
+            int b0, r0, sl;
+            item_origin(gg, t - gg.tile_begin, b0, r0, sl);
+            const int kb1 = min(gg.K, (sl + 1) * gg.slice_k) / KB;
+            const uint32_t bytes = (P == 3 ? 2u : 1u) * (uint32_t)(W_TILE + gg.nb * KB * 2);
+            for (int kb = sl * gg.slice_k / KB; kb < kb1; ++kb, ++kbg) {
                 const int s = kbg % S;
                 if (kbg >= S) ok = mbar_wait(empty_bar(s), ((kbg / S) - 1) & 1, err, 11, true, wait_ns);
                 if (!ok) break;
-                mbar_expect_tx(full_bar(s), CF::stage_bytes);
+                mbar_expect_tx(full_bar(s), bytes);
                 const int kc = kb * KB;
-                tma_load_2d(sAhi(s), &gg.ahi, kc, m0, full_bar(s));
-                tma_load_2d(sWhi(s), &gg.whi, kc, n0, full_bar(s));
+                tma_load_2d(sWhi(s), &gg.whi, kc, r0, full_bar(s));
+                tma_load_2d(sAhi(s), &gg.ahi, kc, b0, full_bar(s));
                 if (P == 3) {
-                    tma_load_2d(sAlo(s), &gg.alo, kc, m0, full_bar(s));
-                    tma_load_2d(sWlo(s), &gg.wlo, kc, n0, full_bar(s));
+                    tma_load_2d(sWlo(s), &gg.wlo, kc, r0, full_bar(s));
+                    tma_load_2d(sAlo(s), &gg.alo, kc, b0, full_bar(s));
                 }
             }
         }
@@ -149,17 +168,16 @@ __global__ void __launch_bounds__(kGThreads, 1)
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++i) {
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
-            const int nk = gg.K / KB;
-            int m0, n0;
-            tile_origin<TN>(gg, t - gg.tile_begin, m0, n0);
-            // a ragged last column tile runs MMAs only as wide as its valid columns (N % 16 == 0)
-            const uint32_t idesc = idesc_n<TN>(min(TN, gg.N - n0));
+            int b0, r0, sl;
+            item_origin(gg, t - gg.tile_begin, b0, r0, sl);
+            const int kb0 = sl * gg.slice_k / KB, kb1 = min(gg.K, (sl + 1) * gg.slice_k) / KB;
+            const uint32_t idesc = idesc_n<TN>(gg.nb);
             const int a = i & 1;
             if (i >= 2) ok = mbar_wait(acce_bar(a), ((i >> 1) - 1) & 1, err, 13, true, wait_ns);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = tmem + (uint32_t)(a * TN);
-            for (int kb = 0; kb < nk; ++kb, ++kbg) {
+            for (int kb = kb0; kb < kb1; ++kb, ++kbg) {
                 const int s = kbg % S;
                 ok = mbar_wait(full_bar(s), (kbg / S) & 1, err, 14, true, wait_ns);
                 if (!ok) break;
@@ -168,11 +186,11 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 for (int k = 0; k < KB / 16; ++k) {
                     const uint32_t koff = 32u * k;    // 16 BF16 further along the swizzled row
                     const uint64_t ahi = kmajor_desc<KB>(sAhi(s) + koff), whi = kmajor_desc<KB>(sWhi(s) + koff);
-                    mma_bf16_desc(acc, ahi, whi, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                    mma_bf16_desc(acc, whi, ahi, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
                     if (P == 3) {
                         const uint64_t alo = kmajor_desc<KB>(sAlo(s) + koff), wlo = kmajor_desc<KB>(sWlo(s) + koff);
-                        mma_bf16_desc(acc, alo, whi, idesc, 1u);
-                        mma_bf16_desc(acc, ahi, wlo, idesc, 1u);
+                        mma_bf16_desc(acc, whi, alo, idesc, 1u);
+                        mma_bf16_desc(acc, wlo, ahi, idesc, 1u);
                     }
                 }
                 mma_commit(empty_bar(s));
@@ -187,27 +205,25 @@ __global__ void __launch_bounds__(kGThreads, 1)
         for (int t = blockIdx.x; t < total_tiles; t += gridDim.x, ++i) {
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
-            int m0, n0;
-            tile_origin<TN>(gg, t - gg.tile_begin, m0, n0);
+            int b0, r0, sl;
+            item_origin(gg, t - gg.tile_begin, b0, r0, sl);
             const int a = i & 1;
             const bool have = mbar_wait(accf_bar(a), (i >> 1) & 1, err, 15, true, wait_ns);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int go = __shfl_sync(0xffffffffu, (have && *(volatile int*)err == 0) ? 1 : 0, 0);
             if (!go) break;
-            const int row = m0 + q * 32 + lane;
+            const int row = r0 + q * 32 + lane;             // operator row = column of C
+            const int nv = min(gg.nb, gg.M - b0);           // islands of this tile
+            float* dst = gg.C + (size_t)sl * gg.plane + (size_t)b0 * gg.ldc + row;
             const uint32_t lane_addr = tmem + (uint32_t)(a * TN) + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
-            for (int c = 0; c < TN && n0 + c < gg.N; c += 32) {   // columns past N were not computed
+            for (int c = 0; c < nv; c += 32, dst += 32 * (size_t)gg.ldc) {   // (a last 32 may read past nb: unused)
                 uint32_t r[32];
                 tmem_ld32(lane_addr + (uint32_t)c, r);
-                const int col = n0 + c;
-                if (row < gg.M && col < gg.N) {
-                    float4* dst = reinterpret_cast<float4*>(gg.C + (size_t)row * gg.ldc + col);
+                if (row < gg.N) {
 #pragma unroll
-                    for (int v = 0; v < 8; ++v)
-                        if (col + 4 * v < gg.N)
-                            dst[v] = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
-                                                 __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
+                    for (int v = 0; v < 32; ++v)
+                        if (c + v < nv) dst[(size_t)v * gg.ldc] = __uint_as_float(r[v]);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -244,8 +260,64 @@ int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err
 
 }  // namespace
 
+int gemm_splits(int islands, int K, int sm_count) {
+    if (islands > 128) return 1;
+    const int tiles = (K + tc::TM - 1) / tc::TM, kb = K / tc::TK;
+    // slices of at least three k-blocks, at most four (the consumers read every plane), no more items than SMs
+    const int want = std::max(1, std::min({4, sm_count / tiles, (kb + 2) / 3}));
+    const int per = (kb + want - 1) / want;
+    return (kb + per - 1) / per;
+}
+
+namespace {
+
+// Time of an MMA of nb islands relative to a 256-wide one's 256: N / 2 cycles of tensor work, or the
+// 128 operator rows and nb island rows of 32 B that it reads from shared memory at 128 B a cycle
+int mma_cost(int nb) { return std::max(nb, 64 + nb / 2); }
+
+// Islands per tile of a group of M islands when no tile may exceed cap: even tiles, a multiple of 16
+int even_tile(int M, int cap) {
+    const int t = (M + cap - 1) / cap;
+    return (((M + t - 1) / t) + 15) / 16 * 16;
+}
+
+// The widest tiles that do not leave SMs idle: over caps of 256 .. 16 islands, the time of the busiest
+// SM as waves of items x cost of an item (k-steps x MMA cost, an item's fixed cost as 12 k-steps).
+// Wide tiles win ties.  One island of 1547 nodes: 148 items of a quarter of K; 200 islands: 148 items
+// of 64 (60 us against 81 with two 128-row tiles); 4096: 608 items of 256 in four waves.
+// share > 1: the product runs beside share - 1 others on as many streams.  It then aims at its share of
+// the SMs, in no whole waves (an SM takes the others' work next), and at a tenth of gain: more CTAs
+// would only hold up the others (4096 islands of 481 nodes: 1.79 ms an interval with 120 items of 208
+// a chain, 1.60 with 96 of 256).
+int tile_cap(const std::vector<GemmOperands>& ops, int tile_n, int sm_count, int share) {
+    int best = tile_n;
+    double best_t = 1e300;
+    for (int cap : {256, 208, 160, 128, 96, 64, 48, 32, 16}) {
+        if (cap > tile_n) continue;
+        long long items = 0;
+        double sum = 0, top = 0;
+        for (const GemmOperands& o : ops) {
+            const int nb = even_tile(o.M, cap);
+            const long long it = (long long)((o.M + nb - 1) / nb) * ((o.N + tc::TM - 1) / tc::TM) * o.splits;
+            const double c = (double)mma_cost(nb) * (o.K / 16.0 / o.splits + 12.0);
+            items += it;
+            sum += it * c;
+            top = std::max(top, c);
+        }
+        const double waves = (double)items * share / sm_count;
+        const double t = std::max(top, (share > 1 ? waves : std::ceil(waves)) * sum / (double)items);
+        if (t < best_t * (share > 1 ? 0.9 : 0.98)) {
+            best_t = t;
+            best = cap;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
 int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, int tile_n, int products, int raster,
-                       int k_block, size_t l2_bytes, int pair) {
+                       int k_block, int sm_count, int pair, int share) {
     if (pair && tile_n != 256) {
         set_error("the CTA-pair GEMM computes 256 x 256 tiles (tile_n 256)");
         return BPM_ERR_ARG;
@@ -263,47 +335,53 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
         return BPM_ERR_ARG;
     }
     std::vector<GemmGroupDev> h(ops.size());
-    int tiles = 0;
+    int tiles = 0, nb_max = 16;
+    const int cap = tile_cap(ops, tile_n, sm_count, share);
     for (size_t g = 0; g < ops.size(); ++g) {
         const GemmOperands& o = ops[g];
-        if (o.M % tc::TM || o.K % tc::TK || o.N % 16 || o.M <= 0 || o.N <= 0) {
-            set_error("grouped GEMM group %zu: M %% 128, K %% 64, N %% 16 required (M=%d N=%d K=%d)", g, o.M, o.N,
-                      o.K);
+        if (o.rows % tc::TM || o.K % tc::TK || o.N % 16 || o.M <= 0 || o.M > o.rows || o.N <= 0 || o.splits < 1) {
+            set_error("grouped GEMM group %zu: rows %% 128, K %% 64, N %% 16 required (M=%d rows=%d N=%d K=%d)", g,
+                      o.M, o.rows, o.N, o.K);
             return BPM_ERR_ARG;
         }
         std::memset(&h[g], 0, sizeof(GemmGroupDev));
-        // a CTA of a pair stages 128 of the tile's 256 W rows
-        const int w_box = pair ? tile_n / 2 : tile_n;
-        BPM_TRY(make_bf16_tensor_map(&h[g].ahi, o.Ahi, o.K, o.M, tc::TM, k_block));
-        BPM_TRY(make_bf16_tensor_map(&h[g].whi, o.Whi, o.K, o.N, w_box, k_block));
+        const int nb = even_tile(o.M, cap);
+        nb_max = std::max(nb_max, nb);
+        // a CTA of a pair stages 128 of the tile's 256 rows of either operand
+        const int a_box = pair ? tc::TM : nb;
+        BPM_TRY(make_bf16_tensor_map(&h[g].ahi, o.Ahi, o.K, o.rows, a_box, k_block));
+        BPM_TRY(make_bf16_tensor_map(&h[g].whi, o.Whi, o.K, o.N, tc::TM, k_block));
         if (products == 3) {
-            BPM_TRY(make_bf16_tensor_map(&h[g].alo, o.Alo, o.K, o.M, tc::TM, k_block));
-            BPM_TRY(make_bf16_tensor_map(&h[g].wlo, o.Wlo, o.K, o.N, w_box, k_block));
+            BPM_TRY(make_bf16_tensor_map(&h[g].alo, o.Alo, o.K, o.rows, a_box, k_block));
+            BPM_TRY(make_bf16_tensor_map(&h[g].wlo, o.Wlo, o.K, o.N, tc::TM, k_block));
         } else {
             h[g].alo = h[g].ahi;
             h[g].wlo = h[g].whi;
         }
         h[g].C = o.C;
-        h[g].M = o.M;
+        h[g].M = pair ? o.rows : o.M;
         h[g].N = o.N;
         h[g].K = o.K;
         h[g].ldc = o.N;
-        h[g].tiles_m = pair ? (o.M + 2 * tc::TM - 1) / (2 * tc::TM) : o.M / tc::TM;
-        h[g].tiles_n = (o.N + tile_n - 1) / tile_n;
+        h[g].nb = nb;
+        h[g].splits = pair ? 1 : o.splits;
+        h[g].slice_k = (o.K / tc::TK + h[g].splits - 1) / h[g].splits * tc::TK;
+        h[g].plane = o.plane;
+        h[g].tiles_m = pair ? (o.rows + 2 * tc::TM - 1) / (2 * tc::TM) : (o.M + nb - 1) / nb;
+        h[g].tiles_n = (o.N + (pair ? 2 : 1) * tc::TM - 1) / ((pair ? 2 : 1) * tc::TM);
         h[g].tile_begin = tiles;
         // AUTO: N-major when the operator has more rows than the batch operand, so that the
         // larger operand is streamed once per launch and the smaller one re-read from L2
-        (void)l2_bytes;
         const bool auto_n = o.N > o.M;
         h[g].n_major = raster == BPM_RASTER_N || (raster == BPM_RASTER_AUTO && auto_n) ? 1 : 0;
-        tiles += h[g].tiles_m * h[g].tiles_n;
+        tiles += h[g].tiles_m * h[g].tiles_n * h[g].splits;
     }
     grouped_gemm_free(gg);
     BPM_CK(cudaMalloc(&gg->d_groups, h.size() * sizeof(GemmGroupDev)));
     BPM_CK(cudaMemcpy(gg->d_groups, h.data(), h.size() * sizeof(GemmGroupDev), cudaMemcpyHostToDevice));
     gg->n_groups = (int)h.size();
     gg->total_tiles = tiles;
-    gg->tile_n = tile_n;
+    gg->tile_n = nb_max <= 128 ? 128 : 256;
     gg->products = products;
     gg->k_block = k_block;
     gg->pair = pair;

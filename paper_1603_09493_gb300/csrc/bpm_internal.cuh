@@ -161,25 +161,34 @@ struct GemmGroupDev {   // CUtensorMap members carry the 64-byte alignment TMA n
     float* C;
     int M, N, K, ldc;
     int tiles_m, tiles_n;             // output tiles of this group along M and N
-    int tile_begin;                   // first tile of this group in the launch's list
+    int tile_begin;                   // first item of this group in the launch's list
     int n_major;                      // tile order: 1 = consecutive tiles share the W rows
+    int nb;                           // islands (rows of A) per tile
+    int splits, slice_k;              // slices of K, columns per slice; slice s writes C + s * plane
+    size_t plane;
 };
 struct GemmOperands {
     const __nv_bfloat16 *Ahi, *Alo, *Whi, *Wlo;
     float* C;
-    int M, N, K;
+    int M, rows, N, K;                // islands, rows of A (a multiple of 128, zeros from M on)
+    int splits;                       // planes of C (gemm_splits of the group)
+    size_t plane;                     // elements of a plane
 };
+// Slices of K of a group's demag product, from its island count (more than 128: one) and K.  The result
+// of a group then depends on nothing else in its batch or launch.
+int gemm_splits(int islands, int K, int sm_count);
 struct GroupedGemm {
     GemmGroupDev* d_groups = nullptr;
-    int n_groups = 0, total_tiles = 0, tile_n = 256, products = 3, k_block = 64;
+    int n_groups = 0, total_tiles = 0, tile_n = 256, products = 3, k_block = 64;   // tile_n: the kernel's widest tile
     unsigned long long wait_ns = 0;   // limit of the non-drain waits (0: the default)
     int pair = 0;                     // 1: 256 x 256 tiles on CTA pairs (tcgen05 cta_group::2)
     int max_pairs = 0;                // co-resident CTA pairs of the pair kernel (0: not yet queried)
 };
 // k_block: K depth of one pipeline stage, 64 (128-byte swizzle) or 32 (64-byte swizzle, twice the stages)
 // pair: 256 x 256 output tiles computed by the two CTAs of a cluster (bpm_gemm_pair.cu)
+// share: products that run side by side with this one, itself included (see tile_cap)
 int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, int tile_n, int products, int raster,
-                       int k_block, size_t l2_bytes, int pair = 0);
+                       int k_block, int sm_count, int pair = 0, int share = 1);
 int grouped_gemm_pair_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err);
 void grouped_gemm_free(GroupedGemm* gg);
 int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err);

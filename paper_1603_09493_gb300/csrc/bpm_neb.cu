@@ -102,7 +102,9 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     BPM_TRY(buf.alloc(&m0, S));
     BPM_TRY(buf.alloc(&m1, S));
     BPM_TRY(buf.alloc(&Bt, S));
-    BPM_TRY(buf.alloc(&Hd, G));
+    const bool tc = prec == BPM_PREC_BF16X3 || prec == BPM_PREC_BF16;
+    const int splits = tc ? gemm_splits(R, K, ctx->sm_count) : 1;   // planes of Hd
+    BPM_TRY(buf.alloc(&Hd, splits * G));
     if (prec == BPM_PREC_FP32) {
         BPM_TRY(buf.alloc(&A32, G));
     } else {
@@ -152,6 +154,8 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     a.moz = H ? H->origin[2] : 0.f;
     a.m = m0;
     a.Hd = Hd;
+    a.hd_planes = splits;
+    a.hd_plane = G;
     a.A32 = A32;
     a.Ahi = Ahi;
     a.Alo = Alo;
@@ -163,11 +167,10 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     a.ipb = 1;
 
     GroupedGemm gg;
-    const bool tc = prec == BPM_PREC_BF16X3 || prec == BPM_PREC_BF16;
     if (tc) {
-        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, Rp, K, K}};
+        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, R, Rp, K, K, splits, G}};
         int r = grouped_gemm_setup(&gg, ops, 256, prec == BPM_PREC_BF16X3 ? 3 : 1, BPM_RASTER_AUTO, 32,
-                                   ctx->l2_bytes);
+                                   ctx->sm_count);
         if (r != BPM_OK) {
             grouped_gemm_free(&gg);
             return r;

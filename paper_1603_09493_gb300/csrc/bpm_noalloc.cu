@@ -172,6 +172,7 @@ extern "C" int bpm_llg_advance_noalloc(bpm_ctx* ctx, const bpm_island* isl, int3
     a.k1 = reinterpret_cast<float*>(s8 + o_k1);
     float* hd = reinterpret_cast<float*>(s8 + o_hd);
     a.Hd = hd;
+    a.hd_planes = 1;
     a.A32 = reinterpret_cast<float*>(s8 + o_a);
     a.prec = BPM_PREC_FP32;
     a.mz_prev = reinterpret_cast<float*>(s8 + o_mzp);

@@ -90,6 +90,25 @@ __device__ __forceinline__ float3 trilinear(const StepArgs& a, float px, float p
     return acc;
 }
 
+// demag field of island b at node i: the planes of the product's K slices, added in order
+__device__ __forceinline__ float3 load_hd(const StepArgs& a, int b, int i) {
+    const float* hd = a.Hd + (size_t)b * a.kp + i;
+    float3 v = f3(__ldcg(hd), __ldcg(hd + a.n_pad), __ldcg(hd + 2 * a.n_pad));
+    if (a.hd_planes > 1) {
+        // at most four planes: all loads at once (a missing plane repeats the last and is dropped)
+        float3 w[3];
+#pragma unroll
+        for (int s = 1; s < 4; ++s) {
+            const float* p = hd + (size_t)min(s, a.hd_planes - 1) * a.hd_plane;
+            w[s - 1] = f3(__ldcg(p), __ldcg(p + a.n_pad), __ldcg(p + 2 * a.n_pad));
+        }
+#pragma unroll
+        for (int s = 1; s < 4; ++s)
+            if (s < a.hd_planes) v = v + w[s - 1];
+    }
+    return v;
+}
+
 // effective field at node i of island b from the source state staged in smem ([3][n_pad])
 __device__ __forceinline__ float3 eff_field(const StepArgs& a, int b, int i, float3 mi, const float* sm, float4 p0,
                                             float4 p1, float4 p2, float ramp, float xh, unsigned mask) {
@@ -97,10 +116,7 @@ __device__ __forceinline__ float3 eff_field(const StepArgs& a, int b, int i, flo
     const int np = a.n_pad;
     // independent per-node loads first, so that their latency overlaps the exchange gather
     float3 hdv = f3(0, 0, 0);
-    if (mask & BPM_TERM_DEMAG) {
-        const float* hd = a.Hd + (size_t)b * a.kp + i;
-        hdv = f3(__ldcg(hd), __ldcg(hd + np), __ldcg(hd + 2 * np));
-    }
+    if (mask & BPM_TERM_DEMAG) hdv = load_hd(a, b, i);
     const float4 pos = __ldg(a.node_pos + i);
     const float an0 = __ldg(&a.node_mat[i].x);
     if (mask & BPM_TERM_EXCHANGE) {
@@ -394,11 +410,6 @@ __device__ __forceinline__ float3 field_from_sums(const StepArgs& a, float3 mi, 
         B = B + ramp * f3(a.uni[0], a.uni[1], a.uni[2]) + f3(p2.y, p2.z, p2.w);
     }
     return B;
-}
-
-__device__ __forceinline__ float3 load_hd(const StepArgs& a, int b, int i) {
-    const float* hd = a.Hd + (size_t)b * a.kp + i;
-    return f3(__ldcg(hd), __ldcg(hd + a.n_pad), __ldcg(hd + 2 * a.n_pad));
 }
 
 // predictor of islands b0 .. b0 + nb - 1 (nb <= IPB); sp: [IPB][3] island parameters in smem

@@ -19,7 +19,9 @@ struct StepArgs {
     float mh, mox, moy, moz;
     float* m;                 // [Bp][3][n_pad]
     float* k1;                // predictor slope
-    const float* Hd;          // demag field of the GEMM input state, tesla, [Bp][kp]
+    const float* Hd;          // demag field of the GEMM input state, tesla, [Bp][kp]: the sum of
+    int hd_planes;            // hd_planes planes hd_plane elements apart (slices of the product's K)
+    size_t hd_plane;
     float* A32;               // GEMM input (FP32), [Bp][kp], Ms * m in MA/m (planes at c n_pad)
     __nv_bfloat16* Ahi;       // GEMM input BF16 hi/lo split
     __nv_bfloat16* Alo;

@@ -30,3 +30,30 @@ def test_operators_of_small_meshes(ctx, rings, hard, soft):
     assert np.abs(N - ops.demag).max() <= 1e-9 * np.abs(ops.demag).max()
     assert abs(info["exchange_lambda_max_T"] - ops.exchange_lambda_max()) <= 1e-9 * ops.exchange_lambda_max()
     ctx.mesh_release(mid)
+
+
+@pytest.mark.parametrize("B", [1, 15, 17, 127, 128, 129, 145, 257])
+@pytest.mark.parametrize("nodes", ["209", "481"])
+def test_demag_product_tile_and_slice_edges(ctx, B, nodes):
+    """Island counts around the GEMM's tile steps (16 islands, 128 where K is no longer sliced, 256) on two operators
+    whose row count is (1536) and is not (704) a multiple of the 128-row tile: the demag field of the split product
+    against the CUDA-core evaluation of the same products, within one rounding of 2^-23 of the field scale per MMA."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    mesh = synth.small_island_mesh() if nodes == "209" else \
+        synth.layered_island_mesh(12.0, 6.0, 6.0, rings=3, hard_slabs=6, soft_slabs=6, seed=7)
+    mid = ctx.mesh_upload(mesh, synth.ecc_materials())
+    K = ctx.mesh_info(mid)["k_pad"]
+    isl = synth.jittered_islands(B, seed=B, mesh_id=mid)
+    p = synth.RunParams(dt_ps=0.1, substeps=1, term_mask=L.TERM_DEMAG)
+    rng = np.random.default_rng(B)
+    m = rng.standard_normal((B, 3, mesh.n_nodes)) * 0.3
+    m[:, 2] += 1.0
+    m = (m / np.linalg.norm(m, axis=1, keepdims=True)).astype(np.float32)
+    out = []
+    for prec in (L.PREC_BF16X3_REF, L.PREC_BF16X3):
+        with ctx.batch(isl, p, precision=prec) as bt:
+            bt.set_state(m, 0.0)
+            out.append(bt.field(0.0, L.TERM_DEMAG))
+    ctx.mesh_release(mid)
+    assert np.abs(out[1] - out[0]).max() <= (3 * K / 16) * 2.0 ** -23 * np.abs(out[0]).max()
