@@ -375,10 +375,42 @@ void launch_stage_all(bpm_batch* bt, const StageLaunches& L, int stage, int j, c
     }
 }
 
+// Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
+// tensor-core product on one stream, every island's CTA resident at once (at most four of 256 threads
+// an SM, two vectors of the state in shared memory each) and at most 3200 nodes an SM.  Beyond that the
+// two-island kernels on two streams, which share the exchange entries between islands, are as fast
+// (interval in us, this way / theirs: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 /
+// 590; 1547 nodes, 300 islands 4177 / 4774, 512 islands 5304 / 5030).  Fills *G.
+bool few_islands(const bpm_batch* bt, StageGroups* G) {
+    if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
+    const int per_sm = (bt->B + bt->ctx->sm_count - 1) / bt->ctx->sm_count;
+    std::memset(G, 0, sizeof(StageGroups));
+    size_t smem = 0;
+    int n = 0;
+    for (const auto& g : bt->groups) {
+        smem = std::max(smem, 2 * stage_smem_bytes(g.args));
+        n = std::max(n, g.mesh->n);
+        G->a[G->ng] = g.args;
+        G->block_begin[G->ng + 1] = G->block_begin[G->ng] + g.B;
+        ++G->ng;
+    }
+    return per_sm <= 4 && per_sm * n <= std::max(3200, n) && per_sm * (smem + 1024) <= 200 * 1024;
+}
+
 // one output interval of every group; groups of a multi-mesh batch are forked
 // over side streams so that their kernels can run concurrently
 int enqueue_interval(bpm_batch* bt, cudaStream_t s) {
-    if (bt->chains > 0) {
+    StageGroups few;
+    if (few_islands(bt, &few)) {
+        int n = 0;
+        for (const auto& g : bt->groups) n = std::max(n, g.mesh->n);
+        const int nt = few_threads(n, bt->B, bt->ctx->sm_count);
+        for (int j = 0; j < bt->p.substeps; ++j)
+            for (int k = 1; k <= 2; ++k) {
+                BPM_TRY(grouped_gemm_launch(s, bt->gg, bt->ctx->sm_count, bt->gemm_err, true));
+                BPM_TRY(launch_few(few, nt, k, j, s));
+            }
+    } else if (bt->chains > 0) {
         // one chain per chunk of islands: chunk 0 on s, chunk c on chain_stream[c - 1] (forked
         // from and joined into s); each chain runs the Heun steps of its own islands in order, so
         // one chain's GEMM can run while another chain's stage kernels do

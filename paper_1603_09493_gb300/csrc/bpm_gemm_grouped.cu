@@ -90,9 +90,13 @@ __global__ void __launch_bounds__(kGThreads, 1)
     extern __shared__ uint8_t smem_raw[];
     {   // an earlier launch gave up: skip (decided once per CTA, so that no thread is left at a barrier)
         __shared__ int s_abort;
+        pdl_trigger();
         if (threadIdx.x == 0) s_abort = *(volatile int*)err;
         __syncthreads();
-        if (s_abort) return;
+        if (s_abort) {
+            pdl_wait();
+            return;
+        }
     }
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -144,18 +148,32 @@ __global__ void __launch_bounds__(kGThreads, 1)
             item_origin(gg, t - gg.tile_begin, b0, r0, sl);
             const int kb1 = min(gg.K, (sl + 1) * gg.slice_k) / KB;
             const uint32_t bytes = (P == 3 ? 2u : 1u) * (uint32_t)(W_TILE + gg.nb * KB * 2);
-            for (int kb = sl * gg.slice_k / KB; kb < kb1; ++kb, ++kbg) {
+            int kb = sl * gg.slice_k / KB;
+            auto load_w = [&](int s, int kc) {
+                mbar_expect_tx(full_bar(s), bytes);
+                tma_load_2d(sWhi(s), &gg.whi, kc, r0, full_bar(s));
+                if (P == 3) tma_load_2d(sWlo(s), &gg.wlo, kc, r0, full_bar(s));
+            };
+            auto load_a = [&](int s, int kc) {
+                tma_load_2d(sAhi(s), &gg.ahi, kc, b0, full_bar(s));
+                if (P == 3) tma_load_2d(sAlo(s), &gg.alo, kc, b0, full_bar(s));
+            };
+            if (t == blockIdx.x) {
+                // the first ring of operator tiles, which no kernel writes, ahead of the wait for the
+                // kernel that writes the islands' operand
+                const int pre = min(S, kb1 - kb);
+                for (int s = 0; s < pre; ++s) load_w(s, (kb + s) * KB);
+                pdl_wait();
+                for (int s = 0; s < pre; ++s) load_a(s, (kb + s) * KB);
+                kb += pre;
+                kbg = pre;
+            }
+            for (; kb < kb1; ++kb, ++kbg) {
                 const int s = kbg % S;
                 if (kbg >= S) ok = mbar_wait(empty_bar(s), ((kbg / S) - 1) & 1, err, 11, true, wait_ns);
                 if (!ok) break;
-                mbar_expect_tx(full_bar(s), bytes);
-                const int kc = kb * KB;
-                tma_load_2d(sWhi(s), &gg.whi, kc, r0, full_bar(s));
-                tma_load_2d(sAhi(s), &gg.ahi, kc, b0, full_bar(s));
-                if (P == 3) {
-                    tma_load_2d(sWlo(s), &gg.wlo, kc, r0, full_bar(s));
-                    tma_load_2d(sAlo(s), &gg.alo, kc, b0, full_bar(s));
-                }
+                load_w(s, kb * KB);
+                load_a(s, kb * KB);
             }
         }
         // drain: the last armed phase of every stage must land before exit
@@ -201,6 +219,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     } else if (warp >= 2) {
         // ---------------- epilogue warps ----------------
         const int q = warp & 3;    // TMEM lane quarter this warp may access
+        pdl_wait();                // C may still be read by the kernel before
         int i = 0;
         for (int t = blockIdx.x; t < total_tiles; t += gridDim.x, ++i) {
             const int g = find_group(G, ng, t);
@@ -243,7 +262,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
 }
 
 template <int P, int TN, int KB>
-int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err) {
+int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err, bool pdl) {
     static bool configured = false;
     if (!configured) {
         BPM_CK(cudaFuncSetAttribute(k_gemm_grouped<P, TN, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -251,9 +270,8 @@ int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err
         configured = true;
     }
     const int grid = std::max(1, std::min(gg.total_tiles, sm_count));
-    k_gemm_grouped<P, TN, KB>
-        <<<grid, kGThreads, GCfg<P, TN, KB>::smem, s>>>(gg.d_groups, gg.n_groups, gg.total_tiles, err,
-                                                        gg.wait_ns ? gg.wait_ns : kWaitNs);
+    BPM_CK(launch_pdl(k_gemm_grouped<P, TN, KB>, dim3(grid), dim3(kGThreads), GCfg<P, TN, KB>::smem, s, pdl,
+                      gg.d_groups, gg.n_groups, gg.total_tiles, err, gg.wait_ns ? gg.wait_ns : kWaitNs));
     BPM_CK(cudaGetLastError());
     return BPM_OK;
 }
@@ -394,7 +412,7 @@ void grouped_gemm_free(GroupedGemm* gg) {
     gg->n_groups = gg->total_tiles = 0;
 }
 
-int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err) {
+int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err, bool pdl) {
     if (!gg.d_groups) {
         set_error("grouped GEMM not set up");
         return BPM_ERR_STATE;
@@ -402,16 +420,16 @@ int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err)
     if (gg.pair) return grouped_gemm_pair_launch(s, gg, sm_count, err);
     if (gg.k_block == 32) {
         if (gg.products == 3)
-            return gg.tile_n == 128 ? launch_grouped<3, 128, 32>(s, gg, sm_count, err)
-                                    : launch_grouped<3, 256, 32>(s, gg, sm_count, err);
-        return gg.tile_n == 128 ? launch_grouped<1, 128, 32>(s, gg, sm_count, err)
-                                : launch_grouped<1, 256, 32>(s, gg, sm_count, err);
+            return gg.tile_n == 128 ? launch_grouped<3, 128, 32>(s, gg, sm_count, err, pdl)
+                                    : launch_grouped<3, 256, 32>(s, gg, sm_count, err, pdl);
+        return gg.tile_n == 128 ? launch_grouped<1, 128, 32>(s, gg, sm_count, err, pdl)
+                                : launch_grouped<1, 256, 32>(s, gg, sm_count, err, pdl);
     }
     if (gg.products == 3)
-        return gg.tile_n == 128 ? launch_grouped<3, 128, 64>(s, gg, sm_count, err)
-                                : launch_grouped<3, 256, 64>(s, gg, sm_count, err);
-    return gg.tile_n == 128 ? launch_grouped<1, 128, 64>(s, gg, sm_count, err)
-                            : launch_grouped<1, 256, 64>(s, gg, sm_count, err);
+        return gg.tile_n == 128 ? launch_grouped<3, 128, 64>(s, gg, sm_count, err, pdl)
+                                : launch_grouped<3, 256, 64>(s, gg, sm_count, err, pdl);
+    return gg.tile_n == 128 ? launch_grouped<1, 128, 64>(s, gg, sm_count, err, pdl)
+                            : launch_grouped<1, 256, 64>(s, gg, sm_count, err, pdl);
 }
 
 }  // namespace bpm

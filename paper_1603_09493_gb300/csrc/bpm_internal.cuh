@@ -102,6 +102,29 @@ struct HeadMap {
     double max_norm = 0;          // largest |B| of a voxel (T)
 };
 
+// Launch with programmatic stream serialization (pdl): the kernel may start while its predecessor on
+// the stream still runs, once every CTA of that one has called pdl_trigger(), and waits for its
+// completion in pdl_wait().  Before pdl_wait() it touches nothing that a kernel in flight writes, and
+// every CTA of it passes pdl_wait(), so that its own completion implies that of everything before it.
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
 struct Mlp;
 void free_mlp(Mlp* m);
 struct Gp;
@@ -191,7 +214,8 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
                        int k_block, int sm_count, int pair = 0, int share = 1);
 int grouped_gemm_pair_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err);
 void grouped_gemm_free(GroupedGemm* gg);
-int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err);
+// pdl: programmatic launch behind the kernel that wrote the operand (see launch_pdl)
+int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err, bool pdl = false);
 // TMA map of a row-major BF16 [rows][inner] matrix, boxes of box_rows x box_inner (64 or 32)
 int make_bf16_tensor_map(CUtensorMap* map, const void* ptr, int inner, int rows, int box_rows, int box_inner = 64);
 

@@ -109,9 +109,11 @@ __device__ __forceinline__ float3 load_hd(const StepArgs& a, int b, int i) {
     return v;
 }
 
-// effective field at node i of island b from the source state staged in smem ([3][n_pad])
+// effective field at node i of island b from the source state staged in smem ([3][n_pad]); head: the
+// head field there, where the caller has it
 __device__ __forceinline__ float3 eff_field(const StepArgs& a, int b, int i, float3 mi, const float* sm, float4 p0,
-                                            float4 p1, float4 p2, float ramp, float xh, unsigned mask) {
+                                            float4 p1, float4 p2, float ramp, float xh, unsigned mask,
+                                            const float3* head = nullptr) {
     float3 B = f3(0, 0, 0);
     const int np = a.n_pad;
     // independent per-node loads first, so that their latency overlaps the exchange gather
@@ -143,7 +145,7 @@ __device__ __forceinline__ float3 eff_field(const StepArgs& a, int b, int i, flo
     }
     if (mask & BPM_TERM_DEMAG) B = B + hdv;
     if ((mask & BPM_TERM_HEAD) && a.map) {
-        B = B + ramp * trilinear(a, pos.x + p1.w - xh, pos.y + p2.x, pos.z);
+        B = B + ramp * (head ? *head : trilinear(a, pos.x + p1.w - xh, pos.y + p2.x, pos.z));
     }
     if (mask & BPM_TERM_UNIFORM) {
         B = B + ramp * f3(a.uni[0], a.uni[1], a.uni[2]) + f3(p2.y, p2.z, p2.w);
@@ -222,6 +224,19 @@ __device__ __forceinline__ void set_clock(StageClock& c, const StepArgs& a, int 
     c.xh = a.x0 + a.v_nm_ps * (float)t;
 }
 
+// switch detector of island b after the step that ends at t with <m_z> = mz (one thread)
+__device__ __forceinline__ void detect_switch(const StepArgs& a, int b, float mz, double t) {
+    const float prev = a.mz_prev[b];
+    if (!a.crossed[b] && mz <= 0.f) {
+        const double d = (double)prev - (double)mz;
+        const double frac = d > 0 ? (double)prev / d : 1.0;
+        a.t_sw[b] = (float)(t - a.h + a.h * frac);
+        a.crossed[b] = 1;
+    }
+    a.mz_prev[b] = mz;
+    if (!isfinite(mz)) a.status[b] |= BPM_ISLAND_NONFINITE;
+}
+
 // predictor of island b (one CTA)
 __device__ __forceinline__ void stage1_body(const StepArgs& a, int b, int j) {
     extern __shared__ float4 smem4[];
@@ -276,15 +291,7 @@ __device__ __forceinline__ void stage2_body(const StepArgs& a, int b, int j, flo
     }
     float mz = block_reduce(mzp, red);
     if (threadIdx.x == 0) {
-        float prev = a.mz_prev[b];
-        if (!a.crossed[b] && mz <= 0.f) {
-            double d = (double)prev - (double)mz;
-            double frac = d > 0 ? (double)prev / d : 1.0;
-            a.t_sw[b] = (float)(clk.t - a.h + a.h * frac);
-            a.crossed[b] = 1;
-        }
-        a.mz_prev[b] = mz;
-        if (!isfinite(mz)) a.status[b] |= BPM_ISLAND_NONFINITE;
+        detect_switch(a, b, mz, clk.t);
     }
 }
 
@@ -517,16 +524,102 @@ __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, f
         const int q = threadIdx.x, b = b0 + q;
         float mz = 0.f;
         for (int w = 0; w < nw; ++w) mz += red[q * nw + w];
-        float prev = a.mz_prev[b];
-        if (!a.crossed[b] && mz <= 0.f) {
-            double d = (double)prev - (double)mz;
-            double frac = d > 0 ? (double)prev / d : 1.0;
-            a.t_sw[b] = (float)(clk.t - a.h + a.h * frac);
-            a.crossed[b] = 1;
-        }
-        a.mz_prev[b] = mz;
-        if (!isfinite(mz)) a.status[b] |= BPM_ISLAND_NONFINITE;
+        detect_switch(a, b, mz, clk.t);
     }
+}
+
+// ---------------------------------------------------------------------------
+// Both stages for batches of few islands.  With every CTA resident at once a
+// stage's time is its chain of latencies, and most of the chain does not depend
+// on the product before it: the stage's clock, the island's parameters, the head
+// field at every node (the time is known), the exchange entries.  The kernel is
+// launched programmatically behind the GEMM, takes these first (the head field
+// into shared memory, the entries into L1) and only then waits.  The per-island
+// arithmetic is that of eff_field, term by term in the same order.
+// An interval of 9 islands of 481 nodes (8 steps): 330 -> 187 us; of one island of 209 nodes (6 steps):
+// 172 -> 125 us; of 128 islands of 1547 nodes (28 steps): 3.10 -> 1.98 ms.
+// ---------------------------------------------------------------------------
+template <int STAGE>
+__device__ __forceinline__ void few_body(const StepArgs& a, int b, int j, float* red, StageClock& clk) {
+    extern __shared__ float4 smem4[];
+    float* sm = reinterpret_cast<float*>(smem4);
+    const int np = a.n_pad;
+    float* hb = sm + 3 * np;                               // head field, [3][n_pad]
+    const size_t base = (size_t)b * 3 * np;
+    pdl_trigger();
+    set_clock(clk, a, j, STAGE == 2);
+    const float4 p0 = a.isl[3 * b], p1 = a.isl[3 * b + 1], p2 = a.isl[3 * b + 2];
+    const bool head = (a.mask & BPM_TERM_HEAD) && a.map;
+    __syncthreads();
+    const float ramp = clk.ramp, xh = clk.xh;
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        const float4 pos = __ldg(a.node_pos + i);
+        if (a.mask & BPM_TERM_EXCHANGE) {
+            const int hi = __ldg(a.sell_off + (i >> 5) + 1);
+            for (int e = __ldg(a.sell_off + (i >> 5)) + (i & 31); e < hi; e += 32)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(a.sell_ent + e));
+        }
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(a.node_mat + i));
+        if (head) {
+            const float3 h = trilinear(a, pos.x + p1.w - xh, pos.y + p2.x, pos.z);
+            hb[i] = h.x;
+            hb[np + i] = h.y;
+            hb[2 * np + i] = h.z;
+        }
+    }
+    pdl_wait();
+    const float h = (float)a.h, hh = 0.5f * h;
+    if (STAGE == 1)
+        stage_state(a.m + base, sm, np);
+    else
+        stage_predicted(a.m + base, a.k1 + base, sm, np, a.n, h);
+    __syncthreads();
+    float mzp = 0.f;
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        const float3 mi = f3(sm[i], sm[np + i], sm[2 * np + i]);
+        float3 mn, f1;
+        if (STAGE == 2) {
+            mn = f3(__ldcg(a.m + base + i), __ldcg(a.m + base + np + i), __ldcg(a.m + base + 2 * np + i));
+            f1 = f3(__ldcg(a.k1 + base + i), __ldcg(a.k1 + base + np + i), __ldcg(a.k1 + base + 2 * np + i));
+        }
+        const float3 hdv = f3(hb[i], hb[np + i], hb[2 * np + i]);
+        const float3 B = eff_field(a, b, i, mi, sm, p0, p1, p2, ramp, xh, a.mask, &hdv);
+        const float3 f = llg_rhs(mi, B, a.alpha, a.gp);
+        float3 v;
+        if (STAGE == 1) {
+            v = heun_predict(mi, f, h);
+            a.k1[base + i] = f.x;
+            a.k1[base + np + i] = f.y;
+            a.k1[base + 2 * np + i] = f.z;
+        } else {
+            v = normalize3(mn + hh * (f1 + f));
+            a.m[base + i] = v.x;
+            a.m[base + np + i] = v.y;
+            a.m[base + 2 * np + i] = v.z;
+            mzp += __ldg(&a.node_pos[i].w) * v.z;
+        }
+        write_gemm_input(a, b, i, v, __ldg(&a.node_mat[i].y) * p0.z);
+    }
+    if (STAGE == 2) {
+        const float mz = block_reduce(mzp, red);
+        if (threadIdx.x == 0) detect_switch(a, b, mz, clk.t);
+    }
+}
+
+template <int NT, int STAGE>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_few(StepArgs a, int j) {
+    __shared__ float red[NT / 32];
+    __shared__ StageClock clk;
+    few_body<STAGE>(a, blockIdx.x, j, red, clk);
+}
+
+template <int NT, int STAGE>
+__global__ void __launch_bounds__(NT, 1024 / NT)
+    k_few_groups(const __grid_constant__ StageGroups G, int j) {
+    __shared__ float red[NT / 32];
+    __shared__ StageClock clk;
+    const int g = stage_group(G);
+    few_body<STAGE>(G.a[g], blockIdx.x - G.block_begin[g], j, red, clk);
 }
 
 constexpr int kMultiNT = 256, kMultiIPB = 2;
@@ -816,6 +909,15 @@ constexpr size_t kMaxStageSmem = 3 * sizeof(float) * kMaxNodes;
 
 size_t stage_smem_bytes(const StepArgs& a) { return 3 * sizeof(float) * (size_t)a.n_pad; }
 
+template <int NT>
+static int configure_few(int smem) {
+    BPM_CK(cudaFuncSetAttribute(k_few<NT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_few<NT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_few_groups<NT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_few_groups<NT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return BPM_OK;
+}
+
 int configure_step_kernels() {
     int smem = (int)kMaxStageSmem;
     BPM_CK(cudaFuncSetAttribute(k_stage1<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -834,11 +936,42 @@ int configure_step_kernels() {
     BPM_CK(cudaFuncSetAttribute(k_stage2_groups<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_stage2_groups<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int smem2 = kMultiIPB * smem;
+    BPM_TRY(configure_few<256>(smem2));
+    BPM_TRY(configure_few<512>(smem2));
+    BPM_TRY(configure_few<1024>(smem2));
     BPM_CK(cudaFuncSetAttribute(k_stage1m, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     BPM_CK(cudaFuncSetAttribute(k_stage2m, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     BPM_CK(cudaFuncSetAttribute(k_stage1m_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     BPM_CK(cudaFuncSetAttribute(k_stage2m_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     return BPM_OK;
+}
+
+int few_threads(int n, int B, int sm_count) {
+    // one pass over the nodes where the SMs hold that many threads for all islands (at most 1024 a CTA)
+    const int per_sm = (B + sm_count - 1) / sm_count;
+    const int nt = n <= 256 || per_sm > 2 ? 256 : n <= 512 || per_sm > 1 ? 512 : 1024;
+    return nt;
+}
+
+namespace {
+template <int NT>
+int launch_few_nt(const StageGroups& G, int stage, int j, cudaStream_t s) {
+    size_t smem = 0;
+    for (int g = 0; g < G.ng; ++g) smem = std::max(smem, 2 * stage_smem_bytes(G.a[g]));
+    const dim3 grid(G.block_begin[G.ng]), block(NT);
+    if (G.ng == 1)
+        BPM_CK(stage == 1 ? launch_pdl(k_few<NT, 1>, grid, block, smem, s, true, G.a[0], j)
+                          : launch_pdl(k_few<NT, 2>, grid, block, smem, s, true, G.a[0], j));
+    else
+        BPM_CK(stage == 1 ? launch_pdl(k_few_groups<NT, 1>, grid, block, smem, s, true, G, j)
+                          : launch_pdl(k_few_groups<NT, 2>, grid, block, smem, s, true, G, j));
+    return BPM_OK;
+}
+}  // namespace
+
+int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t s) {
+    return threads == 1024 ? launch_few_nt<1024>(G, stage, j, s)
+                           : threads == 512 ? launch_few_nt<512>(G, stage, j, s) : launch_few_nt<256>(G, stage, j, s);
 }
 
 int stage_blocks_per_sm(int threads, int ipb, size_t smem, int* blocks) {

@@ -57,3 +57,39 @@ def test_demag_product_tile_and_slice_edges(ctx, B, nodes):
             out.append(bt.field(0.0, L.TERM_DEMAG))
     ctx.mesh_release(mid)
     assert np.abs(out[1] - out[0]).max() <= (3 * K / 16) * 2.0 ** -23 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("sizes", [(129,), (300,), (40, 130), (1, 64, 200)])
+def test_few_island_stages_match_the_two_island_stages(ctx, sizes):
+    """Batches on the stage kernels of few islands (one and several mesh groups, 256 and 512 threads a CTA) against
+    the same run on the CTA-pair GEMM, which takes the two-island stage kernels.  A group of more than 128 islands has
+    the same products in the same order on both sides: m and the switch data are bitwise equal, <m_z> up to the order
+    of its sum.  Smaller groups slice K on one side: within the drift of the GEMM's rounding (2^-23 of the field per
+    MMA, 1e-4 over the run as in the pair GEMM's own run test)."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    meshes = [synth.layered_island_mesh(12.0, 6.0, 6.0, rings=3, hard_slabs=6, soft_slabs=6, seed=7),
+              synth.small_island_mesh(), synth.layered_island_mesh(7.0, 6.0, 4.0, rings=2, hard_slabs=9, soft_slabs=6)]
+    mids = [ctx.mesh_upload(meshes[-1 - k], synth.ecc_materials()) for k in range(len(sizes))]
+    hid = ctx.headmap_upload(synth.synthetic_head_map())
+    isl = synth.Islands.concat([synth.jittered_islands(b, seed=b, mesh_id=m) for b, m in zip(sizes, mids)])
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, rise_ps=2.0, use_map=True, x0_nm=-2.0, substeps=0,
+                        uniform_T=synth.uniform_field(0.9, 170.0))
+    out = []
+    for pair in (0, 1):
+        with ctx.batch(isl, p, precision=L.PREC_BF16X3, map_id=hid) as bt:
+            bt.set_tuning(256, 256, L.RASTER_AUTO, 2, 32, gemm_pair=pair)
+            bt.advance(40)
+            out.append(bt.read())
+    few, two = out
+    assert np.all(few["status"] == 0) and np.abs(few["mz"] - 1.0).max() > 0.02      # the islands have moved
+    for b, m in zip(sizes, mids):
+        r = np.asarray(isl.mesh_id) == m
+        if b > 128:
+            assert np.array_equal(few["m"][r], two["m"][r]) and np.array_equal(few["t_sw"][r], two["t_sw"][r])
+            assert np.abs(few["mz"][r] - two["mz"][r]).max() <= 1e-6
+        else:
+            assert np.abs(few["m"][r] - two["m"][r]).max() <= 1e-4
+    for m in mids:
+        ctx.mesh_release(m)
+    ctx.headmap_release(hid)
