@@ -288,7 +288,7 @@ int run_demag_gemm(bpm_batch* bt, Group& g, cudaStream_t s) {
     const int K = M->K();
     switch (bt->p.precision) {
         case BPM_PREC_FP32:
-            return gemm_f32_nt(s, g.Bp, K, K, g.A32, K, M->N32, K, g.Hd, K);
+            return gemm_f32_nt(s, g.B, K, K, g.A32, K, M->N32, K, g.Hd, K);
         case BPM_PREC_BF16X3_REF:
             return gemm_bf16x3_simt(s, g.Bp, K, K, g.Ahi, g.Alo, M->Nhi, M->Nlo, g.Hd, 3);
         default:

@@ -179,7 +179,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     auto demag = [&]() -> int {
         if (!(p->term_mask & BPM_TERM_DEMAG)) return BPM_OK;
         if (tc) return grouped_gemm_launch(s, gg, ctx->sm_count, err);
-        if (prec == BPM_PREC_FP32) return gemm_f32_nt(s, Rp, K, K, A32, K, M->N32, K, Hd, K);
+        if (prec == BPM_PREC_FP32) return gemm_f32_nt(s, R, K, K, A32, K, M->N32, K, Hd, K);
         return gemm_bf16x3_simt(s, Rp, K, K, Ahi, Alo, M->Nhi, M->Nlo, Hd, 3);
     };
 

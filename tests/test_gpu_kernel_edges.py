@@ -93,3 +93,29 @@ def test_few_island_stages_match_the_two_island_stages(ctx, sizes):
     for m in mids:
         ctx.mesh_release(m)
     ctx.headmap_release(hid)
+
+
+@pytest.mark.parametrize("B", [1, 16, 31, 32, 33, 64, 65, 130])
+def test_fp32_product_tile_edges(ctx, B):
+    """Row counts around the FP32 GEMM's tiles (16 rows up to 32, 64 beyond) on an operator whose columns (704) end
+    inside a 64-column tile: against the FP64 product of the exported FP32 operator and the same FP32 sources.  A sum
+    of K products in FP32 with four partial sums: K/4 * 2^-24 of the sum of magnitudes, K = 704."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    mesh = synth.small_island_mesh()
+    mid = ctx.mesh_upload(mesh, synth.ecc_materials())
+    n = mesh.n_nodes
+    isl = synth.jittered_islands(B, seed=B, mesh_id=mid)
+    rng = np.random.default_rng(B)
+    m = rng.standard_normal((B, 3, n)).astype(np.float32)
+    m /= np.linalg.norm(m, axis=1, keepdims=True)
+    with ctx.batch(isl, synth.RunParams(dt_ps=0.1, substeps=1, term_mask=L.TERM_DEMAG), precision=L.PREC_FP32) as bt:
+        bt.set_state(m, 0.0)
+        got = bt.field(0.0, L.TERM_DEMAG).reshape(B, 3 * n)
+    Ms = (ctx.get_operator(mid, L.OP_NODAL_MS_F64) * 1e-6).astype(np.float32)
+    src = ((Ms[None] * isl.Ms_scale[:, None])[:, None] * m).astype(np.float64).reshape(B, 3 * n)
+    W = ctx.get_operator(mid, L.OP_DEMAG_F32).astype(np.float64)
+    ctx.mesh_release(mid)
+    bound = (176 * 2.0 ** -24 + 2.0 ** -22) * (np.abs(src) @ np.abs(W).T)      # + the sources' own FP32 rounding
+    assert np.all(np.abs(got - src @ W.T) <= bound)
+
