@@ -23,15 +23,18 @@ namespace {
 using namespace tc;
 
 // warp 0 issues the TMA loads and warp 1 the MMAs; all eight warps run the epilogue, warp w
-// on TMEM lane quarter w % 4 (rows) and column half w / 4
+// on TMEM lane quarter w % 4 (rows) and every second 32 columns, from 32 (w / 4)
 constexpr int kThreads = 256;
 
 // The forward layers of the MLP (bias+GELU and output epilogues) have K <= 256, at most four
 // k-blocks: two stages keep their ring full and halve the shared memory, so that two CTAs share
 // an SM and one CTA's epilogue runs beside the other's MMAs.  The other GEMMs (K = batch rows)
 // keep the deep ring.
-// The forward layers launch 128-wide column tiles: at 64 KB of ring a CTA, three CTAs (24 warps)
-// share an SM for the GELU epilogue, which bounds these layers.
+// Column tiles (4096 rows, 256 features; the sums do not depend on the tile): the epilogues bound the
+// forward and input-gradient layers, so their tiles are as narrow as fills the SMs -- forward 64 wide
+// (128 CTAs, 17 us a layer; 128 wide 27), input gradient 64 wide (23 us; 256 wide, 32 CTAs, 71).
+// The weight gradient's K is the batch, a serial walk of 64 k-blocks; 32-wide tiles make it 16 CTAs
+// of 20 us that run beside the input gradients (two CTAs of 27 us in line with them before).
 template <int P, int TN, int EPI>
 struct Cfg {
     static constexpr int W_TILE = Tile<TN>::W_TILE;
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int row = m0 + quarter * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-        for (int c = half * (TN / 2); c < (half + 1) * (TN / 2); c += 32) {
+        for (int c = 32 * half; c < TN; c += 64) {
             uint32_t r[32];
             float colsum[32];
             tmem_ld32(lane_addr + (uint32_t)c, r);
@@ -327,10 +330,11 @@ int gemm_tc(cudaStream_t s, int epi, int M, int N, int K, const __nv_bfloat16* A
         return BPM_ERR_ARG;
     }
     switch (epi) {
-        case TC_EPI_STORE: return launch<1, TC_EPI_STORE>(s, M, N, K, A, A, W, W, e, err_flag);
-        case TC_EPI_BIAS_GELU: return launch<1, TC_EPI_BIAS_GELU, 128>(s, M, N, K, A, A, W, W, e, err_flag);
+        case TC_EPI_STORE: return launch<1, TC_EPI_STORE, 32>(s, M, N, K, A, A, W, W, e, err_flag);
+        case TC_EPI_BIAS_GELU: 
+            return launch<1, TC_EPI_BIAS_GELU, 64>(s, M, N, K, A, A, W, W, e, err_flag);
         case TC_EPI_BIAS_OUT: return launch<1, TC_EPI_BIAS_OUT, 128>(s, M, N, K, A, A, W, W, e, err_flag);
-        case TC_EPI_GELU_BWD: return launch<1, TC_EPI_GELU_BWD>(s, M, N, K, A, A, W, W, e, err_flag);
+        case TC_EPI_GELU_BWD: return launch<1, TC_EPI_GELU_BWD, 64>(s, M, N, K, A, A, W, W, e, err_flag);
         default: set_error("unknown epilogue %d", epi); return BPM_ERR_ARG;
     }
 }

@@ -40,7 +40,10 @@ struct Mlp {
     std::vector<__nv_bfloat16*> H, HT;   // H[l]: input of layer l ([rows][in_pad[l]]), HT its transpose
     std::vector<float*> Z;               // Z[l]: pre-activation of hidden layer l
     float *logits = nullptr, *Y = nullptr, *colsum = nullptr, *loss = nullptr;
-    __nv_bfloat16 *dZa = nullptr, *dZaT = nullptr, *dZb = nullptr, *dZbT = nullptr;
+    std::vector<__nv_bfloat16*> dZ, dZT;  // dZ[l]: gradient at layer l's pre-activation, dZT its transpose
+    // weight gradients run on `side`, beside the chain of input gradients
+    cudaStream_t side = nullptr;
+    std::vector<cudaEvent_t> ev;          // ev[l]: dZ[l] written; ev[L]: the weight gradients are done
     int* err = nullptr;
     int max_pad = 0;
 };
@@ -57,12 +60,11 @@ void free_ws(Mlp* m) {
     cudaFree(m->logits);
     cudaFree(m->Y);
     cudaFree(m->colsum);
-    cudaFree(m->dZa);
-    cudaFree(m->dZaT);
-    cudaFree(m->dZb);
-    cudaFree(m->dZbT);
+    for (auto p : m->dZ) cudaFree(p);
+    for (auto p : m->dZT) cudaFree(p);
+    m->dZ.clear();
+    m->dZT.clear();
     m->logits = m->Y = m->colsum = nullptr;
-    m->dZa = m->dZaT = m->dZb = m->dZbT = nullptr;
     m->ws_rows = 0;
 }
 
@@ -91,10 +93,17 @@ int ensure_ws(Mlp* m, int rows) {
     BPM_TRY(zalloc(&m->logits, (size_t)rows * m->n_out));
     BPM_TRY(zalloc(&m->Y, (size_t)rows * m->n_out));
     BPM_TRY(zalloc(&m->colsum, (size_t)(rows / 32) * m->max_pad));
-    BPM_TRY(zalloc(&m->dZa, (size_t)rows * m->max_pad));
-    BPM_TRY(zalloc(&m->dZaT, (size_t)rows * m->max_pad));
-    BPM_TRY(zalloc(&m->dZb, (size_t)rows * m->max_pad));
-    BPM_TRY(zalloc(&m->dZbT, (size_t)rows * m->max_pad));
+    m->dZ.assign(m->L, nullptr);
+    m->dZT.assign(m->L, nullptr);
+    for (int l = 0; l < m->L; ++l) {
+        BPM_TRY(zalloc(&m->dZ[l], (size_t)rows * m->out_pad[l]));
+        BPM_TRY(zalloc(&m->dZT[l], (size_t)rows * m->out_pad[l]));
+    }
+    if (!m->side) {
+        BPM_CK(cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking));
+        m->ev.assign(m->L + 1, nullptr);
+        for (auto& e : m->ev) BPM_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     m->ws_rows = rows;
     return BPM_OK;
 }
@@ -174,6 +183,7 @@ __global__ void k_colsum_reduce(int nblk, int ncol, int ld, const float* __restr
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncol) return;
     float s = 0.f;
+#pragma unroll 32   // the loads of 32 blocks in flight; the sum stays in order
     for (int k = 0; k < nblk; ++k) s += part[(size_t)k * ld + c];
     db[c] = s;
 }
@@ -281,40 +291,42 @@ int forward(Mlp* m, cudaStream_t s, int rows, int nb, bool infer, bool sigmoid) 
 // backward for the batch in the workspace: gradients into m->grad, loss into loss_slot
 int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
     const int Lm = m->L - 1;
-    BPM_CK(cudaMemsetAsync(m->dZa, 0, sizeof(__nv_bfloat16) * (size_t)rows * m->max_pad, s));
-    BPM_CK(cudaMemsetAsync(m->dZaT, 0, sizeof(__nv_bfloat16) * (size_t)rows * m->max_pad, s));
-    k_loss_head<<<1, 1024, 0, s>>>(nb, m->n_out, m->out_pad[Lm], rows, m->logits, m->Y, m->dZa, m->dZaT,
+    // (the pads of dZ[Lm] are zero from the allocation on; a shorter batch lays its transpose out anew)
+    BPM_CK(cudaMemsetAsync(m->dZ[Lm], 0, sizeof(__nv_bfloat16) * (size_t)rows * m->out_pad[Lm], s));
+    BPM_CK(cudaMemsetAsync(m->dZT[Lm], 0, sizeof(__nv_bfloat16) * (size_t)rows * m->out_pad[Lm], s));
+    k_loss_head<<<1, 1024, 0, s>>>(nb, m->n_out, m->out_pad[Lm], rows, m->logits, m->Y, m->dZ[Lm], m->dZT[Lm],
                                    m->grad + m->b_off[Lm], loss_slot);
     BPM_CK(cudaGetLastError());
-    __nv_bfloat16 *dz = m->dZa, *dzT = m->dZaT, *dzn = m->dZb, *dznT = m->dZbT;
     for (int l = Lm; l >= 0; --l) {
-        // dW_l = dZ_l^T H_l
+        // dW_l = dZ_l^T H_l on the side stream: nothing before the optimiser reads it
+        BPM_CK(cudaEventRecord(m->ev[l], s));
+        BPM_CK(cudaStreamWaitEvent(m->side, m->ev[l], 0));
         TcEpilogue g{};
         g.C = m->grad + m->w_off[l];
         g.ldc = m->in_real[l];
         g.rows_valid = m->out_real[l];
         g.cols_valid = m->in_real[l];
-        BPM_TRY(gemm_tc(s, TC_EPI_STORE, m->out_pad[l], m->in_pad[l], rows, dzT, m->HT[l], g, m->err));
+        BPM_TRY(gemm_tc(m->side, TC_EPI_STORE, m->out_pad[l], m->in_pad[l], rows, m->dZT[l], m->HT[l], g, m->err));
         if (l == 0) break;
         // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1}), bias gradient of layer l-1
         TcEpilogue e{};
         e.Zin = m->Z[l - 1];
         e.ldz = m->out_pad[l - 1];
-        e.H = dzn;
+        e.H = m->dZ[l - 1];
         e.ldh = m->out_pad[l - 1];
-        e.HT = dznT;
+        e.HT = m->dZT[l - 1];
         e.ldht = rows;
         e.colsum = m->colsum;
         e.ldcs = m->in_pad[l];
         e.rows_valid = nb;
         e.cols_valid = m->out_real[l - 1];
-        BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], dz, m->WT[l], e, m->err));
+        BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], m->dZ[l], m->WT[l], e, m->err));
         k_colsum_reduce<<<(m->out_real[l - 1] + 127) / 128, 128, 0, s>>>(rows / 32, m->out_real[l - 1], m->in_pad[l],
                                                                          m->colsum, m->grad + m->b_off[l - 1]);
         BPM_CK(cudaGetLastError());
-        std::swap(dz, dzn);
-        std::swap(dzT, dznT);
     }
+    BPM_CK(cudaEventRecord(m->ev[m->L], m->side));
+    BPM_CK(cudaStreamWaitEvent(s, m->ev[m->L], 0));
     return BPM_OK;
 }
 
@@ -362,7 +374,11 @@ int check_err(Mlp* m, cudaStream_t s) {
 
 void free_mlp(Mlp* m) {
     if (!m) return;
+    if (m->side) cudaStreamSynchronize(m->side);
     free_ws(m);
+    for (auto e : m->ev)
+        if (e) cudaEventDestroy(e);
+    if (m->side) cudaStreamDestroy(m->side);
     for (auto p : m->W) cudaFree(p);
     for (auto p : m->WT) cudaFree(p);
     cudaFree(m->params);
