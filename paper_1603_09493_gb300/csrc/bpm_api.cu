@@ -19,6 +19,34 @@ void set_error(const char* fmt, ...) {
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+int CallBuffers::reserve() {
+    char* base = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (size <= Scratch::kKeep) {
+        lock = std::unique_lock<std::mutex>(ctx->scratch.mu);
+        Scratch& k = ctx->scratch;
+        if (size > k.size) {
+            cudaFree(k.p);          // waits for the work that uses it
+            k.p = nullptr;
+            k.size = 0;
+            e = cudaMalloc(&k.p, size);
+            if (e == cudaSuccess) k.size = size;
+        }
+        base = static_cast<char*>(k.p);
+    } else {
+        e = cudaMalloc(&own, size);
+        base = static_cast<char*>(own);
+    }
+    if (e != cudaSuccess) {
+        set_error("device buffers of %zu bytes: %s", size, cudaGetErrorString(e));
+        return BPM_ERR_OOM;
+    }
+    for (auto& q : at) *q.first = base + q.second;
+    return BPM_OK;
+}
+
+CallBuffers::~CallBuffers() { cudaFree(own); }
+
 // Heun's explicit step is stable on the fastest precession mode when
 // gamma/(1+alpha^2) |B| h <= 1/2; k is the smallest step count per output
 // interval that keeps h = dt/k there for the largest field the run can see.
@@ -127,6 +155,7 @@ struct bpm_batch {
     int B = 0, n_max = 0;
     bpm_run_params p{};
     std::vector<Group> groups;
+    void* arena = nullptr;            // every device buffer of the batch and its groups
     int* gemm_err = nullptr;
     long long* interval = nullptr;
     long long intervals_done = 0;
@@ -193,6 +222,28 @@ int setup_grouped_gemm(bpm_batch* bt) {
                               bt->k_block, bt->ctx->sm_count, bt->pair);
 }
 
+// Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
+// tensor-core product on one stream, every island's CTA resident at once (at most four of 256
+// threads an SM, two vectors of the state in shared memory each) and at most 3200 nodes an SM.  Beyond that the
+// two-island kernels on two streams, which share the exchange entries between islands, are as fast
+// (interval in us, this way / theirs: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 /
+// 590; 1547 nodes, 300 islands 4177 / 4774, 512 islands 5304 / 5030).  Fills *G.
+bool few_islands(const bpm_batch* bt, StageGroups* G) {
+    if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
+    const int per_sm = (bt->B + bt->ctx->sm_count - 1) / bt->ctx->sm_count;
+    std::memset(G, 0, sizeof(StageGroups));
+    size_t smem = 0;
+    int n = 0;
+    for (const auto& g : bt->groups) {
+        smem = std::max(smem, 2 * stage_smem_bytes(g.args));
+        n = std::max(n, g.mesh->n);
+        G->a[G->ng] = g.args;
+        G->block_begin[G->ng + 1] = G->block_begin[G->ng] + g.B;
+        ++G->ng;
+    }
+    return per_sm <= 4 && per_sm * n <= std::max(3200, n) && per_sm * (smem + 1024) <= 200 * 1024;
+}
+
 // The chains of a multi-stream batch: the one group's islands cut into `streams` chunks of a
 // multiple of 128 islands (the GEMM's M tile; the last chunk takes the rest), each with its own
 // GEMM over its operand rows and its own view of the stage arguments.  chains stays 0 where the
@@ -201,7 +252,8 @@ int setup_chains(bpm_batch* bt) {
     for (auto& h : bt->gg_chain) grouped_gemm_free(&h);
     bt->chains = 0;
     for (auto& v : bt->chain_groups) v.clear();
-    if (bt->streams < 2 || !tensor_core_precision(bt)) return BPM_OK;
+    StageGroups few;
+    if (bt->streams < 2 || !tensor_core_precision(bt) || few_islands(bt, &few)) return BPM_OK;
     const int ng = (int)bt->groups.size();
     const int chunk = ng > 1 ? 0 : kIslandPad * ((bt->groups[0].B + bt->streams * kIslandPad - 1) /
                                                  (bt->streams * kIslandPad));
@@ -375,28 +427,6 @@ void launch_stage_all(bpm_batch* bt, const StageLaunches& L, int stage, int j, c
     }
 }
 
-// Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
-// tensor-core product on one stream, every island's CTA resident at once (at most four of 256 threads
-// an SM, two vectors of the state in shared memory each) and at most 3200 nodes an SM.  Beyond that the
-// two-island kernels on two streams, which share the exchange entries between islands, are as fast
-// (interval in us, this way / theirs: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 /
-// 590; 1547 nodes, 300 islands 4177 / 4774, 512 islands 5304 / 5030).  Fills *G.
-bool few_islands(const bpm_batch* bt, StageGroups* G) {
-    if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
-    const int per_sm = (bt->B + bt->ctx->sm_count - 1) / bt->ctx->sm_count;
-    std::memset(G, 0, sizeof(StageGroups));
-    size_t smem = 0;
-    int n = 0;
-    for (const auto& g : bt->groups) {
-        smem = std::max(smem, 2 * stage_smem_bytes(g.args));
-        n = std::max(n, g.mesh->n);
-        G->a[G->ng] = g.args;
-        G->block_begin[G->ng + 1] = G->block_begin[G->ng] + g.B;
-        ++G->ng;
-    }
-    return per_sm <= 4 && per_sm * n <= std::max(3200, n) && per_sm * (smem + 1024) <= 200 * 1024;
-}
-
 // one output interval of every group; groups of a multi-mesh batch are forked
 // over side streams so that their kernels can run concurrently
 int enqueue_interval(bpm_batch* bt, cudaStream_t s) {
@@ -469,11 +499,6 @@ int enqueue_interval(bpm_batch* bt, cudaStream_t s) {
     return BPM_OK;
 }
 
-void free_group(Group& g) {
-    void* ptrs[] = {g.d_idx, g.isl, g.m, g.k1, g.Hd, g.A32, g.Ahi, g.Alo, g.mz_prev, g.t_sw, g.crossed, g.status};
-    for (void* p : ptrs) cudaFree(p);
-}
-
 void drop_graph(bpm_batch* bt) {
     if (bt->exec) {
         cudaGraphExecDestroy(bt->exec);
@@ -489,33 +514,57 @@ void free_batch(bpm_batch* bt) {
     if (!bt) return;
     if (bt->exec) cudaGraphExecDestroy(bt->exec);
     if (bt->graph) cudaGraphDestroy(bt->graph);
-    for (auto& g : bt->groups) free_group(g);
+    cudaFree(bt->arena);
     grouped_gemm_free(&bt->gg);
     for (auto& h : bt->gg_chain) grouped_gemm_free(&h);
     for (auto st : bt->chain_stream)
         if (st) cudaStreamDestroy(st);
     for (auto e : bt->chain_ev)
         if (e) cudaEventDestroy(e);
-    cudaFree(bt->gemm_err);
-    cudaFree(bt->interval);
     for (auto s : bt->side) cudaStreamDestroy(s);
     for (auto e : bt->ev) cudaEventDestroy(e);
     delete bt;
 }
 
-template <class T>
-int dalloc(T** p, size_t count) {
-    cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(1, count) * sizeof(T));
-    if (e != cudaSuccess) {
-        set_error("device allocation of %zu bytes failed: %s", count * sizeof(T), cudaGetErrorString(e));
-        return BPM_ERR_OOM;
+// Device buffers of a batch, 256-byte aligned in one allocation (a batch of twelve meshes made 146,
+// 2.4 ms of a run_batch call).  First pass with base null: the size; second: the addresses.
+struct Arena {
+    char* base;
+    size_t off = 0;
+    template <class T>
+    void take(T** p, size_t count) {
+        *p = base ? reinterpret_cast<T*>(base + off) : nullptr;
+        off = (off + std::max<size_t>(1, count) * sizeof(T) + 255) & ~(size_t)255;
     }
-    e = cudaMemset(*p, 0, std::max<size_t>(1, count) * sizeof(T));
-    if (e != cudaSuccess) {
-        set_error("cudaMemset failed: %s", cudaGetErrorString(e));
-        return BPM_ERR_CUDA;
+};
+
+// the buffers of a batch; the island tables and index lists of all groups come first, as one block
+// that the host uploads (its size: the return value)
+size_t carve(bpm_batch* bt, Arena& A) {
+    for (auto& g : bt->groups) {
+        A.take(&g.isl, 3 * (size_t)g.B);
+        A.take(&g.d_idx, g.B);
     }
-    return BPM_OK;
+    const size_t tables = A.off;
+    A.take(&bt->gemm_err, 4);
+    A.take(&bt->interval, 1);
+    for (auto& g : bt->groups) {
+        const size_t S = (size_t)g.Bp * g.mesh->K();
+        A.take(&g.m, S);
+        A.take(&g.k1, S);
+        A.take(&g.Hd, g.splits * S);
+        if (bt->p.precision == BPM_PREC_FP32) {
+            A.take(&g.A32, S);
+        } else {
+            A.take(&g.Ahi, S);
+            A.take(&g.Alo, S);
+        }
+        A.take(&g.mz_prev, g.B);
+        A.take(&g.t_sw, g.B);
+        A.take(&g.crossed, g.B);
+        A.take(&g.status, g.B);
+    }
+    return tables;
 }
 
 // the batch's interval graph, captured on first use
@@ -661,6 +710,7 @@ void bpm_destroy(bpm_ctx* ctx) {
         }
         delete h;
     }
+    cudaFree(ctx->scratch.p);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -898,53 +948,48 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
     bt->p.substeps = k_steps;
     bt->t0 = p->t0_ps;
     int r = BPM_OK;
-    auto chk = [&](int rr) {
-        if (r == BPM_OK) r = rr;
-    };
-    chk(dalloc(&bt->gemm_err, 4));
-    chk(dalloc(&bt->interval, 1));
     bt->groups.resize(mesh_of_group.size());
-    for (size_t gi = 0; gi < bt->groups.size() && r == BPM_OK; ++gi) {
+    for (size_t gi = 0; gi < bt->groups.size(); ++gi) {
         Group& g = bt->groups[gi];
-        Mesh* M = ctx->meshes[mesh_of_group[gi]];
-        g.mesh = M;
+        g.mesh = ctx->meshes[mesh_of_group[gi]];
         g.user_idx = members[gi];
         g.B = (int)g.user_idx.size();
         g.Bp = round_up(g.B, kIslandPad);
-        bt->n_max = std::max(bt->n_max, M->n);
-        const size_t S = (size_t)g.Bp * M->K();
-        chk(dalloc(&g.d_idx, g.B));
-        chk(dalloc(&g.isl, 3 * (size_t)g.B));
-        chk(dalloc(&g.m, S));
-        chk(dalloc(&g.k1, S));
-        if (tensor_core_precision(bt)) g.splits = gemm_splits(g.B, M->K(), ctx->sm_count);
-        chk(dalloc(&g.Hd, g.splits * S));
-        if (p->precision == BPM_PREC_FP32) {
-            chk(dalloc(&g.A32, S));
-        } else {
-            chk(dalloc(&g.Ahi, S));
-            chk(dalloc(&g.Alo, S));
+        bt->n_max = std::max(bt->n_max, g.mesh->n);
+        if (tensor_core_precision(bt)) g.splits = gemm_splits(g.B, g.mesh->K(), ctx->sm_count);
+    }
+    Arena size{nullptr};
+    const size_t tables = carve(bt, size);
+    cudaError_t ce = cudaMalloc(&bt->arena, size.off);
+    if (ce != cudaSuccess) {
+        set_error("device allocation of %zu bytes failed: %s", size.off, cudaGetErrorString(ce));
+        r = BPM_ERR_OOM;
+    } else {
+        Arena A{static_cast<char*>(bt->arena)};
+        carve(bt, A);
+        std::vector<char> host(tables);
+        for (auto& g : bt->groups) {
+            float4* ip = reinterpret_cast<float4*>(host.data() + (reinterpret_cast<char*>(g.isl) - A.base));
+            for (int k = 0; k < g.B; ++k) {
+                const bpm_island& I = isl[g.user_idx[k]];
+                ip[3 * k] = make_float4(1.f / I.Ms_scale, I.Ku_scale / I.Ms_scale, I.Ms_scale, 0.f);
+                ip[3 * k + 1] = make_float4(I.u[0], I.u[1], I.u[2], I.pos_nm[0]);
+                ip[3 * k + 2] = make_float4(I.pos_nm[1], I.Hext_T[0], I.Hext_T[1], I.Hext_T[2]);
+            }
+            std::memcpy(host.data() + (reinterpret_cast<char*>(g.d_idx) - A.base), g.user_idx.data(),
+                        g.B * sizeof(int));
         }
-        chk(dalloc(&g.mz_prev, g.B));
-        chk(dalloc(&g.t_sw, g.B));
-        chk(dalloc(&g.crossed, g.B));
-        chk(dalloc(&g.status, g.B));
-        if (r != BPM_OK) break;
-        std::vector<float4> ip(3 * (size_t)g.B);
-        for (int k = 0; k < g.B; ++k) {
-            const bpm_island& I = isl[g.user_idx[k]];
-            ip[3 * k] = make_float4(1.f / I.Ms_scale, I.Ku_scale / I.Ms_scale, I.Ms_scale, 0.f);
-            ip[3 * k + 1] = make_float4(I.u[0], I.u[1], I.u[2], I.pos_nm[0]);
-            ip[3 * k + 2] = make_float4(I.pos_nm[1], I.Hext_T[0], I.Hext_T[1], I.Hext_T[2]);
-        }
-        cudaError_t e = cudaMemcpy(g.isl, ip.data(), ip.size() * sizeof(float4), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(g.d_idx, g.user_idx.data(), g.B * sizeof(int), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            set_error("island upload: %s", cudaGetErrorString(e));
+        ce = cudaMemsetAsync(A.base + tables, 0, size.off - tables, ctx->stream);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(A.base, host.data(), tables, cudaMemcpyHostToDevice, ctx->stream);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(ctx->stream);
+        if (ce != cudaSuccess) {
+            set_error("island upload: %s", cudaGetErrorString(ce));
             r = BPM_ERR_CUDA;
-            break;
         }
+    }
+    for (size_t gi = 0; gi < bt->groups.size() && r == BPM_OK; ++gi) {
+        Group& g = bt->groups[gi];
+        Mesh* M = g.mesh;
         StepArgs& a = g.args;
         a.B = g.B;
         a.n = M->n;
@@ -991,7 +1036,7 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
         a.threads = 256;
         a.ipb = 2;
     }
-    if (r == BPM_OK && bt->groups.size() > 1) {
+    if (r == BPM_OK && bt->groups.size() > 1 && !tensor_core_precision(bt)) {
         const int ns = (int)std::min<size_t>(4, bt->groups.size());
         bt->side.resize(ns, nullptr);
         bt->ev.resize(ns + 1, nullptr);

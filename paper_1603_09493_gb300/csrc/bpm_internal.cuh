@@ -7,6 +7,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -132,7 +133,19 @@ void free_gp(Gp* g);
 
 }  // namespace bpm
 
+namespace bpm {
+// Device scratch that a context keeps between calls (at most kKeep bytes; bpm_destroy frees it).  A call
+// holds the lock while it uses the memory; uses follow one another on the context's stream.
+struct Scratch {
+    static constexpr size_t kKeep = size_t(64) << 20;
+    std::mutex mu;
+    void* p = nullptr;
+    size_t size = 0;
+};
+}  // namespace bpm
+
 struct bpm_ctx {
+    bpm::Scratch scratch;
     int device = 0;
     int sm_count = 0;
     size_t l2_bytes = 0;
@@ -156,6 +169,26 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets,
                   const int32_t* region, const bpm_region_mat* mats, int32_t n_regions,
                   uint32_t flags);
 void free_mesh(Mesh* M);
+
+// Buffers of one call: take() every buffer, then reserve(), which sets the pointers.  Up to
+// Scratch::kKeep bytes come from the context's scratch (locked until the object goes), more from an
+// allocation of its own.  Contents are undefined.
+struct CallBuffers {
+    bpm_ctx* ctx;
+    size_t size = 0;
+    void* own = nullptr;
+    std::unique_lock<std::mutex> lock;
+    std::vector<std::pair<void**, size_t>> at;
+    explicit CallBuffers(bpm_ctx* c) : ctx(c) {}
+    CallBuffers(const CallBuffers&) = delete;
+    template <typename T>
+    void take(T** p, size_t count) {
+        at.push_back({reinterpret_cast<void**>(p), size});
+        size += ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+    }
+    int reserve();
+    ~CallBuffers();
+};
 
 // epilogues of the tensor-core GEMM (C = A W^T, BF16 operands, FP32 accumulate)
 enum { TC_EPI_STORE = 0, TC_EPI_BIAS_GELU = 1, TC_EPI_BIAS_OUT = 2, TC_EPI_GELU_BWD = 3 };

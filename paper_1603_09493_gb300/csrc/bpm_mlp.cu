@@ -34,9 +34,12 @@ struct Mlp {
     size_t P = 0;
     float *params = nullptr, *mom1 = nullptr, *mom2 = nullptr, *grad = nullptr;
     std::vector<__nv_bfloat16*> W, WT;
+    __nv_bfloat16 **d_W = nullptr, **d_WT = nullptr;   // the same pointers on the device
+    void *arena = nullptr, *ws = nullptr;              // every buffer above / of the workspace
     long long t = 0;
-    // workspace for up to ws_rows batch rows
+    // workspace for up to ws_rows batch rows; ws_train: with the buffers of the backward pass
     int ws_rows = 0;
+    bool ws_train = false;
     std::vector<__nv_bfloat16*> H, HT;   // H[l]: input of layer l ([rows][in_pad[l]]), HT its transpose
     std::vector<float*> Z;               // Z[l]: pre-activation of hidden layer l
     float *logits = nullptr, *Y = nullptr, *colsum = nullptr, *loss = nullptr;
@@ -51,60 +54,66 @@ struct Mlp {
 namespace {
 
 void free_ws(Mlp* m) {
-    for (auto p : m->H) cudaFree(p);
-    for (auto p : m->HT) cudaFree(p);
-    for (auto p : m->Z) cudaFree(p);
-    m->H.clear();
-    m->HT.clear();
-    m->Z.clear();
-    cudaFree(m->logits);
-    cudaFree(m->Y);
-    cudaFree(m->colsum);
-    for (auto p : m->dZ) cudaFree(p);
-    for (auto p : m->dZT) cudaFree(p);
-    m->dZ.clear();
-    m->dZT.clear();
-    m->logits = m->Y = m->colsum = nullptr;
+    cudaFree(m->ws);
+    m->ws = nullptr;
     m->ws_rows = 0;
 }
 
-template <class T>
-int zalloc(T** p, size_t n) {
-    cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(n, 1) * sizeof(T));
-    if (e == cudaSuccess) e = cudaMemset(*p, 0, std::max<size_t>(n, 1) * sizeof(T));
-    if (e != cudaSuccess) {
-        set_error("device allocation of %zu bytes: %s", n * sizeof(T), cudaGetErrorString(e));
-        return BPM_ERR_OOM;
+// Buffers in one zeroed allocation (a training call on a new surrogate made 47, half of its time):
+// take() every buffer, then reserve(), which sets the pointers
+struct Pack {
+    size_t size = 0;
+    std::vector<std::pair<void**, size_t>> at;
+    template <class T>
+    void take(T** p, size_t n) {
+        at.push_back({reinterpret_cast<void**>(p), size});
+        size += (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~(size_t)255;
     }
-    return BPM_OK;
-}
+    int reserve(void** base, cudaStream_t s) {
+        cudaError_t e = cudaMalloc(base, size);
+        if (e == cudaSuccess) e = cudaMemsetAsync(*base, 0, size, s);
+        if (e != cudaSuccess) {
+            set_error("device allocation of %zu bytes: %s", size, cudaGetErrorString(e));
+            return BPM_ERR_OOM;
+        }
+        for (auto& q : at) *q.first = static_cast<char*>(*base) + q.second;
+        return BPM_OK;
+    }
+};
 
-int ensure_ws(Mlp* m, int rows) {
-    if (rows <= m->ws_rows) return BPM_OK;
+int ensure_ws(Mlp* m, int rows, bool train, cudaStream_t s) {
+    if (rows <= m->ws_rows && (m->ws_train || !train)) return BPM_OK;
+    rows = std::max(rows, m->ws_rows);
+    train = train || m->ws_train;
+    BPM_CK(cudaStreamSynchronize(s));
     free_ws(m);
+    Pack P;
     m->H.assign(m->L, nullptr);
     m->HT.assign(m->L, nullptr);
     m->Z.assign(m->L, nullptr);
-    for (int l = 0; l < m->L; ++l) {
-        BPM_TRY(zalloc(&m->H[l], (size_t)rows * m->in_pad[l]));
-        BPM_TRY(zalloc(&m->HT[l], (size_t)rows * m->in_pad[l]));
-        if (l < m->L - 1) BPM_TRY(zalloc(&m->Z[l], (size_t)rows * m->out_pad[l]));
-    }
-    BPM_TRY(zalloc(&m->logits, (size_t)rows * m->n_out));
-    BPM_TRY(zalloc(&m->Y, (size_t)rows * m->n_out));
-    BPM_TRY(zalloc(&m->colsum, (size_t)(rows / 32) * m->max_pad));
     m->dZ.assign(m->L, nullptr);
     m->dZT.assign(m->L, nullptr);
+    P.take(&m->logits, (size_t)rows * m->n_out);
     for (int l = 0; l < m->L; ++l) {
-        BPM_TRY(zalloc(&m->dZ[l], (size_t)rows * m->out_pad[l]));
-        BPM_TRY(zalloc(&m->dZT[l], (size_t)rows * m->out_pad[l]));
+        P.take(&m->H[l], (size_t)rows * m->in_pad[l]);
+        if (!train) continue;
+        P.take(&m->HT[l], (size_t)rows * m->in_pad[l]);
+        if (l < m->L - 1) P.take(&m->Z[l], (size_t)rows * m->out_pad[l]);
+        P.take(&m->dZ[l], (size_t)rows * m->out_pad[l]);
+        P.take(&m->dZT[l], (size_t)rows * m->out_pad[l]);
     }
-    if (!m->side) {
+    if (train) {
+        P.take(&m->Y, (size_t)rows * m->n_out);
+        P.take(&m->colsum, (size_t)(rows / 32) * m->max_pad);
+    }
+    BPM_TRY(P.reserve(&m->ws, s));
+    m->ws_rows = rows;
+    m->ws_train = train;
+    if (train && !m->side) {
         BPM_CK(cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking));
         m->ev.assign(m->L + 1, nullptr);
         for (auto& e : m->ev) BPM_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
-    m->ws_rows = rows;
     return BPM_OK;
 }
 
@@ -250,16 +259,6 @@ LayerTable table(const Mlp* m) {
     return T;
 }
 
-__nv_bfloat16** device_ptr_table(const std::vector<__nv_bfloat16*>& v, int* err) {
-    __nv_bfloat16** d = nullptr;
-    if (cudaMalloc(&d, v.size() * sizeof(void*)) != cudaSuccess ||
-        cudaMemcpy(d, v.data(), v.size() * sizeof(void*), cudaMemcpyHostToDevice) != cudaSuccess) {
-        *err = 1;
-        return nullptr;
-    }
-    return d;
-}
-
 // forward over `rows` (multiple of 128) batch rows, nb of them valid, input already in H[0]/HT[0]
 // infer: skip the pre-activations and transposes kept for the backward pass;
 // sigmoid: probabilities instead of logits in m->logits
@@ -359,6 +358,18 @@ __global__ void k_screen_mean(double* acc, long long n, int J) {
     if (i < n) acc[i] /= (double)J;
 }
 
+// BF16 copies of the current parameters; returns once they are there
+int publish(Mlp* m, cudaStream_t s) {
+    k_publish<<<(unsigned)((m->P + 255) / 256), 256, 0, s>>>((long long)m->P, table(m), m->params, m->d_W, m->d_WT);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        set_error("surrogate weight publish failed: %s", cudaGetErrorString(e));
+        return BPM_ERR_CUDA;
+    }
+    return BPM_OK;
+}
+
 int check_err(Mlp* m, cudaStream_t s) {
     int e = 0;
     BPM_CK(cudaMemcpyAsync(&e, m->err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -379,14 +390,7 @@ void free_mlp(Mlp* m) {
     for (auto e : m->ev)
         if (e) cudaEventDestroy(e);
     if (m->side) cudaStreamDestroy(m->side);
-    for (auto p : m->W) cudaFree(p);
-    for (auto p : m->WT) cudaFree(p);
-    cudaFree(m->params);
-    cudaFree(m->mom1);
-    cudaFree(m->mom2);
-    cudaFree(m->grad);
-    cudaFree(m->loss);
-    cudaFree(m->err);
+    cudaFree(m->arena);
     delete m;
 }
 
@@ -432,45 +436,35 @@ int bpm_surrogate_create(bpm_ctx* ctx, const bpm_mlp_cfg* cfg, const float* para
     }
     m->P = off;
     for (int l = 0; l < m->L; ++l) m->max_pad = std::max(m->max_pad, std::max(m->in_pad[l], m->out_pad[l]));
-    int r = BPM_OK;
-    auto chk = [&](int rr) {
-        if (r == BPM_OK) r = rr;
-    };
-    chk(zalloc(&m->params, m->P));
-    chk(zalloc(&m->mom1, m->P));
-    chk(zalloc(&m->mom2, m->P));
-    chk(zalloc(&m->grad, m->P));
-    chk(zalloc(&m->loss, 1));
-    chk(zalloc(&m->err, 1));
+    Pack A;
+    A.take(&m->params, m->P);
+    A.take(&m->mom1, m->P);
+    A.take(&m->mom2, m->P);
+    A.take(&m->grad, m->P);
+    A.take(&m->loss, 1);
+    A.take(&m->err, 1);
     m->W.assign(m->L, nullptr);
     m->WT.assign(m->L, nullptr);
-    for (int l = 0; l < m->L && r == BPM_OK; ++l) {
-        chk(zalloc(&m->W[l], (size_t)m->out_pad[l] * m->in_pad[l]));
-        chk(zalloc(&m->WT[l], (size_t)m->out_pad[l] * m->in_pad[l]));
+    for (int l = 0; l < m->L; ++l) {
+        A.take(&m->W[l], (size_t)m->out_pad[l] * m->in_pad[l]);
+        A.take(&m->WT[l], (size_t)m->out_pad[l] * m->in_pad[l]);
     }
+    A.take(&m->d_W, m->L);
+    A.take(&m->d_WT, m->L);
+    cudaStream_t s = ctx->stream;
+    int r = A.reserve(&m->arena, s);
     if (r == BPM_OK) {
-        cudaError_t e = cudaMemcpy(m->params, params, m->P * sizeof(float), cudaMemcpyHostToDevice);
+        cudaError_t e = cudaMemcpyAsync(m->params, params, m->P * sizeof(float), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(m->d_W, m->W.data(), m->L * sizeof(void*), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(m->d_WT, m->WT.data(), m->L * sizeof(void*), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) {
             set_error("parameter upload: %s", cudaGetErrorString(e));
             r = BPM_ERR_CUDA;
         }
     }
-    if (r == BPM_OK) {
-        int terr = 0;
-        __nv_bfloat16** dW = device_ptr_table(m->W, &terr);
-        __nv_bfloat16** dWT = device_ptr_table(m->WT, &terr);
-        if (!terr) {
-            k_publish<<<(unsigned)((m->P + 255) / 256), 256, 0, ctx->stream>>>((long long)m->P, table(m), m->params, dW,
-                                                                               dWT);
-            cudaStreamSynchronize(ctx->stream);
-        }
-        cudaFree(dW);
-        cudaFree(dWT);
-        if (terr || cudaGetLastError() != cudaSuccess) {
-            set_error("surrogate weight publish failed");
-            r = BPM_ERR_CUDA;
-        }
-    }
+    if (r == BPM_OK) r = publish(m, s);
     if (r != BPM_OK) {
         free_mlp(m);
         return r;
@@ -498,7 +492,7 @@ int bpm_surrogate_get_params(bpm_ctx* ctx, int32_t sid, float* out) {
 
 static int load_batch(bpm_ctx* ctx, Mlp* m, const float* Xd, const float* Yd, int nb, int rows) {
     cudaStream_t s = ctx->stream;
-    BPM_TRY(ensure_ws(m, rows));
+    BPM_TRY(ensure_ws(m, rows, Yd != nullptr, s));
     const long long cx = (long long)rows * (m->in_pad[0] / 8), ct = (long long)rows * m->in_pad[0];
     k_load_x<<<(unsigned)((cx + 255) / 256), 256, 0, s>>>(nb, rows, m->n_in, m->in_pad[0], Xd, m->H[0]);
     if (Yd) k_load_xt<<<(unsigned)((ct + 255) / 256), 256, 0, s>>>(nb, rows, m->n_in, m->in_pad[0], Xd, m->HT[0]);
@@ -554,14 +548,7 @@ int bpm_surrogate_train(bpm_ctx* ctx, int32_t sid, const float* X, const float* 
     BPM_CK(cudaMallocAsync(&curve, sizeof(float) * (size_t)steps, s));
     BPM_CK(cudaMemcpyAsync(Xd, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
     BPM_CK(cudaMemcpyAsync(Yd, Y, sizeof(float) * (size_t)N * m->n_out, cudaMemcpyHostToDevice, s));
-    int r = ensure_ws(m, rup(cfg->batch, 128));
-    int terr = 0;
-    __nv_bfloat16** dW = device_ptr_table(m->W, &terr);
-    __nv_bfloat16** dWT = device_ptr_table(m->WT, &terr);
-    if (terr && r == BPM_OK) {
-        set_error("pointer table upload failed");
-        r = BPM_ERR_CUDA;
-    }
+    int r = ensure_ws(m, rup(cfg->batch, 128), true, s);
     const LayerTable T = table(m);
     long long step = 0;
     for (int ep = 0; ep < cfg->epochs && r == BPM_OK; ++ep) {
@@ -577,7 +564,8 @@ int bpm_surrogate_train(bpm_ctx* ctx, int32_t sid, const float* X, const float* 
             const double c2 = 1.0 - std::pow((double)cfg->beta2, (double)m->t);
             k_adamw<<<(unsigned)((m->P + 255) / 256), 256, 0, s>>>((long long)m->P, T, m->params, m->mom1, m->mom2,
                                                                   m->grad, cfg->lr, cfg->weight_decay, cfg->beta1,
-                                                                  cfg->beta2, cfg->eps, (float)c1, (float)c2, dW, dWT);
+                                                                  cfg->beta2, cfg->eps, (float)c1, (float)c2, m->d_W,
+                                                                  m->d_WT);
             if (cudaGetLastError() != cudaSuccess) {
                 set_error("AdamW launch failed");
                 r = BPM_ERR_CUDA;
@@ -593,8 +581,6 @@ int bpm_surrogate_train(bpm_ctx* ctx, int32_t sid, const float* X, const float* 
         }
     }
     cudaStreamSynchronize(s);
-    cudaFree(dW);
-    cudaFree(dWT);
     cudaFreeAsync(Xd, s);
     cudaFreeAsync(Yd, s);
     cudaFreeAsync(curve, s);
@@ -748,20 +734,7 @@ int bpm_surrogate_load(bpm_ctx* ctx, int32_t sid, const char* path) {
     BPM_CK(cudaMemcpy(m->mom1, buf.data() + m->P, m->P * sizeof(float), cudaMemcpyHostToDevice));
     BPM_CK(cudaMemcpy(m->mom2, buf.data() + 2 * m->P, m->P * sizeof(float), cudaMemcpyHostToDevice));
     m->t = t;
-    int terr = 0;
-    __nv_bfloat16** dW = device_ptr_table(m->W, &terr);
-    __nv_bfloat16** dWT = device_ptr_table(m->WT, &terr);
-    if (!terr) {
-        k_publish<<<(unsigned)((m->P + 255) / 256), 256, 0, ctx->stream>>>((long long)m->P, table(m), m->params, dW, dWT);
-        cudaStreamSynchronize(ctx->stream);
-    }
-    cudaFree(dW);
-    cudaFree(dWT);
-    if (terr || cudaGetLastError() != cudaSuccess) {
-        set_error("surrogate weight publish failed");
-        return BPM_ERR_CUDA;
-    }
-    return BPM_OK;
+    return publish(m, ctx->stream);
 }
 
 int bpm_surrogate_destroy(bpm_ctx* ctx, int32_t sid) {
