@@ -85,76 +85,149 @@ __global__ void __launch_bounds__(kGpThreads) k_lhs_min_d2(const double* __restr
     }
 }
 
-// Cholesky factor of the correlation matrix of one theta vector per CTA, in place
-// in A (lower triangle, row-major [n][n]), then z = L^-1 y, w = L^-1 1 and
-// nll = n ln sigma2 + ln det R.  A non-positive pivot gives nll = +inf.
-__global__ void __launch_bounds__(kGpThreads) k_gp_factor(const double* __restrict__ X,
-                                                          const double* __restrict__ y, int n, int d,
-                                                          const double* __restrict__ theta, double nugget,
-                                                          double* __restrict__ Aall, double* __restrict__ zall,
-                                                          double* __restrict__ wall, double* __restrict__ nll,
-                                                          double* __restrict__ stats) {
+// ---------------------------------------------------------------------------
+// Cholesky factors of the correlation matrices of a batch of theta vectors, blocked over the whole GPU.
+// Matrix t is A[t] [n + 2][n], the lower triangle of R with two more rows, y and 1: factoring the first
+// n rows turns them into z = L^-1 y and w = L^-1 1, so the solves cost no pass of their own.  Per block
+// of 32 columns one launch factors the diagonal block (every CTA for itself) and solves 32 rows below
+// it a CTA, one launch subtracts the block's products from 32 x 32 tiles to its right.  An element's
+// products are subtracted in the order of k, one rounding each, as an unblocked factorisation does.
+// An SM does two FP64 multiply-adds a cycle: n = 160, 32 vectors are 22 M for the factors and as many
+// for the correlations, 0.08 ms spread over the GPU.  One CTA a matrix, unblocked from global memory,
+// took 1.40 ms; 0.47 ms now.
+// ---------------------------------------------------------------------------
+constexpr int kPB = 32;
+
+// rows 0 .. n - 1: the lower triangle of R; row n: y; row n + 1: ones
+__global__ void __launch_bounds__(kGpThreads) k_gp_matrix(const double* __restrict__ X, const double* __restrict__ y,
+                                                          int n, int d, const double* __restrict__ theta,
+                                                          double nugget, double* __restrict__ Aall) {
+    const int j = blockIdx.x * kPB + (threadIdx.x & 31), t = blockIdx.z;
+    if ((int)blockIdx.x > (int)blockIdx.y && (int)(blockIdx.y + 1) * kPB < n) return;   // above the diagonal
+    double* A = Aall + (size_t)t * (n + 2) * n;
+    const double* th = theta + (size_t)t * d;
+    for (int i = blockIdx.y * kPB + (threadIdx.x >> 5); i < min(n + 2, (int)(blockIdx.y + 1) * kPB);
+         i += kGpThreads / 32) {
+        if (j >= n || (i < n && j > i)) continue;
+        double v;
+        if (i >= n) {
+            v = i == n ? y[j] : 1.0;
+        } else {
+            double s = 0.0;
+            for (int k = 0; k < d; ++k) {
+                const double u = X[i * d + k] - X[j * d + k];
+                s += th[k] * u * u;
+            }
+            v = exp(-s) + (i == j ? nugget : 0.0);
+        }
+        A[(size_t)i * n + j] = v;
+    }
+}
+
+// Columns k0 .. k0 + 31: factor the diagonal block (written by CTA 0 of the matrix), solve the 32 rows
+// of this CTA below it.  A non-positive pivot marks the matrix as failed.
+__global__ void __launch_bounds__(kGpThreads) k_gp_panel(int n, int k0, double* __restrict__ Aall,
+                                                         int* __restrict__ fail) {
+    __shared__ double D[kPB][kPB + 1], P[kPB][kPB + 1], inv[kPB];
+    __shared__ int s_bad;
+    const int t = blockIdx.y, nb = min(kPB, n - k0), r0 = k0 + nb + kPB * blockIdx.x;
+    if (fail[t]) return;
+    double* A = Aall + (size_t)t * (n + 2) * n;
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_bad = 0;
+    if (w == 0) inv[l] = 0.0;
+    for (int i = w; i < kPB; i += kGpThreads / 32) {
+        D[i][l] = i < nb && l <= i ? A[(size_t)(k0 + i) * n + k0 + l] : 0.0;
+        P[i][l] = r0 + i < n + 2 && l < nb ? A[(size_t)(r0 + i) * n + k0 + l] : 0.0;
+    }
+    __syncthreads();
+    for (int k = 0; k < nb; ++k) {
+        if (w == 0) {                                       // one warp: an FP64 root or quotient costs every lane
+            const double piv = D[k][k];
+            double iv = 0.0;
+            if (l == 0) {
+                iv = rsqrt(piv);                            // one chain of FP64 latencies for root and quotient
+                inv[k] = iv;
+                if (!(piv > 0.0)) s_bad = 1;
+            }
+            iv = __shfl_sync(0xffffffffu, iv, 0);
+            __syncwarp();
+            if (l >= k && l < nb) D[l][k] *= iv;            // L_kk = piv / sqrt(piv)
+        }
+        __syncthreads();
+        if (s_bad) {
+            if (threadIdx.x == 0) fail[t] = 1;              // every CTA of the matrix writes the same
+            return;
+        }
+        for (int i = k + 1 + w; i < nb; i += kGpThreads / 32)
+            if (l > k && l <= i) D[i][l] -= D[i][k] * D[l][k];
+        __syncthreads();
+    }
+    if (blockIdx.x == 0)
+        for (int i = w; i < nb; i += kGpThreads / 32)
+            if (l <= i) A[(size_t)(k0 + i) * n + k0 + l] = D[i][l];
+    // row solve: a warp per four rows, lane = column.  The right-hand sides stay unscaled, the quotients
+    // go into the factor's columns (one multiply-add an element and step) and into the result.
+    double a[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = P[4 * w + q][l];
+    for (int k = 0; k < nb; ++k) {
+        const double c = l > k ? -D[l][k] * inv[k] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] += __shfl_sync(0xffffffffu, a[q], k) * c;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = r0 + 4 * w + q;
+        if (i < n + 2 && l < nb) A[(size_t)i * n + k0 + l] = a[q] * inv[l];
+    }
+}
+
+// Tiles right of the panel: A[i][j] -= sum over its columns of A[i][k] A[j][k] (j <= i for the rows of R)
+__global__ void __launch_bounds__(kGpThreads) k_gp_update(int n, int k0, double* __restrict__ Aall,
+                                                          const int* __restrict__ fail) {
+    __shared__ double Ri[kPB][kPB + 1], Rj[kPB][kPB + 1];
+    const int t = blockIdx.z, j0 = k0 + kPB * (1 + blockIdx.x), i0 = k0 + kPB * (1 + blockIdx.y);
+    if ((i0 + kPB <= n && i0 < j0) || j0 >= n || fail[t]) return;   // above the diagonal; the last row block has y and 1
+    double* A = Aall + (size_t)t * (n + 2) * n;
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int r = w; r < kPB; r += kGpThreads / 32) {
+        Ri[r][l] = i0 + r < n + 2 ? A[(size_t)(i0 + r) * n + k0 + l] : 0.0;
+        Rj[r][l] = j0 + r < n ? A[(size_t)(j0 + r) * n + k0 + l] : 0.0;
+    }
+    __syncthreads();
+    const int j = j0 + l;
+    double acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + 4 * w + q;
+        acc[q] = i < n + 2 && j < n ? A[(size_t)i * n + j] : 0.0;
+    }
+#pragma unroll 8
+    for (int k = 0; k < kPB; ++k) {
+        const double b = Rj[l][k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] -= Ri[4 * w + q][k] * b;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + 4 * w + q;
+        if (i < n + 2 && j < n && (i >= n || j <= i)) A[(size_t)i * n + j] = acc[q];
+    }
+}
+
+// nll = n ln sigma2 + ln det R from the factored matrix (one CTA each); +inf where it failed
+__global__ void __launch_bounds__(kGpThreads) k_gp_stats(int n, const double* __restrict__ Aall,
+                                                         const int* __restrict__ fail, double* __restrict__ nll,
+                                                         double* __restrict__ stats) {
     __shared__ double red[kGpThreads / 32];
-    __shared__ double th[kGpMaxD];
-    __shared__ int s_fail;
     const int t = blockIdx.x;
-    double* A = Aall + (size_t)t * n * n;
-    double* z = zall + (size_t)t * n;
-    double* w = wall + (size_t)t * n;
-    for (int k = threadIdx.x; k < d; k += blockDim.x) th[k] = theta[(size_t)t * d + k];
-    if (threadIdx.x == 0) s_fail = 0;
-    __syncthreads();
-    // lower triangle of R
-    for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) {
-        const int i = (int)(q / n), j = (int)(q % n);
-        if (j > i) continue;
-        double s = 0.0;
-        for (int k = 0; k < d; ++k) {
-            const double u = X[i * d + k] - X[j * d + k];
-            s += th[k] * u * u;
-        }
-        A[q] = exp(-s) + (i == j ? nugget : 0.0);
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int k = 0; k < n; ++k) {
-        __syncthreads();
-        const double piv = A[(size_t)k * n + k];
-        if (!(piv > 0.0)) {
-            if (threadIdx.x == 0) s_fail = 1;
-            break;
-        }
-        const double lkk = sqrt(piv);
-        __syncthreads();                       // every thread has read the pivot
-        if (threadIdx.x == 0) A[(size_t)k * n + k] = lkk;
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[(size_t)i * n + k] /= lkk;
-        __syncthreads();
-        for (int i = k + 1 + warp; i < n; i += nwarps) {
-            const double lik = A[(size_t)i * n + k];
-            for (int j = k + 1 + lane; j <= i; j += 32) A[(size_t)i * n + j] -= lik * A[(size_t)j * n + k];
-        }
-    }
-    __syncthreads();
-    if (s_fail) {
+    if (fail[t]) {
         if (threadIdx.x == 0) nll[t] = INFINITY;
         return;
     }
-    // forward substitution for y and 1 together: z_i = (y_i - sum_j<i L_ij z_j) / L_ii
-    for (int i = 0; i < n; ++i) {
-        double sz = 0.0, sw = 0.0;
-        for (int j = threadIdx.x; j < i; j += blockDim.x) {
-            const double l = A[(size_t)i * n + j];
-            sz += l * z[j];
-            sw += l * w[j];
-        }
-        sz = cta_sum(sz, red);
-        sw = cta_sum(sw, red);
-        if (threadIdx.x == 0) {
-            const double l = A[(size_t)i * n + i];
-            z[i] = (y[i] - sz) / l;
-            w[i] = (1.0 - sw) / l;
-        }
-        __syncthreads();
-    }
+    const double* A = Aall + (size_t)t * (n + 2) * n;
+    const double *z = A + (size_t)n * n, *w = z + n;
     double ww = 0.0, wz = 0.0, ld = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         ww += w[i] * w[i];
@@ -182,16 +255,67 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_factor(const double* __restri
     }
 }
 
-// column j of Linv = L^-1 by forward substitution (one thread per column)
-__global__ void k_gp_linv(const double* __restrict__ L, int n, double* __restrict__ Linv) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    for (int i = 0; i < j; ++i) Linv[(size_t)i * n + j] = 0.0;
-    Linv[(size_t)j * n + j] = 1.0 / L[(size_t)j * n + j];
-    for (int i = j + 1; i < n; ++i) {
-        double s = 0.0;
-        for (int k = j; k < i; ++k) s += L[(size_t)i * n + k] * Linv[(size_t)k * n + j];
-        Linv[(size_t)i * n + j] = -s / L[(size_t)i * n + i];
+// factors and likelihoods of T matrices (A: T (n + 2) n doubles, fail: T ints)
+int gp_factor(cudaStream_t s, const double* X, const double* y, int n, int d, const double* theta, int T,
+              double nugget, double* A, int* fail, double* nll, double* stats) {
+    const int nblk = (n + kPB - 1) / kPB, nrow = (n + 2 + kPB - 1) / kPB;
+    BPM_CK(cudaMemsetAsync(fail, 0, T * sizeof(int), s));
+    for (int t0 = 0; t0 < T; t0 += 32768) {                 // grid y and z limit
+        const int m = std::min(32768, T - t0);
+        double* At = A + (size_t)t0 * (n + 2) * n;
+        k_gp_matrix<<<dim3(nblk, nrow, m), kGpThreads, 0, s>>>(X, y, n, d, theta + (size_t)t0 * d, nugget, At);
+        for (int p = 0; p < nblk; ++p) {
+            const int k0 = p * kPB, below = n + 2 - std::min(n, k0 + kPB);
+            k_gp_panel<<<dim3((below + kPB - 1) / kPB, m), kGpThreads, 0, s>>>(n, k0, At, fail + t0);
+            if (p + 1 < nblk)
+                k_gp_update<<<dim3(nblk - p - 1, nrow - p - 1, m), kGpThreads, 0, s>>>(n, k0, At, fail + t0);
+        }
+        k_gp_stats<<<m, kGpThreads, 0, s>>>(n, At, fail + t0, nll + t0, stats ? stats + 3 * (size_t)t0 : nullptr);
+    }
+    BPM_CK(cudaGetLastError());
+    return BPM_OK;
+}
+
+// Block row i0 .. i0 + 31 of Linv = L^-1 (L: [n + 2][n]): 32 columns a CTA, products of the block rows
+// above (in the order of k) first, then the triangular solve within the block; Linv_ij = -s / L_ii.
+// (One thread per column walked the whole triangle: 0.81 ms at n = 160; 0.26 ms now.)
+__global__ void __launch_bounds__(kGpThreads) k_gp_linv(const double* __restrict__ L, int n, int i0,
+                                                        double* __restrict__ Linv) {
+    __shared__ double Lb[kPB][kPB + 1], Xb[kPB][kPB + 1];
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * kPB + l;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k0 = blockIdx.x * kPB; k0 < i0; k0 += kPB) {   // rows of Linv above column block: zero
+        __syncthreads();
+        for (int r = w; r < kPB; r += kGpThreads / 32) {
+            Lb[r][l] = i0 + r < n ? L[(size_t)(i0 + r) * n + k0 + l] : 0.0;
+            Xb[r][l] = j < n ? Linv[(size_t)(k0 + r) * n + j] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int k = 0; k < kPB; ++k)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] += Lb[4 * w + q][k] * Xb[k][l];
+    }
+    __syncthreads();
+    for (int r = w; r < kPB; r += kGpThreads / 32)
+        Lb[r][l] = i0 + r < n && i0 + l < n && l <= r ? L[(size_t)(i0 + r) * n + i0 + l] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Xb[4 * w + q][l] = s[q];
+    __syncthreads();
+    if (w) return;
+    const double dinv = i0 + l < n ? 1.0 / Lb[l][l] : 0.0;  // of every row at once
+    for (int r = 0; r < kPB && i0 + r < n; ++r) {           // one warp, lane = column
+        const int i = i0 + r;
+        double u[4] = {Xb[r][l], 0.0, 0.0, 0.0};            // four sums: a chain of FP64 latencies otherwise
+        int k = 0;
+        for (; k + 4 <= r; k += 4)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) u[e] += Lb[r][k + e] * Xb[k + e][l];
+        for (; k < r; ++k) u[0] += Lb[r][k] * Xb[k][l];
+        const double q = __shfl_sync(0xffffffffu, dinv, r);
+        const double v = i == j ? q : i > j ? -((u[0] + u[1]) + (u[2] + u[3])) * q : 0.0;
+        Xb[r][l] = v;
+        if (j < n) Linv[(size_t)i * n + j] = v;
     }
 }
 
@@ -234,42 +358,42 @@ __global__ void k_gp_corr(const double* __restrict__ C, const double* __restrict
     Rc[q] = exp(-s);
 }
 
-// V[N][n] = Rc[N][n] * Linv[n][n]^T, FP64, 64 x 64 tiles, 4 x 4 outputs per thread.  B lower
+// V[N][n] = Rc[N][n] * Linv[n][n]^T, FP64, 32 x 64 tiles, 2 x 4 outputs per thread (64 x 64 tiles of
+// 4000 candidates and n = 160 were 189 CTAs of unequal depth on 152 SMs: 329 us, 236 now).  B lower
 // triangular: row r of B is zero past column r, so output columns n0 .. n0 + 63 need K only up
 // to n0 + 64 (the skipped products are exact zeros; the sums are unchanged)
-constexpr int kTM = 64, kTN = 64, kTK = 16;
+constexpr int kTM = 32, kTN = 64, kTK = 16;
 __global__ void __launch_bounds__(256) k_gp_gemm_nt(const double* __restrict__ A, const double* __restrict__ B,
                                                     int M, int N, int K, double* __restrict__ Cout) {
     __shared__ double As[kTK][kTM + 1];
     __shared__ double Bs[kTK][kTN + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int m0 = blockIdx.y * kTM, n0 = blockIdx.x * kTN;
-    double acc[4][4] = {};
+    double acc[2][4] = {};
     const int kend = min(K, n0 + kTN);
     for (int k0 = 0; k0 < kend; k0 += kTK) {
-        for (int e = threadIdx.x; e < kTM * kTK; e += 256) {
+        for (int e = threadIdx.x; e < kTN * kTK; e += 256) {
             const int r = e / kTK, kk = e % kTK;
-            As[kk][r] = (m0 + r < M && k0 + kk < K) ? A[(size_t)(m0 + r) * K + k0 + kk] : 0.0;
+            if (r < kTM) As[kk][r] = (m0 + r < M && k0 + kk < K) ? A[(size_t)(m0 + r) * K + k0 + kk] : 0.0;
             Bs[kk][r] = (n0 + r < N && k0 + kk < K) ? B[(size_t)(n0 + r) * K + k0 + kk] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < kTK; ++kk) {
-            double av[4], bv[4];
+            double av[2], bv[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                av[q] = As[kk][ty + 16 * q];
-                bv[q] = Bs[kk][tx + 16 * q];
-            }
+            for (int q = 0; q < 2; ++q) av[q] = As[kk][ty + 16 * q];
 #pragma unroll
-            for (int p = 0; p < 4; ++p)
+            for (int q = 0; q < 4; ++q) bv[q] = Bs[kk][tx + 16 * q];
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int p = 0; p < 2; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int r = m0 + ty + 16 * p, col = n0 + tx + 16 * q;
@@ -319,29 +443,11 @@ using namespace bpm;
 
 namespace {
 
-// device buffers of one call, freed on every exit path
-struct GpScratch {
-    std::vector<void*> ptrs;
-    template <typename T>
-    int alloc(T** p, size_t count) {
-        cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(1, count) * sizeof(T));
-        if (e != cudaSuccess) {
-            set_error("optimiser buffers: %s", cudaGetErrorString(e));
-            return BPM_ERR_OOM;
-        }
-        ptrs.push_back(*p);
-        return BPM_OK;
-    }
-    template <typename T>
-    int upload(T** p, const T* h, size_t count, cudaStream_t s) {
-        BPM_TRY(alloc(p, count));
-        BPM_CK(cudaMemcpyAsync(*p, h, count * sizeof(T), cudaMemcpyHostToDevice, s));
-        return BPM_OK;
-    }
-    ~GpScratch() {
-        for (void* p : ptrs) cudaFree(p);
-    }
-};
+template <typename T>
+int upload(T* d, const T* h, size_t count, cudaStream_t s) {
+    BPM_CK(cudaMemcpyAsync(d, h, count * sizeof(T), cudaMemcpyHostToDevice, s));
+    return BPM_OK;
+}
 
 int check_design(const double* X, const double* y, int n, int d) {
     if (!X || !y || n < 2 || n > kGpMaxN || d < 1 || d > kGpMaxD) {
@@ -370,10 +476,12 @@ extern "C" int bpm_lhs_maximin(bpm_ctx* ctx, const double* cands, int32_t T, int
     }
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
-    GpScratch sc;
+    CallBuffers sc(ctx);
     double *dC = nullptr, *dD = nullptr;
-    BPM_TRY(sc.upload(&dC, cands, (size_t)T * n * d, s));
-    BPM_TRY(sc.alloc(&dD, T));
+    sc.take(&dC, (size_t)T * n * d);
+    sc.take(&dD, T);
+    BPM_TRY(sc.reserve());
+    BPM_TRY(upload(dC, cands, (size_t)T * n * d, s));
     k_lhs_min_d2<<<T, kGpThreads, 0, s>>>(dC, n, d, dD);
     BPM_CK(cudaGetLastError());
     std::vector<double> h(T);
@@ -397,21 +505,23 @@ extern "C" int bpm_gp_nll(bpm_ctx* ctx, const double* X, const double* y, int32_
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
     // theta vectors per launch: their factors together stay under 1 GiB
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(T, (size_t(1) << 30) / (8 * (size_t)n * n)));
-    GpScratch sc;
-    double *dX = nullptr, *dy = nullptr, *dth = nullptr, *A = nullptr, *z = nullptr, *w = nullptr, *dn = nullptr;
-    BPM_TRY(sc.upload(&dX, X, (size_t)n * d, s));
-    BPM_TRY(sc.upload(&dy, y, n, s));
-    BPM_TRY(sc.upload(&dth, theta, (size_t)T * d, s));
-    BPM_TRY(sc.alloc(&A, (size_t)chunk * n * n));
-    BPM_TRY(sc.alloc(&z, (size_t)chunk * n));
-    BPM_TRY(sc.alloc(&w, (size_t)chunk * n));
-    BPM_TRY(sc.alloc(&dn, T));
-    for (int t0 = 0; t0 < T; t0 += chunk) {
-        const int m = std::min(chunk, T - t0);
-        k_gp_factor<<<m, kGpThreads, 0, s>>>(dX, dy, n, d, dth + (size_t)t0 * d, nugget, A, z, w, dn + t0, nullptr);
-        BPM_CK(cudaGetLastError());
-    }
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(T, (size_t(1) << 30) / (8 * (size_t)(n + 2) * n)));
+    CallBuffers sc(ctx);
+    double *dX = nullptr, *dy = nullptr, *dth = nullptr, *A = nullptr, *dn = nullptr;
+    int* fail = nullptr;
+    sc.take(&dX, (size_t)n * d);
+    sc.take(&dy, n);
+    sc.take(&dth, (size_t)T * d);
+    sc.take(&A, (size_t)chunk * (n + 2) * n);
+    sc.take(&fail, chunk);
+    sc.take(&dn, T);
+    BPM_TRY(sc.reserve());
+    BPM_TRY(upload(dX, X, (size_t)n * d, s));
+    BPM_TRY(upload(dy, y, n, s));
+    BPM_TRY(upload(dth, theta, (size_t)T * d, s));
+    for (int t0 = 0; t0 < T; t0 += chunk)
+        BPM_TRY(gp_factor(s, dX, dy, n, d, dth + (size_t)t0 * d, std::min(chunk, T - t0), nugget, A, fail, dn + t0,
+                          nullptr));
     BPM_CK(cudaMemcpyAsync(nll, dn, T * sizeof(double), cudaMemcpyDeviceToHost, s));
     BPM_CK(cudaStreamSynchronize(s));
     return BPM_OK;
@@ -426,8 +536,9 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
     BPM_TRY(check_design(X, y, n, d));
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
-    GpScratch sc;
-    double *dy = nullptr, *A = nullptr, *z = nullptr, *w = nullptr, *dn = nullptr, *st = nullptr, *u = nullptr;
+    CallBuffers sc(ctx);
+    double *dy = nullptr, *A = nullptr, *dn = nullptr, *st = nullptr, *u = nullptr;
+    int* dfail = nullptr;
     Gp* g = new Gp();
     g->n = n;
     g->d = d;
@@ -436,9 +547,13 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
         return r;
     };
     int r = BPM_OK;
-    if ((r = sc.upload(&dy, y, n, s)) || (r = sc.alloc(&A, (size_t)n * n)) || (r = sc.alloc(&z, n)) ||
-        (r = sc.alloc(&w, n)) || (r = sc.alloc(&dn, 1)) || (r = sc.alloc(&st, 3)) || (r = sc.alloc(&u, n)))
-        return fail(r);
+    sc.take(&dy, n);
+    sc.take(&A, (size_t)(n + 2) * n);
+    sc.take(&dn, 1);
+    sc.take(&st, 3);
+    sc.take(&u, n);
+    sc.take(&dfail, 1);
+    if ((r = sc.reserve()) || (r = upload(dy, y, n, s))) return fail(r);
     cudaError_t e = cudaMalloc(&g->X, (size_t)n * d * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&g->theta, d * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&g->Linv, (size_t)n * n * sizeof(double));
@@ -450,7 +565,7 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
         set_error("kriging model buffers: %s", cudaGetErrorString(e));
         return fail(BPM_ERR_OOM);
     }
-    k_gp_factor<<<1, kGpThreads, 0, s>>>(g->X, dy, n, d, g->theta, nugget, A, z, w, dn, st);
+    if ((r = gp_factor(s, g->X, dy, n, d, g->theta, 1, nugget, A, dfail, dn, st))) return fail(r);
     double hst[3] = {0, 0, 0}, hn = 0;
     e = cudaMemcpyAsync(hst, st, sizeof(hst), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hn, dn, sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -467,7 +582,8 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
     g->sigma2 = hst[1];
     g->one_Ri_1 = hst[2];
     const int nb = (n + 127) / 128;
-    k_gp_linv<<<nb, 128, 0, s>>>(A, n, g->Linv);
+    for (int i0 = 0; i0 < n; i0 += kPB)
+        k_gp_linv<<<(n + kPB - 1) / kPB, kGpThreads, 0, s>>>(A, n, i0, g->Linv);
     k_gp_rows<<<nb, 128, 0, s>>>(g->Linv, dy, g->mu, n, u, g->c);
     k_gp_cols<<<nb, 128, 0, s>>>(g->Linv, u, n, g->a);
     e = cudaGetLastError();
@@ -498,14 +614,15 @@ extern "C" int bpm_gp_predict(bpm_ctx* ctx, int32_t gp_id, const double* C, int6
     cudaStream_t s = ctx->stream;
     const int n = g->n, d = g->d;
     const int chunk = (int)std::min<int64_t>(N, 32768);
-    GpScratch sc;
+    CallBuffers sc(ctx);
     double *dC = nullptr, *Rc = nullptr, *V = nullptr, *dy = nullptr, *ds = nullptr, *de = nullptr;
-    BPM_TRY(sc.alloc(&dC, (size_t)chunk * d));
-    BPM_TRY(sc.alloc(&Rc, (size_t)chunk * n));
-    BPM_TRY(sc.alloc(&V, (size_t)chunk * n));
-    BPM_TRY(sc.alloc(&dy, chunk));
-    BPM_TRY(sc.alloc(&ds, chunk));
-    BPM_TRY(sc.alloc(&de, chunk));
+    sc.take(&dC, (size_t)chunk * d);
+    sc.take(&Rc, (size_t)chunk * n);
+    sc.take(&V, (size_t)chunk * n);
+    sc.take(&dy, chunk);
+    sc.take(&ds, chunk);
+    sc.take(&de, chunk);
+    BPM_TRY(sc.reserve());
     for (int64_t c0 = 0; c0 < N; c0 += chunk) {
         const int m = (int)std::min<int64_t>(chunk, N - c0);
         BPM_CK(cudaMemcpyAsync(dC, C + c0 * d, (size_t)m * d * sizeof(double), cudaMemcpyHostToDevice, s));
