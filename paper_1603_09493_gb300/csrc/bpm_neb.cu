@@ -17,29 +17,6 @@ namespace {
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-// device buffers of one band run, freed on every exit path
-struct NebBuffers {
-    std::vector<void*> ptrs;
-    template <typename T>
-    int alloc(T** p, size_t count) {
-        cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(1, count) * sizeof(T));
-        if (e != cudaSuccess) {
-            set_error("band buffers: %s", cudaGetErrorString(e));
-            return BPM_ERR_OOM;
-        }
-        ptrs.push_back(*p);
-        e = cudaMemset(*p, 0, std::max<size_t>(1, count) * sizeof(T));
-        if (e != cudaSuccess) {
-            set_error("band buffers: %s", cudaGetErrorString(e));
-            return BPM_ERR_CUDA;
-        }
-        return BPM_OK;
-    }
-    ~NebBuffers() {
-        for (void* p : ptrs) cudaFree(p);
-    }
-};
-
 }  // namespace
 }  // namespace bpm
 
@@ -91,29 +68,32 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
 
-    NebBuffers buf;
+    CallBuffers buf(ctx);
     float4* d_isl = nullptr;
     float *m0 = nullptr, *m1 = nullptr, *Bt = nullptr, *Hd = nullptr, *A32 = nullptr, *fmax = nullptr;
     __nv_bfloat16 *Ahi = nullptr, *Alo = nullptr;
     double* E = nullptr;
     int* err = nullptr;
     const size_t S = (size_t)Rp * 3 * np, G = (size_t)Rp * K;
-    BPM_TRY(buf.alloc(&d_isl, 3 * (size_t)R));
-    BPM_TRY(buf.alloc(&m0, S));
-    BPM_TRY(buf.alloc(&m1, S));
-    BPM_TRY(buf.alloc(&Bt, S));
     const bool tc = prec == BPM_PREC_BF16X3 || prec == BPM_PREC_BF16;
     const int splits = tc ? gemm_splits(R, K, ctx->sm_count) : 1;   // planes of Hd
-    BPM_TRY(buf.alloc(&Hd, splits * G));
+    buf.take(&err, 1);
+    buf.take(&m0, S);
+    buf.take(&m1, S);
     if (prec == BPM_PREC_FP32) {
-        BPM_TRY(buf.alloc(&A32, G));
+        buf.take(&A32, G);
     } else {
-        BPM_TRY(buf.alloc(&Ahi, G));
-        BPM_TRY(buf.alloc(&Alo, G));
+        buf.take(&Ahi, G);
+        buf.take(&Alo, G);
     }
-    BPM_TRY(buf.alloc(&E, R));
-    BPM_TRY(buf.alloc(&fmax, R));
-    BPM_TRY(buf.alloc(&err, 1));
+    const size_t zeroed = buf.size;              // pads of the states and the operand stay zero
+    buf.take(&Hd, splits * G);
+    buf.take(&Bt, S);
+    buf.take(&d_isl, 3 * (size_t)R);
+    buf.take(&E, R);
+    buf.take(&fmax, R);
+    BPM_TRY(buf.reserve());
+    BPM_CK(cudaMemsetAsync(err, 0, zeroed, s));
 
     // island parameters, the same for every image of a band
     std::vector<float4> ip(3 * (size_t)R);
@@ -178,7 +158,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     }
     auto demag = [&]() -> int {
         if (!(p->term_mask & BPM_TERM_DEMAG)) return BPM_OK;
-        if (tc) return grouped_gemm_launch(s, gg, ctx->sm_count, err);
+        if (tc) return grouped_gemm_launch(s, gg, ctx->sm_count, err, true);
         if (prec == BPM_PREC_FP32) return gemm_f32_nt(s, R, K, K, A32, K, M->N32, K, Hd, K);
         return gemm_bf16x3_simt(s, Rp, K, K, Ahi, Alo, M->Nhi, M->Nlo, Hd, 3);
     };
@@ -195,10 +175,12 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
         a.m = cur;
         r = demag();
         if (r != BPM_OK) break;
-        launch_neb_energy(a, Bt, E, vol_scale, s);
+        r = launch_neb_energy(a, Bt, E, vol_scale, ctx->sm_count, s);
+        if (r != BPM_OK) break;
         NebArgs nb{P, (p->climb_after >= 0 && it >= p->climb_after) ? 1 : 0, (float)p->step, (float)p->spring,
                    E, Bt, cur, nxt, fmax};
-        launch_neb_step(a, nb, s);
+        r = launch_neb_step(a, nb, ctx->sm_count, s);
+        if (r != BPM_OK) break;
         std::swap(cur, nxt);
         if ((it + 1) % check == 0 || it + 1 == p->max_iters) {
             cudaError_t e = cudaMemcpyAsync(fm.data(), fmax, R * sizeof(float), cudaMemcpyDeviceToHost, s);
@@ -220,7 +202,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
         a.m = cur;
         r = demag();
     }
-    if (r == BPM_OK) launch_neb_energy(a, Bt, E, vol_scale, s);
+    if (r == BPM_OK) r = launch_neb_energy(a, Bt, E, vol_scale, ctx->sm_count, s);
     if (tc) grouped_gemm_free(&gg);
     if (r != BPM_OK) return r;
     cudaError_t e = cudaStreamSynchronize(s);

@@ -539,19 +539,10 @@ __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, f
 // An interval of 9 islands of 481 nodes (8 steps): 330 -> 187 us; of one island of 209 nodes (6 steps):
 // 172 -> 125 us; of 128 islands of 1547 nodes (28 steps): 3.10 -> 1.98 ms.
 // ---------------------------------------------------------------------------
-template <int STAGE>
-__device__ __forceinline__ void few_body(const StepArgs& a, int b, int j, float* red, StageClock& clk) {
-    extern __shared__ float4 smem4[];
-    float* sm = reinterpret_cast<float*>(smem4);
+// the head field at every node (into hb [3][n_pad]) and the exchange entries (into L1)
+__device__ __forceinline__ void prepare_nodes(const StepArgs& a, float4 p1, float4 p2, float xh, float* hb) {
     const int np = a.n_pad;
-    float* hb = sm + 3 * np;                               // head field, [3][n_pad]
-    const size_t base = (size_t)b * 3 * np;
-    pdl_trigger();
-    set_clock(clk, a, j, STAGE == 2);
-    const float4 p0 = a.isl[3 * b], p1 = a.isl[3 * b + 1], p2 = a.isl[3 * b + 2];
     const bool head = (a.mask & BPM_TERM_HEAD) && a.map;
-    __syncthreads();
-    const float ramp = clk.ramp, xh = clk.xh;
     for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
         const float4 pos = __ldg(a.node_pos + i);
         if (a.mask & BPM_TERM_EXCHANGE) {
@@ -567,6 +558,21 @@ __device__ __forceinline__ void few_body(const StepArgs& a, int b, int j, float*
             hb[2 * np + i] = h.z;
         }
     }
+}
+
+template <int STAGE>
+__device__ __forceinline__ void few_body(const StepArgs& a, int b, int j, float* red, StageClock& clk) {
+    extern __shared__ float4 smem4[];
+    float* sm = reinterpret_cast<float*>(smem4);
+    const int np = a.n_pad;
+    float* hb = sm + 3 * np;                               // head field, [3][n_pad]
+    const size_t base = (size_t)b * 3 * np;
+    pdl_trigger();
+    set_clock(clk, a, j, STAGE == 2);
+    const float4 p0 = a.isl[3 * b], p1 = a.isl[3 * b + 1], p2 = a.isl[3 * b + 2];
+    __syncthreads();
+    const float ramp = clk.ramp, xh = clk.xh;
+    prepare_nodes(a, p1, p2, xh, hb);
     pdl_wait();
     const float h = (float)a.h, hh = 0.5f * h;
     if (STAGE == 1)
@@ -670,35 +676,67 @@ __device__ __forceinline__ double block_sum_d(double v, double* red) {
     return s;
 }
 
+// sums over the CTA of N doubles per thread, in a fixed order; every thread gets them.  red: N * NT / 32
+// doubles.  (FP64 runs at two operations a cycle and SM: the warps' sums are added by one warp.)
+template <int NT, int N>
+__device__ __forceinline__ void block_sums_d(double (&v)[N], double* red) {
+    constexpr int NW = NT / 32;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int q = 0; q < N; ++q) red[q * NW + (threadIdx.x >> 5)] = v[q];
+    __syncthreads();
+    if (threadIdx.x < N) {
+        double s = 0.0;
+        for (int w = 0; w < NW; ++w) s += red[threadIdx.x * NW + w];
+        red[threadIdx.x * NW] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = red[q * NW];
+}
+
 // total field Bt of every image and its energy
 //   E = -sum_i V_i Ms_i (B_quad,i / 2 + B_lin,i) . m_i   (J; vol_scale = sum V [nm^3] * 1e-21)
-__global__ void __launch_bounds__(kStepThreads) k_neb_energy(StepArgs a, float* __restrict__ Bt,
-                                                             double* __restrict__ E, double vol_scale) {
+// AHEAD (few images, see few_body): launched programmatically behind the GEMM, with the head field, which
+// does not change along the run, and the exchange entries taken before the wait.  45 images of 481
+// nodes, one band update (GEMM, this and k_neb_step): 40 us one after the other, 34 so.
+template <int NT, bool AHEAD>
+__global__ void __launch_bounds__(NT) k_neb_energy(StepArgs a, float* __restrict__ Bt, double* __restrict__ E,
+                                                   double vol_scale) {
     extern __shared__ float4 smem4[];
-    __shared__ double red[kStepThreads / 32];
+    __shared__ double red[NT / 32];
     float* sm = reinterpret_cast<float*>(smem4);
     const int b = blockIdx.x;
     const int np = a.n_pad;
+    float* hb = sm + 3 * np;
     const size_t base = (size_t)b * 3 * np;
     const float4 p0 = a.isl[3 * b], p1 = a.isl[3 * b + 1], p2 = a.isl[3 * b + 2];
     const float xh = a.x0;
+    pdl_trigger();
+    if (AHEAD) prepare_nodes(a, p1, p2, xh, hb);
+    pdl_wait();
     stage_state(a.m + base, sm, np);
     __syncthreads();
-    double e = 0.0;
-    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+    double e[1] = {0.0};
+    for (int i = threadIdx.x; i < a.n; i += NT) {
         const float3 mi = f3(sm[i], sm[np + i], sm[2 * np + i]);
+        float3 hv = f3(0, 0, 0);
+        if (AHEAD) hv = f3(hb[i], hb[np + i], hb[2 * np + i]);
         const float3 Bq = eff_field(a, b, i, mi, sm, p0, p1, p2, 1.f, xh, a.mask & kQuadTerms);
-        const float3 Bl = eff_field(a, b, i, mi, sm, p0, p1, p2, 1.f, xh, a.mask & kLinTerms);
+        const float3 Bl = eff_field(a, b, i, mi, sm, p0, p1, p2, 1.f, xh, a.mask & kLinTerms, AHEAD ? &hv : nullptr);
         const float3 B = Bq + Bl;
         Bt[base + i] = B.x;
         Bt[base + np + i] = B.y;
         Bt[base + 2 * np + i] = B.z;
         const float msn = __ldg(&a.node_mat[i].y) * p0.z;
         const float w = __ldg(&a.node_pos[i].w);
-        e += (double)(w * msn) * (double)dot3(0.5f * Bq + Bl, mi);
+        e[0] += (double)(w * msn) * (double)dot3(0.5f * Bq + Bl, mi);
     }
-    const double tot = block_sum_d<kStepThreads>(e, red);
-    if (threadIdx.x == 0) E[b] = -vol_scale * tot;
+    block_sums_d<NT, 1>(e, red);
+    if (threadIdx.x == 0) E[b] = -vol_scale * e[0];
 }
 
 __device__ __forceinline__ float3 perp3(float3 v, float3 m) { return v + (-dot3(v, m)) * m; }
@@ -708,14 +746,17 @@ __device__ __forceinline__ float3 load_state(const float* m, size_t base, int np
 }
 
 // one band update of every image (Jacobi: neighbours from m_in, result to m_out)
-__global__ void __launch_bounds__(kStepThreads) k_neb_step(StepArgs a, NebArgs nb) {
-    __shared__ double red[kStepThreads / 32];
+template <int NT>
+__global__ void __launch_bounds__(NT) k_neb_step(StepArgs a, NebArgs nb) {
+    __shared__ double red[4 * NT / 32];
     __shared__ int s_ci;
+    pdl_trigger();
     const int b = blockIdx.x, P = nb.P, d = b / P, k = b - d * P;
     const int np = a.n_pad;
     const size_t S = 3 * (size_t)np, base = (size_t)b * S;
     const float msc = a.isl[3 * b].z;
     const bool end = (k == 0 || k == P - 1);
+    pdl_wait();
     // climbing image of this band: the interior image of highest energy
     if (threadIdx.x == 0) {
         int ci = -1;
@@ -750,8 +791,8 @@ __global__ void __launch_bounds__(kStepThreads) k_neb_step(StepArgs a, NebArgs n
             cm = (float)(Ep > Em ? dmin : dmax);
         }
         // pass 1: |t|^2, <g, t>, |m+ - m|^2, |m - m-|^2
-        double stt = 0.0, sft = 0.0, dn = 0.0, dp = 0.0;
-        for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        double sum[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = threadIdx.x; i < a.n; i += NT) {
             const float w = __ldg(&a.node_pos[i].w);
             const float3 m0 = load_state(nb.m_in, base, np, i);
             const float3 mp = load_state(nb.m_in, base + S, np, i);
@@ -759,23 +800,20 @@ __global__ void __launch_bounds__(kStepThreads) k_neb_step(StepArgs a, NebArgs n
             const float3 dplus = sub3(mp, m0), dminus = sub3(m0, mm);
             const float3 t = perp3(cp * dplus + cm * dminus, m0);
             const float3 g = (__ldg(&a.node_mat[i].y) * msc) * perp3(load_state(nb.Bt, base, np, i), m0);
-            stt += (double)(w * dot3(t, t));
-            sft += (double)(w * dot3(g, t));
-            dn += (double)(w * dot3(dplus, dplus));
-            dp += (double)(w * dot3(dminus, dminus));
+            sum[0] += (double)(w * dot3(t, t));
+            sum[1] += (double)(w * dot3(g, t));
+            sum[2] += (double)(w * dot3(dplus, dplus));
+            sum[3] += (double)(w * dot3(dminus, dminus));
         }
-        stt = block_sum_d<kStepThreads>(stt, red);
-        sft = block_sum_d<kStepThreads>(sft, red);
-        dn = block_sum_d<kStepThreads>(dn, red);
-        dp = block_sum_d<kStepThreads>(dp, red);
-        inv_t = stt > 0.0 ? 1.0 / sqrt(stt) : 0.0;
-        s_ft = sft * inv_t;                                  // <g, t_hat>
-        spring_term = (double)nb.spring * (sqrt(dn) - sqrt(dp));
+        block_sums_d<NT, 4>(sum, red);
+        inv_t = sum[0] > 0.0 ? 1.0 / sqrt(sum[0]) : 0.0;
+        s_ft = sum[1] * inv_t;                               // <g, t_hat>
+        spring_term = (double)nb.spring * (sqrt(sum[2]) - sqrt(sum[3]));
     }
     // pass 2: band force and the normalised step
     const float c_t = climbing ? (float)(-2.0 * s_ft * inv_t) : (float)((spring_term - s_ft) * inv_t);
     float fmax_loc = 0.f;
-    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+    for (int i = threadIdx.x; i < a.n; i += NT) {
         const float3 m0 = load_state(nb.m_in, base, np, i);
         const float msn = __ldg(&a.node_mat[i].y) * msc;
         float3 f = msn * perp3(load_state(nb.Bt, base, np, i), m0);
@@ -793,12 +831,12 @@ __global__ void __launch_bounds__(kStepThreads) k_neb_step(StepArgs a, NebArgs n
         write_gemm_input(a, b, i, v, msn);
     }
     for (int o = 16; o > 0; o >>= 1) fmax_loc = fmaxf(fmax_loc, __shfl_xor_sync(0xffffffffu, fmax_loc, o));
-    __shared__ float redf[kStepThreads / 32];
+    __shared__ float redf[NT / 32];
     if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = fmax_loc;
     __syncthreads();
     if (threadIdx.x == 0) {
         float f = 0.f;
-        for (int w = 0; w < kStepThreads / 32; ++w) f = fmaxf(f, redf[w]);
+        for (int w = 0; w < NT / 32; ++w) f = fmaxf(f, redf[w]);
         nb.fmax[b] = f;
     }
 }
@@ -927,7 +965,9 @@ int configure_step_kernels() {
     BPM_CK(cudaFuncSetAttribute(k_stage2<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_stage2<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_field, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    BPM_CK(cudaFuncSetAttribute(k_neb_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_neb_energy<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_neb_energy<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * smem));
+    BPM_CK(cudaFuncSetAttribute(k_neb_energy<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * smem));
     BPM_CK(cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_stage1_groups<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_stage1_groups<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -949,8 +989,7 @@ int configure_step_kernels() {
 int few_threads(int n, int B, int sm_count) {
     // one pass over the nodes where the SMs hold that many threads for all islands (at most 1024 a CTA)
     const int per_sm = (B + sm_count - 1) / sm_count;
-    const int nt = n <= 256 || per_sm > 2 ? 256 : n <= 512 || per_sm > 1 ? 512 : 1024;
-    return nt;
+    return n <= 256 || per_sm > 2 ? 256 : n <= 512 || per_sm > 1 ? 512 : 1024;
 }
 
 namespace {
@@ -970,8 +1009,9 @@ int launch_few_nt(const StageGroups& G, int stage, int j, cudaStream_t s) {
 }  // namespace
 
 int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t s) {
-    return threads == 1024 ? launch_few_nt<1024>(G, stage, j, s)
-                           : threads == 512 ? launch_few_nt<512>(G, stage, j, s) : launch_few_nt<256>(G, stage, j, s);
+    return threads == 1024  ? launch_few_nt<1024>(G, stage, j, s)
+           : threads == 512 ? launch_few_nt<512>(G, stage, j, s)
+                            : launch_few_nt<256>(G, stage, j, s);
 }
 
 int stage_blocks_per_sm(int threads, int ipb, size_t smem, int* blocks) {
@@ -1054,11 +1094,29 @@ void launch_energy(const StepArgs& a, double t, double vol_scale, double* E, flo
 void launch_neb_init(const StepArgs& a, int P, int great_circle, cudaStream_t s) {
     k_neb_init<<<a.B, kStepThreads, 0, s>>>(a, P, great_circle);
 }
-void launch_neb_energy(const StepArgs& a, float* Bt, double* E, double vol_scale, cudaStream_t s) {
-    k_neb_energy<<<a.B, kStepThreads, stage_smem_bytes(a), s>>>(a, Bt, E, vol_scale);
+// threads of the band kernels, 0 where the rows are too many for the programmatic form (see few_islands)
+static int neb_few(const StepArgs& a, int sm_count) {
+    const int per_sm = (a.B + sm_count - 1) / sm_count;
+    const bool few = per_sm <= 4 && per_sm * a.n <= std::max(3200, a.n) &&
+                     per_sm * (2 * stage_smem_bytes(a) + 1024) <= 200 * 1024;
+    return few ? std::min(512, few_threads(a.n, a.B, sm_count)) : 0;
 }
-void launch_neb_step(const StepArgs& a, const NebArgs& nb, cudaStream_t s) {
-    k_neb_step<<<a.B, kStepThreads, 0, s>>>(a, nb);
+int launch_neb_energy(const StepArgs& a, float* Bt, double* E, double vol_scale, int sm_count, cudaStream_t s) {
+    const size_t sm = stage_smem_bytes(a);
+    switch (neb_few(a, sm_count)) {
+        case 512: BPM_CK(launch_pdl(k_neb_energy<512, true>, dim3(a.B), dim3(512), 2 * sm, s, true, a, Bt, E, vol_scale)); break;
+        case 256: BPM_CK(launch_pdl(k_neb_energy<256, true>, dim3(a.B), dim3(256), 2 * sm, s, true, a, Bt, E, vol_scale)); break;
+        default: k_neb_energy<256, false><<<a.B, 256, sm, s>>>(a, Bt, E, vol_scale); BPM_CK(cudaGetLastError());
+    }
+    return BPM_OK;
+}
+int launch_neb_step(const StepArgs& a, const NebArgs& nb, int sm_count, cudaStream_t s) {
+    const int nt = neb_few(a, sm_count);
+    if (nt == 512)
+        BPM_CK(launch_pdl(k_neb_step<512>, dim3(a.B), dim3(512), 0, s, true, a, nb));
+    else
+        BPM_CK(launch_pdl(k_neb_step<256>, dim3(a.B), dim3(256), 0, s, nt > 0, a, nb));
+    return BPM_OK;
 }
 
 }  // namespace bpm

@@ -89,8 +89,8 @@ struct NebArgs {
 // energy (J) and largest torque |m x B| (T) of each island at time t (a.mask selects the terms)
 void launch_energy(const StepArgs& a, double t, double vol_scale, double* E, float* torque, cudaStream_t s);
 void launch_neb_init(const StepArgs& a, int P, int great_circle, cudaStream_t s);
-void launch_neb_energy(const StepArgs& a, float* Bt, double* E, double vol_scale, cudaStream_t s);
-void launch_neb_step(const StepArgs& a, const NebArgs& nb, cudaStream_t s);
+int launch_neb_energy(const StepArgs& a, float* Bt, double* E, double vol_scale, int sm_count, cudaStream_t s);
+int launch_neb_step(const StepArgs& a, const NebArgs& nb, int sm_count, cudaStream_t s);
 int configure_step_kernels();
 
 }  // namespace bpm
