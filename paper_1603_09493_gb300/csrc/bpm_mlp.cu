@@ -17,7 +17,7 @@
 #include <cmath>
 #include <cstdio>
 
-#include "bpm_internal.cuh"
+#include "bpm_mlp_forward.cuh"
 
 namespace bpm {
 
@@ -49,6 +49,9 @@ struct Mlp {
     std::vector<cudaEvent_t> ev;          // ev[l]: dZ[l] written; ev[L]: the weight gradients are done
     int* err = nullptr;
     int max_pad = 0;
+    // inference in one kernel (networks up to 256 wide); layer by layer otherwise
+    bool one_kernel = false;
+    MlpForward fwd{};
 };
 
 namespace {
@@ -329,6 +332,9 @@ int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
     return BPM_OK;
 }
 
+// forward pass of rows [0, n) of the device array X into out [n][n_out]: logits, or probabilities
+int infer_rows(Mlp* m, bpm_ctx* ctx, const float* X, long long n, bool sigmoid, float* out);
+
 // Screened error rates (Sec. II.C), one chunk of rows [r0, r0 + nb) of the
 // design-major sample list: one warp per (design, output) that has samples in
 // the chunk adds its share to acc[d][k] in FP64, lanes strided over the
@@ -465,6 +471,18 @@ int bpm_surrogate_create(bpm_ctx* ctx, const bpm_mlp_cfg* cfg, const float* para
         }
     }
     if (r == BPM_OK) r = publish(m, s);
+    m->one_kernel = mlp_forward_fits(m->L, m->in_pad.data(), m->out_pad.data());
+    for (int l = 0; l < m->L && m->one_kernel && r == BPM_OK; ++l) {
+        MlpForward& f = m->fwd;
+        f.k_pad[l] = m->in_pad[l];
+        f.n_pad[l] = m->out_pad[l];
+        f.n_real[l] = m->out_real[l];
+        f.n_mma[l] = l + 1 < m->L ? m->out_pad[l] : rup(m->out_real[l], 16);
+        f.bias[l] = m->params + m->b_off[l];
+        f.L = m->L;
+        f.n_in = m->n_in;
+        r = make_bf16_tensor_map(&f.w[l], m->W[l], m->in_pad[l], m->out_pad[l], f.n_mma[l]);
+    }
     if (r != BPM_OK) {
         free_mlp(m);
         return r;
@@ -503,6 +521,36 @@ static int load_batch(bpm_ctx* ctx, Mlp* m, const float* Xd, const float* Yd, in
     }
     return BPM_OK;
 }
+
+}  // extern "C"
+
+namespace bpm {
+namespace {
+int infer_rows(Mlp* m, bpm_ctx* ctx, const float* X, long long n, bool sigmoid, float* out) {
+    cudaStream_t s = ctx->stream;
+    if (m->one_kernel) {
+        MlpForward f = m->fwd;
+        f.N = n;
+        f.X = X;
+        f.out = out;
+        f.sigmoid = sigmoid ? 1 : 0;
+        return mlp_forward_launch(s, f, ctx->sm_count, m->err);
+    }
+    const int chunk = 65536;   // 512 row tiles per layer GEMM: enough CTAs for every SM
+    for (long long s0 = 0; s0 < n; s0 += chunk) {
+        const int nb = (int)std::min<long long>(chunk, n - s0);
+        const int rows = rup(nb, 128);
+        BPM_TRY(load_batch(ctx, m, X + s0 * m->n_in, nullptr, nb, rows));
+        BPM_TRY(forward(m, s, rows, nb, true, sigmoid));
+        BPM_CK(cudaMemcpyAsync(out + s0 * m->n_out, m->logits, sizeof(float) * (size_t)nb * m->n_out,
+                               cudaMemcpyDeviceToDevice, s));
+    }
+    return BPM_OK;
+}
+}  // namespace
+}  // namespace bpm
+
+extern "C" {
 
 int bpm_surrogate_grad(bpm_ctx* ctx, int32_t sid, const float* X, const float* Y, int32_t N, float* grad,
                        float* loss) {
@@ -595,27 +643,20 @@ int bpm_surrogate_infer(bpm_ctx* ctx, int32_t sid, const float* X, int64_t N, fl
     }
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
-    const int chunk = 65536;   // 512 row tiles per layer GEMM: enough CTAs for every SM
     const float* Xd = X;
-    float* Xtmp = nullptr;
+    float *Xtmp = nullptr, *Pd = P;
     if (!on_device) {
-        BPM_CK(cudaMallocAsync(&Xtmp, sizeof(float) * (size_t)N * m->n_in, s));
+        BPM_CK(cudaMallocAsync(&Xtmp, sizeof(float) * (size_t)N * (m->n_in + m->n_out), s));
         BPM_CK(cudaMemcpyAsync(Xtmp, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
         Xd = Xtmp;
+        Pd = Xtmp + (size_t)N * m->n_in;
     }
-    int r = BPM_OK;
-    for (long long s0 = 0; s0 < N && r == BPM_OK; s0 += chunk) {
-        const int nb = (int)std::min<long long>(chunk, N - s0);
-        const int rows = rup(nb, 128);
-        r = load_batch(ctx, m, Xd + s0 * m->n_in, nullptr, nb, std::max(rows, std::min(rup(chunk, 128), rows)));
-        if (r == BPM_OK) r = forward(m, s, rows, nb, true, true);
-        if (r == BPM_OK) {
-            cudaError_t e = cudaMemcpyAsync(P + s0 * m->n_out, m->logits, sizeof(float) * (size_t)nb * m->n_out,
-                                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
-            if (e != cudaSuccess) {
-                set_error("inference copy: %s", cudaGetErrorString(e));
-                r = BPM_ERR_CUDA;
-            }
+    int r = infer_rows(m, ctx, Xd, N, true, Pd);
+    if (r == BPM_OK && !on_device) {
+        cudaError_t e = cudaMemcpyAsync(P, Pd, sizeof(float) * (size_t)N * m->n_out, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) {
+            set_error("inference copy: %s", cudaGetErrorString(e));
+            r = BPM_ERR_CUDA;
         }
     }
     if (Xtmp) cudaFreeAsync(Xtmp, s);
@@ -634,11 +675,13 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
     const long long N = (long long)n_designs * n_jitter;
-    const int chunk = 65536;
+    // logits of at most 2^20 samples at a time
+    const long long chunk = 1 << 20;
     const float* Xd = X;
-    float* Xtmp = nullptr;
+    float *Xtmp = nullptr, *z = nullptr;
     double* acc = nullptr;
     const size_t out_bytes = sizeof(double) * (size_t)n_designs * m->n_out;
+    BPM_CK(cudaMallocAsync(&z, sizeof(float) * (size_t)std::min(N, chunk) * m->n_out, s));
     if (!on_device) {
         BPM_CK(cudaMallocAsync(&Xtmp, sizeof(float) * (size_t)N * m->n_in, s));
         BPM_CK(cudaMemcpyAsync(Xtmp, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
@@ -650,16 +693,14 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
     BPM_CK(cudaMemsetAsync(acc, 0, out_bytes, s));
     int r = BPM_OK;
     for (long long s0 = 0; s0 < N && r == BPM_OK; s0 += chunk) {
-        const int nb = (int)std::min<long long>(chunk, N - s0);
-        const int rows = rup(nb, 128);
-        r = load_batch(ctx, m, Xd + s0 * m->n_in, nullptr, nb, std::max(rows, std::min(rup(chunk, 128), rows)));
-        if (r == BPM_OK) r = forward(m, s, rows, nb, true, false);
+        const int nb = (int)std::min(chunk, N - s0);
+        r = infer_rows(m, ctx, Xd + s0 * m->n_in, nb, false, z);
         if (r == BPM_OK) {
             const long long d_lo = s0 / n_jitter, d_hi = (s0 + nb - 1) / n_jitter;
             const int n_d = (int)(d_hi - d_lo + 1);
             const long long threads = 32LL * n_d * m->n_out;
-            k_screen_accum<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(m->logits, s0, nb, n_jitter, m->n_out,
-                                                                            d_lo, n_d, acc);
+            k_screen_accum<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(z, s0, nb, n_jitter, m->n_out, d_lo, n_d,
+                                                                            acc);
             if (cudaGetLastError() != cudaSuccess) {
                 set_error("screening kernel launch failed");
                 r = BPM_ERR_CUDA;
@@ -676,6 +717,7 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
             r = BPM_ERR_CUDA;
         }
     }
+    cudaFreeAsync(z, s);
     if (Xtmp) cudaFreeAsync(Xtmp, s);
     if (!on_device && acc) cudaFreeAsync(acc, s);
     if (r != BPM_OK) return r;

@@ -119,3 +119,25 @@ def test_fp32_product_tile_edges(ctx, B):
     bound = (176 * 2.0 ** -24 + 2.0 ** -22) * (np.abs(src) @ np.abs(W).T)      # + the sources' own FP32 rounding
     assert np.all(np.abs(got - src @ W.T) <= bound)
 
+
+@pytest.mark.parametrize("shape", [(16, 256, 4, 2), (3, 100, 1, 5), (70, 130, 2, 17), (200, 256, 6, 128)])
+def test_one_kernel_forward_matches_the_layers(ctx, shape):
+    """The forward pass in one kernel at its edges (one input k-block to four, padded and whole widths, depths 1 and 6,
+    one to eight output groups of 16; one sample, a full tile, two and more tiles of an SM) against the layer-by-layer
+    forward pass of the gradient call: the loss of both must agree.  Probabilities and logits go through FP32 once
+    more (a sigmoid and its inverse): 1e-5 of the loss."""
+    from paper_1603_09493_gb300 import synth
+    n_in, width, depth, n_out = shape
+    sizes = [n_in] + [width] * depth + [n_out]
+    sur = ctx.surrogate(shape, synth.mlp_init_params(sizes, seed=sum(shape)))
+    rng = np.random.default_rng(n_in)
+    X = rng.uniform(-1, 1, (152 * 128 * 3 + 77, n_in)).astype(np.float32)
+    P = sur.infer(X)
+    for N in (1, 127, 128, 129, 152 * 128 + 1):
+        assert np.array_equal(sur.infer(X[:N]), P[:N])
+    for lo, N in ((0, 1), (100, 300), (152 * 128 - 60, 500), (152 * 128 * 3 - 50, 127)):
+        x, y = X[lo:lo + N], (rng.random((N, n_out)) < 0.5).astype(np.float32)
+        p = P[lo:lo + N].astype(np.float64)
+        loss = -np.mean(y * np.log(p) + (1 - y) * np.log1p(-p))
+        assert abs(sur.grad(x, y)[1] - loss) <= 1e-5 * max(1.0, loss)
+    sur.destroy()
