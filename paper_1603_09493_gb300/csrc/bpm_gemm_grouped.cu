@@ -18,8 +18,12 @@
 // nodes: 374 -> 172 us an interval of 6 steps; nine of 481 nodes: 689 -> 330 us of
 // 8 steps; 60 of 1547 nodes: 5.2 -> 2.7 ms of 28 steps.
 //
-// The items of all groups form one list; each CTA (one per SM) walks it with a
-// stride of the grid size.  Within a group the tiles run M-major or N-major (chosen
+// The items of all groups are dealt to the CTAs (one per SM) when the GEMM is set
+// up: an item costs its K, so each goes, longest first, to the CTA with the least
+// so far (a walk of the list with the grid as stride left the longest items of
+// eight uneven variants to the last, two-thirds full round: 31.1 ms an interval,
+// 30.9 so, the product then being bound by reading 1.6 GB of operators).  Items of
+// equal cost keep the list's order, one after the other over the CTAs.  Within a group the tiles run M-major or N-major (chosen
 // per group), so that a wave of CTAs shares the larger operand's rows in L2 and it
 // is read from HBM once.  Warp roles:
 //   warp 0  one lane streams the k-blocks of every item with TMA into a ring of
@@ -36,6 +40,8 @@
 // memory or TMEM is given up.
 #include <algorithm>
 #include <cstring>
+#include <functional>
+#include <queue>
 
 #include "bpm_tc_ptx.cuh"
 
@@ -82,7 +88,8 @@ __device__ __forceinline__ void item_origin(const GemmGroupDev& gg, int it, int&
 
 template <int P, int TN, int KB>
 __global__ void __launch_bounds__(kGThreads, 1)
-    k_gemm_grouped(const GemmGroupDev* __restrict__ G, int ng, int total_tiles, int* err, unsigned long long wait_ns) {
+    k_gemm_grouped(const GemmGroupDev* __restrict__ G, int ng, const int* __restrict__ sched, int* err,
+                   unsigned long long wait_ns) {
     using CF = GCfg<P, TN, KB>;
     constexpr int S = CF::stages;
     constexpr int A_TILE = CF::A_BYTES;
@@ -114,6 +121,9 @@ __global__ void __launch_bounds__(kGThreads, 1)
     auto sAlo = [&](int s) { return base + s * CF::stage_bytes + 2 * W_TILE + A_TILE; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // this CTA's items: sched holds gridDim.x + 1 offsets into the list behind them
+    const int* items = sched + gridDim.x + 1;
+    const int q0 = sched[blockIdx.x], q1 = sched[blockIdx.x + 1];
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full_bar(s), 1);
@@ -141,7 +151,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
         // ---------------- TMA producer ----------------
         int kbg = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
+        for (int qi = q0; qi < q1 && ok; ++qi) {
+            const int t = items[qi];
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
@@ -158,7 +169,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 tma_load_2d(sAhi(s), &gg.ahi, kc, b0, full_bar(s));
                 if (P == 3) tma_load_2d(sAlo(s), &gg.alo, kc, b0, full_bar(s));
             };
-            if (t == blockIdx.x) {
+            if (qi == q0) {
                 // the first ring of operator tiles, which no kernel writes, ahead of the wait for the
                 // kernel that writes the islands' operand
                 const int pre = min(S, kb1 - kb);
@@ -183,7 +194,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
         // ---------------- MMA issuer ----------------
         int kbg = 0, i = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++i) {
+        for (int qi = q0; qi < q1 && ok; ++qi, ++i) {
+            const int t = items[qi];
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
@@ -221,7 +233,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const int q = warp & 3;    // TMEM lane quarter this warp may access
         pdl_wait();                // C may still be read by the kernel before
         int i = 0;
-        for (int t = blockIdx.x; t < total_tiles; t += gridDim.x, ++i) {
+        for (int qi = q0; qi < q1; ++qi, ++i) {
+            const int t = items[qi];
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
@@ -269,10 +282,9 @@ int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err
                                     GCfg<P, TN, KB>::smem));
         configured = true;
     }
-    const int grid = std::max(1, std::min(gg.total_tiles, sm_count));
-    BPM_CK(launch_pdl(k_gemm_grouped<P, TN, KB>, dim3(grid), dim3(kGThreads), GCfg<P, TN, KB>::smem, s, pdl,
-                      gg.d_groups, gg.n_groups, gg.total_tiles, err, gg.wait_ns ? gg.wait_ns : kWaitNs));
-    BPM_CK(cudaGetLastError());
+    (void)sm_count;                       // the grid is part of the schedule
+    BPM_CK(launch_pdl(k_gemm_grouped<P, TN, KB>, dim3(gg.grid), dim3(kGThreads), GCfg<P, TN, KB>::smem, s, pdl,
+                      gg.d_groups, gg.n_groups, gg.d_sched, err, gg.wait_ns ? gg.wait_ns : kWaitNs));
     return BPM_OK;
 }
 
@@ -330,6 +342,37 @@ int tile_cap(const std::vector<GemmOperands>& ops, int tile_n, int sm_count, int
         }
     }
     return best;
+}
+
+// Offsets [grid + 1] of each CTA's items, then the items: longest first (list order among equals), each
+// to the CTA with the least cost so far (the lowest index among equals); an item costs the MMAs of its
+// slice and a fixed part (see tile_cap)
+std::vector<int> deal_items(const std::vector<GemmGroupDev>& h, int items, int grid) {
+    struct Item {
+        double cost;
+        int it;
+    };
+    std::vector<Item> list;
+    list.reserve(items);
+    for (const GemmGroupDev& g : h)
+        for (int k = 0; k < g.tiles_m * g.tiles_n * g.splits; ++k) {
+            const int lo = (k % g.splits) * g.slice_k, hi = std::min(g.K, lo + g.slice_k);
+            list.push_back(Item{mma_cost(g.nb) * ((hi - lo) / 16.0 + 12.0), g.tile_begin + k});
+        }
+    std::stable_sort(list.begin(), list.end(), [](const Item& x, const Item& y) { return x.cost > y.cost; });
+    std::vector<std::vector<int>> of(grid);
+    std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<>> load;
+    for (int c = 0; c < grid; ++c) load.push({0.0, c});
+    for (const Item& x : list) {
+        const auto [l, c] = load.top();
+        load.pop();
+        of[c].push_back(x.it);
+        load.push({l + x.cost, c});
+    }
+    std::vector<int> out(1, 0);
+    for (const auto& v : of) out.push_back(out.back() + (int)v.size());
+    for (const auto& v : of) out.insert(out.end(), v.begin(), v.end());
+    return out;
 }
 
 }  // namespace
@@ -395,8 +438,16 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
         tiles += h[g].tiles_m * h[g].tiles_n * h[g].splits;
     }
     grouped_gemm_free(gg);
-    BPM_CK(cudaMalloc(&gg->d_groups, h.size() * sizeof(GemmGroupDev)));
-    BPM_CK(cudaMemcpy(gg->d_groups, h.data(), h.size() * sizeof(GemmGroupDev), cudaMemcpyHostToDevice));
+    const int grid = std::max(1, std::min(tiles, sm_count));
+    const std::vector<int> sched = pair ? std::vector<int>() : deal_items(h, tiles, grid);
+    const size_t gbytes = h.size() * sizeof(GemmGroupDev), sbytes = sched.size() * sizeof(int);
+    std::vector<char> host(gbytes + sbytes);
+    std::memcpy(host.data(), h.data(), gbytes);
+    if (sbytes) std::memcpy(host.data() + gbytes, sched.data(), sbytes);
+    BPM_CK(cudaMalloc(&gg->d_groups, host.size()));
+    BPM_CK(cudaMemcpy(gg->d_groups, host.data(), host.size(), cudaMemcpyHostToDevice));
+    gg->d_sched = reinterpret_cast<int*>(reinterpret_cast<char*>(gg->d_groups) + gbytes);
+    gg->grid = grid;
     gg->n_groups = (int)h.size();
     gg->total_tiles = tiles;
     gg->tile_n = nb_max <= 128 ? 128 : 256;
@@ -409,6 +460,7 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
 void grouped_gemm_free(GroupedGemm* gg) {
     if (gg->d_groups) cudaFree(gg->d_groups);
     gg->d_groups = nullptr;
+    gg->d_sched = nullptr;
     gg->n_groups = gg->total_tiles = 0;
 }
 

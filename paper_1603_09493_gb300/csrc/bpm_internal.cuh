@@ -235,6 +235,8 @@ struct GemmOperands {
 int gemm_splits(int islands, int K, int sm_count);
 struct GroupedGemm {
     GemmGroupDev* d_groups = nullptr;
+    int* d_sched = nullptr;           // the CTAs' items (in d_groups' allocation); grid: CTAs
+    int grid = 0;
     int n_groups = 0, total_tiles = 0, tile_n = 256, products = 3, k_block = 64;   // tile_n: the kernel's widest tile
     unsigned long long wait_ns = 0;   // limit of the non-drain waits (0: the default)
     int pair = 0;                     // 1: 256 x 256 tiles on CTA pairs (tcgen05 cta_group::2)
