@@ -676,38 +676,34 @@ __device__ __forceinline__ double block_sum_d(double v, double* red) {
     return s;
 }
 
-// sums over the CTA of N doubles per thread, in a fixed order; every thread gets them.  red: N * NT / 32
-// doubles.  (FP64 runs at two operations a cycle and SM: the warps' sums are added by one warp.)
+// Sums over the CTA of N doubles per thread, in a fixed order, to lane 0 of warp q for value q (part: N * NT
+// doubles of shared memory; the caller synchronises before it reads what those lanes store).  An SM does
+// two FP64 operations a cycle, and a shuffle tree costs every warp five: one warp a value adds them all.
 template <int NT, int N>
-__device__ __forceinline__ void block_sums_d(double (&v)[N], double* red) {
-    constexpr int NW = NT / 32;
+__device__ __forceinline__ double block_sums_d(const double (&v)[N], double* part) {
 #pragma unroll
-    for (int q = 0; q < N; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-        for (int q = 0; q < N; ++q) red[q * NW + (threadIdx.x >> 5)] = v[q];
+    for (int q = 0; q < N; ++q) part[q * NT + threadIdx.x] = v[q];
     __syncthreads();
-    if (threadIdx.x < N) {
-        double s = 0.0;
-        for (int w = 0; w < NW; ++w) s += red[threadIdx.x * NW + w];
-        red[threadIdx.x * NW] = s;
+    const int w = threadIdx.x >> 5;
+    double s = 0.0;
+    if (w < N) {
+        for (int k = threadIdx.x & 31; k < NT; k += 32) s += part[w * NT + k];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < N; ++q) v[q] = red[q * NW];
+    return s;
 }
 
 // total field Bt of every image and its energy
 //   E = -sum_i V_i Ms_i (B_quad,i / 2 + B_lin,i) . m_i   (J; vol_scale = sum V [nm^3] * 1e-21)
 // AHEAD (few images, see few_body): launched programmatically behind the GEMM, with the head field, which
 // does not change along the run, and the exchange entries taken before the wait.  45 images of 481
-// nodes, one band update (GEMM, this and k_neb_step): 40 us one after the other, 34 so.
+// nodes, one band update (GEMM, this and k_neb_step): 40 us one after the other, 34 so, 27 with
+// the FP64 scalars of the update on one warp.
 template <int NT, bool AHEAD>
 __global__ void __launch_bounds__(NT) k_neb_energy(StepArgs a, float* __restrict__ Bt, double* __restrict__ E,
                                                    double vol_scale) {
     extern __shared__ float4 smem4[];
-    __shared__ double red[NT / 32];
+    __shared__ double part[NT];
     float* sm = reinterpret_cast<float*>(smem4);
     const int b = blockIdx.x;
     const int np = a.n_pad;
@@ -735,8 +731,8 @@ __global__ void __launch_bounds__(NT) k_neb_energy(StepArgs a, float* __restrict
         const float w = __ldg(&a.node_pos[i].w);
         e[0] += (double)(w * msn) * (double)dot3(0.5f * Bq + Bl, mi);
     }
-    block_sums_d<NT, 1>(e, red);
-    if (threadIdx.x == 0) E[b] = -vol_scale * e[0];
+    const double tot = block_sums_d<NT, 1>(e, part);
+    if (threadIdx.x == 0) E[b] = -vol_scale * tot;
 }
 
 __device__ __forceinline__ float3 perp3(float3 v, float3 m) { return v + (-dot3(v, m)) * m; }
@@ -748,8 +744,9 @@ __device__ __forceinline__ float3 load_state(const float* m, size_t base, int np
 // one band update of every image (Jacobi: neighbours from m_in, result to m_out)
 template <int NT>
 __global__ void __launch_bounds__(NT) k_neb_step(StepArgs a, NebArgs nb) {
-    __shared__ double red[4 * NT / 32];
-    __shared__ int s_ci;
+    __shared__ double part[4 * NT], s_sum[4];
+    __shared__ float s_w[3];                     // tangent weights, then the tangent's factor
+    __shared__ int s_climbing;
     pdl_trigger();
     const int b = blockIdx.x, P = nb.P, d = b / P, k = b - d * P;
     const int np = a.n_pad;
@@ -757,39 +754,51 @@ __global__ void __launch_bounds__(NT) k_neb_step(StepArgs a, NebArgs nb) {
     const float msc = a.isl[3 * b].z;
     const bool end = (k == 0 || k == P - 1);
     pdl_wait();
-    // climbing image of this band: the interior image of highest energy
-    if (threadIdx.x == 0) {
+    // One warp takes the band's FP64 scalars.  Climbing image: the interior image of highest energy, the
+    // first of equals.  Improved tangent: weights of (m+ - m) and (m - m-) from the neighbours' energies.
+    if (threadIdx.x < 32 && !end) {
+        double top = -1e300;
         int ci = -1;
-        if (nb.climb) {
-            double emax = -1e300;
-            for (int q = 1; q < P - 1; ++q) {
+        if (nb.climb)
+            for (int q = 1 + threadIdx.x; q < P - 1; q += 32) {
                 const double eq = nb.E[d * P + q];
-                if (eq > emax) {
-                    emax = eq;
+                if (eq > top) {
+                    top = eq;
                     ci = q;
                 }
             }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double t2 = __shfl_xor_sync(0xffffffffu, top, o);
+            const int c2 = __shfl_xor_sync(0xffffffffu, ci, o);
+            if (c2 >= 0 && (ci < 0 || t2 > top || (t2 == top && c2 < ci))) {
+                top = t2;
+                ci = c2;
+            }
         }
-        s_ci = ci;
+        if (threadIdx.x == 0) {
+            s_climbing = k == ci;
+            float cp, cm;
+            const double Em = nb.E[b - 1], E0 = nb.E[b], Ep = nb.E[b + 1];
+            if (Ep > E0 && E0 > Em) {
+                cp = 1.f;
+                cm = 0.f;
+            } else if (Ep < E0 && E0 < Em) {
+                cp = 0.f;
+                cm = 1.f;
+            } else {
+                const double dmax = fmax(fabs(Ep - E0), fabs(Em - E0)), dmin = fmin(fabs(Ep - E0), fabs(Em - E0));
+                cp = (float)(Ep > Em ? dmax : dmin);
+                cm = (float)(Ep > Em ? dmin : dmax);
+            }
+            s_w[0] = cp;
+            s_w[1] = cm;
+        }
     }
     __syncthreads();
-    const bool climbing = (k == s_ci);
-    // improved tangent: weights of (m+ - m) and (m - m-) from the neighbours' energies
-    float cp = 1.f, cm = 0.f;
-    double inv_t = 0.0, s_ft = 0.0, spring_term = 0.0;
+    float cp = 0.f, cm = 0.f, c_t = 0.f;
     if (!end) {
-        const double Em = nb.E[b - 1], E0 = nb.E[b], Ep = nb.E[b + 1];
-        if (Ep > E0 && E0 > Em) {
-            cp = 1.f;
-            cm = 0.f;
-        } else if (Ep < E0 && E0 < Em) {
-            cp = 0.f;
-            cm = 1.f;
-        } else {
-            const double dmax = fmax(fabs(Ep - E0), fabs(Em - E0)), dmin = fmin(fabs(Ep - E0), fabs(Em - E0));
-            cp = (float)(Ep > Em ? dmax : dmin);
-            cm = (float)(Ep > Em ? dmin : dmax);
-        }
+        cp = s_w[0];
+        cm = s_w[1];
         // pass 1: |t|^2, <g, t>, |m+ - m|^2, |m - m-|^2
         double sum[4] = {0.0, 0.0, 0.0, 0.0};
         for (int i = threadIdx.x; i < a.n; i += NT) {
@@ -805,13 +814,19 @@ __global__ void __launch_bounds__(NT) k_neb_step(StepArgs a, NebArgs nb) {
             sum[2] += (double)(w * dot3(dplus, dplus));
             sum[3] += (double)(w * dot3(dminus, dminus));
         }
-        block_sums_d<NT, 4>(sum, red);
-        inv_t = sum[0] > 0.0 ? 1.0 / sqrt(sum[0]) : 0.0;
-        s_ft = sum[1] * inv_t;                               // <g, t_hat>
-        spring_term = (double)nb.spring * (sqrt(sum[2]) - sqrt(sum[3]));
+        const double tot = block_sums_d<NT, 4>(sum, part);
+        if (threadIdx.x < 128 && (threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = tot;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const double inv_t = s_sum[0] > 0.0 ? 1.0 / sqrt(s_sum[0]) : 0.0;
+            const double s_ft = s_sum[1] * inv_t;                               // <g, t_hat>
+            const double spring_term = (double)nb.spring * (sqrt(s_sum[2]) - sqrt(s_sum[3]));
+            s_w[2] = s_climbing ? (float)(-2.0 * s_ft * inv_t) : (float)((spring_term - s_ft) * inv_t);
+        }
+        __syncthreads();
+        c_t = s_w[2];
     }
     // pass 2: band force and the normalised step
-    const float c_t = climbing ? (float)(-2.0 * s_ft * inv_t) : (float)((spring_term - s_ft) * inv_t);
     float fmax_loc = 0.f;
     for (int i = threadIdx.x; i < a.n; i += NT) {
         const float3 m0 = load_state(nb.m_in, base, np, i);
