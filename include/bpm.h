@@ -118,7 +118,7 @@ typedef struct {
     int32_t n_tets, n_boundary;
     int32_t nnz;                 /* exchange CSR entries including the diagonal */
     int32_t cg_iters_neumann, cg_iters_dirichlet;
-    int32_t k_pad;               /* demag GEMM width: 3 n_pad rounded up to 64 */
+    int32_t k_pad;               /* demag GEMM width: 3 n_nodes rounded up to 64 */
     double  volume_nm3;
     double  exchange_lambda_max_T;  /* largest eigenvalue of S (nominal Ms), power iteration */
     double  field_bound_T;          /* lambda_max + max anisotropy field + mu0*max Ms */

@@ -550,8 +550,8 @@ size_t carve(bpm_batch* bt, Arena& A) {
     A.take(&bt->interval, 1);
     for (auto& g : bt->groups) {
         const size_t S = (size_t)g.Bp * g.mesh->K();
-        A.take(&g.m, S);
-        A.take(&g.k1, S);
+        A.take(&g.m, (size_t)g.Bp * 3 * g.mesh->n_pad);
+        A.take(&g.k1, (size_t)g.Bp * 3 * g.mesh->n_pad);
         A.take(&g.Hd, g.splits * S);
         if (bt->p.precision == BPM_PREC_FP32) {
             A.take(&g.A32, S);
@@ -731,7 +731,13 @@ int bpm_mesh_upload(bpm_ctx* ctx, const double* xyz_nm, int32_t n_nodes, const i
     Mesh* M = new Mesh();
     M->n = n_nodes;
     M->n_pad = round_up(n_nodes, kNodePad);
-    M->k_pad = round_up(3 * M->n_pad, kKPad);
+    // The operand's planes lie as close as whole 32-byte sectors of their first nodes allow without a
+    // wider K: planes of n_pad nodes made K 4736 instead of 4672 on the census mesh, 704 instead of 640
+    // on the 209-node one.
+    M->k_pad = round_up(3 * n_nodes, kKPad);
+    M->pitch = n_nodes;
+    for (int u : {4, 8})
+        if (3 * round_up(n_nodes, u) <= M->k_pad) M->pitch = round_up(n_nodes, u);
     M->n_tets = n_tets;
     int r = assemble_mesh(ctx, M, xyz_nm, tets, n_tets, tet_region, mats, n_regions, flags);
     if (r != BPM_OK) {
@@ -754,7 +760,7 @@ int bpm_mesh_get_operator(bpm_ctx* ctx, int32_t mesh_id, int32_t which, void* ds
     Mesh* M = get_mesh(ctx, mesh_id);
     if (!M || !dst) return BPM_ERR_ARG;
     BPM_TRY(ensure_device(ctx));
-    const int n = M->n, np = M->n_pad;
+    const int n = M->n;
     switch (which) {
         case BPM_OP_EXCHANGE_F32: {
             float* S = static_cast<float*>(dst);
@@ -779,11 +785,11 @@ int bpm_mesh_get_operator(bpm_ctx* ctx, int32_t mesh_id, int32_t which, void* ds
             return BPM_OK;
         case BPM_OP_DEMAG_F32: {
             float* D = static_cast<float*>(dst);
-            const int K = M->K();
+            const int K = M->K(), pc = M->pitch;
             for (int c = 0; c < 3; ++c)
                 for (int c2 = 0; c2 < 3; ++c2)
                     BPM_CK(cudaMemcpy2D(D + (size_t)c * n * 3 * n + (size_t)c2 * n, 3 * n * sizeof(float),
-                                        M->N32 + (size_t)c * np * K + (size_t)c2 * np, K * sizeof(float),
+                                        M->N32 + (size_t)c * pc * K + (size_t)c2 * pc, K * sizeof(float),
                                         n * sizeof(float), n, cudaMemcpyDeviceToHost));
             return BPM_OK;
         }
@@ -995,6 +1001,7 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
         a.n = M->n;
         a.n_pad = M->n_pad;
         a.kp = M->k_pad;
+        a.cp = M->pitch;
         a.node_pos = M->node_pos;
         a.node_mat = M->node_mat;
         a.sell_off = M->sell_off;

@@ -57,8 +57,8 @@ struct NodeF64 {
 struct Mesh {
     int n = 0, n_pad = 0, n_tets = 0, nb = 0, nnz = 0;
     // demag GEMM width: the operand row of an island holds its three component planes
-    // [c n_pad, c n_pad + n) and zeros up to k_pad = 3 n_pad rounded up to kKPad
-    int k_pad = 0;
+    // [c pitch, c pitch + n) and zeros elsewhere up to k_pad = 3 n rounded up to kKPad
+    int k_pad = 0, pitch = 0;
     // per node (padded to n_pad; padding nodes have w = 0 and no neighbours)
     float4* node_pos = nullptr;   // x, y, z (nm), w_i = V_i / sum V
     float4* node_mat = nullptr;   // 2 Ku_i / Ms_i (T), Ms_i (MA/m), 0, 0
@@ -70,8 +70,8 @@ struct Mesh {
     // the same entries with col replaced by the byte offset of node col's x component in the
     // interleaved shared state of the two-island stage kernels (see kIlIslands)
     int2* sell_il = nullptr;
-    // demag operator -mu0*1e6*N, row c*n_pad+i, column c'*n_pad+k (T per MA/m); rows and
-    // columns from 3 n_pad to k_pad are zero
+    // demag operator -mu0*1e6*N, row c*pitch+i, column c'*pitch+k (T per MA/m); the other rows and
+    // columns are zero
     float* N32 = nullptr;         // [K][K], K = k_pad
     __nv_bfloat16* Nhi = nullptr; // [K][K]
     __nv_bfloat16* Nlo = nullptr; // [K][K]
@@ -91,6 +91,8 @@ struct Mesh {
     double ms_max = 0;            // max_i Ms_i (A/m)
     bpm_mesh_info info{};
     int K() const { return k_pad; }
+    // floats of a buffer row that holds a state [3][n_pad] or a GEMM row [k_pad]
+    int row_floats() const { return (3 * n_pad + kKPad - 1) / kKPad * kKPad; }
 };
 
 struct HeadMap {

@@ -117,6 +117,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     a.n = n;
     a.n_pad = np;
     a.kp = K;
+    a.cp = M->pitch;
     a.node_pos = M->node_pos;
     a.node_mat = M->node_mat;
     a.sell_off = M->sell_off;

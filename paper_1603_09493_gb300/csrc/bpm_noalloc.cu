@@ -98,7 +98,7 @@ extern "C" int bpm_llg_advance_noalloc(bpm_ctx* ctx, const bpm_island* isl, int3
         return BPM_ERR_ARG;
     }
     // scratch layout
-    const size_t state = (size_t)B * K * sizeof(float);
+    const size_t state = (size_t)B * M->row_floats() * sizeof(float);
     size_t off = 0;
     const size_t o_isl = off;
     off = align256(off + 3 * (size_t)B * sizeof(float4));
@@ -153,6 +153,7 @@ extern "C" int bpm_llg_advance_noalloc(bpm_ctx* ctx, const bpm_island* isl, int3
     a.n = n;
     a.n_pad = np;
     a.kp = K;
+    a.cp = M->pitch;
     a.node_pos = M->node_pos;
     a.node_mat = M->node_mat;
     a.sell_off = M->sell_off;

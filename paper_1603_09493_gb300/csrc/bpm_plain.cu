@@ -277,7 +277,7 @@ extern "C" int bpm_run_plain(bpm_ctx* ctx, const bpm_island* isl, int32_t B, con
     cudaStream_t s = ctx->stream;
     // one region per buffer, each large enough for a state [3][n_pad] and a GEMM row [k_pad]
     int kmax = 0;
-    for (int b = 0; b < B; ++b) kmax = std::max(kmax, ctx->meshes[isl[b].mesh_id]->K());
+    for (int b = 0; b < B; ++b) kmax = std::max(kmax, ctx->meshes[isl[b].mesh_id]->row_floats());
     const size_t S = (size_t)kmax;
     float *buf = nullptr, *scal = nullptr;
     int *iscal = nullptr;
@@ -308,6 +308,7 @@ extern "C" int bpm_run_plain(bpm_ctx* ctx, const bpm_island* isl, int32_t B, con
         a.n = n;
         a.n_pad = np;
         a.kp = K;
+        a.cp = M->pitch;
         a.node_pos = M->node_pos;
         a.node_mat = M->node_mat;
         a.sell_off = M->sell_off;

@@ -93,14 +93,14 @@ __device__ __forceinline__ float3 trilinear(const StepArgs& a, float px, float p
 // demag field of island b at node i: the planes of the product's K slices, added in order
 __device__ __forceinline__ float3 load_hd(const StepArgs& a, int b, int i) {
     const float* hd = a.Hd + (size_t)b * a.kp + i;
-    float3 v = f3(__ldcg(hd), __ldcg(hd + a.n_pad), __ldcg(hd + 2 * a.n_pad));
+    float3 v = f3(__ldcg(hd), __ldcg(hd + a.cp), __ldcg(hd + 2 * a.cp));
     if (a.hd_planes > 1) {
         // at most four planes: all loads at once (a missing plane repeats the last and is dropped)
         float3 w[3];
 #pragma unroll
         for (int s = 1; s < 4; ++s) {
             const float* p = hd + (size_t)min(s, a.hd_planes - 1) * a.hd_plane;
-            w[s - 1] = f3(__ldcg(p), __ldcg(p + a.n_pad), __ldcg(p + 2 * a.n_pad));
+            w[s - 1] = f3(__ldcg(p), __ldcg(p + a.cp), __ldcg(p + 2 * a.cp));
         }
 #pragma unroll
         for (int s = 1; s < 4; ++s)
@@ -164,7 +164,7 @@ __device__ __forceinline__ void write_gemm_input(const StepArgs& a, int b, int i
     float x[3] = {msi * v.x, msi * v.y, msi * v.z};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        size_t oc = o + (size_t)c * a.n_pad;
+        size_t oc = o + (size_t)c * a.cp;
         if (a.prec == BPM_PREC_FP32) {
             a.A32[oc] = x[c];
         } else {

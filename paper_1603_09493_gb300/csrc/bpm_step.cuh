@@ -6,7 +6,7 @@ namespace bpm {
 
 struct StepArgs {
     int B, n, n_pad;
-    int kp;                   // row stride of Hd and the GEMM operand (k_pad >= 3 n_pad)
+    int kp, cp;               // row stride of Hd and the GEMM operand, distance of their component planes
     const float4* node_pos;   // [n_pad] x, y, z, w
     const float4* node_mat;   // [n_pad] 2Ku/Ms (T), Ms (MA/m)
     const int* sell_off;
@@ -22,7 +22,7 @@ struct StepArgs {
     const float* Hd;          // demag field of the GEMM input state, tesla, [Bp][kp]: the sum of
     int hd_planes;            // hd_planes planes hd_plane elements apart (slices of the product's K)
     size_t hd_plane;
-    float* A32;               // GEMM input (FP32), [Bp][kp], Ms * m in MA/m (planes at c n_pad)
+    float* A32;               // GEMM input (FP32), [Bp][kp], Ms * m in MA/m (planes at c cp)
     __nv_bfloat16* Ahi;       // GEMM input BF16 hi/lo split
     __nv_bfloat16* Alo;
     int prec;
