@@ -1130,8 +1130,10 @@ int bpm_batch_set_state(bpm_batch* bt, const float* m, int32_t ld, double t0_ps,
         return BPM_ERR_ARG;
     }
     float* src = const_cast<float*>(m);
+    CallBuffers buf(bt->ctx);
     if (m && !on_device) {
-        BPM_CK(cudaMallocAsync(&src, sizeof(float) * 3 * (size_t)bt->B * ld, s));
+        buf.take(&src, 3 * (size_t)bt->B * ld);
+        BPM_TRY(buf.reserve());
         BPM_CK(cudaMemcpyAsync(src, m, sizeof(float) * 3 * (size_t)bt->B * ld, cudaMemcpyHostToDevice, s));
     }
     for (auto& g : bt->groups) {
@@ -1141,7 +1143,6 @@ int bpm_batch_set_state(bpm_batch* bt, const float* m, int32_t ld, double t0_ps,
         else
             k_fill_plus_z<<<dim3((n + 255) / 256, g.B), 256, 0, s>>>(n, np, g.m);
     }
-    if (m && !on_device) cudaFreeAsync(src, s);
     BPM_CK(cudaMemsetAsync(bt->interval, 0, sizeof(long long), s));
     bt->t0 = t0_ps;
     bt->intervals_done = 0;
@@ -1207,15 +1208,15 @@ int bpm_batch_read(bpm_batch* bt, float* m, int32_t ld, uint8_t* switched, float
     float *dm = on_device ? m : nullptr, *dtsw = on_device ? t_sw_ps : nullptr, *dmz = on_device ? mz : nullptr;
     uint8_t* dsw = on_device ? switched : nullptr;
     int* dst = on_device ? status : nullptr;
+    CallBuffers buf(bt->ctx);
     if (!on_device) {
-        if (m) {
-            BPM_CK(cudaMallocAsync(&dm, sizeof(float) * 3 * (size_t)B * ld, s));
-            BPM_CK(cudaMemsetAsync(dm, 0, sizeof(float) * 3 * (size_t)B * ld, s));
-        }
-        BPM_CK(cudaMallocAsync(&dtsw, sizeof(float) * B, s));
-        BPM_CK(cudaMallocAsync(&dmz, sizeof(float) * B, s));
-        BPM_CK(cudaMallocAsync(&dsw, B, s));
-        BPM_CK(cudaMallocAsync(&dst, sizeof(int) * B, s));
+        buf.take(&dtsw, B);
+        buf.take(&dmz, B);
+        buf.take(&dsw, B);
+        buf.take(&dst, B);
+        if (m) buf.take(&dm, 3 * (size_t)B * ld);
+        BPM_TRY(buf.reserve());
+        if (m) BPM_CK(cudaMemsetAsync(dm, 0, sizeof(float) * 3 * (size_t)B * ld, s));
     }
     for (auto& g : bt->groups) {
         const int n = g.mesh->n, np = g.mesh->n_pad;
@@ -1235,11 +1236,6 @@ int bpm_batch_read(bpm_batch* bt, float* m, int32_t ld, uint8_t* switched, float
     BPM_CK(cudaMemcpyAsync(mzv.data(), dmz, sizeof(float) * B, cudaMemcpyDeviceToHost, s));
     BPM_CK(cudaMemcpyAsync(swv.data(), dsw, B, cudaMemcpyDeviceToHost, s));
     BPM_CK(cudaMemcpyAsync(stv.data(), dst, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
-    if (dm) cudaFreeAsync(dm, s);
-    cudaFreeAsync(dtsw, s);
-    cudaFreeAsync(dmz, s);
-    cudaFreeAsync(dsw, s);
-    cudaFreeAsync(dst, s);
     BPM_CK(cudaStreamSynchronize(s));
     if (gerr) {
         set_error("a bounded wait in the tensor-core demag GEMM gave up (code %d); results are invalid", gerr);

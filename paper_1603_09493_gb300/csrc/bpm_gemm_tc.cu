@@ -49,6 +49,11 @@ __device__ __forceinline__ float gelu_grad(float x) {
     return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // Epilogue of one thread: row `row`, 32 accumulator columns starting at `col`.
 template <int EPI>
 __device__ __forceinline__ void epilogue32(const TcEpilogue& e, int M, int N, int row, int col, const uint32_t (&r)[32],
@@ -70,28 +75,29 @@ __device__ __forceinline__ void epilogue32(const TcEpilogue& e, int M, int N, in
         }
     } else if (EPI == TC_EPI_BIAS_GELU) {
         // z = acc + b; keep z (for the backward pass, optional) and h = GELU(z) row-major and,
-        // optionally, transposed.  N is a multiple of 32 and the rows of H are 16-byte aligned,
-        // so the 32 columns of h go out as four 16-byte stores.
+        // optionally, transposed.  N is a multiple of 32 and the rows of z and H are 16-byte aligned, so
+        // a thread's 32 columns of z and h go out in 16-byte stores (a lane's row is a line of its own:
+        // scalar ones cost a sector each).
         if (col >= N || row >= M) return;
-        uint32_t hp[16];
 #pragma unroll
-        for (int q = 0; q < 32; q += 2) {
-            float h2[2];
+        for (int q = 0; q < 32; q += 8) {
+            float z[8], h[8];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            for (int u = 0; u < 8; ++u) {
                 const int c = col + q + u;
-                const float z = __uint_as_float(r[q + u]) + (c < e.cols_valid ? e.bias[c] : 0.f);
+                z[u] = __uint_as_float(r[q + u]) + (c < e.cols_valid ? e.bias[c] : 0.f);
                 // rows past the valid batch are written as zeros so that no stale value travels on
-                h2[u] = (rok && c < e.cols_valid) ? gelu(z) : 0.f;
-                if (e.C && rok) e.C[(size_t)row * e.ldc + c] = z;
-                if (e.HT) e.HT[(size_t)c * e.ldht + row] = __float2bfloat16_rn(h2[u]);
+                h[u] = (rok && c < e.cols_valid) ? gelu(z[u]) : 0.f;
+                if (e.HT) e.HT[(size_t)c * e.ldht + row] = __float2bfloat16_rn(h[u]);
             }
-            const __nv_bfloat162 pk = __floats2bfloat162_rn(h2[0], h2[1]);
-            hp[q / 2] = *reinterpret_cast<const uint32_t*>(&pk);
+            if (e.C && rok) {
+                float4* zd = reinterpret_cast<float4*>(e.C + (size_t)row * e.ldc + col + q);
+                zd[0] = make_float4(z[0], z[1], z[2], z[3]);
+                zd[1] = make_float4(z[4], z[5], z[6], z[7]);
+            }
+            *reinterpret_cast<uint4*>(e.H + (size_t)row * e.ldh + col + q) =
+                make_uint4(pack2(h[0], h[1]), pack2(h[2], h[3]), pack2(h[4], h[5]), pack2(h[6], h[7]));
         }
-        uint4* dst = reinterpret_cast<uint4*>(e.H + (size_t)row * e.ldh + col);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) dst[v] = make_uint4(hp[4 * v], hp[4 * v + 1], hp[4 * v + 2], hp[4 * v + 3]);
     } else if (EPI == TC_EPI_BIAS_OUT) {
 #pragma unroll
         for (int q = 0; q < 32; ++q) {
@@ -101,19 +107,45 @@ __device__ __forceinline__ void epilogue32(const TcEpilogue& e, int M, int N, in
             e.C[(size_t)row * e.ldc + c] = e.sigmoid ? 1.f / (1.f + expf(-z)) : z;
         }
     } else if (EPI == TC_EPI_GELU_BWD) {
-        // dz = dh * GELU'(z) in both layouts, plus per-column sums for the bias gradient
+        // dz = dh * GELU'(z) in both layouts (16-byte loads and stores along the row), plus per-column
+        // sums for the bias gradient
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            const int c = col + q;
-            float dz = 0.f;
-            if (rok && c < e.cols_valid) dz = __uint_as_float(r[q]) * gelu_grad(e.Zin[(size_t)row * e.ldz + c]);
-            colsum[q] = dz;
-            if (c < N) {
-                if (row < M) e.H[(size_t)row * e.ldh + c] = __float2bfloat16_rn(dz);
-                if (e.HT && row < M) e.HT[(size_t)c * e.ldht + row] = __float2bfloat16_rn(dz);
+        for (int q = 0; q < 32; q += 8) {
+            float z[8], dz[8];
+            if (rok && col + q < N) {
+                const float4* zs = reinterpret_cast<const float4*>(e.Zin + (size_t)row * e.ldz + col + q);
+                const float4 lo = zs[0], hi = zs[1];
+                z[0] = lo.x; z[1] = lo.y; z[2] = lo.z; z[3] = lo.w;
+                z[4] = hi.x; z[5] = hi.y; z[6] = hi.z; z[7] = hi.w;
             }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int c = col + q + u;
+                dz[u] = 0.f;
+                if (rok && c < e.cols_valid) dz[u] = __uint_as_float(r[q + u]) * gelu_grad(z[u]);
+                colsum[q + u] = dz[u];
+                if (c < N && e.HT && row < M) e.HT[(size_t)c * e.ldht + row] = __float2bfloat16_rn(dz[u]);
+            }
+            if (col + q < N && row < M)
+                *reinterpret_cast<uint4*>(e.H + (size_t)row * e.ldh + col + q) =
+                    make_uint4(pack2(dz[0], dz[1]), pack2(dz[2], dz[3]), pack2(dz[4], dz[5]), pack2(dz[6], dz[7]));
         }
     }
+}
+
+// sums over the warp's lanes of 32 values per lane, value q to lane q: the exchange halves the values
+// held at every step (31 shuffles; a tree per value is 160), and adds the same pairs as those trees
+__device__ __forceinline__ float warp_colsums(float (&v)[32], int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < o; ++q) {
+            const float mine = up ? v[q + o] : v[q], other = up ? v[q] : v[q + o];
+            v[q] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+    }
+    return v[0];
 }
 
 template <int P, int EPI, int TN>
@@ -231,13 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             epilogue32<EPI>(e, M, N, row, col, r, colsum);
             if (EPI == TC_EPI_GELU_BWD && e.colsum && col < N) {
                 // fixed-order warp sums -> one partial per (row block of 32, column)
-#pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    float v = colsum[q];
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane == q && col + q < N)
-                        e.colsum[(size_t)(blockIdx.y * 4 + quarter) * e.ldcs + col + q] = v;
-                }
+                const float v = warp_colsums(colsum, lane);
+                if (col + lane < N) e.colsum[(size_t)(blockIdx.y * 4 + quarter) * e.ldcs + col + lane] = v;
             }
         }
     }

@@ -107,7 +107,7 @@ int ensure_ws(Mlp* m, int rows, bool train, cudaStream_t s) {
     }
     if (train) {
         P.take(&m->Y, (size_t)rows * m->n_out);
-        P.take(&m->colsum, (size_t)(rows / 32) * m->max_pad);
+        P.take(&m->colsum, (size_t)m->L * (rows / 32) * m->max_pad);   // one part per layer
     }
     BPM_TRY(P.reserve(&m->ws, s));
     m->ws_rows = rows;
@@ -151,11 +151,24 @@ __global__ void k_load_xt(int nb, int rows, int n_in, int in_pad, const float* _
     H0T[q] = __float2bfloat16_rn(v);
 }
 
-// loss head (one CTA): mean sigmoid-BCE over nb x n_out, dz = (sigmoid(z) - y) / (nb n_out)
-// into dZ [rows][out_pad] and dZ^T [out_pad][rows], bias gradient and loss in fixed order
-__global__ void k_loss_head(int nb, int n_out, int out_pad, int rows, const float* __restrict__ logits,
+// dz = (sigmoid(z) - y) / (nb n_out) into dZ [rows][out_pad] and dZ^T [out_pad][rows]
+__device__ __forceinline__ float loss_grad(float z, float y, float inv) { return (1.f / (1.f + expf(-z)) - y) * inv; }
+
+__global__ void k_loss_grad(int nb, int n_out, int out_pad, int rows, const float* __restrict__ logits,
                             const float* __restrict__ Y, __nv_bfloat16* __restrict__ dZ,
-                            __nv_bfloat16* __restrict__ dZT, float* __restrict__ db, float* __restrict__ loss_out) {
+                            __nv_bfloat16* __restrict__ dZT) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nb * n_out) return;
+    const int r = k / n_out, o = k % n_out;
+    const __nv_bfloat16 b = __float2bfloat16_rn(loss_grad(logits[k], Y[k], 1.f / ((float)nb * (float)n_out)));
+    dZ[(size_t)r * out_pad + o] = b;
+    dZT[(size_t)o * rows + r] = b;
+}
+
+// mean sigmoid-BCE over nb x n_out and the output biases' gradient (one CTA, fixed order); beside the
+// chain of input gradients, which waits for neither (15 us of every step when one kernel did it all)
+__global__ void k_loss_sums(int nb, int n_out, const float* __restrict__ logits, const float* __restrict__ Y,
+                            float* __restrict__ db, float* __restrict__ loss_out) {
     __shared__ float red[32];
     const float inv = 1.f / ((float)nb * (float)n_out);
     float lsum = 0.f;
@@ -163,10 +176,6 @@ __global__ void k_loss_head(int nb, int n_out, int out_pad, int rows, const floa
         for (int o = 0; o < n_out; ++o) {
             float z = logits[(size_t)r * n_out + o], y = Y[(size_t)r * n_out + o];
             lsum += fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))) - y * z;
-            float g = (1.f / (1.f + expf(-z)) - y) * inv;
-            __nv_bfloat16 b = __float2bfloat16_rn(g);
-            dZ[(size_t)r * out_pad + o] = b;
-            dZT[(size_t)o * rows + r] = b;
         }
     auto bsum = [&](float v) {
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -181,10 +190,8 @@ __global__ void k_loss_head(int nb, int n_out, int out_pad, int rows, const floa
     if (threadIdx.x == 0 && loss_out) *loss_out = L * inv;
     for (int o = 0; o < n_out; ++o) {
         float g = 0.f;
-        for (int r = threadIdx.x; r < nb; r += blockDim.x) {
-            float z = logits[(size_t)r * n_out + o], y = Y[(size_t)r * n_out + o];
-            g += (1.f / (1.f + expf(-z)) - y) * inv;
-        }
+        for (int r = threadIdx.x; r < nb; r += blockDim.x)
+            g += loss_grad(logits[(size_t)r * n_out + o], Y[(size_t)r * n_out + o], inv);
         float s = bsum(g);
         if (threadIdx.x == 0) db[o] = s;
     }
@@ -296,13 +303,23 @@ int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
     // (the pads of dZ[Lm] are zero from the allocation on; a shorter batch lays its transpose out anew)
     BPM_CK(cudaMemsetAsync(m->dZ[Lm], 0, sizeof(__nv_bfloat16) * (size_t)rows * m->out_pad[Lm], s));
     BPM_CK(cudaMemsetAsync(m->dZT[Lm], 0, sizeof(__nv_bfloat16) * (size_t)rows * m->out_pad[Lm], s));
-    k_loss_head<<<1, 1024, 0, s>>>(nb, m->n_out, m->out_pad[Lm], rows, m->logits, m->Y, m->dZ[Lm], m->dZT[Lm],
-                                   m->grad + m->b_off[Lm], loss_slot);
+    const int cells = nb * m->n_out;
+    k_loss_grad<<<(cells + 255) / 256, 256, 0, s>>>(nb, m->n_out, m->out_pad[Lm], rows, m->logits, m->Y, m->dZ[Lm],
+                                                    m->dZT[Lm]);
     BPM_CK(cudaGetLastError());
     for (int l = Lm; l >= 0; --l) {
-        // dW_l = dZ_l^T H_l on the side stream: nothing before the optimiser reads it
+        // dW_l = dZ_l^T H_l, the bias gradient and the loss on the side stream: nothing before the optimiser
+        // reads them
         BPM_CK(cudaEventRecord(m->ev[l], s));
         BPM_CK(cudaStreamWaitEvent(m->side, m->ev[l], 0));
+        if (l == Lm) {
+            k_loss_sums<<<1, 1024, 0, m->side>>>(nb, m->n_out, m->logits, m->Y, m->grad + m->b_off[Lm], loss_slot);
+        } else {
+            k_colsum_reduce<<<(m->out_real[l] + 127) / 128, 128, 0, m->side>>>(
+                rows / 32, m->out_real[l], m->in_pad[l + 1], m->colsum + (size_t)(l + 1) * (rows / 32) * m->max_pad,
+                m->grad + m->b_off[l]);
+        }
+        BPM_CK(cudaGetLastError());
         TcEpilogue g{};
         g.C = m->grad + m->w_off[l];
         g.ldc = m->in_real[l];
@@ -318,14 +335,11 @@ int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
         e.ldh = m->out_pad[l - 1];
         e.HT = m->dZT[l - 1];
         e.ldht = rows;
-        e.colsum = m->colsum;
+        e.colsum = m->colsum + (size_t)l * (rows / 32) * m->max_pad;
         e.ldcs = m->in_pad[l];
         e.rows_valid = nb;
         e.cols_valid = m->out_real[l - 1];
         BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], m->dZ[l], m->WT[l], e, m->err));
-        k_colsum_reduce<<<(m->out_real[l - 1] + 127) / 128, 128, 0, s>>>(rows / 32, m->out_real[l - 1], m->in_pad[l],
-                                                                         m->colsum, m->grad + m->b_off[l - 1]);
-        BPM_CK(cudaGetLastError());
     }
     BPM_CK(cudaEventRecord(m->ev[m->L], m->side));
     BPM_CK(cudaStreamWaitEvent(s, m->ev[m->L], 0));
@@ -561,17 +575,17 @@ int bpm_surrogate_grad(bpm_ctx* ctx, int32_t sid, const float* X, const float* Y
     }
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
+    CallBuffers buf(ctx);
     float *Xd = nullptr, *Yd = nullptr;
-    BPM_CK(cudaMallocAsync(&Xd, sizeof(float) * (size_t)N * m->n_in, s));
-    BPM_CK(cudaMallocAsync(&Yd, sizeof(float) * (size_t)N * m->n_out, s));
+    buf.take(&Xd, (size_t)N * m->n_in);
+    buf.take(&Yd, (size_t)N * m->n_out);
+    BPM_TRY(buf.reserve());
     BPM_CK(cudaMemcpyAsync(Xd, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
     BPM_CK(cudaMemcpyAsync(Yd, Y, sizeof(float) * (size_t)N * m->n_out, cudaMemcpyHostToDevice, s));
     const int rows = rup(N, 128);
     int r = load_batch(ctx, m, Xd, Yd, N, rows);
     if (r == BPM_OK) r = forward(m, s, rows, N, false, false);
     if (r == BPM_OK) r = backward(m, s, rows, N, m->loss);
-    cudaFreeAsync(Xd, s);
-    cudaFreeAsync(Yd, s);
     if (r != BPM_OK) return r;
     BPM_TRY(check_err(m, s));
     BPM_CK(cudaMemcpy(grad, m->grad, m->P * sizeof(float), cudaMemcpyDeviceToHost));
@@ -590,10 +604,12 @@ int bpm_surrogate_train(bpm_ctx* ctx, int32_t sid, const float* X, const float* 
     cudaStream_t s = ctx->stream;
     const long long steps_per_epoch = (N + cfg->batch - 1) / cfg->batch;
     const long long steps = steps_per_epoch * cfg->epochs;
+    CallBuffers buf(ctx);
     float *Xd = nullptr, *Yd = nullptr, *curve = nullptr;
-    BPM_CK(cudaMallocAsync(&Xd, sizeof(float) * (size_t)N * m->n_in, s));
-    BPM_CK(cudaMallocAsync(&Yd, sizeof(float) * (size_t)N * m->n_out, s));
-    BPM_CK(cudaMallocAsync(&curve, sizeof(float) * (size_t)steps, s));
+    buf.take(&Xd, (size_t)N * m->n_in);
+    buf.take(&Yd, (size_t)N * m->n_out);
+    buf.take(&curve, (size_t)steps);
+    BPM_TRY(buf.reserve());
     BPM_CK(cudaMemcpyAsync(Xd, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
     BPM_CK(cudaMemcpyAsync(Yd, Y, sizeof(float) * (size_t)N * m->n_out, cudaMemcpyHostToDevice, s));
     int r = ensure_ws(m, rup(cfg->batch, 128), true, s);
@@ -629,9 +645,6 @@ int bpm_surrogate_train(bpm_ctx* ctx, int32_t sid, const float* X, const float* 
         }
     }
     cudaStreamSynchronize(s);
-    cudaFreeAsync(Xd, s);
-    cudaFreeAsync(Yd, s);
-    cudaFreeAsync(curve, s);
     return r;
 }
 
@@ -645,11 +658,13 @@ int bpm_surrogate_infer(bpm_ctx* ctx, int32_t sid, const float* X, int64_t N, fl
     cudaStream_t s = ctx->stream;
     const float* Xd = X;
     float *Xtmp = nullptr, *Pd = P;
+    CallBuffers buf(ctx);
     if (!on_device) {
-        BPM_CK(cudaMallocAsync(&Xtmp, sizeof(float) * (size_t)N * (m->n_in + m->n_out), s));
+        buf.take(&Xtmp, (size_t)N * m->n_in);
+        buf.take(&Pd, (size_t)N * m->n_out);
+        BPM_TRY(buf.reserve());
         BPM_CK(cudaMemcpyAsync(Xtmp, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
         Xd = Xtmp;
-        Pd = Xtmp + (size_t)N * m->n_in;
     }
     int r = infer_rows(m, ctx, Xd, N, true, Pd);
     if (r == BPM_OK && !on_device) {
@@ -659,7 +674,6 @@ int bpm_surrogate_infer(bpm_ctx* ctx, int32_t sid, const float* X, int64_t N, fl
             r = BPM_ERR_CUDA;
         }
     }
-    if (Xtmp) cudaFreeAsync(Xtmp, s);
     if (r != BPM_OK) return r;
     if (!on_device) return check_err(m, s);
     return BPM_OK;
@@ -681,13 +695,18 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
     float *Xtmp = nullptr, *z = nullptr;
     double* acc = nullptr;
     const size_t out_bytes = sizeof(double) * (size_t)n_designs * m->n_out;
-    BPM_CK(cudaMallocAsync(&z, sizeof(float) * (size_t)std::min(N, chunk) * m->n_out, s));
+    CallBuffers buf(ctx);
+    const size_t nz = (size_t)std::min(N, chunk) * m->n_out;
     if (!on_device) {
-        BPM_CK(cudaMallocAsync(&Xtmp, sizeof(float) * (size_t)N * m->n_in, s));
+        buf.take(&Xtmp, (size_t)N * m->n_in);
+        buf.take(&z, nz);
+        buf.take(&acc, (size_t)n_designs * m->n_out);
+        BPM_TRY(buf.reserve());
         BPM_CK(cudaMemcpyAsync(Xtmp, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
         Xd = Xtmp;
-        BPM_CK(cudaMallocAsync(&acc, out_bytes, s));
     } else {
+        // the device form returns with its work in flight: its scratch is stream-ordered memory
+        BPM_CK(cudaMallocAsync(&z, sizeof(float) * nz, s));
         acc = rates;
     }
     BPM_CK(cudaMemsetAsync(acc, 0, out_bytes, s));
@@ -717,9 +736,7 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
             r = BPM_ERR_CUDA;
         }
     }
-    cudaFreeAsync(z, s);
-    if (Xtmp) cudaFreeAsync(Xtmp, s);
-    if (!on_device && acc) cudaFreeAsync(acc, s);
+    if (on_device) cudaFreeAsync(z, s);
     if (r != BPM_OK) return r;
     if (!on_device) return check_err(m, s);
     return BPM_OK;
