@@ -223,25 +223,35 @@ int setup_grouped_gemm(bpm_batch* bt) {
 }
 
 // Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
-// tensor-core product on one stream, every island's CTA resident at once (at most four of 256
-// threads an SM, two vectors of the state in shared memory each) and at most 3200 nodes an SM.  Beyond that the
-// two-island kernels on two streams, which share the exchange entries between islands, are as fast
-// (interval in us, this way / theirs: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 /
-// 590; 1547 nodes, 300 islands 4177 / 4774, 512 islands 5304 / 5030).  Fills *G.
-bool few_islands(const bpm_batch* bt, StageGroups* G) {
+// tensor-core product on one stream, every stage CTA resident at once.  One island a CTA for at most
+// four islands (of 256 threads) and 3200 nodes an SM, two islands a CTA for at most
+// four pairs and 1000 nodes of pairs an SM.  Beyond
+// that the two-island kernels on two streams are as fast (interval in us, one island a CTA this way /
+// two streams: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 / 590; 1547 nodes, 300
+// islands 4177 / 4774, 512 islands 5304 / 5030; two islands a CTA: 209 nodes, 1200 islands 365 / 389; 481
+// nodes, 800 islands 689 / 625).  Fills *G and *threads (launch_few's).
+bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
     if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
-    const int per_sm = (bt->B + bt->ctx->sm_count - 1) / bt->ctx->sm_count;
-    std::memset(G, 0, sizeof(StageGroups));
+    const int sms = bt->ctx->sm_count;
     size_t smem = 0;
-    int n = 0;
+    int n = 0, pairs = 0;
     for (const auto& g : bt->groups) {
         smem = std::max(smem, 2 * stage_smem_bytes(g.args));
         n = std::max(n, g.mesh->n);
+        pairs += (g.B + 1) / 2;
+    }
+    const int ones_sm = (bt->B + sms - 1) / sms, pairs_sm = (pairs + sms - 1) / sms;
+    const bool ones = ones_sm <= 4 && ones_sm * n <= std::max(3200, n) && ones_sm * (smem + 1024) <= 200 * 1024;
+    const bool two = !ones && pairs_sm <= 4 && pairs_sm * n <= 1000 && pairs_sm * (2 * smem + 1024) <= 200 * 1024;
+    if (!ones && !two) return false;
+    std::memset(G, 0, sizeof(StageGroups));
+    for (const auto& g : bt->groups) {
         G->a[G->ng] = g.args;
-        G->block_begin[G->ng + 1] = G->block_begin[G->ng] + g.B;
+        G->block_begin[G->ng + 1] = G->block_begin[G->ng] + (ones ? g.B : (g.B + 1) / 2);
         ++G->ng;
     }
-    return per_sm <= 4 && per_sm * n <= std::max(3200, n) && per_sm * (smem + 1024) <= 200 * 1024;
+    *threads = ones ? few_threads(n, bt->B, sms) : 0;
+    return true;
 }
 
 // The chains of a multi-stream batch: the one group's islands cut into `streams` chunks of a
@@ -253,7 +263,8 @@ int setup_chains(bpm_batch* bt) {
     bt->chains = 0;
     for (auto& v : bt->chain_groups) v.clear();
     StageGroups few;
-    if (bt->streams < 2 || !tensor_core_precision(bt) || few_islands(bt, &few)) return BPM_OK;
+    int few_nt = 0;
+    if (bt->streams < 2 || !tensor_core_precision(bt) || few_islands(bt, &few, &few_nt)) return BPM_OK;
     const int ng = (int)bt->groups.size();
     const int chunk = ng > 1 ? 0 : kIslandPad * ((bt->groups[0].B + bt->streams * kIslandPad - 1) /
                                                  (bt->streams * kIslandPad));
@@ -436,10 +447,8 @@ int launch_stage_all(bpm_batch* bt, const StageLaunches& L, int stage, int j, cu
 // over side streams so that their kernels can run concurrently
 int enqueue_interval(bpm_batch* bt, cudaStream_t s) {
     StageGroups few;
-    if (few_islands(bt, &few)) {
-        int n = 0;
-        for (const auto& g : bt->groups) n = std::max(n, g.mesh->n);
-        const int nt = few_threads(n, bt->B, bt->ctx->sm_count);
+    int nt = 0;
+    if (few_islands(bt, &few, &nt)) {
         for (int j = 0; j < bt->p.substeps; ++j)
             for (int k = 1; k <= 2; ++k) {
                 BPM_TRY(grouped_gemm_launch(s, bt->gg, bt->ctx->sm_count, bt->gemm_err, true));

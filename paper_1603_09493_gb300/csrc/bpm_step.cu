@@ -401,7 +401,7 @@ __device__ __forceinline__ void exchange_sums(const StepArgs& a, int i, const fl
 // effective field of island b at node i from its exchange sum and the local terms
 __device__ __forceinline__ float3 field_from_sums(const StepArgs& a, float3 mi, float3 bex, float3 hdv, float4 p0,
                                                   float4 p1, float4 p2, float4 pos, float an0, float ramp, float xh,
-                                                  unsigned mask) {
+                                                  unsigned mask, const float3* head = nullptr) {
     float3 B = f3(0, 0, 0);
     if (mask & BPM_TERM_EXCHANGE) B = B + p0.x * bex;
     if (mask & BPM_TERM_ANISOTROPY) {
@@ -411,7 +411,7 @@ __device__ __forceinline__ float3 field_from_sums(const StepArgs& a, float3 mi, 
     }
     if (mask & BPM_TERM_DEMAG) B = B + hdv;
     if ((mask & BPM_TERM_HEAD) && a.map) {
-        B = B + ramp * trilinear(a, pos.x + p1.w - xh, pos.y + p2.x, pos.z);
+        B = B + ramp * (head ? *head : trilinear(a, pos.x + p1.w - xh, pos.y + p2.x, pos.z));
     }
     if (mask & BPM_TERM_UNIFORM) {
         B = B + ramp * f3(a.uni[0], a.uni[1], a.uni[2]) + f3(p2.y, p2.z, p2.w);
@@ -419,8 +419,35 @@ __device__ __forceinline__ float3 field_from_sums(const StepArgs& a, float3 mi, 
     return B;
 }
 
-// predictor of islands b0 .. b0 + nb - 1 (nb <= IPB); sp: [IPB][3] island parameters in smem
+// What a programmatic launch takes ahead of its wait (see few_body): the island parameters, the clock,
+// the head field of the islands' nodes (hb [q][3][n_pad]) and the exchange entries (into L1).
 template <int IPB>
+__device__ __forceinline__ void prepare_multi(const StepArgs& a, int nb, const float4* sp, const StageClock& clk,
+                                              float* hb) {
+    __syncthreads();                                       // sp and clk are there
+    const int np = a.n_pad;
+    const bool head = (a.mask & BPM_TERM_HEAD) && a.map;
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        const float4 pos = __ldg(a.node_pos + i);
+        if (a.mask & BPM_TERM_EXCHANGE) {
+            const int hi = __ldg(a.sell_off + (i >> 5) + 1);
+            for (int e = __ldg(a.sell_off + (i >> 5)) + (i & 31); e < hi; e += 32)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(a.sell_il + e));
+        }
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(a.node_mat + i));
+        if (head)
+            for (int q = 0; q < nb; ++q) {
+                const float3 h = trilinear(a, pos.x + sp[3 * q + 1].w - clk.xh, pos.y + sp[3 * q + 2].x, pos.z);
+                float* d = hb + 3 * q * np + i;
+                d[0] = h.x;
+                d[np] = h.y;
+                d[2 * np] = h.z;
+            }
+    }
+}
+
+// predictor of islands b0 .. b0 + nb - 1 (nb <= IPB); sp: [IPB][3] island parameters in smem
+template <int IPB, bool AHEAD = false>
 __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, float4* sp) {
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -429,6 +456,12 @@ __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, f
     if ((int)threadIdx.x < 3 * nb) sp[threadIdx.x] = a.isl[3 * b0 + threadIdx.x];
     __shared__ StageClock clk;
     set_clock(clk, a, j, 0);
+    float* hb = sm + IPB * S;
+    if (AHEAD) {
+        pdl_trigger();
+        prepare_multi<IPB>(a, nb, sp, clk, hb);
+        pdl_wait();
+    }
     for (int q = 0; q < nb; ++q) stage_state_il(a.m + (size_t)(b0 + q) * S, sm, np, q);
     const float hf = (float)a.h;
     const unsigned mask = a.mask;
@@ -451,7 +484,10 @@ __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, f
             const int b = b0 + q;
             const size_t base = (size_t)b * S;
             const float4 p0 = sp[3 * q], p1 = sp[3 * q + 1], p2 = sp[3 * q + 2];
-            float3 B = field_from_sums(a, mi[q], bex[q], hdv[q], p0, p1, p2, pos, nm.x, ramp, xh, mask);
+            float3 hv;
+            if (AHEAD) hv = f3(hb[3 * q * np + i], hb[(3 * q + 1) * np + i], hb[(3 * q + 2) * np + i]);
+            float3 B = field_from_sums(a, mi[q], bex[q], hdv[q], p0, p1, p2, pos, nm.x, ramp, xh, mask,
+                                       AHEAD ? &hv : nullptr);
             float3 f = llg_rhs(mi[q], B, a.alpha, a.gp);
             float3 v = heun_predict(mi[q], f, hf);
             a.k1[base + i] = f.x;
@@ -464,7 +500,7 @@ __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, f
 }
 
 // corrector and switch detectors of islands b0 .. b0 + nb - 1; red: [IPB][NT / 32]
-template <int IPB>
+template <int IPB, bool AHEAD = false>
 __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, float4* sp, float* red) {
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -473,6 +509,12 @@ __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, f
     if ((int)threadIdx.x < 3 * nb) sp[threadIdx.x] = a.isl[3 * b0 + threadIdx.x];
     __shared__ StageClock clk;
     set_clock(clk, a, j, 1);
+    float* hb = sm + IPB * S;
+    if (AHEAD) {
+        pdl_trigger();
+        prepare_multi<IPB>(a, nb, sp, clk, hb);
+        pdl_wait();
+    }
     stage_predicted_il(a.m + (size_t)b0 * S, a.k1 + (size_t)b0 * S, sm, np, a.n, nb, (float)a.h);
     const float hh = 0.5f * (float)a.h;
     const unsigned mask = a.mask;
@@ -500,7 +542,10 @@ __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, f
             const float4 p0 = sp[3 * q], p1 = sp[3 * q + 1], p2 = sp[3 * q + 2];
             const float3 mn = f3(__ldcg(a.m + base + i), __ldcg(a.m + base + np + i), __ldcg(a.m + base + 2 * np + i));
             const float3 f1 = f3(__ldcg(a.k1 + base + i), __ldcg(a.k1 + base + np + i), __ldcg(a.k1 + base + 2 * np + i));
-            float3 B = field_from_sums(a, mi[q], bex[q], hdv[q], p0, p1, p2, pos, nm.x, ramp, xh, mask);
+            float3 hv;
+            if (AHEAD) hv = f3(hb[3 * q * np + i], hb[(3 * q + 1) * np + i], hb[(3 * q + 2) * np + i]);
+            float3 B = field_from_sums(a, mi[q], bex[q], hdv[q], p0, p1, p2, pos, nm.x, ramp, xh, mask,
+                                       AHEAD ? &hv : nullptr);
             float3 f2 = llg_rhs(mi[q], B, a.alpha, a.gp);
             float3 v = normalize3(mn + hh * (f1 + f2));
             a.m[base + i] = v.x;
@@ -653,6 +698,19 @@ __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_stage2m_groups(co
     __shared__ float red[kMultiIPB * kMultiNT / 32];
     const int g = stage_group(G);
     stage2_multi<kMultiIPB>(G.a[g], kMultiIPB * (blockIdx.x - G.block_begin[g]), j, sp, red);
+}
+
+// the same behind a programmatic launch, for more islands than k_few holds at once; stage 1 or 2
+template <int STAGE>
+__global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_few_pairs(const __grid_constant__ StageGroups G, int j) {
+    __shared__ float4 sp[3 * kMultiIPB];
+    __shared__ float red[kMultiIPB * kMultiNT / 32];
+    const int g = stage_group(G);
+    const int b0 = kMultiIPB * (blockIdx.x - G.block_begin[g]);
+    if (STAGE == 1)
+        stage1_multi<kMultiIPB, true>(G.a[g], b0, j, sp);
+    else
+        stage2_multi<kMultiIPB, true>(G.a[g], b0, j, sp, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -991,6 +1049,9 @@ int configure_step_kernels() {
     BPM_CK(cudaFuncSetAttribute(k_stage2_groups<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     BPM_CK(cudaFuncSetAttribute(k_stage2_groups<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int smem2 = kMultiIPB * smem;
+    const int smem3 = std::min(2 * smem2, 200 * 1024);
+    BPM_CK(cudaFuncSetAttribute(k_few_pairs<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3));
+    BPM_CK(cudaFuncSetAttribute(k_few_pairs<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3));
     BPM_TRY(configure_few<256>(smem2));
     BPM_TRY(configure_few<512>(smem2));
     BPM_TRY(configure_few<1024>(smem2));
@@ -1024,6 +1085,14 @@ int launch_few_nt(const StageGroups& G, int stage, int j, cudaStream_t s) {
 }  // namespace
 
 int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t s) {
+    if (threads == 0) {
+        size_t smem = 0;
+        for (int g = 0; g < G.ng; ++g) smem = std::max(smem, 2 * kMultiIPB * stage_smem_bytes(G.a[g]));
+        const dim3 grid(G.block_begin[G.ng]), block(kMultiNT);
+        BPM_CK(stage == 1 ? launch_pdl(k_few_pairs<1>, grid, block, smem, s, true, G, j)
+                          : launch_pdl(k_few_pairs<2>, grid, block, smem, s, true, G, j));
+        return BPM_OK;
+    }
     return threads == 1024  ? launch_few_nt<1024>(G, stage, j, s)
            : threads == 512 ? launch_few_nt<512>(G, stage, j, s)
                             : launch_few_nt<256>(G, stage, j, s);

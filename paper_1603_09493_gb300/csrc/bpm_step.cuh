@@ -61,8 +61,9 @@ void launch_stage2(const StepArgs& a, int j, cudaStream_t s);
 void launch_stage1_groups(const StageGroups& G, int threads, size_t smem, int j, cudaStream_t s);
 void launch_stage2_groups(const StageGroups& G, int threads, size_t smem, int j, cudaStream_t s);
 size_t stage_smem_bytes(const StepArgs& a);
-// The same stages for batches of few islands (see k_few): one island per CTA, programmatic launches.
-// few_threads: CTA size for meshes of up to n nodes in a batch of B islands
+// The same stages for batches of few islands (see k_few), programmatic launches.  threads: CTA size of
+// the one-island kernels (few_threads: for meshes of up to n nodes in a batch of B islands), or 0: two
+// islands a CTA of 256 threads, G's blocks counting pairs
 int few_threads(int n, int B, int sm_count);
 int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t s);
 // resident CTAs per SM of the grouped stage kernels at this CTA size, islands per CTA and
