@@ -866,6 +866,74 @@ __global__ void k_demag_convert(int n, int pitch, int K, const double* __restric
     Wlo[o] = __float2bfloat16_rn((float)(v - (double)__bfloat162float(hi)));
 }
 
+// Sliced-ELL places of the exchange entries: fills the slices' offsets *off [slices + 1] and returns the CSR
+// entry e of each place, ~e for padding (node col[e], value 0).  Entry c of a slice's 32 rows is one gather of
+// the stage kernels, lane l from bank (node mod 32).  Column by column every row, the longest first, takes
+// the neighbour that meets fewest others in its bank so far, and waits for a later column where even that
+// one would lengthen the gather and its row is shorter than the slice; padding reads a node of its row that
+// meets fewest.  1.26 instead of 1.93 wavefronts a gather on the census mesh in row order.
+// An interval of 4096 islands 24.46 -> 24.16 ms, of 1024 islands 6.60 -> 6.48 ms.
+std::vector<int> gather_order(int n, const std::vector<int>& rowptr, const std::vector<int>& col,
+                              std::vector<int>* off) {
+    const int ns = (n + 31) / 32;
+    off->assign(ns + 1, 0);
+    for (int q = 0; q < ns; ++q) {
+        int w = 0;
+        for (int i = 32 * q; i < std::min(n, 32 * q + 32); ++i) w = std::max(w, rowptr[i + 1] - rowptr[i] - 1);
+        (*off)[q + 1] = (*off)[q] + 32 * w;
+    }
+    std::vector<int> slot((*off)[ns]), seen(n, -1), order;
+    std::vector<int> left[32];
+    for (int q = 0; q < ns; ++q) {
+        const int w = ((*off)[q + 1] - (*off)[q]) / 32, rows = std::min(32, n - 32 * q);
+        for (int l = 0; l < rows; ++l) {
+            left[l].clear();
+            for (int e = rowptr[32 * q + l]; e < rowptr[32 * q + l + 1]; ++e)
+                if (col[e] != 32 * q + l) left[l].push_back(e);
+        }
+        order.resize(rows);
+        for (int l = 0; l < rows; ++l) order[l] = l;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int x, int y) { return left[x].size() > left[y].size(); });
+        for (int c = 0; c < w; ++c) {
+            const int tag = (*off)[q] / 32 + c;           // of this column, in seen
+            int bank[32] = {}, deep = 0, any = -1;        // distinct nodes of the column in each bank, their most
+            int* out = &slot[(*off)[q] + 32 * c];
+            auto others = [&](int e) { return bank[col[e] & 31] - (seen[col[e]] == tag ? 1 : 0); };
+            auto place = [&](int e) {
+                if (seen[col[e]] == tag) return;
+                seen[col[e]] = tag;
+                deep = std::max(deep, ++bank[col[e] & 31]);
+            };
+            unsigned padded = 0;
+            for (int l : order) {
+                std::vector<int>& v = left[l];
+                size_t best = 0;
+                int least = 1 << 30;
+                for (size_t k = 0; k < v.size() && least > 0; ++k)
+                    if (const int o = others(v[k]); o < least) least = o, best = k;
+                if (v.empty() || ((int)v.size() < w - c && least >= std::max(1, deep))) {
+                    padded |= 1u << l;
+                    continue;
+                }
+                any = out[l] = v[best];
+                place(out[l]);
+                v.erase(v.begin() + best);
+            }
+            for (int l = 0; l < 32; ++l) {
+                if (l >= rows) out[l] = ~any;
+                if (l >= rows || !(padded >> l & 1)) continue;
+                int pick = rowptr[32 * q + l], least = others(pick);
+                for (int e = pick + 1; e < rowptr[32 * q + l + 1] && least > 0; ++e)
+                    if (const int o = others(e); o < least) least = o, pick = e;
+                place(pick);
+                out[l] = ~pick;
+            }
+        }
+    }
+    return slot;
+}
+
 }  // namespace
 
 void free_mesh(Mesh* M) {
@@ -1183,6 +1251,9 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     BPM_CK(cudaGetLastError());
     double lam = 0;
     BPM_TRY(side.join(st));
+    std::vector<int> off;
+    const std::vector<int> slot = gather_order(n, rowptr, col, &off);   // on the host beside the kernels above
+    M->n_slices = (int)off.size() - 1;
     BPM_CK(cudaMemcpyAsync(&lam, d_lam, sizeof(double), cudaMemcpyDeviceToHost, st));
     BPM_CK(cudaStreamSynchronize(st));
     if (!(flags & BPM_MESH_KEEP_F64)) {
@@ -1205,31 +1276,10 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
         an_max = std::max(an_max, an);
         ms_max = std::max(ms_max, M->Ms[i]);
     }
-    M->n_slices = np / 32;
-    std::vector<int> off(M->n_slices + 1, 0);
-    for (int s = 0; s < M->n_slices; ++s) {
-        int w = 0;
-        for (int l = 0; l < 32; ++l) {
-            int i = 32 * s + l;
-            if (i < n) w = std::max(w, rowptr[i + 1] - rowptr[i] - 1);
-        }
-        off[s + 1] = off[s] + 32 * w;
-    }
-    std::vector<int2> ent(std::max(1, off[M->n_slices]));
-    for (int s = 0; s < M->n_slices; ++s) {
-        int w = (off[s + 1] - off[s]) / 32;
-        for (int l = 0; l < 32; ++l) {
-            int i = 32 * s + l;
-            int q = 0;
-            if (i < n)
-                for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-                    if (col[e] == i) continue;
-                    float v = M->exch_val[e];
-                    ent[off[s] + 32 * q + l] = make_int2(col[e], *reinterpret_cast<int*>(&v));
-                    ++q;
-                }
-            for (; q < w; ++q) ent[off[s] + 32 * q + l] = make_int2(i < n ? i : 0, 0);
-        }
+    std::vector<int2> ent(std::max<size_t>(1, slot.size()), make_int2(0, 0));
+    for (size_t k = 0; k < slot.size(); ++k) {
+        const float v = slot[k] < 0 ? 0.f : M->exch_val[slot[k]];
+        ent[k] = make_int2(col[slot[k] < 0 ? ~slot[k] : slot[k]], *reinterpret_cast<const int*>(&v));
     }
     std::vector<int2> ent_il(ent.size());
     for (size_t k = 0; k < ent.size(); ++k) {

@@ -63,7 +63,8 @@ struct Mesh {
     float4* node_pos = nullptr;   // x, y, z (nm), w_i = V_i / sum V
     float4* node_mat = nullptr;   // 2 Ku_i / Ms_i (T), Ms_i (MA/m), 0, 0
     // exchange operator, difference form, sliced ELL with 32-row slices:
-    // B_ex,i = (1/Ms_scale) sum_e val_e (m_{col_e} - m_i); padding entries val = 0, col = i
+    // B_ex,i = (1/Ms_scale) sum_e val_e (m_{col_e} - m_i); padding entries val = 0, col = i or a
+    // neighbour of i (gather_order)
     int n_slices = 0;
     int* sell_off = nullptr;      // [n_slices + 1] first entry of each slice
     int2* sell_ent = nullptr;     // (col, float bits of val), entry e of row 32 s + l at off[s] + 32 e + l
@@ -150,7 +151,6 @@ struct bpm_ctx {
     bpm::Scratch scratch;
     int device = 0;
     int sm_count = 0;
-    size_t l2_bytes = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     std::vector<bpm::Mesh*> meshes;
