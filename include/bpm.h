@@ -345,8 +345,8 @@ enum { BPM_RASTER_AUTO = 0, BPM_RASTER_M = 1, BPM_RASTER_N = 2 };
  * gemm_k_block 32, gemm_pair 0, and streams 2 for a one-mesh batch, 1 for a
  * multi-mesh batch (the fastest on the census and uneven batches measured).  A
  * batch of few islands (whose stage CTAs all fit the SMs at once) runs one chain
- * with one island per stage CTA whatever stage_threads, stage_islands and
- * streams say, unless gemm_pair is 1. */
+ * with one island per stage CTA, or two where the islands outnumber the SMs,
+ * whatever stage_threads, stage_islands and streams say, unless gemm_pair is 1. */
 typedef struct {
     int32_t gemm_tile_n;     /* islands per demag-GEMM tile at most: 256 or 128 (the library takes
                                 narrower tiles where wide ones would leave SMs idle) */

@@ -223,13 +223,14 @@ int setup_grouped_gemm(bpm_batch* bt) {
 }
 
 // Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
-// tensor-core product on one stream, every stage CTA resident at once.  One island a CTA for at most
-// four islands (of 256 threads) and 3200 nodes an SM, two islands a CTA for at most
-// four pairs and 1000 nodes of pairs an SM.  Beyond
-// that the two-island kernels on two streams are as fast (interval in us, one island a CTA this way /
-// two streams: 209 nodes, 600 islands 304 / 340; 481 nodes, 600 islands 563 / 590; 1547 nodes, 300
-// islands 4177 / 4774, 512 islands 5304 / 5030; two islands a CTA: 209 nodes, 1200 islands 365 / 389; 481
-// nodes, 800 islands 689 / 625).  Fills *G and *threads (launch_few's).
+// tensor-core product on one stream, every stage CTA resident at once.  One island a CTA where each has an
+// SM, two islands a CTA (they share the exchange entries) for at most three pairs and 2000 nodes of pairs an
+// SM (one pair an SM of any mesh).  Beyond that the two-island kernels on two streams are as fast.  An interval in us, this way / two
+// streams, alone and with three batches in turn on as many streams (each a pass): 1547 nodes, 128 islands
+// 2020 / 3900 and 1820 / 1980, 304 islands 4850 / 5600 and 2650 / 2750; 481 nodes, 300 islands 522 / 603 and 219 / 224,
+// 600 islands 606 / 647 and 289 / 281; 209 nodes, 800 islands 343 / 411 and 181 / 177, 1200 islands 470 /
+// 432 and 245 / 220.  One island a CTA and two an SM: 481 nodes, 300 islands 535 and 262; 209 nodes, 600
+// islands 367 and 193 (pairs 344 and 152).
 bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
     if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
     const int sms = bt->ctx->sm_count;
@@ -241,8 +242,8 @@ bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
         pairs += (g.B + 1) / 2;
     }
     const int ones_sm = (bt->B + sms - 1) / sms, pairs_sm = (pairs + sms - 1) / sms;
-    const bool ones = ones_sm <= 4 && ones_sm * n <= std::max(3200, n) && ones_sm * (smem + 1024) <= 200 * 1024;
-    const bool two = !ones && pairs_sm <= 4 && pairs_sm * n <= 1000 && pairs_sm * (2 * smem + 1024) <= 200 * 1024;
+    const bool ones = ones_sm == 1 && smem + 1024 <= 200 * 1024;
+    const bool two = !ones && pairs_sm <= 3 && pairs_sm * n <= std::max(2000, n) && pairs_sm * (2 * smem + 1024) <= 200 * 1024;
     if (!ones && !two) return false;
     std::memset(G, 0, sizeof(StageGroups));
     for (const auto& g : bt->groups) {
@@ -691,7 +692,6 @@ int bpm_create(bpm_ctx** out, int device, void* cuda_stream) {
     bpm_ctx* c = new bpm_ctx();
     c->device = device;
     c->sm_count = prop.multiProcessorCount;
-    c->l2_bytes = (size_t)prop.l2CacheSize;
     if (cuda_stream) {
         c->stream = static_cast<cudaStream_t>(cuda_stream);
     } else {

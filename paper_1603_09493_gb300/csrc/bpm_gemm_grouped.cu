@@ -311,32 +311,38 @@ int even_tile(int M, int cap) {
     return (((M + t - 1) / t) + 15) / 16 * 16;
 }
 
-// The widest tiles that do not leave SMs idle: over caps of 256 .. 16 islands, the time of the busiest
-// SM as waves of items x cost of an item (k-steps x MMA cost, an item's fixed cost as 12 k-steps).
-// Wide tiles win ties.  One island of 1547 nodes: 148 items of a quarter of K; 200 islands: 148 items
-// of 64 (60 us against 81 with two 128-row tiles); 4096: 608 items of 256 in four waves.
-// share > 1: the product runs beside share - 1 others on as many streams.  It then aims at its share of
-// the SMs, in no whole waves (an SM takes the others' work next), and at a tenth of gain: more CTAs
-// would only hold up the others (4096 islands of 481 nodes: 1.79 ms an interval with 120 items of 208
-// a chain, 1.60 with 96 of 256).
+// Islands per tile at most (256 .. 16): the cap with the least of
+//   - the time of the busiest SM: waves of items x cost of an item (k-steps x MMA cost, an item's fixed cost
+//     as 12 k-steps), and
+//   - ten times the launch's own use of the chip, the rows its items read (128 + islands each) as if spread
+//     over every SM: what it takes from the stage kernels, other chains and other batches beside it.
+// Wide tiles win ties.  The second term decides where narrow tiles would read the operator again for each.
+// Without it (the tile that is fastest alone) 200 islands of 1547 nodes took 148 items of 64: an interval
+// 4.25 ms alone but 3.80 with three batches in turn on as many streams (each a pass), against 4.22 and 2.13 so;
+// 512 islands 5.26 and 4.26 against 5.79 and 3.24; nine hundred of 481 nodes 0.64 and 0.52 against 0.73
+// and 0.35; 1318 of 209 nodes 0.41 and 0.29 against 0.46 and 0.23.
+// share > 1: the product runs beside share - 1 others on as many streams and takes no whole waves (an SM
+// takes the others' work next).
 int tile_cap(const std::vector<GemmOperands>& ops, int tile_n, int sm_count, int share) {
     int best = tile_n;
     double best_t = 1e300;
     for (int cap : {256, 208, 160, 128, 96, 64, 48, 32, 16}) {
         if (cap > tile_n) continue;
         long long items = 0;
-        double sum = 0, top = 0;
+        double sum = 0, top = 0, rows = 0;
         for (const GemmOperands& o : ops) {
             const int nb = even_tile(o.M, cap);
             const long long it = (long long)((o.M + nb - 1) / nb) * ((o.N + tc::TM - 1) / tc::TM) * o.splits;
-            const double c = (double)mma_cost(nb) * (o.K / 16.0 / o.splits + 12.0);
+            const double steps = o.K / 16.0 / o.splits + 12.0, c = mma_cost(nb) * steps;
             items += it;
             sum += it * c;
+            rows += it * steps * (128 + nb) / 1.5;          // in the MMA's units at 256 islands
             top = std::max(top, c);
         }
         const double waves = (double)items * share / sm_count;
-        const double t = std::max(top, (share > 1 ? waves : std::ceil(waves)) * sum / (double)items);
-        if (t < best_t * (share > 1 ? 0.9 : 0.98)) {
+        const double busy = std::max(top, (share > 1 ? waves : std::ceil(waves)) * sum / (double)items);
+        const double t = busy + 10.0 * rows / sm_count;
+        if (t < best_t * 0.98) {
             best_t = t;
             best = cap;
         }
