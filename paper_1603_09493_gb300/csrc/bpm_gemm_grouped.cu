@@ -404,6 +404,13 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
     std::vector<GemmGroupDev> h(ops.size());
     int tiles = 0, nb_max = 16;
     const int cap = tile_cap(ops, tile_n, sm_count, share);
+    for (const GemmOperands& o : ops)
+        if (o.M > 0) nb_max = std::max(nb_max, even_tile(o.M, cap));
+    // Tiles of up to 128 islands leave room for three or four stages of 64-deep k-blocks, which read 128 bytes
+    // of a row at a time and take half the barriers: an interval of one island of 1547 nodes 1256 -> 1139 us,
+    // of 60 islands 1655 -> 1522, of eight uneven variants of 14 islands 24.2 -> 23.7 ms.  Wider tiles hold one such
+    // stage only (1024 islands 6.64 ms at 32, 7.00 at 64).
+    if (!pair && nb_max <= 128) k_block = 64;
     for (size_t g = 0; g < ops.size(); ++g) {
         const GemmOperands& o = ops[g];
         if (o.rows % tc::TM || o.K % tc::TK || o.N % 16 || o.M <= 0 || o.M > o.rows || o.N <= 0 || o.splits < 1) {
@@ -413,7 +420,6 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
         }
         std::memset(&h[g], 0, sizeof(GemmGroupDev));
         const int nb = even_tile(o.M, cap);
-        nb_max = std::max(nb_max, nb);
         // a CTA of a pair stages 128 of the tile's 256 rows of either operand
         const int a_box = pair ? tc::TM : nb;
         BPM_TRY(make_bf16_tensor_map(&h[g].ahi, o.Ahi, o.K, o.rows, a_box, k_block));
@@ -456,7 +462,7 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
     gg->grid = grid;
     gg->n_groups = (int)h.size();
     gg->total_tiles = tiles;
-    gg->tile_n = nb_max <= 128 ? 128 : 256;
+    gg->tile_n = nb_max <= 64 ? 64 : nb_max <= 128 ? 128 : 256;
     gg->products = products;
     gg->k_block = k_block;
     gg->pair = pair;
@@ -476,18 +482,15 @@ int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err,
         return BPM_ERR_STATE;
     }
     if (gg.pair) return grouped_gemm_pair_launch(s, gg, sm_count, err);
-    if (gg.k_block == 32) {
-        if (gg.products == 3)
-            return gg.tile_n == 128 ? launch_grouped<3, 128, 32>(s, gg, sm_count, err, pdl)
-                                    : launch_grouped<3, 256, 32>(s, gg, sm_count, err, pdl);
-        return gg.tile_n == 128 ? launch_grouped<1, 128, 32>(s, gg, sm_count, err, pdl)
-                                : launch_grouped<1, 256, 32>(s, gg, sm_count, err, pdl);
-    }
-    if (gg.products == 3)
-        return gg.tile_n == 128 ? launch_grouped<3, 128, 64>(s, gg, sm_count, err, pdl)
-                                : launch_grouped<3, 256, 64>(s, gg, sm_count, err, pdl);
-    return gg.tile_n == 128 ? launch_grouped<1, 128, 64>(s, gg, sm_count, err, pdl)
-                            : launch_grouped<1, 256, 64>(s, gg, sm_count, err, pdl);
+    const bool split = gg.products == 3;
+    if (gg.tile_n == 64) return split ? launch_grouped<3, 64, 64>(s, gg, sm_count, err, pdl)
+                                      : launch_grouped<1, 64, 64>(s, gg, sm_count, err, pdl);
+    if (gg.tile_n == 128) return split ? launch_grouped<3, 128, 64>(s, gg, sm_count, err, pdl)
+                                       : launch_grouped<1, 128, 64>(s, gg, sm_count, err, pdl);
+    if (gg.k_block == 64) return split ? launch_grouped<3, 256, 64>(s, gg, sm_count, err, pdl)
+                                       : launch_grouped<1, 256, 64>(s, gg, sm_count, err, pdl);
+    return split ? launch_grouped<3, 256, 32>(s, gg, sm_count, err, pdl)
+                 : launch_grouped<1, 256, 32>(s, gg, sm_count, err, pdl);
 }
 
 }  // namespace bpm

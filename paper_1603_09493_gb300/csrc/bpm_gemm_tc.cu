@@ -4,11 +4,11 @@
 // Ahi*Wlo; the batched demag product uses the persistent grouped kernel in
 // bpm_gemm_grouped.cu).
 //
-// One CTA computes a 128 x 256 output tile.  Warp 0 (one elected lane) streams the
+// One CTA computes a 128-row output tile of 32 to 256 columns (by epilogue, see Cfg).  Warp 0 (one elected lane) streams the
 // k-blocks (64 BF16 = one 128-byte swizzle atom) of every operand tile with TMA into a
 // ring of shared-memory stages, warp 1 (one elected lane) issues the tcgen05.mma
-// instructions into a 128-lane x 256-column TMEM accumulator, and after the last
-// k-block all four warps read the accumulator back with tcgen05.ld and store it.
+// instructions into a TMEM accumulator of 128 lanes, and after the last
+// k-block all eight warps read the accumulator back with tcgen05.ld and store it.
 // Each stage holds Ahi, Alo, Whi, Wlo for one k-block, so the three products of a
 // k-block share the staged tiles.  Every mbarrier wait is bounded; on timeout the
 // kernel records an error flag, drains its own copies and MMAs, frees TMEM and exits.
