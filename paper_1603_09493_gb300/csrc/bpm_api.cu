@@ -225,12 +225,15 @@ int setup_grouped_gemm(bpm_batch* bt) {
 // Whether the batch's interval runs as the programmatic launches of few islands (launch_few): the
 // tensor-core product on one stream, every stage CTA resident at once.  One island a CTA where each has an
 // SM, two islands a CTA (they share the exchange entries) for at most three pairs and 2000 nodes of pairs an
-// SM (one pair an SM of any mesh).  Beyond that the two-island kernels on two streams are as fast.  An interval in us, this way / two
-// streams, alone and with three batches in turn on as many streams (each a pass): 1547 nodes, 128 islands
-// 2020 / 3900 and 1820 / 1980, 304 islands 4850 / 5600 and 2650 / 2750; 481 nodes, 300 islands 522 / 603 and 219 / 224,
-// 600 islands 606 / 647 and 289 / 281; 209 nodes, 800 islands 343 / 411 and 181 / 177, 1200 islands 470 /
-// 432 and 245 / 220.  One island a CTA and two an SM: 481 nodes, 300 islands 535 and 262; 209 nodes, 600
-// islands 367 and 193 (pairs 344 and 152).
+// SM (one pair an SM of any mesh).  Beyond that the two-island kernels on two streams are as fast.  An
+// interval in us, this way / two streams, alone and with three batches in turn on as many streams (each a
+// pass): 1547 nodes, 128 islands 2020 / 3900 and 1820 / 1980, 304 islands 4850 / 5600 and 2650 / 2750; 481
+// nodes, 300 islands 522 / 603 and 219 / 224, 600 islands 606 / 647 and 289 / 281; 209 nodes, 800 islands
+// 343 / 411 and 181 / 177, 1200 islands 470 / 432 and 245 / 220.  One mesh at one island a CTA and two or
+// more an SM: 481 nodes, 300 islands 535 and 262; 209 nodes, 600 islands 367 and 193 (pairs 344 and 152).
+// Several meshes of over 512 nodes do stay at one island a CTA up to 3200 nodes an SM: their groups are
+// small and sliced, and a pair's 256 threads take four passes over 1000 nodes (518 and 976 nodes, 120
+// islands each: 1410 and 1240, pairs 2620 and 1450).
 bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
     if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
     const int sms = bt->ctx->sm_count;
@@ -242,8 +245,10 @@ bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
         pairs += (g.B + 1) / 2;
     }
     const int ones_sm = (bt->B + sms - 1) / sms, pairs_sm = (pairs + sms - 1) / sms;
-    const bool ones = ones_sm == 1 && smem + 1024 <= 200 * 1024;
-    const bool two = !ones && pairs_sm <= 3 && pairs_sm * n <= std::max(2000, n) && pairs_sm * (2 * smem + 1024) <= 200 * 1024;
+    const bool wide = bt->groups.size() > 1 && n > 512 && ones_sm <= 4 && ones_sm * n <= 3200;
+    const bool ones = (ones_sm == 1 || wide) && ones_sm * (smem + 1024) <= 200 * 1024;
+    const bool two = !ones && pairs_sm <= 3 && pairs_sm * n <= std::max(2000, n) &&
+                     pairs_sm * (2 * smem + 1024) <= 200 * 1024;
     if (!ones && !two) return false;
     std::memset(G, 0, sizeof(StageGroups));
     for (const auto& g : bt->groups) {
