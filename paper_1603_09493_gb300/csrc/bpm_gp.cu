@@ -90,13 +90,19 @@ __global__ void __launch_bounds__(kGpThreads) k_lhs_min_d2(const double* __restr
 // Matrix t is A[t] [n + 2][n], the lower triangle of R with two more rows, y and 1: factoring the first
 // n rows turns them into z = L^-1 y and w = L^-1 1, so the solves cost no pass of their own.  Per block
 // of 32 columns one launch factors the diagonal block (every CTA for itself) and solves 32 rows below
-// it a CTA, one launch subtracts the block's products from 32 x 32 tiles to its right.  An element's
-// products are subtracted in the order of k, one rounding each, as an unblocked factorisation does.
+// it a CTA, one launch subtracts the block's products from 32 x 32 tiles to its right.  The factored
+// diagonal blocks have a place of their own, D[t] [block][32][32]: a CTA of the matrix may start after
+// another has finished, so the block they all load is never written.  An element's products are
+// subtracted in the order of k, one rounding each, as an unblocked factorisation does; the row solve
+// rounds a factor's quotient once more.
 // An SM does two FP64 multiply-adds a cycle: n = 160, 32 vectors are 22 M for the factors and as many
 // for the correlations, 0.08 ms spread over the GPU.  One CTA a matrix, unblocked from global memory,
 // took 1.40 ms; 0.47 ms now.
 // ---------------------------------------------------------------------------
 constexpr int kPB = 32;
+
+// doubles of a matrix's factored diagonal blocks
+__host__ __device__ __forceinline__ size_t diag_doubles(int n) { return (size_t)((n + kPB - 1) / kPB) * kPB * kPB; }
 
 // rows 0 .. n - 1: the lower triangle of R; row n: y; row n + 1: ones
 __global__ void __launch_bounds__(kGpThreads) k_gp_matrix(const double* __restrict__ X, const double* __restrict__ y,
@@ -124,17 +130,19 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_matrix(const double* __restri
     }
 }
 
-// Columns k0 .. k0 + 31: factor the diagonal block (written by CTA 0 of the matrix), solve the 32 rows
-// of this CTA below it.  A non-positive pivot marks the matrix as failed.
+// Columns k0 .. k0 + 31: factor the diagonal block (CTA 0 of the matrix writes it to Dall), solve the
+// 32 rows of this CTA below it.  A non-positive pivot marks the matrix as failed.
 __global__ void __launch_bounds__(kGpThreads) k_gp_panel(int n, int k0, double* __restrict__ Aall,
-                                                         int* __restrict__ fail) {
+                                                         double* __restrict__ Dall, int* __restrict__ fail) {
     __shared__ double D[kPB][kPB + 1], P[kPB][kPB + 1], inv[kPB];
     __shared__ int s_bad;
     const int t = blockIdx.y, nb = min(kPB, n - k0), r0 = k0 + nb + kPB * blockIdx.x;
-    if (fail[t]) return;
+    // one thread reads the mark, which another CTA of the matrix may set meanwhile
+    if (threadIdx.x == 0) s_bad = *(volatile int*)(fail + t);
+    __syncthreads();
+    if (s_bad) return;
     double* A = Aall + (size_t)t * (n + 2) * n;
     const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_bad = 0;
     if (w == 0) inv[l] = 0.0;
     for (int i = w; i < kPB; i += kGpThreads / 32) {
         D[i][l] = i < nb && l <= i ? A[(size_t)(k0 + i) * n + k0 + l] : 0.0;
@@ -163,9 +171,10 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_panel(int n, int k0, double* 
             if (l > k && l <= i) D[i][l] -= D[i][k] * D[l][k];
         __syncthreads();
     }
-    if (blockIdx.x == 0)
-        for (int i = w; i < nb; i += kGpThreads / 32)
-            if (l <= i) A[(size_t)(k0 + i) * n + k0 + l] = D[i][l];
+    if (blockIdx.x == 0) {
+        double* F = Dall + (size_t)t * diag_doubles(n) + (size_t)k0 * kPB;
+        for (int i = w; i < kPB; i += kGpThreads / 32) F[i * kPB + l] = D[i][l];
+    }
     // row solve: a warp per four rows, lane = column.  The right-hand sides stay unscaled, the quotients
     // go into the factor's columns (one multiply-add an element and step) and into the result.
     double a[4];
@@ -218,6 +227,7 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_update(int n, int k0, double*
 
 // nll = n ln sigma2 + ln det R from the factored matrix (one CTA each); +inf where it failed
 __global__ void __launch_bounds__(kGpThreads) k_gp_stats(int n, const double* __restrict__ Aall,
+                                                         const double* __restrict__ Dall,
                                                          const int* __restrict__ fail, double* __restrict__ nll,
                                                          double* __restrict__ stats) {
     __shared__ double red[kGpThreads / 32];
@@ -227,12 +237,12 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_stats(int n, const double* __
         return;
     }
     const double* A = Aall + (size_t)t * (n + 2) * n;
-    const double *z = A + (size_t)n * n, *w = z + n;
+    const double *z = A + (size_t)n * n, *w = z + n, *D = Dall + (size_t)t * diag_doubles(n);
     double ww = 0.0, wz = 0.0, ld = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         ww += w[i] * w[i];
         wz += w[i] * z[i];
-        ld += log(A[(size_t)i * n + i]);
+        ld += log(D[(size_t)i * kPB + (i & (kPB - 1))]);
     }
     ww = cta_sum(ww, red);
     wz = cta_sum(wz, red);
@@ -255,31 +265,33 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_stats(int n, const double* __
     }
 }
 
-// factors and likelihoods of T matrices (A: T (n + 2) n doubles, fail: T ints)
+// factors and likelihoods of T matrices (A: T (n + 2) n doubles, D: T diag_doubles(n), fail: T ints)
 int gp_factor(cudaStream_t s, const double* X, const double* y, int n, int d, const double* theta, int T,
-              double nugget, double* A, int* fail, double* nll, double* stats) {
+              double nugget, double* A, double* D, int* fail, double* nll, double* stats) {
     const int nblk = (n + kPB - 1) / kPB, nrow = (n + 2 + kPB - 1) / kPB;
     BPM_CK(cudaMemsetAsync(fail, 0, T * sizeof(int), s));
     for (int t0 = 0; t0 < T; t0 += 32768) {                 // grid y and z limit
         const int m = std::min(32768, T - t0);
-        double* At = A + (size_t)t0 * (n + 2) * n;
+        double *At = A + (size_t)t0 * (n + 2) * n, *Dt = D + (size_t)t0 * diag_doubles(n);
         k_gp_matrix<<<dim3(nblk, nrow, m), kGpThreads, 0, s>>>(X, y, n, d, theta + (size_t)t0 * d, nugget, At);
         for (int p = 0; p < nblk; ++p) {
             const int k0 = p * kPB, below = n + 2 - std::min(n, k0 + kPB);
-            k_gp_panel<<<dim3((below + kPB - 1) / kPB, m), kGpThreads, 0, s>>>(n, k0, At, fail + t0);
+            k_gp_panel<<<dim3((below + kPB - 1) / kPB, m), kGpThreads, 0, s>>>(n, k0, At, Dt, fail + t0);
             if (p + 1 < nblk)
                 k_gp_update<<<dim3(nblk - p - 1, nrow - p - 1, m), kGpThreads, 0, s>>>(n, k0, At, fail + t0);
         }
-        k_gp_stats<<<m, kGpThreads, 0, s>>>(n, At, fail + t0, nll + t0, stats ? stats + 3 * (size_t)t0 : nullptr);
+        k_gp_stats<<<m, kGpThreads, 0, s>>>(n, At, Dt, fail + t0, nll + t0,
+                                            stats ? stats + 3 * (size_t)t0 : nullptr);
     }
     BPM_CK(cudaGetLastError());
     return BPM_OK;
 }
 
-// Block row i0 .. i0 + 31 of Linv = L^-1 (L: [n + 2][n]): 32 columns a CTA, products of the block rows
+// Block row i0 .. i0 + 31 of Linv = L^-1 (L: [n + 2][n] below its diagonal blocks, which are D): 32 columns a CTA, products of the block rows
 // above (in the order of k) first, then the triangular solve within the block; Linv_ij = -s / L_ii.
 // (One thread per column walked the whole triangle: 0.81 ms at n = 160; 0.26 ms now.)
-__global__ void __launch_bounds__(kGpThreads) k_gp_linv(const double* __restrict__ L, int n, int i0,
+__global__ void __launch_bounds__(kGpThreads) k_gp_linv(const double* __restrict__ L,
+                                                        const double* __restrict__ D, int n, int i0,
                                                         double* __restrict__ Linv) {
     __shared__ double Lb[kPB][kPB + 1], Xb[kPB][kPB + 1];
     const int l = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * kPB + l;
@@ -298,7 +310,7 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_linv(const double* __restrict
     }
     __syncthreads();
     for (int r = w; r < kPB; r += kGpThreads / 32)
-        Lb[r][l] = i0 + r < n && i0 + l < n && l <= r ? L[(size_t)(i0 + r) * n + i0 + l] : 0.0;
+        Lb[r][l] = D[(size_t)(i0 + r) * kPB + l];           // zeros above the diagonal and past n
 #pragma unroll
     for (int q = 0; q < 4; ++q) Xb[4 * w + q][l] = s[q];
     __syncthreads();
@@ -505,14 +517,15 @@ extern "C" int bpm_gp_nll(bpm_ctx* ctx, const double* X, const double* y, int32_
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
     // theta vectors per launch: their factors together stay under 1 GiB
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(T, (size_t(1) << 30) / (8 * (size_t)(n + 2) * n)));
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(T, (size_t(1) << 30) / (8 * ((size_t)(n + 2) * n + diag_doubles(n)))));
     CallBuffers sc(ctx);
-    double *dX = nullptr, *dy = nullptr, *dth = nullptr, *A = nullptr, *dn = nullptr;
+    double *dX = nullptr, *dy = nullptr, *dth = nullptr, *A = nullptr, *D = nullptr, *dn = nullptr;
     int* fail = nullptr;
     sc.take(&dX, (size_t)n * d);
     sc.take(&dy, n);
     sc.take(&dth, (size_t)T * d);
     sc.take(&A, (size_t)chunk * (n + 2) * n);
+    sc.take(&D, (size_t)chunk * diag_doubles(n));
     sc.take(&fail, chunk);
     sc.take(&dn, T);
     BPM_TRY(sc.reserve());
@@ -520,8 +533,8 @@ extern "C" int bpm_gp_nll(bpm_ctx* ctx, const double* X, const double* y, int32_
     BPM_TRY(upload(dy, y, n, s));
     BPM_TRY(upload(dth, theta, (size_t)T * d, s));
     for (int t0 = 0; t0 < T; t0 += chunk)
-        BPM_TRY(gp_factor(s, dX, dy, n, d, dth + (size_t)t0 * d, std::min(chunk, T - t0), nugget, A, fail, dn + t0,
-                          nullptr));
+        BPM_TRY(gp_factor(s, dX, dy, n, d, dth + (size_t)t0 * d, std::min(chunk, T - t0), nugget, A, D, fail,
+                          dn + t0, nullptr));
     BPM_CK(cudaMemcpyAsync(nll, dn, T * sizeof(double), cudaMemcpyDeviceToHost, s));
     BPM_CK(cudaStreamSynchronize(s));
     return BPM_OK;
@@ -537,7 +550,7 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
     CallBuffers sc(ctx);
-    double *dy = nullptr, *A = nullptr, *dn = nullptr, *st = nullptr, *u = nullptr;
+    double *dy = nullptr, *A = nullptr, *D = nullptr, *dn = nullptr, *st = nullptr, *u = nullptr;
     int* dfail = nullptr;
     Gp* g = new Gp();
     g->n = n;
@@ -549,6 +562,7 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
     int r = BPM_OK;
     sc.take(&dy, n);
     sc.take(&A, (size_t)(n + 2) * n);
+    sc.take(&D, diag_doubles(n));
     sc.take(&dn, 1);
     sc.take(&st, 3);
     sc.take(&u, n);
@@ -565,7 +579,7 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
         set_error("kriging model buffers: %s", cudaGetErrorString(e));
         return fail(BPM_ERR_OOM);
     }
-    if ((r = gp_factor(s, g->X, dy, n, d, g->theta, 1, nugget, A, dfail, dn, st))) return fail(r);
+    if ((r = gp_factor(s, g->X, dy, n, d, g->theta, 1, nugget, A, D, dfail, dn, st))) return fail(r);
     double hst[3] = {0, 0, 0}, hn = 0;
     e = cudaMemcpyAsync(hst, st, sizeof(hst), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hn, dn, sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -583,7 +597,7 @@ extern "C" int bpm_gp_create(bpm_ctx* ctx, const double* X, const double* y, int
     g->one_Ri_1 = hst[2];
     const int nb = (n + 127) / 128;
     for (int i0 = 0; i0 < n; i0 += kPB)
-        k_gp_linv<<<(n + kPB - 1) / kPB, kGpThreads, 0, s>>>(A, n, i0, g->Linv);
+        k_gp_linv<<<(n + kPB - 1) / kPB, kGpThreads, 0, s>>>(A, D, n, i0, g->Linv);
     k_gp_rows<<<nb, 128, 0, s>>>(g->Linv, dy, g->mu, n, u, g->c);
     k_gp_cols<<<nb, 128, 0, s>>>(g->Linv, u, n, g->a);
     e = cudaGetLastError();

@@ -141,3 +141,60 @@ def test_one_kernel_forward_matches_the_layers(ctx, shape):
         loss = -np.mean(y * np.log(p) + (1 - y) * np.log1p(-p))
         assert abs(sur.grad(x, y)[1] - loss) <= 1e-5 * max(1.0, loss)
     sur.destroy()
+
+
+@pytest.mark.parametrize("n", [31, 32, 33, 62, 63, 64, 65, 160, 240])
+def test_blocked_kriging_factors(ctx, n):
+    """Design counts around the factorisation's 32-column blocks (one CTA to seven below a block; the rows of y and 1
+    in the last block, in one of their own or on both sides of an edge): likelihoods, the fit and the predictor against
+    the FP64 oracle.  Condition numbers up to 1.4e6, so the bars of well-conditioned models hold: 1e-9 for likelihood,
+    mean and variance, 1e-8 of the data scale for predictions."""
+    from oracle import ego as oego
+    from paper_1603_09493_gb300 import ego, synth
+    X = synth.unit_points(n, 4, 12, 0)
+    y = np.sin(3.0 * X).sum(1)
+    th = 10.0 ** (0.5 + 1.5 * synth.theta_unit_draws(24, 4, 12, 0))
+    got = ego.nll(ctx, X, y, th)
+    assert np.allclose(got, [oego.nll(X, y, t) for t in th], rtol=1e-9, atol=1e-9)
+    gp = oego.fit(X, y, th[0])
+    C = synth.unit_points(333, 4, 9, 1)
+    ry, rs, rei = oego.predict(gp, C, float(y.min()))
+    with ego.Kriging(ctx, X, y, th[0]) as k:
+        assert abs(k.mu - gp["mu"]) <= 1e-9 * np.abs(y).max() and abs(k.sigma2 - gp["sigma2"]) <= 1e-9 * gp["sigma2"]
+        gy, gs, gei = k.predict(C, float(y.min()))
+    scale = np.abs(y).max()
+    assert max(np.abs(gy - ry).max(), np.abs(gs - rs).max(), np.abs(gei - rei).max()) <= 1e-8 * scale
+
+
+@pytest.mark.parametrize("n,T", [(240, 256), (160, 600), (512, 150)])
+def test_more_kriging_factors_than_the_gpu_holds(ctx, n, T):
+    """Batches whose panel launches have more CTAs than are resident at once (1792, 3000 and 2250; eight an SM), so
+    that CTAs of one matrix start after others of it have finished: every likelihood against the FP64 oracle, and
+    bitwise equal to that of the vector in a small batch and of a second call."""
+    from oracle import ego as oego
+    from paper_1603_09493_gb300 import ego, synth
+    X = synth.unit_points(n, 12, 12, 0)
+    y = np.sin(3.0 * X).sum(1)
+    th = 10.0 ** (0.5 + synth.theta_unit_draws(T, 12, 12, 0))
+    got = ego.nll(ctx, X, y, th)
+    assert np.array_equal(got, ego.nll(ctx, X, y, th))
+    assert np.array_equal(got, np.concatenate([ego.nll(ctx, X, y, th[q:q + 50]) for q in range(0, T, 50)]))
+    assert np.allclose(got, [oego.nll(X, y, t) for t in th], rtol=1e-9, atol=1e-9)
+
+
+def test_kriging_pivot_failing_in_a_later_block(ctx):
+    """A matrix whose first 70 pivots are those of the unit matrix and whose pivot 70 is 1 - e^2 (a negative
+    correlation parameter in a direction in which only two designs differ), between good ones: infinity for it alone,
+    as the oracle has it."""
+    from oracle import ego as oego
+    from paper_1603_09493_gb300 import ego
+    n = 100
+    X = np.zeros((n, 2))
+    X[:, 0] = np.arange(n) / n
+    X[70] = [X[45, 0], 1.0]
+    y = np.sin(7.0 * X[:, 0]) + X[:, 1]
+    th = np.array([[1e6, 1.0], [1e6, -1.0], [1e5, 0.5]])
+    got = ego.nll(ctx, X, y, th)
+    ref = [oego.nll(X, y, t) for t in th]
+    assert np.isinf(ref[1]) and np.isfinite(ref[0]) and np.isfinite(ref[2])
+    assert np.isinf(got[1]) and np.allclose(got[[0, 2]], [ref[0], ref[2]], rtol=1e-9, atol=1e-9)
