@@ -168,7 +168,7 @@ def test_blocked_kriging_factors(ctx, n):
 
 @pytest.mark.parametrize("n,T", [(240, 256), (160, 600), (512, 150)])
 def test_more_kriging_factors_than_the_gpu_holds(ctx, n, T):
-    """Batches whose panel launches have more CTAs than are resident at once (1792, 3000 and 2250; eight an SM), so
+    """Batches whose panel launches have more CTAs than are resident at once (1792, 3000 and 2400; eight an SM), so
     that CTAs of one matrix start after others of it have finished: every likelihood against the FP64 oracle, and
     bitwise equal to that of the vector in a small batch and of a second call."""
     from oracle import ego as oego
