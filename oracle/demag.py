@@ -140,18 +140,28 @@ def rhs_matrix(n: int, tets: np.ndarray, vol: np.ndarray, grads: np.ndarray) -> 
     return R
 
 
+def bodies(n: int, tets: np.ndarray) -> np.ndarray:
+    """Body (connected part of the mesh) of each node."""
+    from scipy.sparse import coo_matrix
+    from scipy.sparse.csgraph import connected_components
+    i, j = np.repeat(tets, 4, axis=1).ravel(), np.tile(tets, (1, 4)).ravel()
+    return connected_components(coo_matrix((np.ones(i.size), (i, j)), shape=(n, n)), directed=False)[1]
+
+
 def fredkin_koehler_matrix(xyz, tets, vol, grads, V, return_parts=False):
     """Dense N [3n][3n] with H = -N M (index c*n + i)."""
     from .fem import laplacian
     n = xyz.shape[0]
     K = laplacian(n, tets, vol, grads)
     R = rhs_matrix(n, tets, vol, grads)
-    # 1. Neumann problem with zero-mean gauge (Lagrange multiplier)
-    aug = np.zeros((n + 1, n + 1))
+    # 1. Neumann problem with zero-mean gauge on each body of the mesh (Lagrange multipliers)
+    body = bodies(n, tets)
+    q = int(body.max()) + 1
+    aug = np.zeros((n + q, n + q))
     aug[:n, :n] = K
-    aug[:n, n] = 1.0
-    aug[n, :n] = 1.0
-    rhs = np.zeros((n + 1, 3 * n))
+    aug[np.arange(n), n + body] = 1.0
+    aug[n + body, np.arange(n)] = 1.0
+    rhs = np.zeros((n + q, 3 * n))
     rhs[:n] = R
     u1 = np.linalg.solve(aug, rhs)[:n]
     # 2. boundary values of u2

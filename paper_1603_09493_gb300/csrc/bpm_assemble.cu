@@ -12,9 +12,10 @@
 //   H = -grad(u1 + u2) per tet, lumped to the nodes.
 // The map M -> H is formed as a matrix.  Its source div(M) and its gradient are
 // sparse, so the solves are done for the n nodal sources rather than for the
-// 3n magnetisation components: G = K^+ (Neumann), the harmonic extension E of
-// the boundary values (Dirichlet), Q = G + E (D + diag(..)) G_boundary, and
-// N = P Q R with the sparse R (source) and P (projected gradient).  Both solves
+// 3n magnetisation components: G = K^+ (Neumann; a null vector per body of the
+// mesh), the harmonic extension E of the boundary values (Dirichlet),
+// Q = G + E (D + diag(..)) G_boundary, and N = P Q R with the sparse R (source)
+// and P (projected gradient).  Both solves
 // run as Jacobi-preconditioned CG over row-major blocks of right-hand sides: a
 // CTA owns one or two columns and runs their iterations in shared memory, with
 // reductions in a fixed order so that results are bit-reproducible.
@@ -385,10 +386,16 @@ __global__ void k_apply_source(int n, Sliced A, const double* __restrict__ rv, c
     u[2 * (size_t)n] = s2;
 }
 
-// right-hand sides of the nodal sources of the Neumann problem: e_j - 1/n
-__global__ void k_unit_sources(int n, double* __restrict__ B) {
+// right-hand sides of the nodal sources of the Neumann problem: e_j less its mean over the body that holds
+// j (body: per node; ptr: first node of each body in an order by bodies).  The Laplacian has a null vector
+// per body of the mesh, so a source has to sum to zero over each; div M does, and its potential's constant
+// on a body drops out of u1 + u2.
+__global__ void k_unit_sources(int n, const int* __restrict__ body, const int* __restrict__ ptr,
+                               double* __restrict__ B) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
-    if (j < n) B[(size_t)i * n + j] = (i == j ? 1.0 : 0.0) - 1.0 / n;
+    if (j >= n) return;
+    const int p = body[i];
+    B[(size_t)i * n + j] = (i == j ? 1.0 : 0.0) - (body[j] == p ? 1.0 / (ptr[p + 1] - ptr[p]) : 0.0);
 }
 
 // right-hand sides -K_IB of the harmonic extension (interior rows; B zeroed before)
@@ -605,20 +612,23 @@ __global__ void k_max_ratio(int ncol, const double* __restrict__ rr, const doubl
     }
 }
 
-// subtract each column's mean: 32 columns a CTA, 8 warps over the rows, partial sums in a fixed order
-__global__ void __launch_bounds__(256) k_col_mean_sub(int n, int ncol, double* __restrict__ X) {
+// subtract each column's mean over a body's rows (rows of all bodies, by body): 32 columns of a body a CTA, 8
+// warps over the rows, partial sums in a fixed order
+__global__ void __launch_bounds__(256) k_col_mean_sub(const int* __restrict__ rows, const int* __restrict__ ptr,
+                                                      int ncol, double* __restrict__ X) {
     __shared__ double part[8][32];
     const int l = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + l;
+    const int lo = ptr[blockIdx.y], hi = ptr[blockIdx.y + 1];
     double s = 0;
     if (c < ncol)
-        for (int i = w; i < n; i += 8) s += X[(size_t)i * ncol + c];
+        for (int i = lo + w; i < hi; i += 8) s += X[(size_t)rows[i] * ncol + c];
     part[w][l] = s;
     __syncthreads();
     s = 0;
     for (int k = 0; k < 8; ++k) s += part[k][l];
-    s /= n;
+    s /= hi - lo;
     if (c < ncol)
-        for (int i = w; i < n; i += 8) X[(size_t)i * ncol + c] -= s;
+        for (int i = lo + w; i < hi; i += 8) X[(size_t)rows[i] * ncol + c] -= s;
 }
 
 template <int C>
@@ -1013,6 +1023,25 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
         }
     }
     const int nnz = (int)col.size();
+    // bodies of the mesh (connected parts of the node graph), in the order of their first nodes: body of
+    // each node, nodes by body (ascending), first of each body
+    std::vector<int> body(n, -1), by_body, body_ptr(1, 0);
+    by_body.reserve(n);
+    for (int i = 0; i < n; ++i) {
+        if (body[i] >= 0) continue;
+        const int p = (int)body_ptr.size() - 1;
+        body[i] = p;
+        by_body.push_back(i);
+        for (size_t q = body_ptr[p]; q < by_body.size(); ++q)
+            for (int e = rowptr[by_body[q]]; e < rowptr[by_body[q] + 1]; ++e)
+                if (body[col[e]] < 0) {
+                    body[col[e]] = p;
+                    by_body.push_back(col[e]);
+                }
+        std::sort(by_body.begin() + body_ptr[p], by_body.end());
+        body_ptr.push_back((int)by_body.size());
+    }
+    const int n_bodies = (int)body_ptr.size() - 1;
     // boundary faces: faces of exactly one tet, oriented outward
     struct Face {
         uint64_t key;                      // sorted corners, 21 bits each
@@ -1191,13 +1220,17 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
     BPM_CK(cudaGetLastError());
     int it1 = 0, it2 = 0;
     double res1 = 0, res2 = 0;
-    // G = K^+ for the nodal sources, zero-mean gauge
+    // G = K^+ for the nodal sources, zero-mean gauge on each body
+    int *d_body, *d_by_body, *d_body_ptr;
+    BPM_TRY(upload(pool, &d_body, body));
+    BPM_TRY(upload(pool, &d_by_body, by_body));
+    BPM_TRY(upload(pool, &d_body_ptr, body_ptr));
     double *d_b, *d_G;
     BPM_TRY(pool.alloc(&d_b, NN, false));
     BPM_TRY(pool.alloc(&d_G, NN, false));
-    k_unit_sources<<<dim3((n + 127) / 128, n), 128, 0, st>>>(n, d_b);
+    k_unit_sources<<<dim3((n + 127) / 128, n), 128, 0, st>>>(n, d_body, d_body_ptr, d_b);
     BPM_TRY(pcg(st, pool, n, n, A, d_sval, d_sc, d_b, d_G, 1e-12, 20000, &it1, &res1));
-    k_col_mean_sub<<<(n + 31) / 32, 256, 0, st>>>(n, n, d_G);
+    k_col_mean_sub<<<dim3((n + 31) / 32, n_bodies), 256, 0, st>>>(d_by_body, d_body_ptr, n, d_G);
     // boundary values of u2 from u1
     double *d_omega, *d_Bmat;
     BPM_TRY(pool.alloc(&d_omega, nb, false));

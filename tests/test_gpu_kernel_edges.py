@@ -198,3 +198,31 @@ def test_kriging_pivot_failing_in_a_later_block(ctx):
     ref = [oego.nll(X, y, t) for t in th]
     assert np.isinf(ref[1]) and np.isfinite(ref[0]) and np.isfinite(ref[2])
     assert np.isinf(got[1]) and np.allclose(got[[0, 2]], [ref[0], ref[2]], rtol=1e-9, atol=1e-9)
+
+
+@pytest.mark.parametrize("parts", [2, 3])
+def test_operators_of_meshes_of_several_bodies(ctx, parts):
+    """A hard and a soft prism across a gap and, with three, a single tetrahedron beside them, nodes numbered
+    alternately over the bodies: the Laplacian has a null vector per body, so the nodal sources of the Neumann
+    problem have to sum to zero over each.  FP64 demag matrix against the oracle's, as for one body."""
+    from oracle import fem
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    a = synth.layered_island_mesh(8.0, 5.0, 3.0, rings=2, hard_slabs=3, soft_slabs=2, seed=1)
+    b = synth.layered_island_mesh(9.0, 4.0, 4.0, rings=1, hard_slabs=2, soft_slabs=2, seed=2)
+    xyz, tets, reg = [a.xyz_nm, b.xyz_nm + [0.0, 0.0, 9.0]], [a.tets, b.tets + a.n_nodes], [a.tet_region, b.tet_region]
+    if parts == 3:
+        tets.append(np.arange(4).reshape(1, 4) + a.n_nodes + b.n_nodes)
+        xyz.append(np.array([[14.0, 0, 0], [16.0, 0, 0], [14.0, 2.0, 0], [14.0, 0, 2.0]]))
+        reg.append(np.zeros(1, reg[0].dtype))
+    xyz, tets, reg = np.concatenate(xyz), np.concatenate(tets), np.concatenate(reg)
+    new = np.random.default_rng(parts).permutation(len(xyz))              # node i gets number new[i]
+    mesh = synth.IslandMesh(xyz[np.argsort(new)], new[tets].astype(np.int32), reg.astype(np.int32), 5.0, 17.0)
+    mats = synth.ecc_materials()
+    ops = fem.MeshOperators(mesh.xyz_nm, mesh.tets, mesh.tet_region, mats)
+    mid = ctx.mesh_upload(mesh, mats, keep_f64=True)
+    info = ctx.mesh_info(mid)
+    assert info["cg_residual_neumann"] < 1e-12 and info["cg_residual_dirichlet"] < 1e-12
+    N = ctx.get_operator(mid, L.OP_DEMAG_F64)
+    assert np.abs(N - ops.demag).max() <= 1e-9 * np.abs(ops.demag).max()
+    ctx.mesh_release(mid)

@@ -207,3 +207,24 @@ def test_demag_energy_positive(small_parts):
     for _ in range(20):
         M = rng.standard_normal(3 * ops.n)
         assert M @ (W * (N @ M)) > 0
+
+
+def test_mesh_of_two_bodies():
+    """A prism and a larger one 30 nm beside it in one mesh: the block of a body is its own demag matrix (the other
+    one's surface charges enclose no source of it), and its mean far field is that of a point dipole, within the
+    quadrupole's order (half-extent 5 nm over 30 nm, squared)."""
+    a = synth.layered_island_mesh(8.0, 5.0, 3.0, rings=1, hard_slabs=2, soft_slabs=1, seed=1)
+    b = synth.layered_island_mesh(9.0, 4.0, 4.0, rings=2, hard_slabs=2, soft_slabs=2, seed=2)
+    mats, n = synth.ecc_materials(), a.n_nodes
+    shift = np.array([30.0, 0.0, 0.0])
+    both = fem.MeshOperators(np.concatenate([a.xyz_nm, b.xyz_nm + shift]), np.concatenate([a.tets, b.tets + n]),
+                             np.concatenate([a.tet_region, b.tet_region]), mats)
+    assert len(np.unique(demag.bodies(both.n, np.concatenate([a.tets, b.tets + n])))) == 2
+    N = both.demag.reshape(3, both.n, 3, both.n)
+    for sl, m in ((slice(0, n), a), (slice(n, None), b)):
+        own = fem.MeshOperators(m.xyz_nm, m.tets, m.tet_region, mats).demag.reshape(3, m.n_nodes, 3, m.n_nodes)
+        assert np.abs(N[:, sl, :, sl] - own).max() <= 1e-10 * np.abs(own).max()
+    # H_z in b of a magnetised along z: -V_a M / (4 pi r^3)
+    Va = both.V[:n].sum()
+    H = -(N[2, n:, 2, :n].sum(1) @ both.V[n:]) / both.V[n:].sum()
+    assert abs(H / (-Va / (4 * math.pi * 30.0 ** 3)) - 1.0) <= 3 * (5.0 / 30.0) ** 2
