@@ -1073,6 +1073,10 @@ int assemble_mesh(bpm_ctx* ctx, Mesh* M, const double* xyz, const int32_t* tets_
         faces.push_back(c);
     }
     const int nf = (int)faces.size() / 3;
+    if (nf == 0) {
+        set_error("the mesh has no boundary face: every face belongs to two or more tetrahedra");
+        return BPM_ERR_ARG;
+    }
     std::vector<int> bnodes(faces.begin(), faces.end());
     std::sort(bnodes.begin(), bnodes.end());
     bnodes.erase(std::unique(bnodes.begin(), bnodes.end()), bnodes.end());

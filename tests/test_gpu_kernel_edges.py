@@ -226,3 +226,14 @@ def test_operators_of_meshes_of_several_bodies(ctx, parts):
     N = ctx.get_operator(mid, L.OP_DEMAG_F64)
     assert np.abs(N - ops.demag).max() <= 1e-9 * np.abs(ops.demag).max()
     ctx.mesh_release(mid)
+
+
+def test_mesh_without_a_boundary_is_refused(ctx):
+    """Two tetrahedra on the same four nodes: every face belongs to both, none is on the boundary.  An error from the
+    library's own check of the faces, before the row count of the boundary's weights divides by their number."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    mesh = synth.IslandMesh(np.array([[0.0, 0, 0], [2, 0, 0], [0, 2, 0], [0, 0, 2]]),
+                            np.array([[0, 1, 2, 3], [1, 2, 0, 3]], np.int32), np.zeros(2, np.int32), 1.0, 2.0)
+    with pytest.raises(L.BpmError, match="boundary"):
+        ctx.mesh_upload(mesh, synth.ecc_materials())
