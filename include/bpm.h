@@ -289,7 +289,10 @@ int bpm_stable_substeps(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bp
  * and updates the switch detector.  Magnetisation arrays passed to the batch
  * calls use a leading dimension ld >= the largest mesh's n_nodes; entries past
  * an island's own n_nodes are not read and are left untouched (reads of host
- * arrays leave them zero).
+ * arrays leave them zero).  An island's states have the same bits whatever other
+ * islands share its batch and whatever bpm_batch_set_tuning chooses, on one kind
+ * of GPU and at one number of steps (<m_z> and the crossing time, sums over the
+ * nodes, to rounding).
  * Errors: BPM_ERR_ARG (B < 1, unknown mesh or map id, substeps < 0). */
 int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B,
                      const bpm_run_params* p, bpm_batch** out);

@@ -138,7 +138,7 @@ using namespace bpm;
 struct Group {
     Mesh* mesh = nullptr;
     int B = 0, Bp = 0;
-    int splits = 1;               // planes of Hd: slices of the tensor-core demag product's K
+    int slices = 1, planes = 1;   // of the tensor-core demag product: slices of K, planes of Hd
     std::vector<int> user_idx;    // batch island index of each group row
     int* d_idx = nullptr;
     float4* isl = nullptr;
@@ -213,9 +213,9 @@ int setup_grouped_gemm(bpm_batch* bt) {
     std::vector<GemmOperands> ops;
     for (auto& g : bt->groups) {
         const int K = g.mesh->K();
-        ops.push_back(GemmOperands{g.Ahi, g.Alo, g.mesh->Nhi, g.mesh->Nlo, g.Hd, g.B, g.Bp, K, K, g.splits,
-                                   (size_t)g.Bp * K});
-        g.args.hd_planes = bt->pair ? 1 : g.splits;   // the CTA-pair kernel does not slice K
+        ops.push_back(GemmOperands{g.Ahi, g.Alo, g.mesh->Nhi, g.mesh->Nlo, g.Hd, g.B, g.Bp, K, K, g.slices,
+                                   g.planes, (size_t)g.Bp * K});
+        g.args.hd_planes = bt->pair ? 1 : g.planes;   // the CTA-pair kernel adds the slices itself
         g.args.hd_plane = (size_t)g.Bp * K;
     }
     return grouped_gemm_setup(&bt->gg, ops, bt->tile_n, bt->p.precision == BPM_PREC_BF16X3 ? 3 : 1, bt->raster,
@@ -308,8 +308,8 @@ int setup_chains(bpm_batch* bt) {
             for (int i : bt->chain_groups[c]) {
                 const Group& q = bt->groups[i];
                 const int K = q.mesh->K();
-                ops.push_back(GemmOperands{q.Ahi, q.Alo, q.mesh->Nhi, q.mesh->Nlo, q.Hd, q.B, q.Bp, K, K, q.splits,
-                                           (size_t)q.Bp * K});
+                ops.push_back(GemmOperands{q.Ahi, q.Alo, q.mesh->Nhi, q.mesh->Nlo, q.Hd, q.B, q.Bp, K, K, q.slices,
+                                           q.planes, (size_t)q.Bp * K});
             }
             BPM_TRY(grouped_gemm_setup(&bt->gg_chain[c], ops, bt->tile_n, products, bt->raster, bt->k_block,
                                        bt->ctx->sm_count, bt->pair, chains));
@@ -324,7 +324,7 @@ int setup_chains(bpm_batch* bt) {
         const int rows = c + 1 < chains ? chunk : g.Bp - b0;
         const size_t off = (size_t)b0 * K, S = (size_t)b0 * 3 * g.mesh->n_pad;
         std::vector<GemmOperands> ops{GemmOperands{g.Ahi + off, g.Alo + off, g.mesh->Nhi, g.mesh->Nlo, g.Hd + off,
-                                                   std::min(chunk, g.B - b0), rows, K, K, g.splits, 0}};
+                                                   std::min(chunk, g.B - b0), rows, K, K, g.slices, 1, 0}};
         BPM_TRY(grouped_gemm_setup(&bt->gg_chain[c], ops, bt->tile_n, products, bt->raster, bt->k_block,
                                    bt->ctx->sm_count, bt->pair, chains));
         StepArgs a = g.args;
@@ -572,7 +572,7 @@ size_t carve(bpm_batch* bt, Arena& A) {
         const size_t S = (size_t)g.Bp * g.mesh->K();
         A.take(&g.m, (size_t)g.Bp * 3 * g.mesh->n_pad);
         A.take(&g.k1, (size_t)g.Bp * 3 * g.mesh->n_pad);
-        A.take(&g.Hd, g.splits * S);
+        A.take(&g.Hd, g.planes * S);
         if (bt->p.precision == BPM_PREC_FP32) {
             A.take(&g.A32, S);
         } else {
@@ -981,7 +981,10 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
         g.B = (int)g.user_idx.size();
         g.Bp = round_up(g.B, kIslandPad);
         bt->n_max = std::max(bt->n_max, g.mesh->n);
-        if (tensor_core_precision(bt)) g.splits = gemm_splits(g.B, g.mesh->K(), ctx->sm_count);
+        if (tensor_core_precision(bt)) {
+            g.slices = gemm_slices(g.mesh->K(), ctx->sm_count);
+            g.planes = gemm_planes(g.B, g.slices);
+        }
     }
     Arena size{nullptr};
     const size_t tables = carve(bt, size);

@@ -11,12 +11,18 @@
 // design variants of 135 islands 35.1 ms an interval, 30.2 so).  A tile's accumulator holds operator rows in lanes, so a warp
 // stores 128 contiguous bytes of an island's field per instruction.
 //
-// A group of at most 128 islands has only N_g / 128 tiles, each a serial walk over
-// K.  Its K is cut into up to four slices (gemm_splits), each an item of its own
-// writing its own plane of C; the stage kernels add the planes in order.  The
-// slices depend on K alone, not on what else is in the batch.  One island of 209
-// nodes: 374 -> 172 us an interval of 6 steps; nine of 481 nodes: 689 -> 330 us of
-// 8 steps; 60 of 1547 nodes: 5.2 -> 2.7 ms of 28 steps.
+// K is cut into up to four slices (gemm_slices), from K alone, and an element is the
+// sum of its slices in order, so that an island's field has the same bits in every
+// batch, whatever else is in it and whichever kernel forms it.  A group of at most
+// 128 islands has only N_g / 128 tiles, each a serial walk over K: there a slice is
+// an item of its own writing its own plane of C, and the stage kernels add the
+// planes (one island of 209 nodes: 374 -> 172 us an interval of 6 steps; nine of 481
+// nodes: 689 -> 330 us of 8 steps; 60 of 1547 nodes: 5.2 -> 2.7 ms of 28 steps).
+// Otherwise an item is a tile's whole K: the slices go to the two accumulators in
+// turn, and the epilogue adds them in registers (eight warps of 128 sums a thread, no
+// store before the accumulator is free again; against four warps that stored as they
+// read, one sum of all of K: an interval of 4096 islands of 1547 nodes 24.3 -> 23.9 ms,
+// of 600 of 481 nodes 606 -> 556 us).
 //
 // The items of all groups are dealt to the CTAs (one per SM) when the GEMM is set
 // up: an item costs its K, so each goes, longest first, to the CTA with the least
@@ -28,10 +34,11 @@
 // is read from HBM once.  Warp roles:
 //   warp 0  one lane streams the k-blocks of every item with TMA into a ring of
 //           shared-memory stages (the ring runs across item boundaries);
-//   warp 1  allocates two TMEM accumulators; one lane issues the MMAs, item i
-//           into accumulator i % 2;
-//   warps 2-5  read an accumulator back (tcgen05.ld) and store it, while the
-//           MMAs of the next item run into the other accumulator.
+//   warp 1  allocates two TMEM accumulators; one lane issues the MMAs, slice i of
+//           the CTA's items into accumulator i % 2;
+//   warps 2-9  read an accumulator back (tcgen05.ld; a warp 32 operator rows by half of
+//           the tile's islands), add an item's slices and store them, while the MMAs
+//           of the next slice run into the other accumulator.
 // Per-group tensor maps live in a device array (64-byte aligned entries).
 // Every wait is bounded; on timeout the kernel raises the error flag, drains
 // its copies and MMAs, frees TMEM and exits, and later launches return at once.
@@ -51,7 +58,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kGThreads = 192;
+constexpr int kGThreads = 320, kGEpiWarps = 8;
 
 // KB: K depth of a stage (64: 128 B rows, 128-byte swizzle; 32: 64 B rows, 64-byte swizzle)
 // TN: islands per tile at most
@@ -76,7 +83,7 @@ __device__ __forceinline__ int find_group(const GemmGroupDev* __restrict__ G, in
     return g;
 }
 
-// item it of group gg -> first island, first operator row, k-slice
+// item it of group gg -> first island, first operator row, slice of K that it begins with (0 if it has all)
 __device__ __forceinline__ void item_origin(const GemmGroupDev& gg, int it, int& b0, int& r0, int& slice) {
     slice = it % gg.splits;
     const int lt = it / gg.splits;
@@ -131,7 +138,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(accf_bar(a), 1);
-            mbar_init(acce_bar(a), 4);     // one arrival per epilogue warp
+            mbar_init(acce_bar(a), kGEpiWarps);     // one arrival per epilogue warp
         }
         mbar_init(done_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -157,7 +164,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
             item_origin(gg, t - gg.tile_begin, b0, r0, sl);
-            const int kb1 = min(gg.K, (sl + 1) * gg.slice_k) / KB;
+            const int kb1 = min(gg.K, (sl + gg.segs) * gg.slice_k) / KB;
             const uint32_t bytes = (P == 3 ? 2u : 1u) * (uint32_t)(W_TILE + gg.nb * KB * 2);
             int kb = sl * gg.slice_k / KB;
             auto load_w = [&](int s, int kc) {
@@ -194,73 +201,80 @@ __global__ void __launch_bounds__(kGThreads, 1)
         // ---------------- MMA issuer ----------------
         int kbg = 0, i = 0;
         bool ok = true;
-        for (int qi = q0; qi < q1 && ok; ++qi, ++i) {
+        for (int qi = q0; qi < q1 && ok; ++qi) {
             const int t = items[qi];
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
             item_origin(gg, t - gg.tile_begin, b0, r0, sl);
-            const int kb0 = sl * gg.slice_k / KB, kb1 = min(gg.K, (sl + 1) * gg.slice_k) / KB;
             const uint32_t idesc = idesc_n<TN>(gg.nb);
-            const int a = i & 1;
-            if (i >= 2) ok = mbar_wait(acce_bar(a), ((i >> 1) - 1) & 1, err, 13, true, wait_ns);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t acc = tmem + (uint32_t)(a * TN);
-            for (int kb = kb0; kb < kb1; ++kb, ++kbg) {
-                const int s = kbg % S;
-                ok = mbar_wait(full_bar(s), (kbg / S) & 1, err, 14, true, wait_ns);
+            for (int u = sl; u < sl + gg.segs && ok; ++u, ++i) {
+                const int kb0 = u * gg.slice_k / KB, kb1 = min(gg.K, (u + 1) * gg.slice_k) / KB;
+                const int a = i & 1;
+                if (i >= 2) ok = mbar_wait(acce_bar(a), ((i >> 1) - 1) & 1, err, 13, true, wait_ns);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t acc = tmem + (uint32_t)(a * TN);
+                for (int kb = kb0; kb < kb1; ++kb, ++kbg) {
+                    const int s = kbg % S;
+                    ok = mbar_wait(full_bar(s), (kbg / S) & 1, err, 14, true, wait_ns);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int k = 0; k < KB / 16; ++k) {
-                    const uint32_t koff = 32u * k;    // 16 BF16 further along the swizzled row
-                    const uint64_t ahi = kmajor_desc<KB>(sAhi(s) + koff), whi = kmajor_desc<KB>(sWhi(s) + koff);
-                    mma_bf16_desc(acc, whi, ahi, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                    if (P == 3) {
-                        const uint64_t alo = kmajor_desc<KB>(sAlo(s) + koff), wlo = kmajor_desc<KB>(sWlo(s) + koff);
-                        mma_bf16_desc(acc, whi, alo, idesc, 1u);
-                        mma_bf16_desc(acc, wlo, ahi, idesc, 1u);
+                    for (int k = 0; k < KB / 16; ++k) {
+                        const uint32_t koff = 32u * k;    // 16 BF16 further along the swizzled row
+                        const uint64_t ahi = kmajor_desc<KB>(sAhi(s) + koff), whi = kmajor_desc<KB>(sWhi(s) + koff);
+                        mma_bf16_desc(acc, whi, ahi, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                        if (P == 3) {
+                            const uint64_t alo = kmajor_desc<KB>(sAlo(s) + koff), wlo = kmajor_desc<KB>(sWlo(s) + koff);
+                            mma_bf16_desc(acc, whi, alo, idesc, 1u);
+                            mma_bf16_desc(acc, wlo, ahi, idesc, 1u);
+                        }
                     }
+                    mma_commit(empty_bar(s));
                 }
-                mma_commit(empty_bar(s));
+                if (ok) mma_commit(accf_bar(a));
             }
-            if (ok) mma_commit(accf_bar(a));
         }
         mma_commit(done_bar);      // tracks every MMA issued above, also on the error path
     } else if (warp >= 2) {
         // ---------------- epilogue warps ----------------
         const int q = warp & 3;    // TMEM lane quarter this warp may access
+        const int h0 = (warp - 2) / 4 * (TN / 2);          // its islands of the tile: h0 .. h0 + TN / 2
+        constexpr int NC = TN / 32;                        // in pieces of 16
         pdl_wait();                // C may still be read by the kernel before
         int i = 0;
-        for (int qi = q0; qi < q1; ++qi, ++i) {
+        bool go = true;
+        for (int qi = q0; qi < q1 && go; ++qi) {
             const int t = items[qi];
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int b0, r0, sl;
             item_origin(gg, t - gg.tile_begin, b0, r0, sl);
-            const int a = i & 1;
-            const bool have = mbar_wait(accf_bar(a), (i >> 1) & 1, err, 15, true, wait_ns);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int go = __shfl_sync(0xffffffffu, (have && *(volatile int*)err == 0) ? 1 : 0, 0);
-            if (!go) break;
             const int row = r0 + q * 32 + lane;             // operator row = column of C
-            const int nv = min(gg.nb, gg.M - b0);           // islands of this tile
-            float* dst = gg.C + (size_t)sl * gg.plane + (size_t)b0 * gg.ldc + row;
-            const uint32_t lane_addr = tmem + (uint32_t)(a * TN) + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-            for (int c = 0; c < nv; c += 32, dst += 32 * (size_t)gg.ldc) {   // (a last 32 may read past nb: unused)
-                uint32_t r[32];
-                tmem_ld32(lane_addr + (uint32_t)c, r);
-                if (row < gg.N) {
+            const int nv = min(gg.nb, gg.M - b0) - h0;      // islands of this tile from h0 on
+            float sum[NC][16];
+            for (int u = 0; u < gg.segs; ++u, ++i) {
+                const int a = i & 1;
+                const bool have = mbar_wait(accf_bar(a), (i >> 1) & 1, err, 15, true, wait_ns);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                go = __shfl_sync(0xffffffffu, (have && *(volatile int*)err == 0) ? 1 : 0, 0) != 0;
+                if (!go) break;
+                const uint32_t lane_addr = tmem + (uint32_t)(a * TN + h0) + ((uint32_t)(q * 32) << 16);
 #pragma unroll
-                    for (int v = 0; v < 32; ++v)
-                        if (c + v < nv) dst[(size_t)v * gg.ldc] = __uint_as_float(r[v]);
-                }
+                for (int c = 0; c < NC; ++c)
+                    if (16 * c < nv) tmem_sum16(lane_addr + 16u * c, u > 0, sum[c]);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acce_bar(a));
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acce_bar(a));
+            if (!go || row >= gg.N) continue;
+            float* dst = gg.C + (size_t)sl * gg.plane + (size_t)(b0 + h0) * gg.ldc + row;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int v = 0; v < 16; ++v)
+                    if (16 * c + v < nv) dst[(size_t)(16 * c + v) * gg.ldc] = sum[c][v];
         }
     }
     __syncwarp();
@@ -290,8 +304,7 @@ int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err
 
 }  // namespace
 
-int gemm_splits(int islands, int K, int sm_count) {
-    if (islands > 128) return 1;
+int gemm_slices(int K, int sm_count) {
     const int tiles = (K + tc::TM - 1) / tc::TM, kb = K / tc::TK;
     // slices of at least three k-blocks, at most four (the consumers read every plane), no more items than SMs
     const int want = std::max(1, std::min({4, sm_count / tiles, (kb + 2) / 3}));
@@ -332,8 +345,8 @@ int tile_cap(const std::vector<GemmOperands>& ops, int tile_n, int sm_count, int
         double sum = 0, top = 0, rows = 0;
         for (const GemmOperands& o : ops) {
             const int nb = even_tile(o.M, cap);
-            const long long it = (long long)((o.M + nb - 1) / nb) * ((o.N + tc::TM - 1) / tc::TM) * o.splits;
-            const double steps = o.K / 16.0 / o.splits + 12.0, c = mma_cost(nb) * steps;
+            const long long it = (long long)((o.M + nb - 1) / nb) * ((o.N + tc::TM - 1) / tc::TM) * o.planes;
+            const double steps = o.K / 16.0 / o.planes + 12.0, c = mma_cost(nb) * steps;
             items += it;
             sum += it * c;
             rows += it * steps * (128 + nb) / 1.5;          // in the MMA's units at 256 islands
@@ -362,7 +375,7 @@ std::vector<int> deal_items(const std::vector<GemmGroupDev>& h, int items, int g
     list.reserve(items);
     for (const GemmGroupDev& g : h)
         for (int k = 0; k < g.tiles_m * g.tiles_n * g.splits; ++k) {
-            const int lo = (k % g.splits) * g.slice_k, hi = std::min(g.K, lo + g.slice_k);
+            const int lo = (k % g.splits) * g.slice_k, hi = std::min(g.K, lo + g.segs * g.slice_k);
             list.push_back(Item{mma_cost(g.nb) * ((hi - lo) / 16.0 + 12.0), g.tile_begin + k});
         }
     std::stable_sort(list.begin(), list.end(), [](const Item& x, const Item& y) { return x.cost > y.cost; });
@@ -413,7 +426,8 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
     if (!pair && nb_max <= 128) k_block = 64;
     for (size_t g = 0; g < ops.size(); ++g) {
         const GemmOperands& o = ops[g];
-        if (o.rows % tc::TM || o.K % tc::TK || o.N % 16 || o.M <= 0 || o.M > o.rows || o.N <= 0 || o.splits < 1) {
+        if (o.rows % tc::TM || o.K % tc::TK || o.N % 16 || o.M <= 0 || o.M > o.rows || o.N <= 0 || o.slices < 1 ||
+            (o.planes != 1 && o.planes != o.slices)) {
             set_error("grouped GEMM group %zu: rows %% 128, K %% 64, N %% 16 required (M=%d rows=%d N=%d K=%d)", g,
                       o.M, o.rows, o.N, o.K);
             return BPM_ERR_ARG;
@@ -437,8 +451,9 @@ int grouped_gemm_setup(GroupedGemm* gg, const std::vector<GemmOperands>& ops, in
         h[g].K = o.K;
         h[g].ldc = o.N;
         h[g].nb = nb;
-        h[g].splits = pair ? 1 : o.splits;
-        h[g].slice_k = (o.K / tc::TK + h[g].splits - 1) / h[g].splits * tc::TK;
+        h[g].splits = pair ? 1 : o.planes;
+        h[g].segs = o.slices / h[g].splits;
+        h[g].slice_k = (o.K / tc::TK + o.slices - 1) / o.slices * tc::TK;
         h[g].plane = o.plane;
         h[g].tiles_m = pair ? (o.rows + 2 * tc::TM - 1) / (2 * tc::TM) : (o.M + nb - 1) / nb;
         h[g].tiles_n = (o.N + (pair ? 2 : 1) * tc::TM - 1) / ((pair ? 2 : 1) * tc::TM);

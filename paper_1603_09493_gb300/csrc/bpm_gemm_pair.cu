@@ -16,12 +16,13 @@
 //           barrier (so each CTA waits for its own copies alone before it gives
 //           up its shared memory);
 //   warp 1  allocates TMEM with the peer (two accumulators of 256 columns); in
-//           the even CTA one lane issues the MMAs, tile i into accumulator i % 2,
-//           and commits them to both CTAs' barriers; in the odd CTA one lane
+//           the even CTA one lane issues the MMAs, slice i of K (gemm_slices) over the
+//           pair's tiles into accumulator i % 2, and commits them to both CTAs' barriers; in the odd CTA one lane
 //           forwards every landed stage to a second barrier of the stage in the
 //           even CTA;
-//   warps 2-5  read the CTA's accumulator rows back and store them, then arrive
-//           on the even CTA's accumulator-empty barrier.
+//   warps 2-9  read the CTA's accumulator rows back (a warp 32 rows by half of the
+//           columns), arrive on the even CTA's accumulator-empty barrier, add a
+//           tile's slices in order and store them.
 // Every wait is bounded as in k_gemm_grouped; both CTAs of a pair take the same
 // abort decision before any collective step, and leave through one cluster
 // barrier after every MMA (drained in both CTAs) has completed.
@@ -35,7 +36,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPThreads = 192;
+constexpr int kPThreads = 320;
 constexpr int PTN = 256;      // output columns of a pair tile
 constexpr int PHALF = 128;    // rows of A and of W staged by each CTA
 
@@ -162,7 +163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(accf_bar(a), 1);
-            mbar_init(acce_bar(a), 8);     // one arrival per epilogue warp of both CTAs (even CTA only)
+            mbar_init(acce_bar(a), 16);    // one arrival per epilogue warp of both CTAs (even CTA only)
         }
         mbar_init(done_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -227,15 +228,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
         // ---------------- MMA issuer (even CTA) ----------------
         int kbg = 0, i = 0;
         bool ok = true;
-        for (int t = cluster; t < total_tiles && ok; t += n_clusters, ++i) {
+        for (int t = cluster; t < total_tiles && ok; t += n_clusters) {
             const GemmGroupDev& gg = G[find_group(G, ng, t)];
-            const int nk = gg.K / KB;
-            const int a = i & 1;
-            if (i >= 2) ok = mbar_wait(acce_bar(a), ((i >> 1) - 1) & 1, err, 24, true, wait_ns);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t acc = tmem + (uint32_t)(a * PTN);
-            for (int kb = 0; kb < nk; ++kb, ++kbg) {
+            const int nk = gg.K / KB, per = gg.slice_k / KB;
+            // a slice begins with a wait for its accumulator and ends with a commit to it
+            for (int kb = 0; kb < nk && ok; ++kb, ++kbg) {
+                const int a = i & 1;
+                const bool first = kb % per == 0;
+                if (first) {
+                    if (i >= 2) ok = mbar_wait(acce_bar(a), ((i >> 1) - 1) & 1, err, 24, true, wait_ns);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                const uint32_t acc = tmem + (uint32_t)(a * PTN);
                 const int s = kbg % S;
                 // the odd CTA's copies of the stage have landed when its forwarder arrives (it saw
                 // them complete on its own barrier first)
@@ -247,7 +252,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
                 for (int k = 0; k < KB / 16; ++k) {
                     const uint32_t koff = 32u * k;    // 16 BF16 further along the swizzled row
                     const uint64_t ahi = pair_desc<KB>(sAhi(s) + koff), whi = pair_desc<KB>(sWhi(s) + koff);
-                    mma_pair(acc, ahi, whi, (kb > 0 || k > 0) ? 1u : 0u);
+                    mma_pair(acc, ahi, whi, (!first || k > 0) ? 1u : 0u);
                     if (P == 3) {
                         const uint64_t alo = pair_desc<KB>(sAlo(s) + koff), wlo = pair_desc<KB>(sWlo(s) + koff);
                         mma_pair(acc, alo, whi, 1u);
@@ -255,44 +260,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
                     }
                 }
                 commit_pair(empty_bar(s));
+                if ((kb + 1) % per == 0 || kb + 1 == nk) {
+                    commit_pair(accf_bar(a));
+                    ++i;
+                }
             }
-            if (ok) commit_pair(accf_bar(a));
         }
         commit_pair(done_bar);     // tracks every MMA issued above, also on the error path
     } else if (warp >= 2) {
         // ---------------- epilogue warps: this CTA's 128 rows of each tile ----------------
         const int q = warp & 3;    // TMEM lane quarter this warp may access
+        const int h0 = (warp - 2) / 4 * (PTN / 2);         // its columns of the tile: h0 .. h0 + 127
+        constexpr int NC = PTN / 32;                       // in pieces of 16
         const uint32_t acce_even[2] = {map_to(acce_bar(0), 0), map_to(acce_bar(1), 0)};
         int i = 0;
-        for (int t = cluster; t < total_tiles; t += n_clusters, ++i) {
+        bool go = true;
+        for (int t = cluster; t < total_tiles && go; t += n_clusters) {
             const int g = find_group(G, ng, t);
             const GemmGroupDev& gg = G[g];
             int m0, n0;
             pair_origin(gg, t - gg.tile_begin, m0, n0);
-            const int a = i & 1;
-            const bool have = mbar_wait(accf_bar(a), (i >> 1) & 1, err, 26, true, wait_ns);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int go = __shfl_sync(0xffffffffu, (have && *(volatile int*)err == 0) ? 1 : 0, 0);
-            if (!go) break;
-            const int row = m0 + PHALF * (int)rank + q * 32 + lane;
-            const uint32_t lane_addr = tmem + (uint32_t)(a * PTN) + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-            for (int c = 0; c < PTN && n0 + c < gg.N; c += 32) {   // columns past N were zero operands
-                uint32_t r[32];
-                tmem_ld32(lane_addr + (uint32_t)c, r);
-                const int col = n0 + c;
-                if (row < gg.M) {
-                    float4* dst = reinterpret_cast<float4*>(gg.C + (size_t)row * gg.ldc + col);
+            const int row = m0 + PHALF * (int)rank + q * 32 + lane, col0 = n0 + h0;
+            float sum[NC][16];
+            for (int u = 0; u < gg.segs; ++u, ++i) {
+                const int a = i & 1;
+                const bool have = mbar_wait(accf_bar(a), (i >> 1) & 1, err, 26, true, wait_ns);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                go = __shfl_sync(0xffffffffu, (have && *(volatile int*)err == 0) ? 1 : 0, 0) != 0;
+                if (!go) break;
+                const uint32_t lane_addr = tmem + (uint32_t)(a * PTN + h0) + ((uint32_t)(q * 32) << 16);
 #pragma unroll
-                    for (int v = 0; v < 8; ++v)
-                        if (col + 4 * v < gg.N)
-                            dst[v] = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
-                                                 __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
-                }
+                for (int c = 0; c < NC; ++c)
+                    if (col0 + 16 * c < gg.N) tmem_sum16(lane_addr + 16u * c, u > 0, sum[c]);   // (zero operands past N)
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) remote_arrive(acce_even[a]);
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) remote_arrive(acce_even[a]);
+            if (!go || row >= gg.M) continue;
+            float4* dst = reinterpret_cast<float4*>(gg.C + (size_t)row * gg.ldc + col0);
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (col0 + 16 * c < gg.N)                  // N % 16 == 0
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        dst[4 * c + v] = make_float4(sum[c][4 * v], sum[c][4 * v + 1], sum[c][4 * v + 2],
+                                                     sum[c][4 * v + 3]);
         }
     }
     __syncwarp();

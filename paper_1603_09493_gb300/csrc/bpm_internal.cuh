@@ -222,19 +222,21 @@ struct GemmGroupDev {   // CUtensorMap members carry the 64-byte alignment TMA n
     int tile_begin;                   // first item of this group in the launch's list
     int n_major;                      // tile order: 1 = consecutive tiles share the W rows
     int nb;                           // islands (rows of A) per tile
-    int splits, slice_k;              // slices of K, columns per slice; slice s writes C + s * plane
+    int splits, segs, slice_k;        // items of a tile (item s writes C + s * plane), slices of K each, columns a slice
     size_t plane;
 };
 struct GemmOperands {
     const __nv_bfloat16 *Ahi, *Alo, *Whi, *Wlo;
     float* C;
     int M, rows, N, K;                // islands, rows of A (a multiple of 128, zeros from M on)
-    int splits;                       // planes of C (gemm_splits of the group)
+    int slices, planes;               // slices of K (gemm_slices), planes of C (gemm_planes)
     size_t plane;                     // elements of a plane
 };
-// Slices of K of a group's demag product, from its island count (more than 128: one) and K.  The result
-// of a group then depends on nothing else in its batch or launch.
-int gemm_splits(int islands, int K, int sm_count);
+// Slices of K of a demag product: an element is the sum of its slices in order, so that an island's field has the
+// same bits whatever else is in its batch or launch
+int gemm_slices(int K, int sm_count);
+// planes of C that hold the slices of a group: one each up to 128 islands, else one with their sum
+inline int gemm_planes(int islands, int slices) { return islands <= 128 ? slices : 1; }
 struct GroupedGemm {
     GemmGroupDev* d_groups = nullptr;
     int* d_sched = nullptr;           // the CTAs' items (in d_groups' allocation); grid: CTAs

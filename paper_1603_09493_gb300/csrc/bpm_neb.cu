@@ -76,7 +76,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     int* err = nullptr;
     const size_t S = (size_t)Rp * 3 * np, G = (size_t)Rp * K;
     const bool tc = prec == BPM_PREC_BF16X3 || prec == BPM_PREC_BF16;
-    const int splits = tc ? gemm_splits(R, K, ctx->sm_count) : 1;   // planes of Hd
+    const int slices = tc ? gemm_slices(K, ctx->sm_count) : 1, planes = gemm_planes(R, slices);   // planes of Hd
     buf.take(&err, 1);
     buf.take(&m0, S);
     buf.take(&m1, S);
@@ -87,7 +87,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
         buf.take(&Alo, G);
     }
     const size_t zeroed = buf.size;              // pads of the states and the operand stay zero
-    buf.take(&Hd, splits * G);
+    buf.take(&Hd, planes * G);
     buf.take(&Bt, S);
     buf.take(&d_isl, 3 * (size_t)R);
     buf.take(&E, R);
@@ -135,7 +135,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     a.moz = H ? H->origin[2] : 0.f;
     a.m = m0;
     a.Hd = Hd;
-    a.hd_planes = splits;
+    a.hd_planes = planes;
     a.hd_plane = G;
     a.A32 = A32;
     a.Ahi = Ahi;
@@ -149,7 +149,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
 
     GroupedGemm gg;
     if (tc) {
-        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, R, Rp, K, K, splits, G}};
+        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, R, Rp, K, K, slices, planes, G}};
         int r = grouped_gemm_setup(&gg, ops, 256, prec == BPM_PREC_BF16X3 ? 3 : 1, BPM_RASTER_AUTO, 32,
                                    ctx->sm_count);
         if (r != BPM_OK) {

@@ -237,3 +237,40 @@ def test_mesh_without_a_boundary_is_refused(ctx):
                             np.array([[0, 1, 2, 3], [1, 2, 0, 3]], np.int32), np.zeros(2, np.int32), 1.0, 2.0)
     with pytest.raises(L.BpmError, match="boundary"):
         ctx.mesh_upload(mesh, synth.ecc_materials())
+
+
+@pytest.mark.parametrize("nodes", ["209", "481", "1547"])
+def test_an_island_has_the_same_bits_in_every_batch(ctx, nodes):
+    """The demag product's slices of K come from K alone, and their sum has one order: the field and the states of an
+    island are bitwise the same in a batch of 300, in parts of it on either side of the 128 islands from which on a
+    slice is no longer an item of its own, and on the CTA-pair product; with the split and the single product."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    mesh = {"209": synth.small_island_mesh, "1547": synth.census_island_mesh}.get(
+        nodes, lambda: synth.layered_island_mesh(12.0, 6.0, 6.0, rings=3, hard_slabs=6, soft_slabs=6, seed=7))()
+    mid = ctx.mesh_upload(mesh, synth.ecc_materials())
+    B = 300
+    isl = synth.jittered_islands(B, seed=4, mesh_id=mid)
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, rise_ps=1.0, substeps=4, uniform_T=synth.uniform_field(0.9, 170.0))
+    rng = np.random.default_rng(5)
+    m = rng.standard_normal((B, 3, mesh.n_nodes)) * 0.3
+    m[:, 2] += 1.0
+    m = (m / np.linalg.norm(m, axis=1, keepdims=True)).astype(np.float32)
+
+    def run(rows, prec, pair=0):
+        with ctx.batch(isl.subset(rows), p, precision=prec) as bt:
+            if pair:
+                bt.set_tuning(256, 256, L.RASTER_AUTO, 2, 32, gemm_pair=1)
+            bt.set_state(m[rows], 0.0)
+            field = bt.field(0.0, L.TERM_DEMAG)
+            bt.advance(2)
+            return field, bt.read()["m"]
+
+    for prec in (L.PREC_BF16X3, L.PREC_BF16):
+        field, state = run(np.arange(B), prec)
+        assert np.abs(state - m).max() > 1e-3                             # the islands have moved
+        for rows in (np.arange(1), np.arange(17, 34), np.arange(B - 128, B), np.arange(100, 229)):
+            for pair in (0, 1):
+                f, s = run(rows, prec, pair)
+                assert np.array_equal(f, field[rows]) and np.array_equal(s, state[rows])
+    ctx.mesh_release(mid)
