@@ -330,7 +330,9 @@ int bpm_batch_field(bpm_batch* bt, double t_ps, uint32_t term_mask, float* B_out
 /* Time the kernels of one integrator step with CUDA events on the context
  * stream: runs `reps` Heun steps launch by launch (outside the graph) and
  * returns the average duration in ms of one demag GEMM, one predictor stage
- * and one corrector stage.  The state advances by those steps but the batch
+ * and one corrector stage, in the kernels that the batch's intervals run.  The
+ * intervals of a batch of few islands (see bpm_tuning) are shorter than the sum:
+ * their launches overlap.  The state advances by those steps but the batch
  * clock does not; call bpm_batch_set_state afterwards to restart a run. */
 int bpm_batch_kernel_times(bpm_batch* bt, int32_t reps, double* gemm_ms, double* stage1_ms,
                            double* stage2_ms);
@@ -347,16 +349,22 @@ enum { BPM_RASTER_AUTO = 0, BPM_RASTER_M = 1, BPM_RASTER_N = 2 };
  * gemm_tile_n 256, stage_threads 256, gemm_raster AUTO, stage_islands 2,
  * gemm_k_block 32, gemm_pair 0, and streams 2 for a one-mesh batch, 1 for a
  * multi-mesh batch (the fastest on the census and uneven batches measured).  A
- * batch of few islands (whose stage CTAs all fit the SMs at once) runs one chain
- * with one island per stage CTA, or two where the islands outnumber the SMs,
- * whatever stage_threads, stage_islands and streams say, unless gemm_pair is 1. */
+ * batch of few islands at a tensor-core precision runs one chain of overlapping
+ * launches, whatever stage_threads, stage_islands and streams say, unless
+ * gemm_pair is 1: with one island per stage CTA where every island has an SM, or
+ * where several meshes, the largest of more than 512 nodes, have up to four islands
+ * and 3200 nodes an SM; else with two where that is one pair an SM, or up to three
+ * pairs and 2000 nodes of pairs an SM (nodes of the largest mesh; a batch of more
+ * than 32 meshes, or whose state does not fit the SMs' shared memory, is not one of
+ * few islands). */
 typedef struct {
     int32_t gemm_tile_n;     /* islands per demag-GEMM tile at most: 256 or 128 (the library takes
                                 narrower tiles where wide ones would leave SMs idle) */
     int32_t stage_threads;   /* threads per Heun-stage CTA: 128, 256 or 512 */
     int32_t gemm_raster;     /* BPM_RASTER_*: tile order of the tensor-core GEMM */
     int32_t stage_islands;   /* islands per Heun-stage CTA: 1 (0 = 1), or 2 with 256 threads */
-    int32_t gemm_k_block;    /* K depth of a tensor-core GEMM pipeline stage: 32 (0 = 32) or 64 */
+    int32_t gemm_k_block;    /* K depth of a tensor-core GEMM pipeline stage: 32 (0 = 32) or 64; one-SM
+                                tiles of up to 128 islands always take 64 */
     int32_t gemm_pair;       /* 1: 256 x 256 GEMM tiles on the two SMs of a CTA pair (tcgen05
                                 cta_group::2; needs gemm_tile_n 256), 0: tiles of 128 operator rows
                                 by up to gemm_tile_n islands on one SM */
@@ -374,7 +382,9 @@ typedef struct {
 /* Autotuner: time every (gemm_tile_n, gemm_raster, gemm_k_block, gemm_pair) candidate of the demag GEMM
  * and every (stage_threads, stage_islands) candidate on this batch with CUDA events (reps Heun
  * steps each, kernel by kernel), apply the fastest of each, then time reps whole intervals with
- * streams 1 .. 4 where several chains apply, and report the choice in *chosen (nullable).  The
+ * streams 1 .. 4 where several chains apply, and report the choice in *chosen (nullable).  For a
+ * batch of few islands the one-SM GEMM candidates are timed by reps whole intervals each, and the
+ * CTA pair with its stage candidates is taken where its intervals are shorter.  The
  * state advances by the timed steps but the batch clock does not; call
  * bpm_batch_set_state afterwards to restart a run.  Tile shapes are an
  * implementation choice of this library, not of the paper. */

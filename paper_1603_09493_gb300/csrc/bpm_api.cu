@@ -1373,8 +1373,12 @@ int bpm_batch_kernel_times(bpm_batch* bt, int32_t reps, double* gemm_ms, double*
     for (auto& e : ev) BPM_CK(cudaEventCreate(&e));
     double acc[3] = {0, 0, 0};
     StageLaunches L;
+    StageGroups few;
+    int few_nt = 0;
+    const bool is_few = few_islands(bt, &few, &few_nt);    // the stage kernels that its intervals run
     int r = bt->groups.size() > 1 && tensor_core_precision(bt) ? build_stage_launches(bt, &L) : BPM_OK;
     auto stage = [&](int k, int j) -> int {
+        if (is_few) return launch_few(few, few_nt, k, j, s);
         if (tensor_core_precision(bt)) return launch_stage_all(bt, L, k, j, s);
         for (auto& g : bt->groups) (k == 1 ? launch_stage1 : launch_stage2)(g.args, j, s);
         return BPM_OK;
@@ -1453,10 +1457,32 @@ int bpm_batch_autotune(bpm_batch* bt, int32_t reps, bpm_tuning* chosen) {
     const int kblocks[2] = {64, 32};
     const int threads[3] = {256, 128, 512};
     const bool tc = tensor_core_precision(bt);
+    // a batch of few islands has one stage form and one chain, and its launches overlap: on one-SM tiles
+    // only the GEMM is chosen, by whole intervals.  The CTA pair has none of that: it comes out of the
+    // search below, and is taken where its own intervals are the shorter ones.
+    bpm_tuning best_few{256, 256, BPM_RASTER_AUTO, 2, 32, 0, 1, 0, 0};
+    double few_ms = 1e300;
+    BPM_TRY(bpm_batch_set_tuning(bt, &best_few));
+    StageGroups few_g;
+    int few_nt = 0;
+    const bool few = few_islands(bt, &few_g, &few_nt);
+    for (int ti = 0; ti < 2 && few; ++ti)
+        for (int ri = 0; ri < 3; ++ri)
+            for (int ki = 0; ki < 2; ++ki) {
+                const bpm_tuning t{tiles[ti], 256, rasters[ri], 2, kblocks[ki], 0, 1, 0, 0};
+                BPM_TRY(bpm_batch_set_tuning(bt, &t));
+                double ms = 0;
+                BPM_TRY(time_intervals(bt, 1, &ms));   // capture and warm-up
+                BPM_TRY(time_intervals(bt, reps, &ms));
+                if (ms < few_ms) {
+                    few_ms = ms;
+                    best_few = t;
+                }
+            }
     double best_g = 1e300, best_s = 1e300;
     int bt_n = 256, bt_r = BPM_RASTER_AUTO, bt_t = 256, bt_k = 64, bt_p = 0;
     // the GEMM candidates at the default stage CTA size, then the stage CTA sizes at the best GEMM
-    for (int ti = 0; ti < (tc ? 3 : 1); ++ti)
+    for (int ti = few ? 2 : 0; ti < (tc ? 3 : 1); ++ti)
         for (int ri = 0; ri < (tc ? 3 : 1); ++ri)
             for (int ki = 0; ki < (tc ? 2 : 1); ++ki) {
                 bpm_tuning t{tiles[ti], 256, rasters[ri], 1, kblocks[ki], pairs[ti], 1, 0, 0};
@@ -1489,9 +1515,10 @@ int bpm_batch_autotune(bpm_batch* bt, int32_t reps, bpm_tuning* chosen) {
     }
     // one chain or several: whole intervals of the interval graph, where several chains apply
     int bt_s = 1;
-    if (tensor_core_precision(bt) && (bt->groups.size() > 1 || bt->groups[0].B > kIslandPad)) {
-        double best_i = 1e300;
-        for (int ns = 1; ns <= kMaxChains; ++ns) {
+    double best_i = 1e300;
+    const bool several = tc && (bt->groups.size() > 1 || bt->groups[0].B > kIslandPad);
+    if (several || few) {
+        for (int ns = 1; ns <= (several ? kMaxChains : 1); ++ns) {
             bpm_tuning t{bt_n, bt_t, bt_r, bt_i, bt_k, bt_p, ns, 0, 0};
             BPM_TRY(bpm_batch_set_tuning(bt, &t));
             double ms = 0;
@@ -1504,7 +1531,14 @@ int bpm_batch_autotune(bpm_batch* bt, int32_t reps, bpm_tuning* chosen) {
         }
     }
     bpm_tuning t{bt_n, bt_t, bt_r, bt_i, bt_k, bt_p, bt_s, best_g, best_s};
+    const bool take_few = few && few_ms <= best_i;
+    if (take_few) t = best_few;
     BPM_TRY(bpm_batch_set_tuning(bt, &t));
+    if (take_few) {
+        double s1 = 0, s2 = 0;
+        BPM_TRY(bpm_batch_kernel_times(bt, reps, &t.gemm_ms, &s1, &s2));
+        t.stage_ms = s1 + s2;
+    }
     if (chosen) *chosen = t;
     return BPM_OK;
 }

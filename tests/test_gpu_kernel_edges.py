@@ -274,3 +274,31 @@ def test_an_island_has_the_same_bits_in_every_batch(ctx, nodes):
                 f, s = run(rows, prec, pair)
                 assert np.array_equal(f, field[rows]) and np.array_equal(s, state[rows])
     ctx.mesh_release(mid)
+
+
+@pytest.mark.parametrize("nodes,B", [("209", 40), ("209", 600), ("481", 300)])
+def test_autotuned_few_islands_keep_their_intervals(ctx, nodes, B):
+    """The autotuner times what a batch of few islands runs, overlapping launches in whole intervals: its choice is no
+    slower than a new batch's default, within what two timings of one batch differ by (best of seven each, 15 %)."""
+    import time
+    from paper_1603_09493_gb300 import synth
+    mesh = synth.small_island_mesh() if nodes == "209" else \
+        synth.layered_island_mesh(12.0, 6.0, 6.0, rings=3, hard_slabs=6, soft_slabs=6, seed=7)
+    mid = ctx.mesh_upload(mesh, synth.ecc_materials())
+    isl = synth.jittered_islands(B, seed=4, mesh_id=mid)
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, substeps=8, uniform_T=synth.uniform_field(0.9, 170.0))
+
+    def interval(bt):
+        best = 1e9
+        for _ in range(8):
+            t = time.perf_counter()
+            bt.advance(20)
+            bt.read()
+            best = min(best, time.perf_counter() - t)
+        return best
+
+    with ctx.batch(isl, p) as default, ctx.batch(isl, p) as tuned:
+        t = tuned.autotune(reps=3)
+        assert t["gemm_ms"] > 0 and t["stage_ms"] > 0
+        assert interval(tuned) <= 1.15 * interval(default)
+    ctx.mesh_release(mid)
