@@ -297,8 +297,8 @@ int forward(Mlp* m, cudaStream_t s, int rows, int nb, bool infer, bool sigmoid) 
     return BPM_OK;
 }
 
-// backward for the batch in the workspace: gradients into m->grad, loss into loss_slot
-int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
+// launches of backward() on s and the side stream
+int backward_chain(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
     const int Lm = m->L - 1;
     // (the pads of dZ[Lm] are zero from the allocation on; a shorter batch lays its transpose out anew)
     BPM_CK(cudaMemsetAsync(m->dZ[Lm], 0, sizeof(__nv_bfloat16) * (size_t)rows * m->out_pad[Lm], s));
@@ -341,8 +341,17 @@ int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
         e.cols_valid = m->out_real[l - 1];
         BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], m->dZ[l], m->WT[l], e, m->err));
     }
-    BPM_CK(cudaEventRecord(m->ev[m->L], m->side));
-    BPM_CK(cudaStreamWaitEvent(s, m->ev[m->L], 0));
+    return BPM_OK;
+}
+
+// backward for the batch in the workspace: gradients into m->grad, loss into loss_slot.  The side stream is
+// joined into s after an error too: what it was given still writes the gradients and the call's loss curve.
+int backward(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
+    const int r = backward_chain(m, s, rows, nb, loss_slot);
+    cudaError_t e = cudaEventRecord(m->ev[m->L], m->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, m->ev[m->L], 0);
+    if (r != BPM_OK) return r;
+    BPM_CK(e);
     return BPM_OK;
 }
 
