@@ -302,3 +302,99 @@ def test_autotuned_few_islands_keep_their_intervals(ctx, nodes, B):
         assert t["gemm_ms"] > 0 and t["stage_ms"] > 0
         assert interval(tuned) <= 1.15 * interval(default)
     ctx.mesh_release(mid)
+
+
+def test_chains_of_islands_beyond_the_few(ctx):
+    """Tuning streams on batches that are not of few islands (over three pairs an SM; 152 SMs): 1100 and 1300 islands
+    of 209 nodes in chunks of a multiple of 128 (two of 640 or three of 384, two of 768, three of 512 or four of 384,
+    the last one ragged), and three groups dealt to chains.  A chain has its own kernels of the interval graph; every island sees the same ones, so all results are
+    bitwise those of one chain.  A GEMM wait that runs out inside a several-chain graph reports the timeout."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    meshes = [synth.small_island_mesh(), synth.layered_island_mesh(7.0, 6.0, 4.0, rings=2, hard_slabs=9, soft_slabs=6, seed=5),
+              synth.layered_island_mesh(6.0, 5.0, 3.0, rings=2, hard_slabs=7, soft_slabs=4, seed=6)]
+    mids = [ctx.mesh_upload(m, synth.ecc_materials()) for m in meshes]
+    hid = ctx.headmap_upload(synth.synthetic_head_map())
+    p = synth.RunParams(dt_ps=0.1, substeps=4, alpha=0.1, rise_ps=10.0, use_map=True, x0_nm=-3.0,
+                        uniform_T=synth.uniform_field(0.7, 170.0))
+    one = synth.jittered_islands(1100, seed=1, mesh_id=mids[0])
+    three = synth.Islands.concat([synth.jittered_islands(b, seed=b, mesh_id=m) for b, m in zip((501, 600, 257), mids)])
+    for isl, chains in ((one, (1, 2, 3, 3)), (synth.jittered_islands(1300, seed=2, mesh_id=mids[0]), (1, 2, 3, 4)),
+                        (three, None)):
+        outs = []
+        for streams in (1, 2, 3, 4):
+            with ctx.batch(isl, p, precision=L.PREC_BF16X3, map_id=hid) as bt:
+                bt.set_tuning(256, 256, L.RASTER_AUTO, 2, 32, streams=streams)
+                bt.advance(20)
+                outs.append((bt.read(), bt.graph_kernels()))
+        if chains:
+            assert [k for _, k in outs] == [1 + 16 * c for c in chains]   # four kernels a step and chain, and the clock
+        for o, _ in outs:
+            for key in ("m", "switched", "t_sw", "mz", "status"):
+                assert np.array_equal(o[key], outs[0][0][key]), key
+            assert np.all(o["status"] == 0) and np.abs(o["m"][:, :2]).max() > 1e-2     # the islands have moved
+    with ctx.batch(one, p, precision=L.PREC_BF16X3, map_id=hid) as bt:
+        bt.set_tuning(256, 256, L.RASTER_AUTO, 2, 32, streams=3)
+        L.check(ctx.lib.bpm_debug_set_gemm_wait(bt.h, 1000.0))        # 1 us
+        bt.advance(2)
+        with pytest.raises(L.BpmError) as e:
+            bt.read()
+        assert e.value.code == L.BPM_ERR_TIMEOUT
+    for m in mids:
+        ctx.mesh_release(m)
+    ctx.headmap_release(hid)
+
+
+@pytest.mark.parametrize("sizes", [(20,), (120, 120), (300, 200), (40, 150, 90)])
+def test_few_islands_of_larger_meshes(ctx, sizes):
+    """The stage kernels of few islands on meshes of over 512 nodes (1024 threads a CTA, or 512 where SMs hold several
+    islands; several groups at one island a CTA), against the same run on the two-island stage kernels behind the
+    CTA-pair product, whose sums are the same: m bitwise, <m_z> up to the order of its sum."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    variants = synth.design_variants()[:4:2] + [dict(mesh=synth.layered_island_mesh(7.0, 6.0, 4.0, rings=3, hard_slabs=9,
+                                                                                    soft_slabs=6))]
+    meshes = [v["mesh"] for v in variants][:len(sizes)]
+    assert all(m.n_nodes > 512 for m in meshes)
+    mids = [ctx.mesh_upload(m, synth.ecc_materials()) for m in meshes]
+    hid = ctx.headmap_upload(synth.synthetic_head_map())
+    isl = synth.Islands.concat([synth.jittered_islands(b, seed=b, mesh_id=m) for b, m in zip(sizes, mids)])
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, rise_ps=2.0, use_map=True, x0_nm=-2.0, substeps=8,
+                        uniform_T=synth.uniform_field(0.9, 170.0))
+    out = []
+    for pair in (0, 1):
+        with ctx.batch(isl, p, precision=L.PREC_BF16X3, map_id=hid) as bt:
+            bt.set_tuning(256, 256, L.RASTER_AUTO, 2, 32, gemm_pair=pair)
+            bt.advance(20)
+            out.append(bt.read())
+    few, two = out
+    assert np.all(few["status"] == 0) and np.abs(few["m"][:, :2]).max() > 1e-2         # the islands have moved
+    assert np.array_equal(few["m"], two["m"]) and np.abs(few["mz"] - two["mz"]).max() <= 1e-6
+    for m in mids:
+        ctx.mesh_release(m)
+    ctx.headmap_release(hid)
+
+
+@pytest.mark.parametrize("B", [33, 64, 65, 130])
+def test_fp32_product_column_remainder(ctx, B):
+    """The FP32 GEMM's 128-column tiles on an operator of 1472 columns, the last tile half empty: as in
+    test_fp32_product_tile_edges, K/4 * 2^-24 of the sum of magnitudes, K = 1472, and the sources' own rounding."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    mesh = synth.layered_island_mesh(12.0, 6.0, 6.0, rings=3, hard_slabs=6, soft_slabs=6, seed=7)
+    mid = ctx.mesh_upload(mesh, synth.ecc_materials())
+    n = mesh.n_nodes
+    assert ctx.mesh_info(mid)["k_pad"] % 128 == 64
+    isl = synth.jittered_islands(B, seed=B, mesh_id=mid)
+    rng = np.random.default_rng(B)
+    m = rng.standard_normal((B, 3, n)).astype(np.float32)
+    m /= np.linalg.norm(m, axis=1, keepdims=True)
+    with ctx.batch(isl, synth.RunParams(dt_ps=0.1, substeps=1, term_mask=L.TERM_DEMAG), precision=L.PREC_FP32) as bt:
+        bt.set_state(m, 0.0)
+        got = bt.field(0.0, L.TERM_DEMAG).reshape(B, 3 * n)
+    Ms = (ctx.get_operator(mid, L.OP_NODAL_MS_F64) * 1e-6).astype(np.float32)
+    src = ((Ms[None] * isl.Ms_scale[:, None])[:, None] * m).astype(np.float64).reshape(B, 3 * n)
+    W = ctx.get_operator(mid, L.OP_DEMAG_F32).astype(np.float64)
+    ctx.mesh_release(mid)
+    bound = (368 * 2.0 ** -24 + 2.0 ** -22) * (np.abs(src) @ np.abs(W).T)
+    assert np.all(np.abs(got - src @ W.T) <= bound)
