@@ -30,11 +30,14 @@ constexpr int kThreads = 256;
 // k-blocks: two stages keep their ring full and halve the shared memory, so that two CTAs share
 // an SM and one CTA's epilogue runs beside the other's MMAs.  The other GEMMs (K = batch rows)
 // keep the deep ring.
-// Column tiles (4096 rows, 256 features; the sums do not depend on the tile): the epilogues bound the
-// forward and input-gradient layers, so their tiles are as narrow as fills the SMs -- forward 64 wide
-// (128 CTAs, 17 us a layer; 128 wide 27), input gradient 64 wide (23 us; 256 wide, 32 CTAs, 71).
-// The weight gradient's K is the batch, a serial walk of 64 k-blocks; 32-wide tiles make it 16 CTAs
-// of 20 us that run beside the input gradients (two CTAs of 27 us in line with them before).
+// Column tiles: the widest whose CTAs fill the SMs (tile_width), narrow ones where they would not.  The sums do
+// not depend on the tile.  The epilogues bound the small layers, which want every SM; wide tiles read the
+// row operand fewer times, which bounds the large ones.  4096 rows of 256 features: forward 64 wide 17 us
+// a layer (128 CTAs; 128 wide 27), input gradient 64 wide 23 us (256 wide, 32 CTAs, 71), weight gradient
+// 32 wide 20 us in 16 CTAs beside the input gradients (its K is the batch, a serial walk; 256 wide two
+// CTAs of 27 us).  Inference of 65536 samples, 64 / 128 / 256 wide: width 512 445 / 407 / 462 us, width 2048
+// 1127 / 894 / 954, width 4096 3132 / 2306 / 2384.  A training step of 4096 rows of 2048 features: input
+// gradient 64 / 128 / 256 wide 592 / 541 / 519 us, weight gradient 32 / 64 / 128 / 256 wide 592 / 525 / 492 / 485.
 template <int P, int TN, int EPI>
 struct Cfg {
     static constexpr int W_TILE = Tile<TN>::W_TILE;
@@ -350,18 +353,42 @@ int make_bf16_tensor_map(CUtensorMap* map, const void* ptr, int inner, int rows,
     return BPM_OK;
 }
 
+// the widest column tile, halved from `most` down to `least`, of which the M x N outputs have `ctas` or more
+static int tile_width(int M, int N, int most, int least, int ctas) {
+    int t = most;
+    while (t > least && (long long)(M / tc::TM) * ((N + t - 1) / t) < ctas) t /= 2;
+    return t;
+}
+
 int gemm_tc(cudaStream_t s, int epi, int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* W,
-            const TcEpilogue& e, int* err_flag) {
+            const TcEpilogue& e, int sm_count, int* err_flag) {
     if (M % TM || K % TK || N % 16 || M <= 0 || N <= 0) {
         set_error("tensor-core GEMM needs M %% %d == 0, K %% %d == 0, N %% 16 == 0 (M=%d N=%d K=%d)", TM, TK, M, N, K);
         return BPM_ERR_ARG;
     }
+    // The forward layers alone on the GPU take 128 columns where that gives every SM a CTA (128 CTAs: width
+    // 512 at 4096 rows 108 us 64 wide, 111 so; 256 CTAs: 134 and 123).  The gradients share it, and take the widest
+    // tile with a CTA for every second SM (64 CTAs of 256 columns, width 1024 at 2048 rows: 271 us a step, 259 at
+    // 128; 128 CTAs, 4096 rows: 372 and 386).
     switch (epi) {
-        case TC_EPI_STORE: return launch<1, TC_EPI_STORE, 32>(s, M, N, K, A, A, W, W, e, err_flag);
-        case TC_EPI_BIAS_GELU: 
-            return launch<1, TC_EPI_BIAS_GELU, 64>(s, M, N, K, A, A, W, W, e, err_flag);
+        case TC_EPI_STORE:
+            switch (tile_width(M, N, 256, 32, sm_count / 2)) {
+                case 256: return launch<1, TC_EPI_STORE, 256>(s, M, N, K, A, A, W, W, e, err_flag);
+                case 128: return launch<1, TC_EPI_STORE, 128>(s, M, N, K, A, A, W, W, e, err_flag);
+                case 64: return launch<1, TC_EPI_STORE, 64>(s, M, N, K, A, A, W, W, e, err_flag);
+                default: return launch<1, TC_EPI_STORE, 32>(s, M, N, K, A, A, W, W, e, err_flag);
+            }
+        case TC_EPI_BIAS_GELU:
+            return tile_width(M, N, 128, 64, sm_count) == 128
+                       ? launch<1, TC_EPI_BIAS_GELU, 128>(s, M, N, K, A, A, W, W, e, err_flag)
+                       : launch<1, TC_EPI_BIAS_GELU, 64>(s, M, N, K, A, A, W, W, e, err_flag);
         case TC_EPI_BIAS_OUT: return launch<1, TC_EPI_BIAS_OUT, 128>(s, M, N, K, A, A, W, W, e, err_flag);
-        case TC_EPI_GELU_BWD: return launch<1, TC_EPI_GELU_BWD, 64>(s, M, N, K, A, A, W, W, e, err_flag);
+        case TC_EPI_GELU_BWD:
+            switch (tile_width(M, N, 256, 64, sm_count / 2)) {
+                case 256: return launch<1, TC_EPI_GELU_BWD, 256>(s, M, N, K, A, A, W, W, e, err_flag);
+                case 128: return launch<1, TC_EPI_GELU_BWD, 128>(s, M, N, K, A, A, W, W, e, err_flag);
+                default: return launch<1, TC_EPI_GELU_BWD, 64>(s, M, N, K, A, A, W, W, e, err_flag);
+            }
         default: set_error("unknown epilogue %d", epi); return BPM_ERR_ARG;
     }
 }

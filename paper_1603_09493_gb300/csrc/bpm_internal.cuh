@@ -210,7 +210,7 @@ struct TcEpilogue {
     int sigmoid = 0;               // BIAS_OUT: apply the logistic function
 };
 int gemm_tc(cudaStream_t s, int epi, int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* W,
-            const TcEpilogue& e, int* err_flag);
+            const TcEpilogue& e, int sm_count, int* err_flag);
 
 // grouped persistent tensor-core GEMM (bpm_gemm_grouped.cu): one launch over the
 // output tiles of every mesh group of a batch

@@ -48,7 +48,7 @@ struct Mlp {
     cudaStream_t side = nullptr;
     std::vector<cudaEvent_t> ev;          // ev[l]: dZ[l] written; ev[L]: the weight gradients are done
     int* err = nullptr;
-    int max_pad = 0;
+    int max_pad = 0, sm_count = 0;
     // inference in one kernel (networks up to 256 wide); layer by layer otherwise
     bool one_kernel = false;
     MlpForward fwd{};
@@ -286,12 +286,12 @@ int forward(Mlp* m, cudaStream_t s, int rows, int nb, bool infer, bool sigmoid) 
             e.ldh = m->in_pad[l + 1];
             e.HT = infer ? nullptr : m->HT[l + 1];
             e.ldht = rows;
-            BPM_TRY(gemm_tc(s, TC_EPI_BIAS_GELU, rows, m->out_pad[l], m->in_pad[l], m->H[l], m->W[l], e, m->err));
+            BPM_TRY(gemm_tc(s, TC_EPI_BIAS_GELU, rows, m->out_pad[l], m->in_pad[l], m->H[l], m->W[l], e, m->sm_count, m->err));
         } else {
             e.C = m->logits;
             e.ldc = m->n_out;
             e.sigmoid = sigmoid ? 1 : 0;
-            BPM_TRY(gemm_tc(s, TC_EPI_BIAS_OUT, rows, m->out_pad[l], m->in_pad[l], m->H[l], m->W[l], e, m->err));
+            BPM_TRY(gemm_tc(s, TC_EPI_BIAS_OUT, rows, m->out_pad[l], m->in_pad[l], m->H[l], m->W[l], e, m->sm_count, m->err));
         }
     }
     return BPM_OK;
@@ -325,7 +325,7 @@ int backward_chain(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
         g.ldc = m->in_real[l];
         g.rows_valid = m->out_real[l];
         g.cols_valid = m->in_real[l];
-        BPM_TRY(gemm_tc(m->side, TC_EPI_STORE, m->out_pad[l], m->in_pad[l], rows, m->dZT[l], m->HT[l], g, m->err));
+        BPM_TRY(gemm_tc(m->side, TC_EPI_STORE, m->out_pad[l], m->in_pad[l], rows, m->dZT[l], m->HT[l], g, m->sm_count, m->err));
         if (l == 0) break;
         // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1}), bias gradient of layer l-1
         TcEpilogue e{};
@@ -339,7 +339,7 @@ int backward_chain(Mlp* m, cudaStream_t s, int rows, int nb, float* loss_slot) {
         e.ldcs = m->in_pad[l];
         e.rows_valid = nb;
         e.cols_valid = m->out_real[l - 1];
-        BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], m->dZ[l], m->WT[l], e, m->err));
+        BPM_TRY(gemm_tc(s, TC_EPI_GELU_BWD, rows, m->in_pad[l], m->out_pad[l], m->dZ[l], m->WT[l], e, m->sm_count, m->err));
     }
     return BPM_OK;
 }
@@ -450,6 +450,7 @@ int bpm_surrogate_create(bpm_ctx* ctx, const bpm_mlp_cfg* cfg, const float* para
     m->depth = cfg->depth;
     m->n_out = cfg->n_out;
     m->L = cfg->depth + 1;
+    m->sm_count = ctx->sm_count;
     size_t off = 0;
     for (int l = 0; l < m->L; ++l) {
         int in = l == 0 ? m->n_in : m->width;

@@ -166,3 +166,28 @@ def test_screen_rejects_bad_arguments(ctx):
     with pytest.raises(ValueError):
         sur.screen(X, 3, 3)
     sur.destroy()
+
+
+@pytest.mark.parametrize("width,rows", [(512, 12000), (1024, 2048), (1536, 1280), (2048, 1280)])
+def test_wide_layers_take_other_tiles(ctx, width, rows):
+    """Layers wider than 256: 64- or 128-wide forward tiles, 64 to 256 wide ones for input gradients and 32 to 256 for
+    weight gradients, by the CTAs they give.  Probabilities of a batch are bitwise those of its parts, which take
+    narrower tiles; gradients against the oracle within this file's bounds."""
+    sizes = [16, width, width, 2]
+    params = synth.mlp_init_params(sizes, seed=3)
+    sur = ctx.surrogate((16, width, 2, 2), params)
+    X, Y = dataset(rows, 1)
+    P = sur.infer(X)
+    assert np.array_equal(np.concatenate([sur.infer(X[k:k + 700]) for k in range(0, rows, 700)]), P)
+    X, Y = X[:2048], Y[:2048]
+    g, loss = sur.grad(X, Y)
+    W = synth.unflatten_params(bf16_round(params), sizes)
+    logits, cache = omlp.forward(W, bf16_round(X).astype(np.float64))
+    assert np.abs(P[:2048] - omlp.sigmoid(logits)).max() <= 0.02
+    assert abs(loss - omlp.loss(logits, Y)) <= 1e-2 * abs(loss)
+    off = 0
+    for part in (q.ravel() for layer in omlp.backward(W, cache, logits, Y) for q in layer):
+        gg = g[off:off + part.size].astype(np.float64)
+        off += part.size
+        assert np.linalg.norm(gg - part) <= 1e-2 * np.linalg.norm(part)
+    sur.destroy()
