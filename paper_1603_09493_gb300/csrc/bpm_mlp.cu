@@ -48,6 +48,9 @@ struct Mlp {
     cudaStream_t side = nullptr;
     std::vector<cudaEvent_t> ev;          // ev[l]: dZ[l] written; ev[L]: the weight gradients are done
     int* err = nullptr;
+    // logits of a chunk of a screening call on device arrays, which returns with its work in flight
+    float* z = nullptr;
+    size_t z_size = 0;
     int max_pad = 0, sm_count = 0;
     // inference in one kernel (networks up to 256 wide); layer by layer otherwise
     bool one_kernel = false;
@@ -419,6 +422,7 @@ void free_mlp(Mlp* m) {
     for (auto e : m->ev)
         if (e) cudaEventDestroy(e);
     if (m->side) cudaStreamDestroy(m->side);
+    cudaFree(m->z);
     cudaFree(m->arena);
     delete m;
 }
@@ -699,8 +703,8 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
     BPM_CK(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
     const long long N = (long long)n_designs * n_jitter;
-    // logits of at most 2^20 samples at a time
-    const long long chunk = 1 << 20;
+    // logits of at most 2^20 samples or 32 MB at a time
+    const long long chunk = std::min(1 << 20, (8 << 20) / m->n_out / 128 * 128);
     const float* Xd = X;
     float *Xtmp = nullptr, *z = nullptr;
     double* acc = nullptr;
@@ -715,8 +719,16 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
         BPM_CK(cudaMemcpyAsync(Xtmp, X, sizeof(float) * (size_t)N * m->n_in, cudaMemcpyHostToDevice, s));
         Xd = Xtmp;
     } else {
-        // the device form returns with its work in flight: its scratch is stream-ordered memory
-        BPM_CK(cudaMallocAsync(&z, sizeof(float) * nz, s));
+        // kept with the surrogate: stream-ordered memory cost 130 us a call (the pool is empty after every
+        // synchronisation): 384000 samples of width 256 0.83 -> 0.61 ms, of width 512 2.48 -> 2.22
+        if (nz > m->z_size) {
+            cudaFree(m->z);             // waits for the call that uses it
+            m->z = nullptr;
+            m->z_size = 0;
+            BPM_CK(cudaMalloc(&m->z, sizeof(float) * nz));
+            m->z_size = nz;
+        }
+        z = m->z;
         acc = rates;
     }
     BPM_CK(cudaMemsetAsync(acc, 0, out_bytes, s));
@@ -746,7 +758,6 @@ int bpm_surrogate_screen(bpm_ctx* ctx, int32_t sid, const float* X, int64_t n_de
             r = BPM_ERR_CUDA;
         }
     }
-    if (on_device) cudaFreeAsync(z, s);
     if (r != BPM_OK) return r;
     if (!on_device) return check_err(m, s);
     return BPM_OK;

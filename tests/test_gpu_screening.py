@@ -61,3 +61,20 @@ def test_surrogate_screening_gain():
         assert acc >= 0.9 and a0 >= 0.95
         assert hit >= 0.98 and hit > rate + 0.2
         sur.destroy()
+
+
+@pytest.mark.parametrize("n_out,D,J", [(2, 1100, 1000), (128, 700, 100)])
+def test_screening_device_arrays_in_chunks(n_out, D, J):
+    """Device arrays of more samples than a chunk's logits hold (2^20 of two outputs, 65536 of 128): the rates of host
+    arrays, bit for bit; a smaller call after it and a repeated one too."""
+    import torch
+    from paper_1603_09493_gb300 import api, synth
+    with api.Context(0) as ctx:
+        sur = ctx.surrogate((16, 64, 1, n_out), synth.mlp_init_params([16, 64, n_out], seed=3))
+        X = np.random.default_rng(n_out).uniform(-1, 1, (D * J, 16)).astype(np.float32)
+        Xd = torch.from_numpy(X).cuda()
+        R = sur.screen(X, D, J)
+        for _ in range(2):
+            assert np.array_equal(sur.screen(Xd, D, J).cpu().numpy(), R)
+            assert np.array_equal(sur.screen(Xd[:7 * J], 7, J).cpu().numpy(), R[:7])
+        sur.destroy()
