@@ -214,9 +214,9 @@ int setup_grouped_gemm(bpm_batch* bt) {
     for (auto& g : bt->groups) {
         const int K = g.mesh->K();
         ops.push_back(GemmOperands{g.Ahi, g.Alo, g.mesh->Nhi, g.mesh->Nlo, g.Hd, g.B, g.Bp, K, K, g.slices,
-                                   g.planes, (size_t)g.Bp * K});
+                                   g.planes, (size_t)g.B * K});
         g.args.hd_planes = bt->pair ? 1 : g.planes;   // the CTA-pair kernel adds the slices itself
-        g.args.hd_plane = (size_t)g.Bp * K;
+        g.args.hd_plane = (size_t)g.B * K;
     }
     return grouped_gemm_setup(&bt->gg, ops, bt->tile_n, bt->p.precision == BPM_PREC_BF16X3 ? 3 : 1, bt->raster,
                               bt->k_block, bt->ctx->sm_count, bt->pair);
@@ -309,7 +309,7 @@ int setup_chains(bpm_batch* bt) {
                 const Group& q = bt->groups[i];
                 const int K = q.mesh->K();
                 ops.push_back(GemmOperands{q.Ahi, q.Alo, q.mesh->Nhi, q.mesh->Nlo, q.Hd, q.B, q.Bp, K, K, q.slices,
-                                           q.planes, (size_t)q.Bp * K});
+                                           q.planes, (size_t)q.B * K});
             }
             BPM_TRY(grouped_gemm_setup(&bt->gg_chain[c], ops, bt->tile_n, products, bt->raster, bt->k_block,
                                        bt->ctx->sm_count, bt->pair, chains));
@@ -572,7 +572,9 @@ size_t carve(bpm_batch* bt, Arena& A) {
         const size_t S = (size_t)g.Bp * g.mesh->K();
         A.take(&g.m, (size_t)g.Bp * 3 * g.mesh->n_pad);
         A.take(&g.k1, (size_t)g.Bp * 3 * g.mesh->n_pad);
-        A.take(&g.Hd, g.planes * S);
+        // planes of the islands' rows alone: a batch of up to a hundred islands of 209 nodes then stays below the
+        // 2 MB that cudaMalloc maps anew (created and destroyed 231 -> 59 us)
+        A.take(&g.Hd, std::max(S, (size_t)g.planes * g.B * g.mesh->K()));
         if (bt->p.precision == BPM_PREC_FP32) {
             A.take(&g.A32, S);
         } else {

@@ -230,7 +230,7 @@ struct GemmOperands {
     float* C;
     int M, rows, N, K;                // islands, rows of A (a multiple of 128, zeros from M on)
     int slices, planes;               // slices of K (gemm_slices), planes of C (gemm_planes)
-    size_t plane;                     // elements of a plane
+    size_t plane;                     // elements of a plane: the islands' rows
 };
 // Slices of K of a demag product: an element is the sum of its slices in order, so that an island's field has the
 // same bits whatever else is in its batch or launch

@@ -87,7 +87,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
         buf.take(&Alo, G);
     }
     const size_t zeroed = buf.size;              // pads of the states and the operand stay zero
-    buf.take(&Hd, planes * G);
+    buf.take(&Hd, std::max(G, (size_t)planes * R * K));
     buf.take(&Bt, S);
     buf.take(&d_isl, 3 * (size_t)R);
     buf.take(&E, R);
@@ -136,7 +136,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
     a.m = m0;
     a.Hd = Hd;
     a.hd_planes = planes;
-    a.hd_plane = G;
+    a.hd_plane = (size_t)R * K;
     a.A32 = A32;
     a.Ahi = Ahi;
     a.Alo = Alo;
@@ -149,7 +149,7 @@ extern "C" int bpm_neb_run(bpm_ctx* ctx, const bpm_island* isl, int32_t D, const
 
     GroupedGemm gg;
     if (tc) {
-        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, R, Rp, K, K, slices, planes, G}};
+        std::vector<GemmOperands> ops{GemmOperands{Ahi, Alo, M->Nhi, M->Nlo, Hd, R, Rp, K, K, slices, planes, (size_t)R * K}};
         int r = grouped_gemm_setup(&gg, ops, 256, prec == BPM_PREC_BF16X3 ? 3 : 1, BPM_RASTER_AUTO, 32,
                                    ctx->sm_count);
         if (r != BPM_OK) {
