@@ -209,6 +209,25 @@ bool tensor_core_precision(const bpm_batch* bt) {
 }
 
 // (re)encode the grouped tensor-core GEMM of the batch for its current tile width
+// Whether the groups' tiles go as whole items although some groups are small enough for a plane per slice of
+// K.  Planes spread few tiles over the SMs and even out the SMs' shares, but the stages read every one.  They go
+// where the tiles alone give every SM an item, or three SMs of four while the planes' traffic is a twelfth of
+// the operators'.  Intervals of uneven variants, with planes / without, three batches in turn on as many
+// streams and alone (ms): 6 variants of 120 islands 12.4 / 11.3 and 16.1 / 15.6; 5 of 60 6.2 / 5.8 and 8.9 / 7.9; 8 of
+// 12 17.7 / 17.5 and 18.7 / 19.8; below an SM each, 4 of 90 4.26 / 3.57 and 6.8 / 6.9, but 4 of 36 3.34 / 3.17 and
+// 3.88 / 4.56.
+bool whole_tiles(const bpm_batch* bt) {
+    double items = 0, planes = 0, ops = 0;
+    for (const auto& g : bt->groups) {
+        const double K = g.mesh->K();
+        items += (double)((g.B + 255) / 256) * ((g.mesh->K() + 127) / 128);
+        planes += 2.0 * (g.planes - 1) * g.B * K;          // floats written and read beyond one plane
+        ops += K * K;                                      // an operator's two halves
+    }
+    const int sms = bt->ctx->sm_count;
+    return items >= sms || (items >= 0.75 * sms && planes >= ops / 12);
+}
+
 int setup_grouped_gemm(bpm_batch* bt) {
     std::vector<GemmOperands> ops;
     for (auto& g : bt->groups) {
@@ -988,6 +1007,8 @@ int bpm_batch_create(bpm_ctx* ctx, const bpm_island* isl, int32_t B, const bpm_r
             g.planes = gemm_planes(g.B, g.slices);
         }
     }
+    if (bt->groups.size() > 1 && tensor_core_precision(bt) && whole_tiles(bt))
+        for (auto& g : bt->groups) g.planes = 1;
     Arena size{nullptr};
     const size_t tables = carve(bt, size);
     cudaError_t ce = cudaMalloc(&bt->arena, size.off);

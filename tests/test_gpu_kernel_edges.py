@@ -398,3 +398,42 @@ def test_fp32_product_column_remainder(ctx, B):
     ctx.mesh_release(mid)
     bound = (368 * 2.0 ** -24 + 2.0 ** -22) * (np.abs(src) @ np.abs(W).T)
     assert np.all(np.abs(got - src @ W.T) <= bound)
+
+
+@pytest.mark.parametrize("sizes", [(12, 9, 30, 5, 14, 120), (80, 90, 100, 110), (300, 20, 1, 40, 17)])
+def test_groups_of_whole_tiles_have_the_bits_of_their_own_batches(ctx, sizes):
+    """Batches of several large meshes, whose tiles fill the SMs without a plane per slice of K (six and five meshes by
+    their tiles alone, four by the planes' traffic): field and states of each group bitwise those of a batch of its
+    own, which takes the planes where it has up to 128 islands."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    meshes = [v["mesh"] for v in synth.design_variants()[:2 * len(sizes):2]]
+    mids = [ctx.mesh_upload(m, synth.ecc_materials()) for m in meshes]
+    parts = [synth.jittered_islands(b, seed=b, mesh_id=m) for b, m in zip(sizes, mids)]
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, rise_ps=1.0, substeps=3, uniform_T=synth.uniform_field(0.9, 170.0))
+    n_max = max(m.n_nodes for m in meshes)
+    rng = np.random.default_rng(5)
+    state = []
+    for b, mesh in zip(sizes, meshes):
+        m = rng.standard_normal((b, 3, mesh.n_nodes)) * 0.3
+        m[:, 2] += 1.0
+        state.append((m / np.linalg.norm(m, axis=1, keepdims=True)).astype(np.float32))
+
+    def run(isl, m):
+        with ctx.batch(isl, p) as bt:
+            bt.set_state(m, 0.0)
+            field = bt.field(0.0, L.TERM_DEMAG)
+            bt.advance(1)
+            return field, bt.read()["m"]
+
+    whole = np.concatenate([np.pad(m, ((0, 0), (0, 0), (0, n_max - m.shape[2]))) for m in state])
+    field, out = run(synth.Islands.concat(parts), whole)
+    at = 0
+    for isl, m in zip(parts, state):
+        f, s = run(isl, m)
+        rows = slice(at, at + len(m))
+        at += len(m)
+        assert np.array_equal(field[rows, :, :m.shape[2]], f) and np.array_equal(out[rows, :, :m.shape[2]], s)
+        assert np.abs(s - m).max() > 1e-3                                 # the islands have moved
+    for mid in mids:
+        ctx.mesh_release(mid)
