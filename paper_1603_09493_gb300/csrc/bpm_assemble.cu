@@ -135,12 +135,6 @@ __global__ void k_tet_geom(int nt, const double* __restrict__ xyz, const int* __
     }
 }
 
-__device__ inline int local_index(const int* tet, int node) {
-    for (int a = 0; a < 4; ++a)
-        if (tet[a] == node) return a;
-    return 0;
-}
-
 // position of a node in a tet, -1 if the tet does not hold it
 __device__ inline int tet_slot(const int* tet, int node) {
     for (int a = 0; a < 4; ++a)
@@ -186,7 +180,7 @@ __global__ void k_csr_values(int n, const int* __restrict__ rowptr, const int* _
             const int* tt = tets + 4 * t;
             const int b = tet_slot(tt, j);
             if (b < 0) continue;
-            const int a = local_index(tt, i);
+            const int a = tet_slot(tt, i);
             const double* g = grads + 12 * t;
             const double gg = g[3 * a] * g[3 * b] + g[3 * a + 1] * g[3 * b + 1] + g[3 * a + 2] * g[3 * b + 2];
             kl += vol[t] * gg;

@@ -289,14 +289,13 @@ __global__ void __launch_bounds__(kGThreads, 1)
 }
 
 template <int P, int TN, int KB>
-int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int sm_count, int* err, bool pdl) {
+int launch_grouped(cudaStream_t s, const GroupedGemm& gg, int* err, bool pdl) {
     static bool configured = false;
     if (!configured) {
         BPM_CK(cudaFuncSetAttribute(k_gemm_grouped<P, TN, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     GCfg<P, TN, KB>::smem));
         configured = true;
     }
-    (void)sm_count;                       // the grid is part of the schedule
     BPM_CK(launch_pdl(k_gemm_grouped<P, TN, KB>, dim3(gg.grid), dim3(kGThreads), GCfg<P, TN, KB>::smem, s, pdl,
                       gg.d_groups, gg.n_groups, gg.d_sched, err, gg.wait_ns ? gg.wait_ns : kWaitNs));
     return BPM_OK;
@@ -498,14 +497,14 @@ int grouped_gemm_launch(cudaStream_t s, GroupedGemm& gg, int sm_count, int* err,
     }
     if (gg.pair) return grouped_gemm_pair_launch(s, gg, sm_count, err);
     const bool split = gg.products == 3;
-    if (gg.tile_n == 64) return split ? launch_grouped<3, 64, 64>(s, gg, sm_count, err, pdl)
-                                      : launch_grouped<1, 64, 64>(s, gg, sm_count, err, pdl);
-    if (gg.tile_n == 128) return split ? launch_grouped<3, 128, 64>(s, gg, sm_count, err, pdl)
-                                       : launch_grouped<1, 128, 64>(s, gg, sm_count, err, pdl);
-    if (gg.k_block == 64) return split ? launch_grouped<3, 256, 64>(s, gg, sm_count, err, pdl)
-                                       : launch_grouped<1, 256, 64>(s, gg, sm_count, err, pdl);
-    return split ? launch_grouped<3, 256, 32>(s, gg, sm_count, err, pdl)
-                 : launch_grouped<1, 256, 32>(s, gg, sm_count, err, pdl);
+    if (gg.tile_n == 64) return split ? launch_grouped<3, 64, 64>(s, gg, err, pdl)
+                                      : launch_grouped<1, 64, 64>(s, gg, err, pdl);
+    if (gg.tile_n == 128) return split ? launch_grouped<3, 128, 64>(s, gg, err, pdl)
+                                       : launch_grouped<1, 128, 64>(s, gg, err, pdl);
+    if (gg.k_block == 64) return split ? launch_grouped<3, 256, 64>(s, gg, err, pdl)
+                                       : launch_grouped<1, 256, 64>(s, gg, err, pdl);
+    return split ? launch_grouped<3, 256, 32>(s, gg, err, pdl)
+                 : launch_grouped<1, 256, 32>(s, gg, err, pdl);
 }
 
 }  // namespace bpm

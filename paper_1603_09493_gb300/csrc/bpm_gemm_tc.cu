@@ -1,17 +1,16 @@
 // Tensor-core GEMM with fused epilogues (tcgen05, sm_103a), used by the surrogate MLP:
 //   C[M][N] = A[M][K] * W[N][K]^T, BF16 operands, FP32 accumulate in TMEM
-// (the kernel also supports the BF16 hi/lo split, products = 3: Ahi*Whi + Alo*Whi +
-// Ahi*Wlo; the batched demag product uses the persistent grouped kernel in
+// (the batched demag product uses the persistent grouped kernel in
 // bpm_gemm_grouped.cu).
 //
-// One CTA computes a 128-row output tile of 32 to 256 columns (by epilogue, see Cfg).  Warp 0 (one elected lane) streams the
-// k-blocks (64 BF16 = one 128-byte swizzle atom) of every operand tile with TMA into a
-// ring of shared-memory stages, warp 1 (one elected lane) issues the tcgen05.mma
-// instructions into a TMEM accumulator of 128 lanes, and after the last
-// k-block all eight warps read the accumulator back with tcgen05.ld and store it.
-// Each stage holds Ahi, Alo, Whi, Wlo for one k-block, so the three products of a
-// k-block share the staged tiles.  Every mbarrier wait is bounded; on timeout the
-// kernel records an error flag, drains its own copies and MMAs, frees TMEM and exits.
+// One CTA computes a 128-row output tile of 32 to 256 columns (by epilogue and
+// size, see Cfg and gemm_tc).  Warp 0 (one elected lane) streams the k-blocks (64
+// BF16 = one 128-byte swizzle atom) of both operand tiles with TMA into a ring of
+// shared-memory stages, warp 1 (one elected lane) issues the tcgen05.mma
+// instructions into a TMEM accumulator of 128 lanes, and after the last k-block
+// all eight warps read the accumulator back with tcgen05.ld and store it.
+// Every mbarrier wait is bounded; on timeout the kernel records an error flag,
+// drains its own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>
 
 #include "bpm_tc_ptx.cuh"
@@ -38,12 +37,12 @@ constexpr int kThreads = 256;
 // CTAs of 27 us).  Inference of 65536 samples, 64 / 128 / 256 wide: width 512 445 / 407 / 462 us, width 2048
 // 1127 / 894 / 954, width 4096 3132 / 2306 / 2384.  A training step of 4096 rows of 2048 features: input
 // gradient 64 / 128 / 256 wide 592 / 541 / 519 us, weight gradient 32 / 64 / 128 / 256 wide 592 / 525 / 492 / 485.
-template <int P, int TN, int EPI>
+template <int TN, int EPI>
 struct Cfg {
     static constexpr int W_TILE = Tile<TN>::W_TILE;
-    static constexpr int stage_bytes = (P == 3 ? 2 : 1) * (A_TILE + W_TILE);
+    static constexpr int stage_bytes = A_TILE + W_TILE;
     static constexpr bool forward_layer = EPI == 1 || EPI == 2;   // TC_EPI_BIAS_GELU, TC_EPI_BIAS_OUT
-    static constexpr int stages = forward_layer ? 2 : (192 * 1024) / stage_bytes;   // 2 .. 6
+    static constexpr int stages = forward_layer ? 2 : (192 * 1024) / stage_bytes;   // 2, or 4 (256 wide) .. 9 (32 wide)
     static constexpr int smem = stages * stage_bytes + 1024 /*align*/ + 256 /*barriers*/;
 };
 
@@ -151,13 +150,11 @@ __device__ __forceinline__ float warp_colsums(float (&v)[32], int lane) {
     return v[0];
 }
 
-template <int P, int EPI, int TN>
+template <int EPI, int TN>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_gemm_tc(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
-              const __grid_constant__ CUtensorMap mWhi, const __grid_constant__ CUtensorMap mWlo, int M, int N, int K,
+    k_gemm_tc(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mW, int M, int N, int K,
               const TcEpilogue e, int* err) {
-    using CF = Cfg<P, TN, EPI>;
-    constexpr int W_TILE = CF::W_TILE;
+    using CF = Cfg<TN, EPI>;
     constexpr int S = CF::stages;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -198,10 +195,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
-    auto sAhi = [&](int s) { return base + s * CF::stage_bytes; };
-    auto sWhi = [&](int s) { return base + s * CF::stage_bytes + A_TILE; };
-    auto sAlo = [&](int s) { return base + s * CF::stage_bytes + A_TILE + W_TILE; };
-    auto sWlo = [&](int s) { return base + s * CF::stage_bytes + 2 * A_TILE + W_TILE; };
+    auto sA = [&](int s) { return base + s * CF::stage_bytes; };
+    auto sW = [&](int s) { return base + s * CF::stage_bytes + A_TILE; };
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer ----------------
@@ -213,12 +208,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             mbar_expect_tx(full_bar(s), CF::stage_bytes);
             const int kc = kb * TK;
-            tma_load_2d(sAhi(s), &mAhi, kc, m0, full_bar(s));
-            tma_load_2d(sWhi(s), &mWhi, kc, n0, full_bar(s));
-            if (P == 3) {
-                tma_load_2d(sAlo(s), &mAlo, kc, m0, full_bar(s));
-                tma_load_2d(sWlo(s), &mWlo, kc, n0, full_bar(s));
-            }
+            tma_load_2d(sA(s), &mA, kc, m0, full_bar(s));
+            tma_load_2d(sW(s), &mW, kc, n0, full_bar(s));
             issued = kb + 1;
         }
         // drain: every stage armed so far must have landed before the CTA may exit
@@ -235,13 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int k = 0; k < TK / 16; ++k) {
                 const uint32_t koff = 32u * k;
-                const uint64_t ahi = sw128_desc(sAhi(s) + koff), whi = sw128_desc(sWhi(s) + koff);
-                mma_bf16<TN>(tmem, ahi, whi, (kb > 0 || k > 0) ? 1u : 0u);
-                if (P == 3) {
-                    const uint64_t alo = sw128_desc(sAlo(s) + koff), wlo = sw128_desc(sWlo(s) + koff);
-                    mma_bf16<TN>(tmem, alo, whi, 1u);
-                    mma_bf16<TN>(tmem, ahi, wlo, 1u);
-                }
+                mma_bf16<TN>(tmem, sw128_desc(sA(s) + koff), sw128_desc(sW(s) + koff), (kb > 0 || k > 0) ? 1u : 0u);
             }
             mma_commit(empty_bar(s));
         }
@@ -279,27 +264,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-template <int P, int EPI, int TN = 256>
-int launch(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo,
-           const __nv_bfloat16* Whi, const __nv_bfloat16* Wlo, const TcEpilogue& e, int* err) {
+template <int EPI, int TN>
+int launch(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* W, const TcEpilogue& e,
+           int* err) {
     static bool configured = false;
     if (!configured) {
-        BPM_CK(cudaFuncSetAttribute(k_gemm_tc<P, EPI, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    Cfg<P, TN, EPI>::smem));
+        BPM_CK(cudaFuncSetAttribute(k_gemm_tc<EPI, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    Cfg<TN, EPI>::smem));
         configured = true;
     }
-    CUtensorMap mAhi, mAlo, mWhi, mWlo;
-    BPM_TRY(make_bf16_tensor_map(&mAhi, Ahi, K, M, TM));
-    BPM_TRY(make_bf16_tensor_map(&mWhi, Whi, K, N, TN));
-    if (P == 3) {
-        BPM_TRY(make_bf16_tensor_map(&mAlo, Alo, K, M, TM));
-        BPM_TRY(make_bf16_tensor_map(&mWlo, Wlo, K, N, TN));
-    } else {
-        mAlo = mAhi;
-        mWlo = mWhi;
-    }
+    CUtensorMap mA, mW;
+    BPM_TRY(make_bf16_tensor_map(&mA, A, K, M, TM));
+    BPM_TRY(make_bf16_tensor_map(&mW, W, K, N, TN));
     dim3 grid((N + TN - 1) / TN, M / TM);
-    k_gemm_tc<P, EPI, TN><<<grid, kThreads, Cfg<P, TN, EPI>::smem, s>>>(mAhi, mAlo, mWhi, mWlo, M, N, K, e, err);
+    k_gemm_tc<EPI, TN><<<grid, kThreads, Cfg<TN, EPI>::smem, s>>>(mA, mW, M, N, K, e, err);
     BPM_CK(cudaGetLastError());
     return BPM_OK;
 }
@@ -373,21 +351,21 @@ int gemm_tc(cudaStream_t s, int epi, int M, int N, int K, const __nv_bfloat16* A
     switch (epi) {
         case TC_EPI_STORE:
             switch (tile_width(M, N, 256, 32, sm_count / 2)) {
-                case 256: return launch<1, TC_EPI_STORE, 256>(s, M, N, K, A, A, W, W, e, err_flag);
-                case 128: return launch<1, TC_EPI_STORE, 128>(s, M, N, K, A, A, W, W, e, err_flag);
-                case 64: return launch<1, TC_EPI_STORE, 64>(s, M, N, K, A, A, W, W, e, err_flag);
-                default: return launch<1, TC_EPI_STORE, 32>(s, M, N, K, A, A, W, W, e, err_flag);
+                case 256: return launch<TC_EPI_STORE, 256>(s, M, N, K, A, W, e, err_flag);
+                case 128: return launch<TC_EPI_STORE, 128>(s, M, N, K, A, W, e, err_flag);
+                case 64: return launch<TC_EPI_STORE, 64>(s, M, N, K, A, W, e, err_flag);
+                default: return launch<TC_EPI_STORE, 32>(s, M, N, K, A, W, e, err_flag);
             }
         case TC_EPI_BIAS_GELU:
             return tile_width(M, N, 128, 64, sm_count) == 128
-                       ? launch<1, TC_EPI_BIAS_GELU, 128>(s, M, N, K, A, A, W, W, e, err_flag)
-                       : launch<1, TC_EPI_BIAS_GELU, 64>(s, M, N, K, A, A, W, W, e, err_flag);
-        case TC_EPI_BIAS_OUT: return launch<1, TC_EPI_BIAS_OUT, 128>(s, M, N, K, A, A, W, W, e, err_flag);
+                       ? launch<TC_EPI_BIAS_GELU, 128>(s, M, N, K, A, W, e, err_flag)
+                       : launch<TC_EPI_BIAS_GELU, 64>(s, M, N, K, A, W, e, err_flag);
+        case TC_EPI_BIAS_OUT: return launch<TC_EPI_BIAS_OUT, 128>(s, M, N, K, A, W, e, err_flag);
         case TC_EPI_GELU_BWD:
             switch (tile_width(M, N, 256, 64, sm_count / 2)) {
-                case 256: return launch<1, TC_EPI_GELU_BWD, 256>(s, M, N, K, A, A, W, W, e, err_flag);
-                case 128: return launch<1, TC_EPI_GELU_BWD, 128>(s, M, N, K, A, A, W, W, e, err_flag);
-                default: return launch<1, TC_EPI_GELU_BWD, 64>(s, M, N, K, A, A, W, W, e, err_flag);
+                case 256: return launch<TC_EPI_GELU_BWD, 256>(s, M, N, K, A, W, e, err_flag);
+                case 128: return launch<TC_EPI_GELU_BWD, 128>(s, M, N, K, A, W, e, err_flag);
+                default: return launch<TC_EPI_GELU_BWD, 64>(s, M, N, K, A, W, e, err_flag);
             }
         default: set_error("unknown epilogue %d", epi); return BPM_ERR_ARG;
     }
