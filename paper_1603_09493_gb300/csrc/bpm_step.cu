@@ -90,11 +90,14 @@ __device__ __forceinline__ float3 trilinear(const StepArgs& a, float px, float p
     return acc;
 }
 
-// demag field of island b at node i: the planes of the product's K slices, added in order
+// demag field of island b at node i: the planes of the product's K slices, added in order.  PLANES false: for
+// one plane (the loads of four held registers and slots that the two-island predictor misses: 4096 islands
+// of 1547 nodes 157 us with them, 142 without)
+template <bool PLANES = true>
 __device__ __forceinline__ float3 load_hd(const StepArgs& a, int b, int i) {
     const float* hd = a.Hd + (size_t)b * a.kp + i;
     float3 v = f3(__ldcg(hd), __ldcg(hd + a.cp), __ldcg(hd + 2 * a.cp));
-    if (a.hd_planes > 1) {
+    if (PLANES && a.hd_planes > 1) {
         // at most four planes: all loads at once (a missing plane repeats the last and is dropped)
         float3 w[3];
 #pragma unroll
@@ -447,7 +450,7 @@ __device__ __forceinline__ void prepare_multi(const StepArgs& a, int nb, const f
 }
 
 // predictor of islands b0 .. b0 + nb - 1 (nb <= IPB); sp: [IPB][3] island parameters in smem
-template <int IPB, bool AHEAD = false>
+template <int IPB, bool AHEAD, bool PLANES>
 __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, float4* sp) {
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -473,7 +476,7 @@ __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, f
 #pragma unroll
         for (int q = 0; q < IPB; ++q) {
             mi[q] = f3(sm[wi + 32 * (3 * q)], sm[wi + 32 * (3 * q + 1)], sm[wi + 32 * (3 * q + 2)]);
-            hdv[q] = (mask & BPM_TERM_DEMAG) && q < nb ? load_hd(a, b0 + q, i) : f3(0, 0, 0);
+            hdv[q] = (mask & BPM_TERM_DEMAG) && q < nb ? load_hd<PLANES>(a, b0 + q, i) : f3(0, 0, 0);
         }
         const float4 pos = __ldg(a.node_pos + i);
         const float4 nm = __ldg(a.node_mat + i);
@@ -500,7 +503,7 @@ __device__ __forceinline__ void stage1_multi(const StepArgs& a, int b0, int j, f
 }
 
 // corrector and switch detectors of islands b0 .. b0 + nb - 1; red: [IPB][NT / 32]
-template <int IPB, bool AHEAD = false>
+template <int IPB, bool AHEAD, bool PLANES>
 __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, float4* sp, float* red) {
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -529,7 +532,7 @@ __device__ __forceinline__ void stage2_multi(const StepArgs& a, int b0, int j, f
 #pragma unroll
         for (int q = 0; q < IPB; ++q) {
             mi[q] = f3(sm[wi + 32 * (3 * q)], sm[wi + 32 * (3 * q + 1)], sm[wi + 32 * (3 * q + 2)]);
-            hdv[q] = (mask & BPM_TERM_DEMAG) && q < nb ? load_hd(a, b0 + q, i) : f3(0, 0, 0);
+            hdv[q] = (mask & BPM_TERM_DEMAG) && q < nb ? load_hd<PLANES>(a, b0 + q, i) : f3(0, 0, 0);
         }
         const float4 pos = __ldg(a.node_pos + i);
         const float4 nm = __ldg(a.node_mat + i);
@@ -677,40 +680,44 @@ constexpr int kMultiNT = 256, kMultiIPB = 2;
 // 4 CTAs (8 islands) per SM: up to 64 registers a thread; 2 x 18.8 KB of state per CTA at 1568 nodes
 constexpr int kMultiMinBlocks = 4;
 
+template <bool PLANES>
 __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_stage1m(StepArgs a, int j) {
     __shared__ float4 sp[3 * kMultiIPB];
-    stage1_multi<kMultiIPB>(a, kMultiIPB * blockIdx.x, j, sp);
+    stage1_multi<kMultiIPB, false, PLANES>(a, kMultiIPB * blockIdx.x, j, sp);
 }
+template <bool PLANES>
 __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_stage2m(StepArgs a, int j) {
     __shared__ float4 sp[3 * kMultiIPB];
     __shared__ float red[kMultiIPB * kMultiNT / 32];
-    stage2_multi<kMultiIPB>(a, kMultiIPB * blockIdx.x, j, sp, red);
+    stage2_multi<kMultiIPB, false, PLANES>(a, kMultiIPB * blockIdx.x, j, sp, red);
 }
+template <bool PLANES>
 __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_stage1m_groups(const __grid_constant__ StageGroups G,
                                                                              int j) {
     __shared__ float4 sp[3 * kMultiIPB];
     const int g = stage_group(G);
-    stage1_multi<kMultiIPB>(G.a[g], kMultiIPB * (blockIdx.x - G.block_begin[g]), j, sp);
+    stage1_multi<kMultiIPB, false, PLANES>(G.a[g], kMultiIPB * (blockIdx.x - G.block_begin[g]), j, sp);
 }
+template <bool PLANES>
 __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_stage2m_groups(const __grid_constant__ StageGroups G,
                                                                              int j) {
     __shared__ float4 sp[3 * kMultiIPB];
     __shared__ float red[kMultiIPB * kMultiNT / 32];
     const int g = stage_group(G);
-    stage2_multi<kMultiIPB>(G.a[g], kMultiIPB * (blockIdx.x - G.block_begin[g]), j, sp, red);
+    stage2_multi<kMultiIPB, false, PLANES>(G.a[g], kMultiIPB * (blockIdx.x - G.block_begin[g]), j, sp, red);
 }
 
 // the same behind a programmatic launch, for more islands than k_few holds at once; stage 1 or 2
-template <int STAGE>
+template <int STAGE, bool PLANES>
 __global__ void __launch_bounds__(kMultiNT, kMultiMinBlocks) k_few_pairs(const __grid_constant__ StageGroups G, int j) {
     __shared__ float4 sp[3 * kMultiIPB];
     __shared__ float red[kMultiIPB * kMultiNT / 32];
     const int g = stage_group(G);
     const int b0 = kMultiIPB * (blockIdx.x - G.block_begin[g]);
     if (STAGE == 1)
-        stage1_multi<kMultiIPB, true>(G.a[g], b0, j, sp);
+        stage1_multi<kMultiIPB, true, PLANES>(G.a[g], b0, j, sp);
     else
-        stage2_multi<kMultiIPB, true>(G.a[g], b0, j, sp, red);
+        stage2_multi<kMultiIPB, true, PLANES>(G.a[g], b0, j, sp, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -1029,6 +1036,24 @@ static int configure_few(int smem) {
     return BPM_OK;
 }
 
+template <bool PLANES>
+static int configure_multi(int smem, int smem_few) {
+    BPM_CK(cudaFuncSetAttribute(k_few_pairs<1, PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_few));
+    BPM_CK(cudaFuncSetAttribute(k_few_pairs<2, PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_few));
+    BPM_CK(cudaFuncSetAttribute(k_stage1m<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_stage2m<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_stage1m_groups<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BPM_CK(cudaFuncSetAttribute(k_stage2m_groups<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return BPM_OK;
+}
+
+// whether a group of a launch has its demag field in several planes
+static bool has_planes(const StageGroups& G) {
+    bool any = false;
+    for (int g = 0; g < G.ng; ++g) any = any || G.a[g].hd_planes > 1;
+    return any;
+}
+
 int configure_step_kernels() {
     int smem = (int)kMaxStageSmem;
     BPM_CK(cudaFuncSetAttribute(k_stage1<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -1050,15 +1075,11 @@ int configure_step_kernels() {
     BPM_CK(cudaFuncSetAttribute(k_stage2_groups<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int smem2 = kMultiIPB * smem;
     const int smem3 = std::min(2 * smem2, 200 * 1024);
-    BPM_CK(cudaFuncSetAttribute(k_few_pairs<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3));
-    BPM_CK(cudaFuncSetAttribute(k_few_pairs<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3));
+    BPM_TRY(configure_multi<false>(smem2, smem3));
+    BPM_TRY(configure_multi<true>(smem2, smem3));
     BPM_TRY(configure_few<256>(smem2));
     BPM_TRY(configure_few<512>(smem2));
     BPM_TRY(configure_few<1024>(smem2));
-    BPM_CK(cudaFuncSetAttribute(k_stage1m, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
-    BPM_CK(cudaFuncSetAttribute(k_stage2m, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
-    BPM_CK(cudaFuncSetAttribute(k_stage1m_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
-    BPM_CK(cudaFuncSetAttribute(k_stage2m_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     return BPM_OK;
 }
 
@@ -1089,8 +1110,12 @@ int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t
         size_t smem = 0;
         for (int g = 0; g < G.ng; ++g) smem = std::max(smem, 2 * kMultiIPB * stage_smem_bytes(G.a[g]));
         const dim3 grid(G.block_begin[G.ng]), block(kMultiNT);
-        BPM_CK(stage == 1 ? launch_pdl(k_few_pairs<1>, grid, block, smem, s, true, G, j)
-                          : launch_pdl(k_few_pairs<2>, grid, block, smem, s, true, G, j));
+        if (has_planes(G))
+            BPM_CK(stage == 1 ? launch_pdl(k_few_pairs<1, true>, grid, block, smem, s, true, G, j)
+                              : launch_pdl(k_few_pairs<2, true>, grid, block, smem, s, true, G, j));
+        else
+            BPM_CK(stage == 1 ? launch_pdl(k_few_pairs<1, false>, grid, block, smem, s, true, G, j)
+                              : launch_pdl(k_few_pairs<2, false>, grid, block, smem, s, true, G, j));
         return BPM_OK;
     }
     return threads == 1024  ? launch_few_nt<1024>(G, stage, j, s)
@@ -1101,8 +1126,8 @@ int launch_few(const StageGroups& G, int threads, int stage, int j, cudaStream_t
 int stage_blocks_per_sm(int threads, int ipb, size_t smem, int* blocks) {
     int b1 = 0, b2 = 0;
     if (ipb == kMultiIPB) {
-        BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_stage1m_groups, kMultiNT, smem));
-        BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_stage2m_groups, kMultiNT, smem));
+        BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_stage1m_groups<true>, kMultiNT, smem));
+        BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_stage2m_groups<true>, kMultiNT, smem));
     } else if (threads == 128) {
         BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_stage1_groups<128>, 128, smem));
         BPM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_stage2_groups<128>, 128, smem));
@@ -1122,7 +1147,7 @@ int stage_islands_per_cta(const StepArgs& a) { return a.ipb == kMultiIPB ? kMult
 void launch_stage1(const StepArgs& a, int j, cudaStream_t s) {
     const size_t sm = stage_smem_bytes(a);
     if (a.ipb == kMultiIPB)
-        k_stage1m<<<(a.B + kMultiIPB - 1) / kMultiIPB, kMultiNT, kMultiIPB * sm, s>>>(a, j);
+        (a.hd_planes > 1 ? k_stage1m<true> : k_stage1m<false>)<<<(a.B + kMultiIPB - 1) / kMultiIPB, kMultiNT, kMultiIPB * sm, s>>>(a, j);
     else if (a.threads == 128)
         k_stage1<128><<<a.B, 128, sm, s>>>(a, j);
     else if (a.threads == 512)
@@ -1133,7 +1158,7 @@ void launch_stage1(const StepArgs& a, int j, cudaStream_t s) {
 void launch_stage2(const StepArgs& a, int j, cudaStream_t s) {
     const size_t sm = stage_smem_bytes(a);
     if (a.ipb == kMultiIPB)
-        k_stage2m<<<(a.B + kMultiIPB - 1) / kMultiIPB, kMultiNT, kMultiIPB * sm, s>>>(a, j);
+        (a.hd_planes > 1 ? k_stage2m<true> : k_stage2m<false>)<<<(a.B + kMultiIPB - 1) / kMultiIPB, kMultiNT, kMultiIPB * sm, s>>>(a, j);
     else if (a.threads == 128)
         k_stage2<128><<<a.B, 128, sm, s>>>(a, j);
     else if (a.threads == 512)
@@ -1144,7 +1169,7 @@ void launch_stage2(const StepArgs& a, int j, cudaStream_t s) {
 void launch_stage1_groups(const StageGroups& G, int threads, size_t smem, int j, cudaStream_t s) {
     const int blocks = G.block_begin[G.ng];
     if (G.a[0].ipb == kMultiIPB)
-        k_stage1m_groups<<<blocks, kMultiNT, smem, s>>>(G, j);
+        (has_planes(G) ? k_stage1m_groups<true> : k_stage1m_groups<false>)<<<blocks, kMultiNT, smem, s>>>(G, j);
     else if (threads == 128)
         k_stage1_groups<128><<<blocks, 128, smem, s>>>(G, j);
     else if (threads == 512)
@@ -1155,7 +1180,7 @@ void launch_stage1_groups(const StageGroups& G, int threads, size_t smem, int j,
 void launch_stage2_groups(const StageGroups& G, int threads, size_t smem, int j, cudaStream_t s) {
     const int blocks = G.block_begin[G.ng];
     if (G.a[0].ipb == kMultiIPB)
-        k_stage2m_groups<<<blocks, kMultiNT, smem, s>>>(G, j);
+        (has_planes(G) ? k_stage2m_groups<true> : k_stage2m_groups<false>)<<<blocks, kMultiNT, smem, s>>>(G, j);
     else if (threads == 128)
         k_stage2_groups<128><<<blocks, 128, smem, s>>>(G, j);
     else if (threads == 512)

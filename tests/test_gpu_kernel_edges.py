@@ -437,3 +437,33 @@ def test_groups_of_whole_tiles_have_the_bits_of_their_own_batches(ctx, sizes):
         assert np.abs(s - m).max() > 1e-3                                 # the islands have moved
     for mid in mids:
         ctx.mesh_release(mid)
+
+
+@pytest.mark.parametrize("sizes", [(900, 700, 60), (1500, 1, 400), (1200,)])
+def test_stages_of_one_plane_and_of_several(ctx, sizes):
+    """Batches beyond the few islands on the two-island stage kernels, with a group of at most 128 islands (whose field
+    comes in a plane per slice of K, in every stage launch that holds one) and without: states of each group bitwise
+    those of parts of 100 islands in batches of their own, which are of few islands."""
+    from paper_1603_09493_gb300 import _lib as L
+    from paper_1603_09493_gb300 import synth
+    meshes = [synth.small_island_mesh(), synth.layered_island_mesh(7.0, 6.0, 4.0, rings=2, hard_slabs=9, soft_slabs=6, seed=5),
+              synth.layered_island_mesh(6.0, 5.0, 3.0, rings=2, hard_slabs=7, soft_slabs=4, seed=6)]
+    mids = [ctx.mesh_upload(m, synth.ecc_materials()) for m in meshes[:len(sizes)]]
+    parts = [synth.jittered_islands(b, seed=b, mesh_id=m) for b, m in zip(sizes, mids)]
+    p = synth.RunParams(dt_ps=0.1, alpha=0.1, rise_ps=1.0, substeps=4, uniform_T=synth.uniform_field(0.9, 170.0))
+
+    def run(isl):
+        with ctx.batch(isl, p, precision=L.PREC_BF16X3) as bt:
+            bt.advance(10)
+            return bt.read()["m"]
+
+    out, at = run(synth.Islands.concat(parts)), 0
+    assert np.abs(out[:, :2]).max() > 1e-2                                # the islands have moved
+    for isl, mesh in zip(parts, meshes):
+        n = mesh.n_nodes
+        for q in range(0, len(isl), 100):
+            rows = np.arange(q, min(q + 100, len(isl)))
+            assert np.array_equal(run(isl.subset(rows))[:, :, :n], out[at + rows][:, :, :n])
+        at += len(isl)
+    for m in mids:
+        ctx.mesh_release(m)
