@@ -246,13 +246,14 @@ int setup_grouped_gemm(bpm_batch* bt) {
 // SM, two islands a CTA (they share the exchange entries) for at most three pairs and 2000 nodes of pairs an
 // SM (one pair an SM of any mesh).  Beyond that the two-island kernels on two streams are as fast.  An
 // interval in us, this way / two streams, alone and with three batches in turn on as many streams (each a
-// pass): 1547 nodes, 128 islands 2020 / 3900 and 1820 / 1980, 304 islands 4850 / 5600 and 2650 / 2750; 481
-// nodes, 300 islands 522 / 603 and 219 / 224, 600 islands 606 / 647 and 289 / 281; 209 nodes, 800 islands
-// 343 / 411 and 181 / 177, 1200 islands 470 / 432 and 245 / 220.  One mesh at one island a CTA and two or
-// more an SM: 481 nodes, 300 islands 535 and 262; 209 nodes, 600 islands 367 and 193 (pairs 344 and 152).
+// pass): 1547 nodes, 128 islands 1770 / 3110 and 1630 / 1790, 304 islands 4700 / 5300 and 2600 / 2610; 481
+// nodes, 300 islands 485 / 515 and 208 / 198, 600 islands 557 / 609 and 272 / 269; 209 nodes, 800 islands
+// 309 / 393 and 171 / 163; 1200 islands were slower both ways (470 / 432 and 245 / 220, before the product took
+// its present form).  One mesh at one island a CTA and two or more an SM: 481 nodes, 300 islands 501 and 252;
+// 209 nodes, 600 islands 336 and 181 (pairs 313 and 144).
 // Several meshes of over 512 nodes do stay at one island a CTA up to 3200 nodes an SM: their groups are
 // small and sliced, and a pair's 256 threads take four passes over 1000 nodes (518 and 976 nodes, 120
-// islands each: 1410 and 1240, pairs 2620 and 1450).
+// islands each: 1295 and 1144, pairs 2490 and 1345).
 bool few_islands(const bpm_batch* bt, StageGroups* G, int* threads) {
     if (!tensor_core_precision(bt) || bt->pair || bt->groups.size() > kMaxStageGroups) return false;
     const int sms = bt->ctx->sm_count;

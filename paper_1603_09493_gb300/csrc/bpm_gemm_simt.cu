@@ -18,8 +18,8 @@ constexpr int BM = 128, BN = 128, BK = 8;
 // warps take the fours of k in turn: an output has four sums, added at the end, and nothing is shuffled
 // into pairs.  A warp holds TM rows of A (its loads are broadcasts) by 32 TN rows of W; rows of 36 words
 // put the eight rows of a quarter warp's load in distinct banks.
-// The bound is the FP32 FMA rate (80 TFLOP/s).  64 x 128 outputs of 2 x 8 warps: 200 rows of a 4736 x
-// 4736 operator are 148 CTAs, one an SM, 0.27 ms (0.32 with one group: two warps a scheduler do not
+// The bound is the FP32 FMA rate (80 TFLOP/s).  64 x 128 outputs of 2 x 8 warps: 200 rows of a 4672 x
+// 4672 operator are 148 CTAs, one an SM, 0.29 ms (0.32 with one group: two warps a scheduler do not
 // cover the FMAs' latency; 1.04 with 128 x 128 tiles, 74 CTAs, and scalar loads and FMAs).  Up to 32 rows
 // take 16 x 32 tiles, so that their few rows still give every SM a CTA.  The sum of an output does not
 // depend on the tile.
