@@ -272,9 +272,10 @@ __global__ void __launch_bounds__(kGThreads, 1)
             float* dst = gg.C + (size_t)sl * gg.plane + (size_t)(b0 + h0) * gg.ldc + row;
 #pragma unroll
             for (int c = 0; c < NC; ++c)
+                if (16 * c < nv)                            // (one island: 16 guarded stores, not all)
 #pragma unroll
-                for (int v = 0; v < 16; ++v)
-                    if (16 * c + v < nv) dst[(size_t)(16 * c + v) * gg.ldc] = sum[c][v];
+                    for (int v = 0; v < 16; ++v)
+                        if (16 * c + v < nv) dst[(size_t)(16 * c + v) * gg.ldc] = sum[c][v];
         }
     }
     __syncwarp();
