@@ -119,10 +119,10 @@ def gemm_peak(pk):
 # (dram__bytes_read.sum + dram__bytes_write.sum, mean of two launches), keyed by
 # (precision, islands, nodes) of the captured workload:
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum \
-#       --clock-control none -k regex:k_gemm_grouped -s 10 -c 2 --csv \
-#       python bench.py --steps 2 --warmup 1 --no-cpu --no-e2e --no-extras --no-autotune
-# (k_gemm_grouped<3,256,32>, N-major tile order).  Remove an entry when the kernel changes.
-NCU_GEMM_TRAFFIC = {(1, 4096, 1547): 412.97e6 + 60.92e6}
+#       --clock-control none -k regex:k_gemm_ -s 3 -c 2 --csv python -c "..."
+# on Batch.kernel_times of the census batch (profiles/demag_gemm_grouped_census_2048.md;
+# k_gemm_grouped<3,256,32>, N-major tile order).  Remove an entry when the kernel changes.
+NCU_GEMM_TRAFFIC = {(1, 4096, 1547): 397.32e6 + 61.01e6}
 
 
 def gemm_traffic(prec, B, n):
@@ -131,9 +131,9 @@ def gemm_traffic(prec, B, n):
 
 # Warp instructions per island-node of the Heun stage kernels (two islands per CTA, BF16x3
 # operand) from ncu's smsp__inst_executed.sum of one launch over the 1024 islands of one chain
-# (2048 islands, two chains) of the 1547-node mesh (profiles/heun_stages_census_2048.md: 24.30 M
-# and 26.87 M).  Remove when the kernels change.
-NCU_STAGE_WARP_INSTR = {1547: (24.30e6 / (1024 * 1547), 26.87e6 / (1024 * 1547))}
+# (2048 islands, two chains) of the 1547-node mesh (profiles/heun_stages_census_2048.md: 24.19 M
+# and 26.55 M).  Remove when the kernels change.
+NCU_STAGE_WARP_INSTR = {1547: (24.19e6 / (1024 * 1547), 26.55e6 / (1024 * 1547))}
 SM_COUNT = 152
 ISSUE_PER_SM_CLK = 4           # one warp instruction per scheduler per cycle, four schedulers per SM
 

@@ -287,8 +287,9 @@ int gp_factor(cudaStream_t s, const double* X, const double* y, int n, int d, co
     return BPM_OK;
 }
 
-// Block row i0 .. i0 + 31 of Linv = L^-1 (L: [n + 2][n] below its diagonal blocks, which are D): 32 columns a CTA, products of the block rows
-// above (in the order of k) first, then the triangular solve within the block; Linv_ij = -s / L_ii.
+// Block row i0 .. i0 + 31 of Linv = L^-1 (L: [n + 2][n] below its diagonal blocks, which are D): 32 columns
+// a CTA, products of the block rows above (in the order of k) first, then the triangular solve within the
+// block; Linv_ij = -s / L_ii.
 // (One thread per column walked the whole triangle: 0.81 ms at n = 160; 0.26 ms now.)
 __global__ void __launch_bounds__(kGpThreads) k_gp_linv(const double* __restrict__ L,
                                                         const double* __restrict__ D, int n, int i0,
